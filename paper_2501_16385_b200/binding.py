@@ -1,8 +1,9 @@
-"""ctypes binding of libfbq.so.  Argument marshalling only.
+"""Binding of libfbq.so.  Argument marshalling only.
 
 Tensors are torch CUDA tensors (PyTorch supplies device memory and streams);
 their data pointers and the current stream's handle are passed straight to the
-C ABI declared in include/fbq.h.
+C ABI declared in include/fbq.h: by the native module _fbq_torch for the calls
+of a decode loop, through ctypes for the rest.
 """
 from __future__ import annotations
 
@@ -16,6 +17,7 @@ STATUS = {0: "FBQ_OK", -1: "FBQ_ERR_BADARG", -2: "FBQ_ERR_UNSUPPORTED", -3: "FBQ
           -4: "FBQ_ERR_CUDA", -5: "FBQ_ERR_TIMEOUT"}
 
 _lib = None
+_native = None
 
 
 class FbqError(RuntimeError):
@@ -74,6 +76,22 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def native():
+    """The module _fbq_torch (csrc/fbq_torch.cpp), which marshals the calls of a decode loop."""
+    global _native
+    if _native is None:
+        import torch  # noqa: F401  (its libraries have to be in the process first)
+        lib()
+        if not os.path.exists(_build.TORCH_LIB):
+            _build.build()
+        import importlib.util
+        spec = importlib.util.spec_from_file_location("_fbq_torch", _build.TORCH_LIB)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        _native = mod
+    return _native
+
+
 def _check(code: int, where: str) -> None:
     if code != 0:
         raise FbqError(code, where)
@@ -125,21 +143,10 @@ def dequant(qweight, scales, zeros, N: int, K: int, group: int, bits: int, strea
 def linear(x, qweight, scales, zeros, A, B, N: int, group: int, bits: int, y=None, stream=None):
     """fbq_linear (fp16 x) or fbq_linear_bf16 (bf16 x).  x: [M, K]; A: [rank, K] or None;
     B: [N, rank] or None.  Returns y [M, N] in the dtype of x."""
-    import torch
-    assert x.is_cuda and x.is_contiguous() and x.dim() == 2
-    M, K = x.shape
-    rank = 0 if A is None else A.shape[0]
-    if y is None:
-        y = torch.empty((M, N), dtype=x.dtype, device=x.device)
-    if x.dtype == torch.float16:
-        fn, name = lib().fbq_linear, "fbq_linear"
-    elif x.dtype == torch.bfloat16:
-        fn, name = lib().fbq_linear_bf16, "fbq_linear_bf16"
-    else:
-        raise TypeError("x must be float16 or bfloat16")
-    _check(fn(_ptr(x), _ptr(qweight), _ptr(scales), _ptr(zeros), _ptr(A), _ptr(B), _ptr(y),
-              M, N, K, group, bits, rank, _stream(stream)), name)
-    return y
+    r = (_native or native()).linear(x, qweight, scales, zeros, A, B, N, group, bits, y, stream)
+    if r.__class__ is int:
+        raise FbqError(r, "fbq_linear" if str(x.dtype) == "torch.float16" else "fbq_linear_bf16")
+    return r
 
 
 def linear_hostio(x_host, qweight, scales, zeros, A, B, y_host, N: int, group: int, bits: int,
@@ -249,8 +256,7 @@ def linear_batch(problems, group: int, bits: int, stream=None, batch=None, host_
     descriptor array made earlier by make_batch (``batch``).  The y tensors are written.  With
     host_io the x and y tensors are (pinned) CPU tensors: fbq_linear_batch_hostio."""
     arr, n, M, rank, bf16 = batch if batch is not None else make_batch(problems)
-    fn = lib().fbq_linear_batch_hostio if host_io else lib().fbq_linear_batch
-    _check(fn(arr, n, M, group, bits, rank, bf16, _stream(stream)), "fbq_linear_batch")
+    _check((_native or native()).linear_batch(ctypes.addressof(arr), n, M, group, bits, rank, bf16, host_io, stream), "fbq_linear_batch")
 
 
 def select_kernel(M, N, K, group, bits, rank, bf16=False) -> int:

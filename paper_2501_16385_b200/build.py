@@ -1,4 +1,5 @@
-"""Builds libfbq.so (CUDA kernels + C ABI) in-tree with nvcc for sm_100a.
+"""Builds libfbq.so (CUDA kernels + C ABI) in-tree with nvcc for sm_100a, and beside it
+_fbq_torch.so, the native part of the Python binding (g++, torch's headers).
 
 Every source file is compiled to an object of its own (in parallel, and only
 when it or a header changed), then the objects are linked into the shared
@@ -16,7 +17,9 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libfbq.so")
-SOURCES = ["fbq_api.cu", "fbq_pack.cu", "fbq_generic.cu", "fbq_decode.cu", "fbq_gemv.cu", "fbq_prefill.cu", "fbq_noalloc.cu",
+TORCH_SRC = "fbq_torch.cpp"
+TORCH_LIB = os.path.join(HERE, "_fbq_torch.so")
+SOURCES = ["fbq_api.cu", "fbq_maps.cu", "fbq_pack.cu", "fbq_generic.cu", "fbq_decode.cu", "fbq_gemv.cu", "fbq_prefill.cu", "fbq_noalloc.cu",
            "fbq_quant.cu", "fbq_reconstruct.cu"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 COMPILE_FLAGS = ARCH + ["-lineinfo", "-O3", "-std=c++17", "-Xptxas=-v", "-Xcompiler", "-fPIC", "-rdc=false"]
@@ -42,12 +45,31 @@ def _stale_obj(src: str, force: bool) -> bool:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(TORCH_LIB):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(TORCH_LIB))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
     deps.append(os.path.join(HERE, "..", "include", "fbq.h"))
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _build_binding() -> None:
+    import sysconfig
+
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    inc = include_paths() + [sysconfig.get_paths()["include"], "/usr/local/cuda/include"]
+    tmp = TORCH_LIB + ".tmp%d" % os.getpid()
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi()]
+    cmd += [f for d in inc for f in ("-isystem", d)] + [os.path.join(CSRC, TORCH_SRC), "-o", tmp]
+    # torch's libraries are in the process before the module is imported; libfbq.so is found beside it
+    cmd += ["-L" + os.path.join(os.path.dirname(torch.__file__), "lib"), "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10", "-lc10_cuda"]
+    cmd += ["-L" + HERE, "-l:libfbq.so", "-Wl,-rpath,$ORIGIN"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("g++ failed building _fbq_torch.so")
+    os.replace(tmp, TORCH_LIB)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -80,6 +102,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if res.returncode != 0:
         raise RuntimeError("nvcc failed linking libfbq.so")
     os.replace(tmp, LIB)
+    if force or not os.path.exists(TORCH_LIB) or any(os.path.getmtime(d) > os.path.getmtime(TORCH_LIB)
+                                                     for d in (os.path.join(CSRC, TORCH_SRC), os.path.join(HERE, "..", "include", "fbq.h"))):
+        _build_binding()
+    else:
+        os.utime(TORCH_LIB)
     return LIB
 
 

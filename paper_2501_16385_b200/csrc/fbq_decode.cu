@@ -34,15 +34,13 @@
 // worst, handed to the warp that completes t: then nothing spins on another
 // CTA.  All waits are bounded.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 
 #include <cstdio>
 #include <cstdlib>
-#include <mutex>
 #include <type_traits>
-#include <vector>
 
 #include "fbq_common.cuh"
+#include "fbq_maps.h"
 
 #ifndef FBQ_NACC
 #define FBQ_NACC 2
@@ -1928,7 +1926,8 @@ Plan make_plan(const LinearArgs &a, const DecodeTuning &tune)
         for (int sk = 1; sk <= min(G, 4) && !pl.ok; ++sk) pl.ok = either(sk, kSmemBudget);
         for (int sk = 1; sk <= G && !pl.ok; ++sk) pl.ok = either(sk, kSmemMax);
     }
-    if (getenv("FBQ_PLAN"))
+    static const bool print_plans = getenv("FBQ_PLAN") != nullptr;
+    if (print_plans)
         fprintf(stderr, "plan M %d N %d K %d r %d: ok %d SK %d R %d CHG %d NS %d nbuf %d a_cap %d b_rows %d smem %zu (meta %d x %d ring@%d) i8 %d heavy %d alias %d n_t %d\n", a.M, a.N, a.K,
                 a.rank, (int)pl.ok, pl.SK, pl.R, pl.CHG, pl.NS, pl.nbuf, pl.a_cap, pl.b_cap_rows, pl.smem, pl.off_x - pl.off_meta,
                 pl.off_px - pl.off_x, pl.off_ring, (int)pl.i8, (int)pl.heavy, pl.ab_alias, pl.n_t);
@@ -1952,49 +1951,18 @@ Plan make_plan(const LinearArgs &a, const DecodeTuning &tune)
 
 // 3-D tensor map of the packed codes for the weight stream: (word in group, weight row, group), boxes of
 // one group's words x 16 rows x CHG groups, which land in shared memory as [group][row][GB bytes].
-// Encoding takes a microsecond or two on the host, so the last maps are kept (they depend on the
-// weights' address and the plan only).
-struct MapKey {
-    const void *qw;
-    int N, G, bits, chg;
-    bool operator==(const MapKey &o) const { return qw == o.qw && N == o.N && G == o.G && bits == o.bits && chg == o.chg; }
-};
 cudaError_t weight_map(CUtensorMap *map, const LinearArgs &a, const Plan &pl)
 {
-    static std::mutex mu;
-    static std::vector<std::pair<MapKey, CUtensorMap>> cache;
-    static size_t next = 0;
-    static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-    const MapKey key{a.qw, a.N, a.K / kGroupFast, a.bits, pl.CHG};
-    std::lock_guard<std::mutex> lk(mu);
-    for (const auto &e : cache)
-        if (e.first == key) {
-            *map = e.second;
-            return cudaSuccess;
-        }
-    if (!encode) {
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
-        if (e != cudaSuccess) return e;
-        if (qres != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-        encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
-    const cuuint32_t wpg = (a.bits == 4) ? 16 : 12;
-    const cuuint64_t dims[3] = {wpg, (cuuint64_t)a.N, (cuuint64_t)key.G};
-    const cuuint64_t strides[2] = {(cuuint64_t)key.G * wpg * 4, (cuuint64_t)wpg * 4};
-    const cuuint32_t box[3] = {wpg, (cuuint32_t)kTileRows, (cuuint32_t)pl.CHG};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    if (encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<uint32_t *>(a.qw), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    constexpr size_t kKeep = 256;
-    if (cache.size() < kKeep)
-        cache.emplace_back(key, *map);
-    else
-        cache[next++ % kKeep] = std::make_pair(key, *map);
-    return cudaSuccess;
+    const int wpg = (a.bits == 4) ? 16 : 12, G = a.K / kGroupFast;
+    MapSpec m{};
+    m.base = a.qw;
+    m.type = CU_TENSOR_MAP_DATA_TYPE_UINT32;
+    m.ndim = 3;
+    m.dims[0] = (cuuint64_t)wpg; m.dims[1] = (cuuint64_t)a.N; m.dims[2] = (cuuint64_t)G;
+    m.strides[0] = (cuuint64_t)G * wpg * 4; m.strides[1] = (cuuint64_t)wpg * 4;
+    m.box[0] = (cuuint32_t)wpg; m.box[1] = (cuuint32_t)kTileRows; m.box[2] = (cuuint32_t)pl.CHG;
+    m.swizzle = CU_TENSOR_MAP_SWIZZLE_NONE;
+    return cached_map(map, m);
 }
 
 template <int BITS, typename T, int MT, bool HEAVY, bool I8>

@@ -28,15 +28,14 @@
 // partial t to scratch; an arrival counter tells the main CTAs' epilogue warps when all chunks are
 // there (bounded polling; FBQ_ERR_TIMEOUT instead of a hang), which then add the chunks in order.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 
 #include <cstdio>
 #include <cstdlib>
-#include <mutex>
+#include <cstring>
 #include <type_traits>
-#include <vector>
 
 #include "fbq_common.cuh"
+#include "fbq_maps.h"
 #include "fbq_ptx.cuh"
 
 namespace fbq {
@@ -1735,6 +1734,12 @@ struct Plan {
 int g_sm_count = 0;
 constexpr size_t kSmemMax = 227 * 1024;
 
+bool print_plans()
+{
+    static const bool on = getenv("FBQ_PLAN") != nullptr;
+    return on;
+}
+
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Fewer t CTAs (two blocks per warp, chunks of A up to 192 KB) where that saves every main CTA a tile: the main
@@ -1844,7 +1849,7 @@ Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
     p.poll_limit = tune.poll_limit > 0 ? (uint32_t)tune.poll_limit : (1u << 20);
     p.test_skip_arrive = tune.test_skip_arrive;
     pl.ok = true;
-    if (getenv("FBQ_PLAN"))
+    if (print_plans())
         fprintf(stderr, "gemv plan M %d N %d K %d r %d: n_main %d n_t %d (t_kb %d) NS %d nmeta %d nbuf %d nb %d smem %zu (t CTA %zu)\n",
                 a.M, a.N, a.K, a.rank, p.n_main, p.n_t, p.t_kb, p.NS, p.nmeta, p.nbuf, p.nb, need, need_t);
     return pl;
@@ -1956,54 +1961,31 @@ Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
     p.poll_limit = tune.poll_limit > 0 ? (uint32_t)tune.poll_limit : (1u << 20);
     p.test_skip_arrive = tune.test_skip_arrive;
     pl.ok = true;
-    if (getenv("FBQ_PLAN"))
+    if (print_plans())
         fprintf(stderr, "gemv wide plan M %d N %d K %d r %d: R %d SK %d (slice %d groups) n_t %d NS %d nmeta %d nbuf %d nb %d smem %zu (t CTA %zu)\n",
                 a.M, a.N, a.K, a.rank, p.R, p.SK, p.slice_groups, p.n_t, p.NS, p.nmeta, p.nbuf, p.nb, need, need_t);
     return pl;
 }
 
-// Tensor maps are encoded on the host once per (pointer, shape) and kept: they hold addresses and
-// extents only, never data.
-struct MapKey {
-    const void *ptr;
-    int kind, d0, d1, d2, b0, b1;
-    bool operator==(const MapKey &o) const
-    {
-        return ptr == o.ptr && kind == o.kind && d0 == o.d0 && d1 == o.d1 && d2 == o.d2 && b0 == o.b0 && b1 == o.b1;
-    }
-};
-PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-std::mutex g_map_mu;
-std::vector<std::pair<MapKey, CUtensorMap>> g_maps;
-size_t g_map_next = 0;
-
-cudaError_t cached_map(CUtensorMap *out, const MapKey &key, CUtensorMapDataType dt, int ndim, const cuuint64_t *dims,
-                       const cuuint64_t *strides, const cuuint32_t *box, CUtensorMapSwizzle swz_mode)
+// A plan is a function of the shape and the tuning alone and a call needs it twice (scratch, launch): the host thread
+// keeps the plans of the shapes it met last (a decoder has three or four).
+const Plan &plan_for(const LinearArgs &a, const GemvTuning &tune)
 {
-    std::lock_guard<std::mutex> lk(g_map_mu);
-    for (const auto &e : g_maps)
-        if (e.first == key) {
-            *out = e.second;
-            return cudaSuccess;
-        }
-    if (!g_encode) {
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
-        if (e != cudaSuccess) return e;
-        if (qres != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-        g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+    struct Entry {
+        int key[8] = {-1};
+        Plan plan;
+    };
+    static thread_local Entry table[16];
+    const int key[8] = {a.M, a.N, a.K, a.bits, a.rank, tune.max_ctas, tune.poll_limit, tune.test_skip_arrive};
+    unsigned h = 0;
+    for (int k : key) h = (h ^ (unsigned)k) * 0x9E3779B1u;
+    Entry &e = table[h >> 28];
+    if (memcmp(e.key, key, sizeof key) != 0) {
+        e.plan = a.M > 2 ? make_plan_wide(a, tune) : make_plan(a, tune);
+        memcpy(e.key, key, sizeof key);
+        if (!e.plan.ok) e.key[0] = -1;            // not kept: asked again
     }
-    const cuuint32_t estr[3] = {1, 1, 1};
-    if (g_encode(out, dt, ndim, const_cast<void *>(key.ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz_mode,
-                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    constexpr size_t kKeep = 1024;
-    if (g_maps.size() < kKeep)
-        g_maps.emplace_back(key, *out);
-    else
-        g_maps[g_map_next++ % kKeep] = std::make_pair(key, *out);
-    return cudaSuccess;
+    return e.plan;
 }
 
 template <int BITS, typename T, int MT>
@@ -2093,7 +2075,7 @@ bool gemv_supported(const LinearArgs &a)
 void gemv_workspace_need(const LinearArgs &a, const GemvTuning &tune, size_t *tpart_floats, int *counters, size_t *partial_floats)
 {
     const bool wide = a.M > 2;
-    const Plan pl = wide ? make_plan_wide(a, tune) : make_plan(a, tune);
+    const Plan &pl = plan_for(a, tune);
     *tpart_floats = (size_t)(std::max(pl.p.n_t, 1) + 1) * std::max(pl.p.slot_elems, 32);
     *counters = 8 + (wide ? pl.p.NT : 0);
     *partial_floats = (wide && pl.p.SK > 1) ? (size_t)pl.p.NT * pl.p.SK * a.M * kTile : 0;
@@ -2102,7 +2084,7 @@ void gemv_workspace_need(const LinearArgs &a, const GemvTuning &tune, size_t *tp
 cudaError_t launch_gemv(const LinearArgs &a, Workspace &ws, const GemvTuning &tune, cudaStream_t s, int *launches)
 {
     const bool wide = a.M > 2;
-    Plan pl = wide ? make_plan_wide(a, tune) : make_plan(a, tune);
+    Plan pl = plan_for(a, tune);
     if (!pl.ok) return cudaErrorInvalidConfiguration;
     GemvParams &p = pl.p;
     p.x = a.x; p.scales = a.scales; p.zeros = a.zeros; p.y = a.y;
@@ -2120,30 +2102,24 @@ cudaError_t launch_gemv(const LinearArgs &a, Workspace &ws, const GemvTuning &tu
     }
     CUtensorMap wmap, bmap, amap;
     {
-        const cuuint32_t wpg = (a.bits == 4) ? 16 : 12;
-        const cuuint64_t dims[3] = {wpg, (cuuint64_t)a.N, (cuuint64_t)p.G};
-        const cuuint64_t strides[2] = {(cuuint64_t)p.G * wpg * 4, (cuuint64_t)wpg * 4};
-        const int chg = wide ? kCHGW : kCHG;
-        const cuuint32_t box[3] = {wpg, (cuuint32_t)kTile, (cuuint32_t)chg};
-        const MapKey key{a.qw, 0, (int)wpg, a.N, p.G, kTile, chg};
-        if (cudaError_t e = cached_map(&wmap, key, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
-            e != cudaSuccess)
-            return e;
+        const int wpg = (a.bits == 4) ? 16 : 12;
+        MapSpec m{};
+        m.base = a.qw;
+        m.type = CU_TENSOR_MAP_DATA_TYPE_UINT32;
+        m.ndim = 3;
+        m.dims[0] = (cuuint64_t)wpg; m.dims[1] = (cuuint64_t)a.N; m.dims[2] = (cuuint64_t)p.G;
+        m.strides[0] = (cuuint64_t)p.G * wpg * 4; m.strides[1] = (cuuint64_t)wpg * 4;
+        m.box[0] = (cuuint32_t)wpg; m.box[1] = (cuuint32_t)kTile; m.box[2] = (cuuint32_t)(wide ? kCHGW : kCHG);
+        m.swizzle = CU_TENSOR_MAP_SWIZZLE_NONE;
+        if (cudaError_t e = cached_map(&wmap, m); e != cudaSuccess) return e;
     }
     bmap = wmap;
     amap = wmap;
     if (a.rank > 0) {
-        const cuuint64_t bd[2] = {(cuuint64_t)a.rank, (cuuint64_t)a.N}, bs[1] = {(cuuint64_t)a.rank * 2};
-        const cuuint32_t bb[2] = {(cuuint32_t)p.b_box_cols, (cuuint32_t)kTile};
         const CUtensorMapSwizzle sw = p.b_swz == 7 ? CU_TENSOR_MAP_SWIZZLE_128B : (p.b_swz == 3 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
         const CUtensorMapDataType dt = a.bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-        if (cudaError_t e = cached_map(&bmap, MapKey{a.B, 1, a.rank, a.N, a.bf16, p.b_box_cols, kTile}, dt, 2, bd, bs, bb, sw); e != cudaSuccess)
-            return e;
-        const cuuint64_t ad[2] = {(cuuint64_t)a.K, (cuuint64_t)a.rank}, as[1] = {(cuuint64_t)a.K * 2};
-        const cuuint32_t ab[2] = {(cuuint32_t)kTKB, (cuuint32_t)a.rank};
-        if (cudaError_t e = cached_map(&amap, MapKey{a.A, 2, a.K, a.rank, a.bf16, kTKB, a.rank}, dt, 2, ad, as, ab, CU_TENSOR_MAP_SWIZZLE_128B);
-            e != cudaSuccess)
-            return e;
+        if (cudaError_t e = cached_map(&bmap, matrix_map(a.B, dt, 2, a.rank, a.N, p.b_box_cols, kTile, sw)); e != cudaSuccess) return e;
+        if (cudaError_t e = cached_map(&amap, matrix_map(a.A, dt, 2, a.K, a.rank, kTKB, a.rank, CU_TENSOR_MAP_SWIZZLE_128B)); e != cudaSuccess) return e;
     }
     const bool pdl = tune.pdl != 0;
     cudaError_t e = cudaErrorInvalidConfiguration;

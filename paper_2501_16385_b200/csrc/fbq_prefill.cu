@@ -49,9 +49,9 @@
 // All waits are bounded: a wait that runs out raises FBQ_ERR_TIMEOUT in the
 // status word and every role falls through to the common exit.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 
 #include "fbq_common.cuh"
+#include "fbq_maps.h"
 
 namespace fbq {
 namespace {
@@ -1557,27 +1557,13 @@ cudaError_t launch_pair_kernel(const CUtensorMap &xmap, const CUtensorMap &wmap,
 int g_pair = 0;
 
 // 2-D tensor map of a row-major matrix: `cols` elements per row (16- or 32-bit), `rows` rows,
-// boxes of box_cols x box_rows.  Reads outside the matrix return zero.
+// boxes of box_cols x box_rows.  Maps of weights are kept (`keep`), those of activations are not.
 cudaError_t make_map(CUtensorMap *map, const void *base, bool elem32, size_t cols, size_t rows, int box_cols, int box_rows,
-                     CUtensorMapSwizzle swizzle)
+                     CUtensorMapSwizzle swizzle, bool keep)
 {
-    static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-    if (!encode) {
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
-        if (e != cudaSuccess) return e;
-        if (qres != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-        encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
-    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)cols * (elem32 ? 4 : 2)};
-    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = encode(map, elem32 ? CU_TENSOR_MAP_DATA_TYPE_UINT32 : CU_TENSOR_MAP_DATA_TYPE_UINT16, 2,
-                              const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+    const MapSpec m = matrix_map(base, elem32 ? CU_TENSOR_MAP_DATA_TYPE_UINT32 : CU_TENSOR_MAP_DATA_TYPE_UINT16, elem32 ? 4 : 2, cols, rows, box_cols,
+                                 box_rows, swizzle);
+    return keep ? cached_map(map, m) : encode_map(map, m);
 }
 
 // K splits of a main tile when all tokens fit one tile of 128: as many as keep the CTA count near the
@@ -1630,13 +1616,13 @@ cudaError_t run_prefill(const LinearArgs &a, Workspace &ws, cudaStream_t s, int 
     p.test_skip_flag = g_pf_skip_flag;
     CUtensorMap xmap, qmap, amap, bmap, ymap;
     cudaError_t e;
-    if ((e = make_map(&xmap, a.x, false, (size_t)a.K, (size_t)a.M, kBK, PAIR ? 128 : TOK, CU_TENSOR_MAP_SWIZZLE_128B)) != cudaSuccess)
+    if ((e = make_map(&xmap, a.x, false, (size_t)a.K, (size_t)a.M, kBK, PAIR ? 128 : TOK, CU_TENSOR_MAP_SWIZZLE_128B, false)) != cudaSuccess)
         return e;
     const int wpg = (a.bits == 4) ? 16 : 12;
     if ((e = make_map(&qmap, a.qw, true, (size_t)(a.K / kGroupFast) * wpg, (size_t)a.N, wpg, kBN,
-                      a.bits == 4 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE)) != cudaSuccess)
+                      a.bits == 4 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE, true)) != cudaSuccess)
         return e;
-    if ((e = make_map(&ymap, a.y, false, (size_t)a.N, (size_t)a.M, kBN, TOK / 4, CU_TENSOR_MAP_SWIZZLE_NONE)) != cudaSuccess) return e;
+    if ((e = make_map(&ymap, a.y, false, (size_t)a.N, (size_t)a.M, kBN, TOK / 4, CU_TENSOR_MAP_SWIZZLE_NONE, false)) != cudaSuccess) return e;
     amap = bmap = xmap;
     CUtensorMap tmap = xmap;
     p.t16 = nullptr;
@@ -1644,11 +1630,11 @@ cudaError_t run_prefill(const LinearArgs &a, Workspace &ws, cudaStream_t s, int 
     if (!PAIR && a.rank > 0 && p.splitt == 1) {
         // t goes from the t CTAs to the main CTAs in the activation type, laid out like x, behind the fp32 slices of t
         p.t16 = ws.t_gen + (((size_t)a.M * a.rank + 3) & ~(size_t)3);
-        if ((e = make_map(&tmap, p.t16, false, (size_t)p.rank_pad, (size_t)a.M, kBK, TOK, CU_TENSOR_MAP_SWIZZLE_128B)) != cudaSuccess) return e;
+        if ((e = make_map(&tmap, p.t16, false, (size_t)p.rank_pad, (size_t)a.M, kBK, TOK, CU_TENSOR_MAP_SWIZZLE_128B, false)) != cudaSuccess) return e;
     }
     if (a.rank > 0) {
-        if ((e = make_map(&amap, a.A, false, (size_t)a.K, (size_t)a.rank, kBK, kBN, CU_TENSOR_MAP_SWIZZLE_128B)) != cudaSuccess) return e;
-        if ((e = make_map(&bmap, a.B, false, (size_t)a.rank, (size_t)a.N, kBK, kBN, CU_TENSOR_MAP_SWIZZLE_128B)) != cudaSuccess) return e;
+        if ((e = make_map(&amap, a.A, false, (size_t)a.K, (size_t)a.rank, kBK, kBN, CU_TENSOR_MAP_SWIZZLE_128B, true)) != cudaSuccess) return e;
+        if ((e = make_map(&bmap, a.B, false, (size_t)a.rank, (size_t)a.N, kBK, kBN, CU_TENSOR_MAP_SWIZZLE_128B, true)) != cudaSuccess) return e;
     }
     const unsigned grid = (unsigned)p.n_t + (unsigned)p.nt * (unsigned)mt * (unsigned)p.splitk;
     if (PAIR)

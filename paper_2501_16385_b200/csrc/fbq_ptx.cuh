@@ -53,7 +53,7 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
 }
 // Bounded wait: false when the time limit is hit (never spins forever).  The first look is inline; the
 // polling loop is one out-of-line function, so that the many wait sites cost little code.
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, uint32_t sleep_ns)
+static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, uint32_t sleep_ns)
 {
     const unsigned long long t0 = global_ns();
 #pragma unroll 1

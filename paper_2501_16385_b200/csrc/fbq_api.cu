@@ -1,6 +1,7 @@
 // extern "C" boundary of libfbq: argument validation, kernel selection,
 // per-stream scratch space, launch bookkeeping.  Declarations and the contract
 // of every entry point are in include/fbq.h.
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <map>
@@ -215,6 +216,16 @@ int run_linear(const LinearArgs &a, cudaStream_t s, int decode_ctas = 0)
         size_t have_c = (size_t)ws->n_counters, need_t = 0, need_p = 0;
         int need_c = 0;
         prefill_workspace_need(a, &need_c, &need_t, &need_p);
+        if (prefill_dense(a)) {
+            size_t need_w = 0, need_tags = 0, tf = 0;
+            dense_workspace_need(a, &need_w, &need_tags, &tf);
+            char *w16 = static_cast<char *>(ws->w16);
+            e = grow(w16, ws->w16_bytes, need_w, 1, s);
+            ws->w16 = w16;
+            if (e == cudaSuccess) e = grow(ws->tags, ws->n_tags, need_tags, sizeof(uint32_t), s);
+            if (e != cudaSuccess) return grow_status(e);
+            need_t = std::max(need_t, tf);
+        }
         if ((e = grow(ws->counters, have_c, (size_t)need_c, sizeof(int), s)) != cudaSuccess) return grow_status(e);
         ws->n_counters = (int)have_c;
         if (need_t > 0 && (e = grow(ws->t_gen, ws->t_gen_floats, need_t, sizeof(float), s)) != cudaSuccess) return grow_status(e);
@@ -661,6 +672,7 @@ int fbq_poll_status(void *stream)
         cudaMemset(ws->counters, 0, sizeof(int) * (size_t)ws->n_counters);
         if (ws->t) cudaMemset(ws->t, 0, sizeof(float) * ws->t_floats);
         if (ws->tslots) cudaMemset(ws->tslots, 0, sizeof(float) * ws->tslots_floats);
+        if (ws->tags) cudaMemset(ws->tags, 0, sizeof(uint32_t) * ws->n_tags);
     }
     return st;
 }
@@ -688,6 +700,8 @@ int fbq_release_workspaces(void)
         cudaFree(w.trace);
         cudaFree(w.stage_x);
         cudaFree(w.stage_y);
+        cudaFree(w.w16);
+        cudaFree(w.tags);
     }
     g_ws.clear();
     return FBQ_OK;

@@ -42,6 +42,10 @@ struct Workspace {
     void *stage_x = nullptr;      // staging for the host-buffer entry point
     void *stage_y = nullptr;
     size_t stage_x_bytes = 0, stage_y_bytes = 0;
+    void *w16 = nullptr;          // dequantised weights of the dense prefill kernel (no invariant)
+    size_t w16_bytes = 0;
+    uint32_t *tags = nullptr;     // its launch number and tags (starts at zero)
+    size_t n_tags = 0;
 };
 constexpr int kCtrT = 0, kCtrDone = 1, kCtrStatus = 2;   // the decode kernel defines the rest
 
@@ -105,7 +109,17 @@ bool decode_batch_need(const LinearArgs *a, int count, const int *ctas, const De
                        size_t *t_floats, int *counters);
 cudaError_t launch_decode_batch(const LinearArgs *a, int count, const int *ctas, Workspace &ws, const DecodeTuning &tune,
                                 cudaStream_t s, int *launches);
+// The dense prefill kernel (fbq_dense.cu).
+struct PrefillTuning {
+    int pdl = 1;
+    int flag_polls = 0;        // 0: waits for t end by time, else after this many looks
+    int test_skip_flag = 0;    // test switch: t is not announced (the wait for it must run out)
+};
+void dense_workspace_need(const LinearArgs &a, size_t *w16_bytes, size_t *tags, size_t *t_floats);
+cudaError_t launch_dense(const LinearArgs &a, Workspace &ws, const PrefillTuning &tune, cudaStream_t s, int *launches);
+
 bool prefill_supported(const LinearArgs &a);
+bool prefill_dense(const LinearArgs &a);       // the dense kernel takes this call (fbq_dense.cu)
 void prefill_workspace_need(const LinearArgs &a, int *counters, size_t *t_floats, size_t *partial_floats);
 cudaError_t launch_prefill(const LinearArgs &a, Workspace &ws, cudaStream_t s, int *launches);
 

@@ -1,0 +1,31 @@
+"""The prefill kernel that dequantises the weights once per call (many tiles): ragged tokens and features, K that is not
+a multiple of its dequantisation units, every sub-branch width of its blocks, both activation types; call after call."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_utils import DeviceLinear, check_parity, torch_to_f64
+from workloads import make_exact_class, make_linear
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("bits,dtype,M,N,K,rank", [(4, "bf16", 2090, 7432, 384, 64), (3, "f16", 3001, 5128, 256, 200),
+                                                   (4, "f16", 2500, 6920, 128, 0), (3, "bf16", 700, 22024, 640, 8)])
+def test_dense_prefill_edges(bits, dtype, M, N, K, rank):
+    import paper_2501_16385_b200 as fbq
+    inp = make_linear(M, N, K, bits, rank, dtype=dtype, seed=3000 + M, outlier_frac=0.01)
+    rows = np.unique(np.concatenate([np.arange(9), np.arange(N - 9, N), np.random.default_rng(M).choice(N, 20)]))
+    check_parity(inp, fbq, expect_kernel=fbq.KERNEL_PREFILL, n_list=rows, threads=16, floor=2e-5)
+
+
+def test_dense_prefill_exact_class_is_bitwise_and_repeats():
+    import paper_2501_16385_b200 as fbq
+    inp = make_exact_class(1100, 13064, 512, 4, 64, seed=3100, x_nnz=32, x_max=2)
+    dev = DeviceLinear(inp, fbq)
+    rows = np.arange(5, inp.N, 97)
+    want = oracle.linear_inputs(inp, n_list=rows, threads=16)
+    for _ in range(3):
+        y = torch_to_f64(dev.run(fbq), "f16")
+        assert fbq.poll_status() == 0
+        assert np.array_equal(y[:, rows], want)

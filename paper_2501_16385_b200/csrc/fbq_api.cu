@@ -248,6 +248,34 @@ int run_linear(const LinearArgs &a, cudaStream_t s, int decode_ctas = 0)
     return FBQ_OK;
 }
 
+// Runs f(scratch, status word, &launches) with `need` bytes of the stream's scratch; where that would have to grow during a
+// stream capture, with memory that belongs to the captured graph.
+template <typename F>
+int with_scratch(size_t need, cudaStream_t s, F f)
+{
+    Workspace *ws = workspace_for(s);
+    if (!ws) return FBQ_ERR_CUDA;
+    int launches = 0, rc;
+    size_t have_c = (size_t)ws->n_counters;
+    if (grow(ws->counters, have_c, 16, sizeof(int), s) == cudaSuccess) ws->n_counters = (int)have_c;
+    int *status = ws->counters ? ws->counters + kCtrStatus : nullptr;
+    char *rec = static_cast<char *>(ws->rec);
+    const cudaError_t e = grow(rec, ws->rec_bytes, need, 1, s);
+    ws->rec = rec;
+    if (e == cudaSuccess) {
+        rc = f(ws->rec, status, &launches);
+    } else if (e == cudaErrorStreamCaptureUnsupported) {
+        void *tmp = nullptr;
+        if (cudaMallocAsync(&tmp, need, s) != cudaSuccess) return FBQ_ERR_CUDA;
+        rc = f(tmp, status, &launches);
+        if (cudaFreeAsync(tmp, s) != cudaSuccess) rc = FBQ_ERR_CUDA;
+    } else {
+        return FBQ_ERR_CUDA;
+    }
+    g_launches += launches;
+    return rc;
+}
+
 int *option_slot(const char *name)
 {
     if (!name) return nullptr;
@@ -375,9 +403,8 @@ size_t fbq_reconstruct_workspace_floats(int N, int K, int rank)
 int fbq_gram(const float *X, float *H, int T, int K, void *stream)
 {
     if (!X || !H || T < 1 || K < 1) return FBQ_ERR_BADARG;
-    const int rc = run_gram(X, H, T, K, static_cast<cudaStream_t>(stream));
-    if (rc == FBQ_OK) ++g_launches;
-    return rc;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return with_scratch(gram_scratch_bytes(T, K), s, [&](void *scratch, int *status, int *n) { return run_gram(X, H, T, K, scratch, status, s, n); });
 }
 
 int fbq_reconstruct_step(const float *W, const float *H, float *A, float *B, float lr, float *loss, float *workspace, int N,
@@ -386,9 +413,10 @@ int fbq_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
     if (N < 1 || K < 1 || rank < 1 || group < 1 || group > 1024 || K % group != 0 || K / group > 65535) return FBQ_ERR_BADARG;
     if (bits != 3 && bits != 4) return FBQ_ERR_BADARG;
     if (!W || !H || !A || !B || !workspace) return FBQ_ERR_BADARG;
-    const int rc = run_reconstruct_step(W, H, A, B, lr, loss, workspace, N, K, group, bits, rank, static_cast<cudaStream_t>(stream));
-    if (rc == FBQ_OK) g_launches += loss ? 8 : 6;       // quantiser, three GEMMs, (two-stage reduction), two updates
-    return rc;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return with_scratch(reconstruct_scratch_bytes(N, K, rank), s, [&](void *scratch, int *status, int *n) {
+        return run_reconstruct_step(W, H, A, B, lr, loss, workspace, N, K, group, bits, rank, scratch, status, s, n);
+    });
 }
 
 // Hands the process-wide switches to the kernel files before a launch.
@@ -702,6 +730,7 @@ int fbq_release_workspaces(void)
         cudaFree(w.stage_y);
         cudaFree(w.w16);
         cudaFree(w.tags);
+        cudaFree(w.rec);
     }
     g_ws.clear();
     return FBQ_OK;

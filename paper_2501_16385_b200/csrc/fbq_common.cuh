@@ -46,6 +46,8 @@ struct Workspace {
     size_t w16_bytes = 0;
     uint32_t *tags = nullptr;     // its launch number and tags (starts at zero)
     size_t n_tags = 0;
+    void *rec = nullptr;          // split operands of the Gram matrix and the reconstruction step (no invariant)
+    size_t rec_bytes = 0;
 };
 constexpr int kCtrT = 0, kCtrDone = 1, kCtrStatus = 2;   // the decode kernel defines the rest
 
@@ -73,12 +75,12 @@ cudaError_t launch_sub_branch_unfused(const void *x, const void *A, const void *
 cudaError_t launch_quantize_feedback(const float *W, const void *A, const void *B, uint8_t *codes, __half *scales,
                                      __half *zeros, float *WF, float *Delta, int N, int K, int group, int bits, int rank,
                                      int ab_kind, cudaStream_t s);
-cudaError_t launch_scaled_dot(const float *a, const float *b, size_t n, float scale, float *partial, float *out, cudaStream_t s);
-cudaError_t launch_axpy(float *y, const float *x, float alpha, size_t n, cudaStream_t s);
 size_t reconstruct_workspace_floats(int N, int K, int rank);
-int run_gram(const float *X, float *H, int T, int K, cudaStream_t s);
+size_t gram_scratch_bytes(int T, int K);
+size_t reconstruct_scratch_bytes(int N, int K, int rank);
+int run_gram(const float *X, float *H, int T, int K, void *scratch, int *status, cudaStream_t s, int *launches);
 int run_reconstruct_step(const float *W, const float *H, float *A, float *B, float lr, float *loss, float *ws, int N, int K,
-                         int group, int bits, int rank, cudaStream_t s);
+                         int group, int bits, int rank, void *scratch, int *status, cudaStream_t s, int *launches);
 
 struct DecodeTuning {
     int sk = 0, chunk = 0, depth = 0, max_ctas = 0, pdl = 1;

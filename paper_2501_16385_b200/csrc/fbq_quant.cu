@@ -359,49 +359,4 @@ cudaError_t launch_quantize_feedback(const float *W, const void *A, const void *
     return ab_kind == 2 ? go(float{}) : ab_kind == 1 ? go(__nv_bfloat16{}) : go(__half{});
 }
 
-// ---- reconstruction step helpers (Algorithm 1 lines 7-9) ---------------------------------
-// partial[b] = sum over this block's slice of a[i]*b[i]; a second launch with one block adds the
-// partials in index order and writes scale * sum.  Fixed order: the result is reproducible.
-__global__ void dot_partial_kernel(const float *__restrict__ a, const float *__restrict__ b, size_t n, float *partial)
-{
-    __shared__ float sh[32];
-    float v = 0.f;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) v = fmaf(a[i], b[i], v);
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-        partial[blockIdx.x] = t;
-    }
-}
-__global__ void dot_final_kernel(const float *partial, int n, float scale, float *out)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double t = 0.0;
-        for (int i = 0; i < n; ++i) t += (double)partial[i];
-        *out = (float)(t * (double)scale);
-    }
-}
-__global__ void axpy_kernel(float *__restrict__ y, const float *__restrict__ x, float alpha, size_t n)
-{
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        y[i] = fmaf(alpha, x[i], y[i]);
-}
-
-cudaError_t launch_scaled_dot(const float *a, const float *b, size_t n, float scale, float *partial /*>= 256*/, float *out,
-                              cudaStream_t s)
-{
-    dot_partial_kernel<<<256, 256, 0, s>>>(a, b, n, partial);
-    dot_final_kernel<<<1, 32, 0, s>>>(partial, 256, scale, out);
-    return cudaGetLastError();
-}
-cudaError_t launch_axpy(float *y, const float *x, float alpha, size_t n, cudaStream_t s)
-{
-    const unsigned blocks = (unsigned)((n + 255) / 256 < 1184 ? (n + 255) / 256 : 1184);
-    axpy_kernel<<<blocks ? blocks : 1, 256, 0, s>>>(y, x, alpha, n);
-    return cudaGetLastError();
-}
-
 }  // namespace fbq

@@ -1,0 +1,57 @@
+"""The tensor-core products behind fbq_gram and fbq_reconstruct_step where their tiles end, and how close to float64 they come."""
+import numpy as np
+import pytest
+
+from oracle import reconstruct as rec
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T,K", [(1, 5), (65, 257), (300, 512), (129, 255), (1000, 770)])
+def test_gram_tile_edges(T, K):
+    import torch
+    import paper_2501_16385_b200 as fbq
+    rng = np.random.default_rng(T)
+    X = (rng.standard_normal((T, K)) * (1.0 + 4.0 * (rng.random(K) < 0.05))).astype(np.float32)
+    H = fbq.gram(torch.from_numpy(X).cuda()).cpu().numpy()
+    assert fbq.poll_status() == 0
+    want = X.astype(np.float64).T @ X.astype(np.float64)
+    assert np.linalg.norm(H - want) <= 3e-7 * np.linalg.norm(want)
+    assert np.abs(H - want).max() <= 1e-6 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("N,K,rank", [(1, 128, 1), (257, 384, 33), (130, 640, 260)])
+def test_step_tile_edges(N, K, rank):
+    import torch
+    import paper_2501_16385_b200 as fbq
+    rng = np.random.default_rng(N)
+    W = (rng.standard_normal((N, K)) * 0.05).astype(np.float32)
+    X = rng.standard_normal((200, K)).astype(np.float32)
+    A = (rng.standard_normal((rank, K)) * 0.05).astype(np.float32)
+    B = (rng.standard_normal((N, rank)) * 0.05).astype(np.float32)
+    H = rec.gram(X)
+    lr = 0.05 / (np.linalg.eigvalsh(H)[-1] * max(np.linalg.norm(A, 2), np.linalg.norm(B, 2)) ** 2)
+    Ad, Bd = torch.from_numpy(A.copy()).cuda(), torch.from_numpy(B.copy()).cuda()
+    loss, _ = fbq.reconstruct_step(torch.from_numpy(W).cuda(), torch.from_numpy(H.astype(np.float32)).cuda(), Ad, Bd, lr, 128, 4)
+    assert fbq.poll_status() == 0
+    loss_o, A_o, B_o = rec.step(W, H, A, B, lr, 128, 4)
+    assert np.isclose(float(loss.item()), loss_o, rtol=2e-6)
+    assert np.linalg.norm(Ad.cpu().numpy() - A_o) <= 1e-6 * np.linalg.norm(A_o)
+    assert np.linalg.norm(Bd.cpu().numpy() - B_o) <= 1e-6 * np.linalg.norm(B_o)
+
+
+def test_gram_captured_before_the_stream_has_scratch():
+    import torch
+    import paper_2501_16385_b200 as fbq
+    X = torch.randn((96, 320), device="cuda")
+    fbq.gram(X[:, :64].contiguous())                   # the kernels are loaded
+    H = torch.zeros((320, 320), device="cuda")
+    stream = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        with torch.cuda.graph(g, stream=stream):
+            H.copy_(fbq.gram(X))
+    g.replay()
+    torch.cuda.synchronize()
+    want = X.double().T @ X.double()
+    assert float((H.double() - want).norm() / want.norm()) < 3e-7

@@ -213,15 +213,16 @@ int fbq_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
  * activation type; N and K are per problem.  No y_i may overlap another problem's inputs.
  *   - `problems` is a HOST array of `count` (<= FBQ_BATCH_MAX) descriptors of DEVICE
  *     pointers (layouts and alignment as for fbq_linear); it is read before the call returns.
- *   - When every problem is decode sized (M <= 16 and the decode kernel's domain) the
- *     problems run concurrently, each with a share of "batch_ctas" CTAs in proportion to its
- *     share of the codes, so that the whole batch is resident at once.  Up to 8 problems run
- *     as ONE launch of the decode kernel over a problem list, on `stream` ("batch_single" = 1,
- *     the default); more problems, or "batch_single" = 0, run one launch per problem on side
- *     streams of the library, forked from and joined to `stream` with events (legal under
- *     stream capture; make the first such call on a device outside a capture: it creates the
- *     side streams and events, which are kept until the process exits).  Either way work
- *     queued on `stream` after the call sees every y_i.
+ *   - When every problem is decode sized (M <= 16 and the decode kernels' domain) the problems run
+ *     concurrently.  Up to 8 problems of the streaming kernel that read the same x (q, k, v; gate,
+ *     up) are ONE launch of it on `stream`, the SMs shared out so that no CTA has much more than
+ *     another ("batch_single" = 1, the default).  Up to 8 problems outside the streaming kernel's
+ *     domain run as ONE launch of the other decode kernel over a problem list, each with a share
+ *     of "batch_ctas" CTAs in proportion to its share of the codes.  Everything else, or
+ *     "batch_single" = 0, runs one launch per problem on side streams of the library, forked from
+ *     and joined to `stream` with events (legal under stream capture; make the first such call on
+ *     a device outside a capture: it creates the side streams and events, which are kept until the
+ *     process exits).  Either way work queued on `stream` after the call sees every y_i.
  *   - Otherwise the problems run one after the other on `stream`.
  * Returns the first error, or FBQ_OK. */
 #define FBQ_BATCH_MAX 16
@@ -238,8 +239,11 @@ typedef struct fbq_problem {
 int fbq_linear_batch(const fbq_problem *problems, int count, int M, int group, int bits, int rank,
                      int act_is_bf16, void *stream);
 /* The same with every problem's x and y in HOST memory (pinned for asynchronous copies), the
- * weights on the device as before: per problem the library copies x to a staging buffer it
- * keeps per stream, runs the linear, and copies y back, all on the stream the problem runs on.
+ * weights on the device as before.  Up to 8 problems of the streaming kernel are two launches on
+ * `stream`: one reads every distinct x over the bus into a staging buffer kept per stream (copies,
+ * where it is not pinned), the other computes all problems and writes y straight to the caller's
+ * buffers where they are pinned.  Otherwise each problem is copied in, computed and copied out on
+ * the stream it runs on.
  * y is complete once work queued on `stream` after the call has run (synchronise `stream`
  * before reading it).  The end-to-end path of the benchmark. */
 int fbq_linear_batch_hostio(const fbq_problem *problems, int count, int M, int group, int bits, int rank,

@@ -39,24 +39,83 @@ struct Options {
     int test_prefill_skip_flag = 0, prefill_flag_polls = 0;
     int decode_trace = 0;
 } g_opt;
+constexpr int kGemvBatchMost = 8;                     // problems of one launch of the streaming kernel
 constexpr size_t kTraceBytes = 512 * 18 * 16 * 8;   // 512 CTAs x up to 18 warps x 16 marks
 
 bool misaligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
 
-// The host-buffer entry points write a small y straight into the caller's buffer when that is pinned host memory
-// which the GPU can address (unified addressing): the kernel's stores cross the bus instead of a copy that would
-// have to be queued behind the kernel.  Returns the buffer's device alias, or nullptr (pageable memory, unaligned,
-// large, switched off): then y goes through the stream's staging buffer and a copy.
-void *direct_y_alias(void *y_host, size_t bytes)
+// Device alias of a pinned host buffer which the GPU can address (unified addressing), 16-byte aligned; nullptr for
+// pageable or other memory.
+void *pinned_alias(const void *host)
 {
-    if (!g_opt.hostio_direct_y || bytes > (256u << 10)) return nullptr;
     cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, y_host) != cudaSuccess) {
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
         (void)cudaGetLastError();
         return nullptr;
     }
     if (at.type != cudaMemoryTypeHost || !at.devicePointer || misaligned16(at.devicePointer)) return nullptr;
     return at.devicePointer;
+}
+// The host-buffer entry points write a small y straight into the caller's buffer where it is pinned: the kernel's stores
+// cross the bus instead of a copy that would have to be queued behind the kernel.  nullptr (pageable memory, unaligned,
+// large, switched off): y goes through the stream's staging buffer and a copy.
+void *direct_y_alias(void *y_host, size_t bytes) { return !g_opt.hostio_direct_y || bytes > (256u << 10) ? nullptr : pinned_alias(y_host); }
+
+// Copies of a call's x into its staging buffer.  Small pinned ones are read over the bus by one kernel, all of them
+// together: a copy of the copy engine costs several microseconds each, and the kernel that reads the staging buffer sets
+// itself up meanwhile (dependent launch).
+constexpr size_t kGatherMost = 512u << 10;
+struct GatherList {
+    int n = 0;
+    unsigned first[FBQ_BATCH_MAX + 1] = {};      // 16-byte units before segment i
+    const uint4 *src[FBQ_BATCH_MAX];
+    uint4 *dst[FBQ_BATCH_MAX];
+};
+__global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ GatherList g)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const unsigned u = blockIdx.x * 256u + threadIdx.x;
+    int i = 0;
+    for (int k = 1; k < g.n; ++k)
+        if (u >= g.first[k]) i = k;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (u < g.first[g.n]) v = g.src[i][u - g.first[i]];
+    asm volatile("griddepcontrol.wait;" ::: "memory");       // the kernel before may still be reading the staging buffer
+    if (u < g.first[g.n]) g.dst[i][u - g.first[i]] = v;
+}
+cudaError_t copy_in(int n, const void *const *src, void *const *dst, const size_t *bytes, cudaStream_t s)
+{
+    GatherList g;
+    size_t total = 0;
+    bool gather = true;
+    for (int i = 0; i < n; ++i) {
+        total += bytes[i];
+        gather = gather && bytes[i] % 16 == 0;
+    }
+    for (int i = 0; gather && total <= kGatherMost && i < n; ++i) {
+        g.src[i] = static_cast<const uint4 *>(pinned_alias(src[i]));
+        g.dst[i] = static_cast<uint4 *>(dst[i]);
+        g.first[i + 1] = g.first[i] + (unsigned)(bytes[i] / 16);
+        gather = g.src[i] != nullptr;
+    }
+    if (gather && total <= kGatherMost && total > 0) {
+        g.n = n;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((g.first[n] + 255u) / 256u);
+        cfg.blockDim = dim3(256);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = g_opt.decode.pdl ? 1 : 0;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, gather_kernel, g);
+        if (e == cudaSuccess) ++g_launches;
+        return e;
+    }
+    for (int i = 0; i < n; ++i)
+        if (const cudaError_t e = cudaMemcpyAsync(dst[i], src[i], bytes[i], cudaMemcpyHostToDevice, s); e != cudaSuccess) return e;
+    return cudaSuccess;
 }
 
 bool well_formed(int M, int N, int K, int group, int bits, int rank)
@@ -141,6 +200,38 @@ Workspace *workspace_for(cudaStream_t s)
 
 int grow_status(cudaError_t e) { return e == cudaErrorStreamCaptureUnsupported ? FBQ_ERR_UNSUPPORTED : FBQ_ERR_CUDA; }
 
+int check_args(const LinearArgs &a)
+{
+    if (!a.x || !a.qw || !a.scales || !a.zeros || !a.y) return FBQ_ERR_BADARG;
+    if (a.rank > 0 && (!a.A || !a.B)) return FBQ_ERR_BADARG;
+    if (misaligned16(a.x) || misaligned16(a.qw) || misaligned16(a.y) || (a.rank > 0 && (misaligned16(a.A) || misaligned16(a.B))))
+        return FBQ_ERR_ALIGN;
+    if ((reinterpret_cast<uintptr_t>(a.scales) & 1u) || (reinterpret_cast<uintptr_t>(a.zeros) & 1u)) return FBQ_ERR_ALIGN;
+    return FBQ_OK;
+}
+
+// Several problems of the streaming kernel as one launch on `s`; FBQ_ERR_UNSUPPORTED where they cannot share one.
+int run_gemv_batch(const LinearArgs *a, int count, cudaStream_t s)
+{
+    for (int i = 0; i < count; ++i)
+        if (const int rc = check_args(a[i]); rc != FBQ_OK) return rc;
+    Workspace *ws = workspace_for(s);
+    if (!ws) return FBQ_ERR_CUDA;
+    GemvTuning gt = g_opt.gemv;
+    gt.pdl = g_opt.decode.pdl;
+    size_t slots = 0;
+    int nc = 0, launches = 0;
+    if (gt.max_ctas > 0 || g_opt.decode_trace || !gemv_batch_need(a, count, gt, &slots, &nc)) return FBQ_ERR_UNSUPPORTED;
+    size_t have_c = (size_t)ws->n_counters;
+    cudaError_t e;
+    if ((e = grow(ws->tslots, ws->tslots_floats, slots, sizeof(float), s)) != cudaSuccess) return grow_status(e);
+    if ((e = grow(ws->counters, have_c, (size_t)nc, sizeof(int), s)) != cudaSuccess) return grow_status(e);
+    ws->n_counters = (int)have_c;
+    if (launch_gemv_batch(a, count, *ws, gt, s, &launches) != cudaSuccess) return FBQ_ERR_CUDA;
+    g_launches += launches;
+    return FBQ_OK;
+}
+
 // decode_ctas > 0 overrides the decode kernel's grid-size bound for this call.
 int run_linear(const LinearArgs &a, cudaStream_t s, int decode_ctas = 0)
 {
@@ -148,11 +239,7 @@ int run_linear(const LinearArgs &a, cudaStream_t s, int decode_ctas = 0)
     if (decode_ctas > 0) tune.max_ctas = decode_ctas;
     if (!well_formed(a.M, a.N, a.K, a.group, a.bits, a.rank)) return FBQ_ERR_BADARG;
     if (a.M == 0) return FBQ_OK;
-    if (!a.x || !a.qw || !a.scales || !a.zeros || !a.y) return FBQ_ERR_BADARG;
-    if (a.rank > 0 && (!a.A || !a.B)) return FBQ_ERR_BADARG;
-    if (misaligned16(a.x) || misaligned16(a.qw) || misaligned16(a.y) || (a.rank > 0 && (misaligned16(a.A) || misaligned16(a.B))))
-        return FBQ_ERR_ALIGN;
-    if ((reinterpret_cast<uintptr_t>(a.scales) & 1u) || (reinterpret_cast<uintptr_t>(a.zeros) & 1u)) return FBQ_ERR_ALIGN;
+    if (const int rc = check_args(a); rc != FBQ_OK) return rc;
 
     Workspace *ws = workspace_for(s);
     if (!ws) return FBQ_ERR_CUDA;
@@ -481,6 +568,65 @@ static BatchLanes *lanes_for(int want)
     return &b;
 }
 
+// A decode-sized batch with host buffers as two launches: x (each distinct one once) into the stream's staging buffer, then
+// all problems; y goes straight to the caller's buffers where that is possible.  FBQ_ERR_UNSUPPORTED: nothing was queued.
+static int host_batch(const LinearArgs *in, const fbq_problem *problems, int count, int M, cudaStream_t s)
+{
+    LinearArgs a[FBQ_BATCH_MAX];
+    const void *src[FBQ_BATCH_MAX];
+    void *dst[FBQ_BATCH_MAX];
+    size_t bytes[FBQ_BATCH_MAX], x_bytes = 0, y_bytes = 0, off[FBQ_BATCH_MAX];
+    int nx = 0, which[FBQ_BATCH_MAX];
+    auto padded = [](size_t n) { return (n + 255) & ~(size_t)255; };
+    Workspace *ws = workspace_for(s);
+    if (!ws) return FBQ_ERR_CUDA;
+    for (int i = 0; i < count; ++i) {
+        a[i] = in[i];
+        if (!a[i].x || !a[i].y) return FBQ_ERR_BADARG;
+        int k = 0;
+        while (k < nx && !(src[k] == a[i].x && bytes[k] == (size_t)M * a[i].K * 2)) ++k;
+        if (k == nx) {
+            src[nx] = a[i].x;
+            bytes[nx] = (size_t)M * a[i].K * 2;
+            off[nx] = x_bytes;
+            x_bytes += padded(bytes[nx++]);
+        }
+        which[i] = k;
+    }
+    char *sx = static_cast<char *>(ws->stage_x), *sy = static_cast<char *>(ws->stage_y);
+    cudaError_t e = grow(sx, ws->stage_x_bytes, x_bytes, 1, s);
+    ws->stage_x = sx;
+    if (e != cudaSuccess) return grow_status(e);
+    bool staged[FBQ_BATCH_MAX];
+    for (int i = 0; i < count; ++i) {
+        a[i].x = sx + off[which[i]];
+        void *alias = direct_y_alias(a[i].y, (size_t)M * a[i].N * 2);
+        staged[i] = alias == nullptr;
+        a[i].y = alias ? alias : reinterpret_cast<void *>(y_bytes);        // (an offset until the buffer is there)
+        if (staged[i]) y_bytes += padded((size_t)M * a[i].N * 2);
+    }
+    if (y_bytes > 0) {
+        e = grow(sy, ws->stage_y_bytes, y_bytes, 1, s);
+        ws->stage_y = sy;
+        if (e != cudaSuccess) return grow_status(e);
+    }
+    for (int i = 0; i < count; ++i)
+        if (staged[i]) a[i].y = sy + reinterpret_cast<size_t>(a[i].y);
+    {                                                                      // before anything is queued
+        size_t slots = 0;
+        int nc = 0;
+        GemvTuning gt = g_opt.gemv;
+        if (gt.max_ctas > 0 || g_opt.decode_trace || !gemv_batch_need(a, count, gt, &slots, &nc)) return FBQ_ERR_UNSUPPORTED;
+    }
+    for (int k = 0; k < nx; ++k) dst[k] = sx + off[k];
+    if (copy_in(nx, src, dst, bytes, s) != cudaSuccess) return FBQ_ERR_CUDA;
+    const int rc = run_gemv_batch(a, count, s);
+    if (rc != FBQ_OK) return rc == FBQ_ERR_UNSUPPORTED ? FBQ_ERR_CUDA : rc;
+    for (int i = 0; i < count; ++i)
+        if (staged[i] && cudaMemcpyAsync(problems[i].y, a[i].y, (size_t)M * a[i].N * 2, cudaMemcpyDeviceToHost, s) != cudaSuccess) return FBQ_ERR_CUDA;
+    return FBQ_OK;
+}
+
 static int linear_batch_common(const fbq_problem *problems, int count, int M, int group, int bits, int rank, int act_is_bf16,
                                void *stream, bool host_io)
 {
@@ -516,7 +662,9 @@ static int linear_batch_common(const fbq_problem *problems, int count, int M, in
         char *sx = static_cast<char *>(ws->stage_x), *sy = static_cast<char *>(ws->stage_y);
         if (grow(sx, ws->stage_x_bytes, xb, 1, st) != cudaSuccess) return FBQ_ERR_CUDA;
         ws->stage_x = sx;
-        if (cudaMemcpyAsync(sx, la.x, xb, cudaMemcpyHostToDevice, st) != cudaSuccess) return FBQ_ERR_CUDA;
+        const void *from[1] = {la.x};
+        void *to[1] = {sx};
+        if (copy_in(1, from, to, &xb, st) != cudaSuccess) return FBQ_ERR_CUDA;
         la.x = sx;
         if (void *alias = direct_y_alias(la.y, yb)) {
             la.y = alias;                             // the kernel writes the caller's buffer itself
@@ -552,6 +700,19 @@ static int linear_batch_common(const fbq_problem *problems, int count, int M, in
     // the same sums, as fbq_linear); the single launch over a problem list is the other decode kernel's.
     bool all_gemv = g_opt.use_gemv != 0;
     for (int i = 0; i < count; ++i) all_gemv = all_gemv && gemv_supported(a[i]);
+    // Problems that read the same x (q, k and v; gate and up) share one launch of it on the caller's stream, and so do all
+    // problems of a call with host buffers, whose x arrive together.
+    if (all_gemv && g_opt.batch_single && count > 1 && count <= kGemvBatchMost) {
+        bool one_x = true;
+        for (int i = 1; i < count; ++i) one_x = one_x && a[i].x == a[0].x && a[i].K == a[0].K;
+        if (one_x && !host_io) {
+            const int rc = run_gemv_batch(a, count, main);
+            if (rc != FBQ_ERR_UNSUPPORTED) return rc;
+        } else if (host_io) {
+            const int rc = host_batch(a, problems, count, M, main);
+            if (rc != FBQ_ERR_UNSUPPORTED) return rc;
+        }
+    }
     if (g_opt.batch_single && !host_io && count <= decode_batch_max() && !all_gemv) {
         // One launch: the decode kernel over a problem list, on the caller's stream.  (With host
         // buffers the per-problem streams below are faster: their small copies overlap.)
@@ -629,7 +790,9 @@ int fbq_linear_hostio(const void *x_host, const uint32_t *qweight, const void *s
     char *sx = static_cast<char *>(ws->stage_x), *sy = static_cast<char *>(ws->stage_y);
     if (grow(sx, ws->stage_x_bytes, xb, 1, s) != cudaSuccess) return FBQ_ERR_CUDA;
     ws->stage_x = sx;
-    if (cudaMemcpyAsync(sx, x_host, xb, cudaMemcpyHostToDevice, s) != cudaSuccess) return FBQ_ERR_CUDA;
+    const void *from[1] = {x_host};
+    void *to[1] = {sx};
+    if (copy_in(1, from, to, &xb, s) != cudaSuccess) return FBQ_ERR_CUDA;
     if (void *alias = direct_y_alias(y_host, yb))       // the kernel writes the caller's buffer itself
         return linear_common(sx, qweight, scales, zeros, A, B, alias, M, N, K, group, bits, rank, act_is_bf16 != 0, stream);
     if (grow(sy, ws->stage_y_bytes, yb, 1, s) != cudaSuccess) return FBQ_ERR_CUDA;

@@ -99,12 +99,18 @@ struct GemvTuning {
     int max_ctas = 0;          // 0: one main CTA per SM
     int pdl = 1;
     int poll_limit = 0;        // 0: default number of looks at the "t complete" counter
+    int main_ctas = 0;         // > 0: this many main CTAs (a problem of a batch)
     int test_skip_arrive = 0;  // test switch: the t CTAs do not report their arrival (the wait for t must run out)
 };
 int gemv_k_slices(int M, int K);      // K slices the streaming decode kernel cuts a shape into (1: x of all K fits)
 bool gemv_supported(const LinearArgs &a);
 void gemv_workspace_need(const LinearArgs &a, const GemvTuning &tune, size_t *tpart_floats, int *counters, size_t *partial_floats);
 cudaError_t launch_gemv(const LinearArgs &a, Workspace &ws, const GemvTuning &tune, cudaStream_t s, int *launches);
+
+// Several problems of the streaming kernel in one launch: scratch, then launch.  false where they cannot share one (other
+// forms, plans that do not fit): then they are launched one by one.
+bool gemv_batch_need(const LinearArgs *a, int count, const GemvTuning &tune, size_t *tslots_floats, int *counters);
+cudaError_t launch_gemv_batch(const LinearArgs *a, int count, Workspace &ws, const GemvTuning &tune, cudaStream_t s, int *launches);
 
 int decode_batch_max();
 bool decode_batch_need(const LinearArgs *a, int count, const int *ctas, const DecodeTuning &tune, size_t *partial_floats,

@@ -55,6 +55,7 @@ constexpr int kTile = 16;                    // weight rows of a tile
 constexpr int kCHG = 2 * kCW;                // quantisation groups of a stage (one pair per compute warp at M = 1)
 constexpr int kMaxNS = 8, kMaxBuf = 8, kMaxB = 4, kMaxMeta = 8;
 constexpr int kMaxSub = 8;                   // tiles whose t.B^T may be formed ahead of their main sums
+constexpr int kGemvBatchMax = 8;             // problems of one launch
 constexpr int kTKB = 64;                     // k extent of one block of A in a t CTA (128 bytes: the swizzle span)
 
 struct GemvParams {
@@ -671,7 +672,7 @@ __device__ __forceinline__ bool look_slots(const uint32_t *tpart, size_t slot_el
 }
 
 template <typename T, bool RANKED>
-__device__ __forceinline__ bool epilogue(const GemvParams &p, uint8_t *smem, const CUtensorMap *bmap, int lane, int tile_first, int ntile)
+__device__ __forceinline__ bool epilogue(const GemvParams &p, uint8_t *smem, const CUtensorMap *bmap, int lane, int tile_first, int ntile, int cta)
 {
     const int g = lane >> 2, tq = lane & 3;
     const uint32_t sbase = smem_u32(smem), bars = sbase + p.off_bar;
@@ -688,7 +689,7 @@ __device__ __forceinline__ bool epilogue(const GemvParams &p, uint8_t *smem, con
     };
     if (RANKED && lane == 0)
         for (int ts = 0; ts < min(ntile, p.nb); ++ts) request_b(ts, ts);   // rows of B are weights: before the wait
-    prefetch_x(p, (int)blockIdx.x - p.n_t, lane, (int)sizeof(T));
+    prefetch_x(p, cta, lane, (int)sizeof(T));
     // Everything this warp does per tile runs alone on its latencies, so what does not depend on the tile is done
     // once, and before the wait: this lane's (swizzled) byte offsets into a tile of B, as MMA row fragments of the
     // four 16-wide blocks of a 64-column box.
@@ -1179,7 +1180,7 @@ __device__ __forceinline__ bool compute_w16(const GemvParams &p, uint8_t *smem, 
 // With K slices the tile's partial sums meet in scratch and the slice that arrives last finishes the tile.
 template <typename T>
 __device__ __forceinline__ bool epilogue_wide(const GemvParams &p, uint8_t *smem, const CUtensorMap *bmap, int lane, int tile_first,
-                                              int ntile, int slice)
+                                              int ntile, int slice, int cta)
 {
     const int g = lane >> 2, tq = lane & 3;
     const uint32_t sbase = smem_u32(smem), bars = sbase + p.off_bar;
@@ -1197,7 +1198,7 @@ __device__ __forceinline__ bool epilogue_wide(const GemvParams &p, uint8_t *smem
     if (rank > 0 && lane == 0)
         for (int ts = 0; ts < min(ntile, p.nb); ++ts) request_b(ts);   // rows of B are weights: before the wait
 
-    prefetch_x(p, (int)blockIdx.x - p.n_t, lane, (int)sizeof(T));
+    prefetch_x(p, cta, lane, (int)sizeof(T));
     uint32_t *s_tf = reinterpret_cast<uint32_t *>(smem + p.off_tf);      // [cb][kb][lane][2]
     for (int i = lane; i < ncb * nkb * 64; i += 32) s_tf[i] = 0u;
     __syncwarp();
@@ -1604,10 +1605,9 @@ __device__ __forceinline__ void t_cta(const GemvParams &p, uint8_t *smem, const 
 }
 
 // ------------------------------------------------------------------------ kernel
+// Block `block` (t CTAs first, then main CTAs) of one problem, integer form.
 template <int BITS, typename T, int M, bool RANKED>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm)
-gemv_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap,
-            const __grid_constant__ CUtensorMap bmap, const __grid_constant__ CUtensorMap amap)
+__device__ __forceinline__ void gemv_body(const GemvParams &p, const CUtensorMap *wmap, const CUtensorMap *bmap, const CUtensorMap *amap, int block)
 {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);     // the swizzled tiles want 1024-byte alignment
@@ -1616,18 +1616,18 @@ gemv_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap,
     pdl_launch_dependents();
     mark(p, 0);
     if constexpr (RANKED) {
-        if ((int)blockIdx.x < p.n_t) {
-            t_cta<T>(p, smem, &amap, (int)blockIdx.x);
+        if (block < p.n_t) {
+            t_cta<T>(p, smem, amap, block);
             return;
         }
     }
-    const int cta = (int)blockIdx.x - p.n_t;
+    const int cta = block - p.n_t;
     const int tile_first = (int)((long long)cta * p.NT / p.n_main);
     const int ntile = (int)((long long)(cta + 1) * p.NT / p.n_main) - tile_first;
     const uint32_t bars = smem_u32(smem) + p.off_bar;
     if (tid == 0) {
-        prefetch_tensormap(&wmap);
-        if (p.rank > 0) prefetch_tensormap(&bmap);
+        prefetch_tensormap(wmap);
+        if (p.rank > 0) prefetch_tensormap(bmap);
         for (int i = 0; i < p.NS; ++i) {
             mbar_init(bars + 8u * (kBarFull + i), 1);
             mbar_init(bars + 8u * (kBarEmpty + i), kCW);
@@ -1645,9 +1645,9 @@ gemv_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap,
 
     bool ok = true;
     if (warp == kProdWarp) {
-        if (lane == 0) ok = produce(p, smem, &wmap, tile_first, ntile);
+        if (lane == 0) ok = produce(p, smem, wmap, tile_first, ntile);
     } else if (warp == kEpiWarp) {
-        ok = epilogue<T, RANKED>(p, smem, &bmap, lane, tile_first, ntile);
+        ok = epilogue<T, RANKED>(p, smem, bmap, lane, tile_first, ntile, cta);
     } else {
         pdl_wait();                                  // x may come from the preceding kernel
         mark(p, 2);
@@ -1658,33 +1658,37 @@ gemv_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap,
     }
     if (!ok && lane == 0) give_up(p);
 }
-
+template <int BITS, typename T, int M, bool RANKED>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+gemv_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap,
+            const __grid_constant__ CUtensorMap bmap, const __grid_constant__ CUtensorMap amap)
+{
+    gemv_body<BITS, T, M, RANKED>(p, &wmap, &bmap, &amap, (int)blockIdx.x);
+}
 
 // The 16-bit form: main CTA `cta` is row block cta / SK, K slice cta % SK.
 template <int BITS, typename T, int MT>
-__global__ void __launch_bounds__(kThreads, 1)
-gemv_wide_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap bmap,
-                 const __grid_constant__ CUtensorMap amap)
+__device__ __forceinline__ void gemv_wide_body(const GemvParams &p, const CUtensorMap *wmap, const CUtensorMap *bmap, const CUtensorMap *amap, int block)
 {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     pdl_launch_dependents();
     mark(p, 0);
-    if ((int)blockIdx.x < p.n_t) {
+    if (block < p.n_t) {
         if (p.pair) cluster_arrive();                // the cluster's barrier counts every thread; nobody here waits on it
-        t_cta<T>(p, smem, &amap, (int)blockIdx.x);
+        t_cta<T>(p, smem, amap, block);
         return;
     }
-    const int cta = (int)blockIdx.x - p.n_t;
+    const int cta = block - p.n_t;
     const int rb = cta / p.SK, slice = cta - rb * p.SK;
     const int tile_first = (int)((long long)rb * p.NT / p.R);
     const int ntile = (int)((long long)(rb + 1) * p.NT / p.R) - tile_first;
     const int g_begin = slice * p.slice_groups, g_count = min(p.slice_groups, p.G - g_begin);
     const uint32_t bars = smem_u32(smem) + p.off_bar;
     if (tid == 0) {
-        prefetch_tensormap(&wmap);
-        if (p.rank > 0) prefetch_tensormap(&bmap);
+        prefetch_tensormap(wmap);
+        if (p.rank > 0) prefetch_tensormap(bmap);
         for (int i = 0; i < p.NS; ++i) {
             mbar_init(bars + 8u * (kBarFull + i), 1);
             mbar_init(bars + 8u * (kBarEmpty + i), kCW);
@@ -1702,10 +1706,10 @@ gemv_wide_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap, c
     bool ok = true;
     if (warp == kProdWarp) {
         if (p.pair) cluster_arrive();
-        if (lane == 0) ok = produce(p, smem, &wmap, tile_first, ntile, g_begin, g_count, kCHGW);
+        if (lane == 0) ok = produce(p, smem, wmap, tile_first, ntile, g_begin, g_count, kCHGW);
     } else if (warp == kEpiWarp) {
         if (p.pair) cluster_arrive();
-        ok = epilogue_wide<T>(p, smem, &bmap, lane, tile_first, ntile, slice);
+        ok = epilogue_wide<T>(p, smem, bmap, lane, tile_first, ntile, slice, cta);
     } else {
         pdl_wait();                                  // x may come from the preceding kernel
         mark(p, 2);
@@ -1720,6 +1724,46 @@ gemv_wide_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap, c
         ok = compute_w16<BITS, T, MT>(p, smem, warp, lane, ntile, g_begin, g_count);
     }
     if (!ok && lane == 0) give_up(p);
+}
+template <int BITS, typename T, int MT>
+__global__ void __launch_bounds__(kThreads, 1)
+gemv_wide_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap bmap,
+                 const __grid_constant__ CUtensorMap amap)
+{
+    gemv_wide_body<BITS, T, MT>(p, &wmap, &bmap, &amap, (int)blockIdx.x);
+}
+
+// Several problems of one form in one launch: the t CTAs of all of them, then their main CTAs.  A block runs the program
+// of its problem with that problem's scratch, counters and plan; nothing synchronises across problems.  What a launch costs
+// besides its weights (the wait for the kernel before, reading and converting x, the last tile's finish) is paid once.
+struct GemvBatch {
+    int n, n_t;                          // problems, t CTAs of all
+    int first_t[kGemvBatchMax], first_main[kGemvBatchMax];
+    GemvParams p[kGemvBatchMax];
+    CUtensorMap w[kGemvBatchMax], b[kGemvBatchMax], a[kGemvBatchMax];
+};
+__device__ __forceinline__ int batch_problem(const GemvBatch &g, int &block)
+{
+    const bool t = block < g.n_t;
+    int i = 0;
+    for (int k = 1; k < g.n; ++k)
+        if (block >= (t ? g.first_t[k] : g.first_main[k])) i = k;
+    block = t ? block - g.first_t[i] : g.p[i].n_t + block - g.first_main[i];
+    return i;
+}
+template <int BITS, typename T, int M, bool RANKED>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) gemv_batch_kernel(const __grid_constant__ GemvBatch g)
+{
+    int block = (int)blockIdx.x;
+    const int i = batch_problem(g, block);
+    gemv_body<BITS, T, M, RANKED>(g.p[i], g.w + i, g.b + i, g.a + i, block);
+}
+template <int BITS, typename T, int MT>
+__global__ void __launch_bounds__(kThreads, 1) gemv_wide_batch_kernel(const __grid_constant__ GemvBatch g)
+{
+    int block = (int)blockIdx.x;
+    const int i = batch_problem(g, block);
+    gemv_wide_body<BITS, T, MT>(g.p[i], g.w + i, g.b + i, g.a + i, block);
 }
 
 // ------------------------------------------------------------------ host side
@@ -1779,13 +1823,13 @@ Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
     if (a.rank > 0) {
         const int per = std::min(kCW, std::max(1, (int)((128 * 1024) / ((size_t)a.rank * 128))));     // one block per warp
         p.n_t = std::min(64, std::max((nblk + per - 1) / per, std::min(nblk, 8)));
-        p.n_t = balanced_t_ctas(p.n_t, nblk, a.rank, p.NT, want);
+        if (tune.main_ctas == 0) p.n_t = balanced_t_ctas(p.n_t, nblk, a.rank, p.NT, want);
         p.t_kb = (nblk + p.n_t - 1) / p.n_t;
         p.n_t = (nblk + p.t_kb - 1) / p.t_kb;
     }
     // All CTAs of a launch, t CTAs included, within one per SM: then every CTA of the NEXT launch finds a free half
     // SM at once.  (Measured: the t CTAs on top of one main CTA per SM cost more, 81 against 72 us per layer step.)
-    p.n_main = std::max(1, std::min(std::max(want - p.n_t, want / 2), p.NT));
+    p.n_main = std::max(1, std::min(tune.main_ctas > 0 ? tune.main_ctas : std::max(want - p.n_t, want / 2), p.NT));
     const int nseg = (p.NT + p.n_main - 1) / p.n_main;
     p.b_box_cols = a.rank <= 16 ? 16 : (a.rank <= 32 ? 32 : 64);      // columns past the rank arrive as zeros
     p.b_swz = p.b_box_cols >= 64 ? 7 : (p.b_box_cols >= 32 ? 3 : 1);
@@ -1888,7 +1932,9 @@ Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
     if (a.rank > 0) {
         const int per = std::min(kCW, std::max(1, (int)((128 * 1024) / ((size_t)a.rank * 128))));     // one block per warp
         p.n_t = std::min(64, std::max((nblk + per - 1) / per, std::min(nblk, 8)));
-        p.n_t = balanced_t_ctas(p.n_t, nblk, a.rank, p.NT, want);
+        // (in a batch every CTA has an SM to itself, so as few t CTAs as fit)
+        p.n_t = tune.main_ctas > 0 ? std::max((nblk + 2 * kCW - 1) / (2 * kCW), (int)(((size_t)nblk * a.rank * 128 + 192 * 1024 - 1) / (192 * 1024)))
+                                   : balanced_t_ctas(p.n_t, nblk, a.rank, p.NT, want);
         p.t_kb = (nblk + p.n_t - 1) / p.n_t;
         p.n_t = (nblk + p.t_kb - 1) / p.t_kb;
     }
@@ -1900,7 +1946,7 @@ Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
     // even number of t CTAs, the odd one out idle, and of main CTAs keeps the clusters among their own kind).
     p.pair = (p.SK == 1 && p.NT >= 2 && want >= 4) ? 1 : 0;
     if (p.pair && (p.n_t & 1)) ++p.n_t;
-    p.R = std::max(1, std::min(std::max(want - p.n_t, want / 2) / p.SK, p.NT));
+    p.R = std::max(1, std::min((tune.main_ctas > 0 ? tune.main_ctas : std::max(want - p.n_t, want / 2)) / p.SK, p.NT));
     if (p.pair && (p.R & 1)) --p.R;
     p.n_main = p.R * p.SK;
     const int nseg = (p.NT + p.R - 1) / p.R;
@@ -1972,11 +2018,11 @@ Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
 const Plan &plan_for(const LinearArgs &a, const GemvTuning &tune)
 {
     struct Entry {
-        int key[8] = {-1};
+        int key[9] = {-1};
         Plan plan;
     };
     static thread_local Entry table[16];
-    const int key[8] = {a.M, a.N, a.K, a.bits, a.rank, tune.max_ctas, tune.poll_limit, tune.test_skip_arrive};
+    const int key[9] = {a.M, a.N, a.K, a.bits, a.rank, tune.max_ctas, tune.poll_limit, tune.test_skip_arrive, tune.main_ctas};
     unsigned h = 0;
     for (int k : key) h = (h ^ (unsigned)k) * 0x9E3779B1u;
     Entry &e = table[h >> 28];
@@ -2081,6 +2127,158 @@ void gemv_workspace_need(const LinearArgs &a, const GemvTuning &tune, size_t *tp
     *partial_floats = (wide && pl.p.SK > 1) ? (size_t)pl.p.NT * pl.p.SK * a.M * kTile : 0;
 }
 
+namespace {
+// Tensor maps of a problem's packed codes, B and A.
+cudaError_t make_maps(const LinearArgs &a, const GemvParams &p, CUtensorMap *wmap, CUtensorMap *bmap, CUtensorMap *amap)
+{
+    const int wpg = (a.bits == 4) ? 16 : 12;
+    MapSpec m{};
+    m.base = a.qw;
+    m.type = CU_TENSOR_MAP_DATA_TYPE_UINT32;
+    m.ndim = 3;
+    m.dims[0] = (cuuint64_t)wpg; m.dims[1] = (cuuint64_t)a.N; m.dims[2] = (cuuint64_t)p.G;
+    m.strides[0] = (cuuint64_t)p.G * wpg * 4; m.strides[1] = (cuuint64_t)wpg * 4;
+    m.box[0] = (cuuint32_t)wpg; m.box[1] = (cuuint32_t)kTile; m.box[2] = (cuuint32_t)(a.M > 2 ? kCHGW : kCHG);
+    m.swizzle = CU_TENSOR_MAP_SWIZZLE_NONE;
+    if (cudaError_t e = cached_map(wmap, m); e != cudaSuccess) return e;
+    *bmap = *amap = *wmap;
+    if (a.rank == 0) return cudaSuccess;
+    const CUtensorMapSwizzle sw = p.b_swz == 7 ? CU_TENSOR_MAP_SWIZZLE_128B : (p.b_swz == 3 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+    const CUtensorMapDataType dt = a.bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+    if (cudaError_t e = cached_map(bmap, matrix_map(a.B, dt, 2, a.rank, a.N, p.b_box_cols, kTile, sw)); e != cudaSuccess) return e;
+    return cached_map(amap, matrix_map(a.A, dt, 2, a.K, a.rank, kTKB, a.rank, CU_TENSOR_MAP_SWIZZLE_128B));
+}
+
+// Plans of a batch's problems: the main CTAs are shared out so that the fullest one has as little as possible (tiles times
+// stages per tile).  Integer form: two CTAs per SM (a launch of several problems lasts long enough that filling the
+// SMs with its own CTAs pays more than letting the next launch's in; 4096 -> 3 x 4096 INT3 rank 64: 8.8 us, 11.3 with one,
+// 15.4 as three launches; 4096 -> 2 x 11008: 12.7, 15.6, 17.2); 16-bit form: one (its CTAs take a whole SM; four tokens:
+// 17.9 and 26.1 us, one by one 28.1 and 31.5).
+struct BatchPlan {
+    Plan plan[kGemvBatchMax];
+    bool ok = false;
+};
+BatchPlan plan_batch(const LinearArgs *a, int count, const GemvTuning &tune)
+{
+    BatchPlan bp;
+    if (count < 1 || count > kGemvBatchMax) return bp;
+    const bool wide = a[0].M > 2;
+    GemvTuning t = tune;
+    t.max_ctas = 0;
+    int n_t = 0;
+    for (int i = 0; i < count; ++i) {
+        t.main_ctas = 2;
+        const Plan &pl = plan_for(a[i], t);
+        if (!pl.ok || (wide && (pl.p.SK != 1 || !pl.p.pair))) return bp;
+        n_t += pl.p.n_t;
+    }
+    auto stages = [&](int i) { const int chg = wide ? kCHGW : kCHG, G = a[i].K / kGroupFast; return (G + chg - 1) / chg; };
+    auto share = [&](int i, int load) {                          // main CTAs with which problem i stays within `load`
+        const int nt = (a[i].N + kTile - 1) / kTile, most = std::max(1, load / stages(i)), c = (nt + most - 1) / most;
+        return wide ? std::max(2, (c + 1) / 2 * 2) : c;
+    };
+    const int budget = std::max(2 * count, (wide ? 1 : 2) * g_sm_count - n_t);
+    int lo = 1, hi = 1;
+    auto total = [&](int load) { int c = 0; for (int i = 0; i < count; ++i) c += share(i, load); return c; };
+    while (total(hi) > budget && hi < (1 << 24)) hi *= 2;
+    while (lo < hi) {
+        const int mid = (lo + hi) / 2;
+        if (total(mid) <= budget) hi = mid;
+        else lo = mid + 1;
+    }
+    for (int i = 0; i < count; ++i) {
+        t.main_ctas = share(i, lo);
+        bp.plan[i] = plan_for(a[i], t);
+        if (!bp.plan[i].ok || (wide && (bp.plan[i].p.R & 1 || bp.plan[i].p.R < 2))) return bp;
+    }
+    bp.ok = true;
+    return bp;
+}
+size_t slot_floats(const GemvParams &p) { return (size_t)(std::max(p.n_t, 1) + 1) * std::max(p.slot_elems, 32); }
+}  // namespace
+
+bool gemv_batch_need(const LinearArgs *a, int count, const GemvTuning &tune, size_t *tslots_floats, int *counters)
+{
+    const BatchPlan bp = plan_batch(a, count, tune);
+    *tslots_floats = 0;
+    *counters = 8 * (count + 1);
+    if (bp.ok)
+        for (int i = 0; i < count; ++i) *tslots_floats += slot_floats(bp.plan[i].p);
+    return bp.ok;
+}
+
+cudaError_t launch_gemv_batch(const LinearArgs *a, int count, Workspace &ws, const GemvTuning &tune, cudaStream_t s, int *launches)
+{
+    const BatchPlan bp = plan_batch(a, count, tune);
+    if (!bp.ok) return cudaErrorInvalidConfiguration;
+    GemvBatch g{};
+    g.n = count;
+    size_t smem = 0, slots = 0;
+    int main_ctas = 0;
+    for (int i = 0; i < count; ++i) {
+        GemvParams &p = g.p[i];
+        p = bp.plan[i].p;
+        p.x = a[i].x; p.scales = a[i].scales; p.zeros = a[i].zeros; p.y = a[i].y;
+        p.tpart = reinterpret_cast<uint32_t *>(ws.tslots) + slots;
+        p.ctr = ws.counters + 8 * (i + 1);
+        p.status = ws.counters + kCtrStatus;
+        slots += slot_floats(p);
+        smem = std::max(smem, bp.plan[i].smem);
+        g.first_t[i] = g.n_t;
+        g.n_t += p.n_t;
+        if (cudaError_t e = make_maps(a[i], p, &g.w[i], &g.b[i], &g.a[i]); e != cudaSuccess) return e;
+    }
+    for (int i = 0; i < count; ++i) {
+        g.first_main[i] = g.n_t + main_ctas;
+        main_ctas += g.p[i].n_main;
+    }
+    const bool wide = a[0].M > 2;
+    auto launch = [&](auto kern, bool &attr_set) {
+        if (!attr_set) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+            if (e != cudaSuccess) return e;
+            attr_set = true;
+        }
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(g.n_t + main_ctas));
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cudaLaunchAttribute at[2];
+        unsigned na = 0;
+        if (tune.pdl) {
+            at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at[na].val.programmaticStreamSerializationAllowed = 1;
+            ++na;
+        }
+        if (wide) {
+            at[na].id = cudaLaunchAttributeClusterDimension;
+            at[na].val.clusterDim.x = 2;
+            at[na].val.clusterDim.y = 1;
+            at[na].val.clusterDim.z = 1;
+            ++na;
+        }
+        cfg.attrs = at;
+        cfg.numAttrs = na;
+        return cudaLaunchKernelEx(&cfg, kern, g);
+    };
+    auto go = [&](auto bits, auto type) {
+        using T = typename decltype(type)::type;
+        constexpr int B = decltype(bits)::value;
+        static bool set[6] = {};
+        if (a[0].M > 8) return launch(gemv_wide_batch_kernel<B, T, 2>, set[0]);
+        if (a[0].M > 2) return launch(gemv_wide_batch_kernel<B, T, 1>, set[1]);
+        if (a[0].rank == 0) return a[0].M == 1 ? launch(gemv_batch_kernel<B, T, 1, false>, set[2]) : launch(gemv_batch_kernel<B, T, 2, false>, set[3]);
+        return a[0].M == 1 ? launch(gemv_batch_kernel<B, T, 1, true>, set[4]) : launch(gemv_batch_kernel<B, T, 2, true>, set[5]);
+    };
+    const bool bf16 = a[0].bf16;
+    const cudaError_t e = a[0].bits == 4 ? (bf16 ? go(std::integral_constant<int, 4>{}, TypeTag<__nv_bfloat16>{}) : go(std::integral_constant<int, 4>{}, TypeTag<__half>{}))
+                                         : (bf16 ? go(std::integral_constant<int, 3>{}, TypeTag<__nv_bfloat16>{}) : go(std::integral_constant<int, 3>{}, TypeTag<__half>{}));
+    if (e == cudaSuccess) ++*launches;
+    return e;
+}
+
 cudaError_t launch_gemv(const LinearArgs &a, Workspace &ws, const GemvTuning &tune, cudaStream_t s, int *launches)
 {
     const bool wide = a.M > 2;
@@ -2101,26 +2299,7 @@ cudaError_t launch_gemv(const LinearArgs &a, Workspace &ws, const GemvTuning &tu
         if (p.n_t + p.n_main > 256) p.trace = nullptr;
     }
     CUtensorMap wmap, bmap, amap;
-    {
-        const int wpg = (a.bits == 4) ? 16 : 12;
-        MapSpec m{};
-        m.base = a.qw;
-        m.type = CU_TENSOR_MAP_DATA_TYPE_UINT32;
-        m.ndim = 3;
-        m.dims[0] = (cuuint64_t)wpg; m.dims[1] = (cuuint64_t)a.N; m.dims[2] = (cuuint64_t)p.G;
-        m.strides[0] = (cuuint64_t)p.G * wpg * 4; m.strides[1] = (cuuint64_t)wpg * 4;
-        m.box[0] = (cuuint32_t)wpg; m.box[1] = (cuuint32_t)kTile; m.box[2] = (cuuint32_t)(wide ? kCHGW : kCHG);
-        m.swizzle = CU_TENSOR_MAP_SWIZZLE_NONE;
-        if (cudaError_t e = cached_map(&wmap, m); e != cudaSuccess) return e;
-    }
-    bmap = wmap;
-    amap = wmap;
-    if (a.rank > 0) {
-        const CUtensorMapSwizzle sw = p.b_swz == 7 ? CU_TENSOR_MAP_SWIZZLE_128B : (p.b_swz == 3 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
-        const CUtensorMapDataType dt = a.bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-        if (cudaError_t e = cached_map(&bmap, matrix_map(a.B, dt, 2, a.rank, a.N, p.b_box_cols, kTile, sw)); e != cudaSuccess) return e;
-        if (cudaError_t e = cached_map(&amap, matrix_map(a.A, dt, 2, a.K, a.rank, kTKB, a.rank, CU_TENSOR_MAP_SWIZZLE_128B)); e != cudaSuccess) return e;
-    }
+    if (cudaError_t me = make_maps(a, p, &wmap, &bmap, &amap); me != cudaSuccess) return me;
     const bool pdl = tune.pdl != 0;
     cudaError_t e = cudaErrorInvalidConfiguration;
     auto go = [&](auto bits, auto type) {

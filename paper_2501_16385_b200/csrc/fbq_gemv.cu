@@ -1799,7 +1799,7 @@ int balanced_t_ctas(int n_t, int nblk, int rank, int tiles, int want)
     return best;
 }
 
-Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
+Plan make_plan_on(const LinearArgs &a, const GemvTuning &tune, int per_sm)
 {
     Plan pl{};
     pl.ok = false;
@@ -1812,7 +1812,7 @@ Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
     const int GB = (a.bits == 4) ? 64 : 48, G = a.K / kGroupFast;
     p.M = a.M; p.N = a.N; p.K = a.K; p.G = G; p.rank = a.rank;
     p.NT = (a.N + kTile - 1) / kTile;
-    const int want = tune.max_ctas > 0 ? tune.max_ctas : g_sm_count;
+    const int want = tune.max_ctas > 0 ? tune.max_ctas : per_sm * g_sm_count;
     const int SPT = (G + kCHG - 1) / kCHG;
     p.stage_bytes = kTile * kCHG * GB;
     p.meta_pitch = (int)align_up((size_t)kTile * G * 2, 16);
@@ -1889,6 +1889,7 @@ Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
     if (need_t > kSmemMax) return pl;
     p.slot_elems = (a.M * a.rank + 31) / 32 * 32;
     p.t_final = (p.n_t * a.M * a.rank > 1024) ? 1 : 0;    // many entries: one t CTA adds the slots for everybody
+    if (per_sm == 2 && std::max(need, need_t) > budget) return pl;
     pl.smem = std::max(need, need_t) + 1024;       // slack for the alignment of the dynamic window
     p.poll_limit = tune.poll_limit > 0 ? (uint32_t)tune.poll_limit : (1u << 20);
     p.test_skip_arrive = tune.test_skip_arrive;
@@ -1897,6 +1898,21 @@ Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
         fprintf(stderr, "gemv plan M %d N %d K %d r %d: n_main %d n_t %d (t_kb %d) NS %d nmeta %d nbuf %d nb %d smem %zu (t CTA %zu)\n",
                 a.M, a.N, a.K, a.rank, p.n_main, p.n_t, p.t_kb, p.NS, p.nmeta, p.nbuf, p.nb, need, need_t);
     return pl;
+}
+
+// Main CTAs: one per SM leaves room for the next launch's, which set themselves up and prefetch; two per SM halve what each
+// has to do, and their compute warps (eight each, alone on their latencies) fill the SM better.  Measured, us per layer of
+// seven linears in a row, one / two per SM: 7B INT4 one token rank 0 40.6 / 38.9, rank 64 47.1 / 45.1, two tokens 54.2 /
+// 46.3, 59.8 / 50.9; 13B INT4 rank 64 79.1 / 70.6, two tokens 96.1 / 76.4; 4096 -> 32000 36.2 / 27.4.  Not where the t CTAs
+// need a whole SM (rank above 64: 51.8 / 73.8, with smaller chunks of A 62.9), nor for INT3 at one token without a
+// sub-branch (40.8 / 41.7: its smaller stages already keep more of them in flight).
+Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
+{
+    if (tune.max_ctas == 0 && tune.main_ctas == 0 && a.rank <= 64 && !(a.bits == 3 && a.rank == 0 && a.M == 1)) {
+        const Plan pl = make_plan_on(a, tune, 2);
+        if (pl.ok) return pl;
+    }
+    return make_plan_on(a, tune, 1);
 }
 
 // Groups per K slice of the 16-bit form: the smallest power-of-two count of slices whose part of x (16-bit, all

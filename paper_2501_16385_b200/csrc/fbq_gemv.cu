@@ -80,7 +80,8 @@ struct GemvParams {
     int off_tA, off_tred;                   // t CTA: blocks of A, reduction buffer
     // 16-bit form (M >= 3): K may be cut into SK slices (CTA = row block x slice) whose partial tiles meet in scratch
     int SK, R;                              // n_main = R * SK
-    int slice_groups;                       // groups per K slice (a multiple of the stage's groups; the last slice takes the rest)
+    int slice_groups;                       // groups per K slice (a multiple of eight; the last slice takes the rest)
+    int chg;                                // groups of a stage: kCW or kGPW * kCW
     int x_pitch;                            // elements between tokens of the staged x
     int off_px, off_tf;                     // (P, X0) table; t as MMA column operands
     int off_sub;                            // t.B^T of the tiles ahead (integer form)
@@ -980,8 +981,12 @@ template <int BITS> __device__ __forceinline__ int frag_pos(int c)
     const int i = c / 10, f = c - 10 * i;
     return (f < 5) ? 2 * (5 * i + f) : 2 * (5 * i + f - 5) + 1;
 }
-constexpr int kCHGW = 8;                     // groups of a stage in the 16-bit form: one per compute warp
-static_assert(kCHGW == kCW, "the 16-bit form gives every compute warp one group of a stage");
+// Groups of a stage in the 16-bit form, per compute warp: two, or one where the shared memory is short (the plan says).  What
+// bounded long runs of tiles here was what a stage costs by itself (its request, its barriers; 0.4 us each with the
+// multiplications left out), not the bytes in flight (sixteen stages instead of eight: nothing).  One group per warp:
+// 4096 -> 44032 INT4 at eight tokens 45.6 us (2.0 TB/s), two: 30.9 (2.9); 4096 -> 11008 16.0 / 12.1.  Four gain another 7 %
+// on the longest launches, but then a long x and two stages no longer fit together.
+constexpr int kGPW = 2;
 
 // x of this CTA's K slice (groups g_begin .. g_begin + g_count) for M tokens: per token and group the sixteen
 // fragment-order pairs of a lane's run as 16-byte units [h_index / 4][lane t][h_index % 4]; (P, X0) per (group, token).
@@ -1065,7 +1070,7 @@ __device__ __forceinline__ void convert_x16(const GemvParams &p, uint8_t *smem, 
     }
 }
 
-// Compute warps of the 16-bit form: stages of eight groups, one group per warp; MT blocks of eight tokens.
+// Compute warps of the 16-bit form: stages of sixteen groups, two per warp; MT blocks of eight tokens.
 template <int BITS, typename T, int MT>
 __device__ __forceinline__ bool compute_w16(const GemvParams &p, uint8_t *smem, int warp, int lane, int ntile, int g_begin, int g_count)
 {
@@ -1073,7 +1078,7 @@ __device__ __forceinline__ bool compute_w16(const GemvParams &p, uint8_t *smem, 
     constexpr int GB = (BITS == 4) ? 64 : 48;
     const int g = lane >> 2, tq = lane & 3;
     const uint32_t sbase = smem_u32(smem), bars = sbase + p.off_bar;
-    const int G = p.G, NS = p.NS, M = p.M, SPT = (g_count + kCHGW - 1) / kCHGW;
+    const int G = p.G, NS = p.NS, M = p.M, chg = p.chg, SPT = (g_count + chg - 1) / chg;
     const uint32_t w_lane = sbase + p.off_ring + (uint32_t)(warp * (kTile * GB) + g * GB + tq * (GB / 4));
     const uint32_t meta0 = sbase + p.off_meta, zoff = (uint32_t)p.meta_pitch, row8 = (uint32_t)(8 * G * 2);
     const uint32_t px_lane = sbase + p.off_px + (uint32_t)(2 * tq) * 8u;
@@ -1093,52 +1098,55 @@ __device__ __forceinline__ bool compute_w16(const GemvParams &p, uint8_t *smem, 
             if (!mbar_wait(bars + 8u * (kBarFull + slot), par)) return false;
             if (first) mark(p, 4);
             first = false;
-            const int gl = st * kCHGW + warp;                          // group of the slice
-            if (gl < g_count) {
-                const uint32_t wa = w_lane + (uint32_t)slot * (uint32_t)p.stage_bytes;
-                uint32_t w0[NW], w1[NW];
-                if constexpr (BITS == 4) {
-                    const uint4 va = lds_v4(wa), vb = lds_v4(wa + 8 * GB);
-                    w0[0] = va.x; w0[1] = va.y; w0[2] = va.z; w0[3] = va.w;
-                    w1[0] = vb.x; w1[1] = vb.y; w1[2] = vb.z; w1[3] = vb.w;
-                } else {
 #pragma unroll
-                    for (int i = 0; i < NW; ++i) {
-                        w0[i] = lds_u32(wa + 4 * i);
-                        w1[i] = lds_u32(wa + 8 * GB + 4 * i);
-                    }
-                }
-                const uint32_t ma = mslot + (uint32_t)(g_begin + gl) * 2u;
-                const float sg = half_bits_to_float(lds_u16(ma)), zg = half_bits_to_float(lds_u16(ma + zoff));
-                const float sh = half_bits_to_float(lds_u16(ma + row8)), zh = half_bits_to_float(lds_u16(ma + row8 + zoff));
-                const float szg = sg * zg, szh = sh * zh;
-                uint32_t ha[16], hb[16];
-                Unpack16<BITS, T>::run(w0, ha);
-                Unpack16<BITS, T>::run(w1, hb);
+            for (int u = 0; u < kGPW; ++u) {
+                const int gl = st * chg + u * kCW + warp;              // group of the slice
+                if (u * kCW < chg && gl < g_count) {
+                    const uint32_t wa = w_lane + (uint32_t)slot * (uint32_t)p.stage_bytes + (uint32_t)(u * kCW * kTile * GB);
+                    uint32_t w0[NW], w1[NW];
+                    if constexpr (BITS == 4) {
+                        const uint4 va = lds_v4(wa), vb = lds_v4(wa + 8 * GB);
+                        w0[0] = va.x; w0[1] = va.y; w0[2] = va.z; w0[3] = va.w;
+                        w1[0] = vb.x; w1[1] = vb.y; w1[2] = vb.z; w1[3] = vb.w;
+                    } else {
 #pragma unroll
-                for (int b = 0; b < MT; ++b) {
-                    // (P, X0) of tokens 8b + 2tq and 8b + 2tq + 1 for this group; one MMA chain starts at -P
-                    const float4 px = lds_f4(px_lane + (uint32_t)(gl * 8 * MT + 8 * b) * 8u);
-                    float t0[4] = {-px.x, -px.z, -px.x, -px.z}, t1[4] = {0.f, 0.f, 0.f, 0.f};
-                    const int token = 8 * b + g;                        // as an MMA column
-                    const uint32_t xg = x_lane + (uint32_t)token * x_tok + (uint32_t)gl * (kGroupFast * 2);
-                    const uint32_t on = token < M ? 1u : 0u;
-#pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        const uint4 xv = lds_v4_if(xg + (uint32_t)q4 * 64u, on);
-                        if (q4 & 1) {
-                            Mma16<T>::run(t1, ha[4 * q4 + 0], hb[4 * q4 + 0], ha[4 * q4 + 1], hb[4 * q4 + 1], xv.x, xv.y);
-                            Mma16<T>::run(t1, ha[4 * q4 + 2], hb[4 * q4 + 2], ha[4 * q4 + 3], hb[4 * q4 + 3], xv.z, xv.w);
-                        } else {
-                            Mma16<T>::run(t0, ha[4 * q4 + 0], hb[4 * q4 + 0], ha[4 * q4 + 1], hb[4 * q4 + 1], xv.x, xv.y);
-                            Mma16<T>::run(t0, ha[4 * q4 + 2], hb[4 * q4 + 2], ha[4 * q4 + 3], hb[4 * q4 + 3], xv.z, xv.w);
+                        for (int i = 0; i < NW; ++i) {
+                            w0[i] = lds_u32(wa + 4 * i);
+                            w1[i] = lds_u32(wa + 8 * GB + 4 * i);
                         }
                     }
-                    // s (mma - P) - (s z) X0
-                    acc[b][0] = fmaf(-szg, px.y, fmaf(sg, t0[0] + t1[0], acc[b][0]));
-                    acc[b][1] = fmaf(-szg, px.w, fmaf(sg, t0[1] + t1[1], acc[b][1]));
-                    acc[b][2] = fmaf(-szh, px.y, fmaf(sh, t0[2] + t1[2], acc[b][2]));
-                    acc[b][3] = fmaf(-szh, px.w, fmaf(sh, t0[3] + t1[3], acc[b][3]));
+                    const uint32_t ma = mslot + (uint32_t)(g_begin + gl) * 2u;
+                    const float sg = half_bits_to_float(lds_u16(ma)), zg = half_bits_to_float(lds_u16(ma + zoff));
+                    const float sh = half_bits_to_float(lds_u16(ma + row8)), zh = half_bits_to_float(lds_u16(ma + row8 + zoff));
+                    const float szg = sg * zg, szh = sh * zh;
+                    uint32_t ha[16], hb[16];
+                    Unpack16<BITS, T>::run(w0, ha);
+                    Unpack16<BITS, T>::run(w1, hb);
+#pragma unroll
+                    for (int b = 0; b < MT; ++b) {
+                        // (P, X0) of tokens 8b + 2tq and 8b + 2tq + 1 for this group; one MMA chain starts at -P
+                        const float4 px = lds_f4(px_lane + (uint32_t)(gl * 8 * MT + 8 * b) * 8u);
+                        float t0[4] = {-px.x, -px.z, -px.x, -px.z}, t1[4] = {0.f, 0.f, 0.f, 0.f};
+                        const int token = 8 * b + g;                        // as an MMA column
+                        const uint32_t xg = x_lane + (uint32_t)token * x_tok + (uint32_t)gl * (kGroupFast * 2);
+                        const uint32_t on = token < M ? 1u : 0u;
+#pragma unroll
+                        for (int q4 = 0; q4 < 4; ++q4) {
+                            const uint4 xv = lds_v4_if(xg + (uint32_t)q4 * 64u, on);
+                            if (q4 & 1) {
+                                Mma16<T>::run(t1, ha[4 * q4 + 0], hb[4 * q4 + 0], ha[4 * q4 + 1], hb[4 * q4 + 1], xv.x, xv.y);
+                                Mma16<T>::run(t1, ha[4 * q4 + 2], hb[4 * q4 + 2], ha[4 * q4 + 3], hb[4 * q4 + 3], xv.z, xv.w);
+                            } else {
+                                Mma16<T>::run(t0, ha[4 * q4 + 0], hb[4 * q4 + 0], ha[4 * q4 + 1], hb[4 * q4 + 1], xv.x, xv.y);
+                                Mma16<T>::run(t0, ha[4 * q4 + 2], hb[4 * q4 + 2], ha[4 * q4 + 3], hb[4 * q4 + 3], xv.z, xv.w);
+                            }
+                        }
+                        // s (mma - P) - (s z) X0
+                        acc[b][0] = fmaf(-szg, px.y, fmaf(sg, t0[0] + t1[0], acc[b][0]));
+                        acc[b][1] = fmaf(-szg, px.w, fmaf(sg, t0[1] + t1[1], acc[b][1]));
+                        acc[b][2] = fmaf(-szh, px.y, fmaf(sh, t0[2] + t1[2], acc[b][2]));
+                        acc[b][3] = fmaf(-szh, px.w, fmaf(sh, t0[3] + t1[3], acc[b][3]));
+                    }
                 }
             }
             __syncwarp();
@@ -1706,7 +1714,7 @@ __device__ __forceinline__ void gemv_wide_body(const GemvParams &p, const CUtens
     bool ok = true;
     if (warp == kProdWarp) {
         if (p.pair) cluster_arrive();
-        if (lane == 0) ok = produce(p, smem, wmap, tile_first, ntile, g_begin, g_count, kCHGW);
+        if (lane == 0) ok = produce(p, smem, wmap, tile_first, ntile, g_begin, g_count, p.chg);
     } else if (warp == kEpiWarp) {
         if (p.pair) cluster_arrive();
         ok = epilogue_wide<T>(p, smem, bmap, lane, tile_first, ntile, slice, cta);
@@ -1915,18 +1923,20 @@ Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
     return make_plan_on(a, tune, 1);
 }
 
-// Groups per K slice of the 16-bit form: the smallest power-of-two count of slices whose part of x (16-bit, all
-// tokens, whole stages) stays below 136 KB of shared memory.
-int wide_slice_groups(int M, int G)
+// Groups per K slice of the 16-bit form (a multiple of eight: the compute warps then have equally many): the smallest
+// power-of-two count of slices whose part of x (16-bit, all tokens) stays within `x_limit` bytes of shared memory.
+constexpr size_t kXLimit = 136 * 1024;           // leaves every shape of the domain room for its stages
+constexpr size_t kXLimitWide = 184 * 1024;       // leaves room only with few tokens or a small rank: tried first
+int wide_slice_groups(int M, int G, size_t x_limit)
 {
     int sk = 1;
-    auto slice_of = [&](int k) { return ((G + k - 1) / k + kCHGW - 1) / kCHGW * kCHGW; };
-    while (sk < 16 && (size_t)M * ((size_t)slice_of(sk) * kGroupFast + 32) * 2 > 136 * 1024) sk *= 2;
+    auto slice_of = [&](int k) { return ((G + k - 1) / k + kCW - 1) / kCW * kCW; };
+    while (sk < 16 && (size_t)M * ((size_t)slice_of(sk) * kGroupFast + 32) * 2 > x_limit) sk *= 2;
     return slice_of(sk);
 }
 
 // Plan of the 16-bit form (3 <= M <= 16): one CTA per SM; K in SK slices when x of all K does not fit.
-Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
+Plan make_plan_wide_on(const LinearArgs &a, const GemvTuning &tune, size_t x_limit, int chg)
 {
     Plan pl{};
     pl.ok = false;
@@ -1940,7 +1950,8 @@ Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
     p.M = a.M; p.N = a.N; p.K = a.K; p.G = G; p.rank = a.rank;
     p.NT = (a.N + kTile - 1) / kTile;
     const int want = tune.max_ctas > 0 ? tune.max_ctas : g_sm_count;
-    p.stage_bytes = kTile * kCHGW * GB;
+    p.chg = chg;
+    p.stage_bytes = kTile * chg * GB;
     p.meta_pitch = (int)align_up((size_t)kTile * G * 2, 16);
     p.n_t = 0;
     p.t_kb = 0;
@@ -1954,8 +1965,7 @@ Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
         p.t_kb = (nblk + p.n_t - 1) / p.n_t;
         p.n_t = (nblk + p.t_kb - 1) / p.t_kb;
     }
-    // K slices: the smallest power of two whose slice of x (16-bit, all tokens) stays below 136 KB
-    p.slice_groups = wide_slice_groups(a.M, G);
+    p.slice_groups = wide_slice_groups(a.M, G, x_limit);
     p.SK = (G + p.slice_groups - 1) / p.slice_groups;
     p.x_pitch = p.slice_groups * kGroupFast + 32;
     // One K slice: the main CTAs all stage the same x, so they come in clusters of two that stage half of it each (an
@@ -1969,7 +1979,7 @@ Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
     // stages per tile of the shortest slice (the last one): the producer runs at most NS stages ahead, that is
     // NS / SPT tiles, and every tile ahead holds a slot of scales and zero points
     const int last_groups = G - (p.SK - 1) * p.slice_groups;
-    const int SPT = (std::min(p.slice_groups, last_groups) + kCHGW - 1) / kCHGW;
+    const int SPT = (std::min(p.slice_groups, last_groups) + chg - 1) / chg;
     p.b_box_cols = a.rank <= 16 ? 16 : (a.rank <= 32 ? 32 : 64);
     p.b_swz = p.b_box_cols >= 64 ? 7 : (p.b_box_cols >= 32 ? 3 : 1);
     p.b_slot_bytes = (int)align_up((size_t)((a.rank + 63) / 64) * kTile * p.b_box_cols * 2, 1024);
@@ -2024,9 +2034,23 @@ Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
     p.test_skip_arrive = tune.test_skip_arrive;
     pl.ok = true;
     if (print_plans())
-        fprintf(stderr, "gemv wide plan M %d N %d K %d r %d: R %d SK %d (slice %d groups) n_t %d NS %d nmeta %d nbuf %d nb %d smem %zu (t CTA %zu)\n",
-                a.M, a.N, a.K, a.rank, p.R, p.SK, p.slice_groups, p.n_t, p.NS, p.nmeta, p.nbuf, p.nb, need, need_t);
+        fprintf(stderr, "gemv wide plan M %d N %d K %d r %d: R %d SK %d (slice %d groups, stage %d) n_t %d NS %d nmeta %d nbuf %d nb %d smem %zu (t CTA %zu)\n",
+                a.M, a.N, a.K, a.rank, p.R, p.SK, p.slice_groups, p.chg, p.n_t, p.NS, p.nmeta, p.nbuf, p.nb, need, need_t);
     return pl;
+}
+
+// Whole K with three stages of sixteen groups, else whole K with stages of eight, else slices.  A slice's partial tiles go
+// through scratch and a counter per tile, which costs more than a shallow ring: 11008 -> 4096 INT4, two slices / whole K:
+// seven tokens rank 64 28.6 / 20.9 us, eight tokens rank 0 25.9 / 22.3; 13824 -> 5120 rank 64, five tokens 38.4 / 30.0, six
+// 40.0 / 33.7.  (Which kernel a call gets does not depend on this: gemv_k_slices counts with kXLimit.)
+Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
+{
+    Plan pl = make_plan_wide_on(a, tune, kXLimitWide, kGPW * kCW);
+    if (pl.ok && pl.p.NS >= 3) return pl;
+    pl = make_plan_wide_on(a, tune, kXLimitWide, kCW);
+    if (pl.ok && pl.p.SK == 1) return pl;
+    pl = make_plan_wide_on(a, tune, kXLimit, kGPW * kCW);
+    return pl.ok ? pl : make_plan_wide_on(a, tune, kXLimit, kCW);
 }
 
 // A plan is a function of the shape and the tuning alone and a call needs it twice (scratch, launch): the host thread
@@ -2119,7 +2143,7 @@ cudaError_t launch_variant(const Plan &pl, const CUtensorMap &wmap, const CUtens
 int gemv_k_slices(int M, int K)
 {
     if (M <= 2 || K < kGroupFast) return 1;
-    const int G = K / kGroupFast, sg = wide_slice_groups(M, G);
+    const int G = K / kGroupFast, sg = wide_slice_groups(M, G, kXLimit);
     return (G + sg - 1) / sg;
 }
 
@@ -2154,7 +2178,7 @@ cudaError_t make_maps(const LinearArgs &a, const GemvParams &p, CUtensorMap *wma
     m.ndim = 3;
     m.dims[0] = (cuuint64_t)wpg; m.dims[1] = (cuuint64_t)a.N; m.dims[2] = (cuuint64_t)p.G;
     m.strides[0] = (cuuint64_t)p.G * wpg * 4; m.strides[1] = (cuuint64_t)wpg * 4;
-    m.box[0] = (cuuint32_t)wpg; m.box[1] = (cuuint32_t)kTile; m.box[2] = (cuuint32_t)(a.M > 2 ? kCHGW : kCHG);
+    m.box[0] = (cuuint32_t)wpg; m.box[1] = (cuuint32_t)kTile; m.box[2] = (cuuint32_t)(a.M > 2 ? p.chg : kCHG);
     m.swizzle = CU_TENSOR_MAP_SWIZZLE_NONE;
     if (cudaError_t e = cached_map(wmap, m); e != cudaSuccess) return e;
     *bmap = *amap = *wmap;
@@ -2188,7 +2212,7 @@ BatchPlan plan_batch(const LinearArgs *a, int count, const GemvTuning &tune)
         if (!pl.ok || (wide && (pl.p.SK != 1 || !pl.p.pair))) return bp;
         n_t += pl.p.n_t;
     }
-    auto stages = [&](int i) { const int chg = wide ? kCHGW : kCHG, G = a[i].K / kGroupFast; return (G + chg - 1) / chg; };
+    auto stages = [&](int i) { const int chg = wide ? kCW : kCHG, G = a[i].K / kGroupFast; return (G + chg - 1) / chg; };
     auto share = [&](int i, int load) {                          // main CTAs with which problem i stays within `load`
         const int nt = (a[i].N + kTile - 1) / kTile, most = std::max(1, load / stages(i)), c = (nt + most - 1) / most;
         return wide ? std::max(2, (c + 1) / 2 * 2) : c;

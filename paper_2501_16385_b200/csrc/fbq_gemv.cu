@@ -1186,14 +1186,15 @@ __device__ __forceinline__ bool compute_w16(const GemvParams &p, uint8_t *smem, 
 // Epilogue warp of the 16-bit form.  Lane (g, tq) finishes rows g and g + 8 of the tile for the tokens 4cb + tq
 // (cb = column block of the up-projection MMA, whose columns 2tq, 2tq + 1 are that token's two 16-bit terms).
 // With K slices the tile's partial sums meet in scratch and the slice that arrives last finishes the tile.
-template <typename T>
+template <typename T, int MT>
 __device__ __forceinline__ bool epilogue_wide(const GemvParams &p, uint8_t *smem, const CUtensorMap *bmap, int lane, int tile_first,
                                               int ntile, int slice, int cta)
 {
     const int g = lane >> 2, tq = lane & 3;
     const uint32_t sbase = smem_u32(smem), bars = sbase + p.off_bar;
     const uint32_t bring = sbase + p.off_B;
-    const int rank = p.rank, M = p.M, nkb = rank / 16, ncb = (M + 3) / 4, SK = p.SK;
+    const int rank = p.rank, M = p.M, nkb = rank / 16, nkb4 = (nkb + 3) & ~3, SK = p.SK;
+    constexpr int NCB = 2 * MT;                                           // column blocks of four tokens
     const int nbox = (rank + 63) / 64;
     const uint32_t box_bytes = (uint32_t)kTile * (uint32_t)p.b_box_cols * 2u;
     auto request_b = [&](int ts) {
@@ -1208,7 +1209,7 @@ __device__ __forceinline__ bool epilogue_wide(const GemvParams &p, uint8_t *smem
 
     prefetch_x(p, cta, lane, (int)sizeof(T));
     uint32_t *s_tf = reinterpret_cast<uint32_t *>(smem + p.off_tf);      // [cb][kb][lane][2]
-    for (int i = lane; i < ncb * nkb * 64; i += 32) s_tf[i] = 0u;
+    for (int i = lane; i < NCB * nkb4 * 16; i += 32) reinterpret_cast<uint4 *>(s_tf)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
     pdl_wait();
     mark(p, 2);
@@ -1274,7 +1275,7 @@ __device__ __forceinline__ bool epilogue_wide(const GemvParams &p, uint8_t *smem
             const uint32_t pk_hi = (uint32_t)(*reinterpret_cast<const uint16_t *>(&h0)) | ((uint32_t)(*reinterpret_cast<const uint16_t *>(&h1)) << 16);
             const uint32_t pk_lo = (uint32_t)(*reinterpret_cast<const uint16_t *>(&l0)) | ((uint32_t)(*reinterpret_cast<const uint16_t *>(&l1)) << 16);
             const int cb = tok >> 2, kb = k0 >> 4, h = (k0 >> 3) & 1, q = (k0 & 7) >> 1;
-            uint32_t *dst = s_tf + ((size_t)(cb * nkb + kb) * 32 + (2 * (tok & 3)) * 4 + q) * 2 + h;
+            uint32_t *dst = s_tf + ((size_t)(cb * nkb4 + kb) * 32 + (2 * (tok & 3)) * 4 + q) * 2 + h;
             dst[0] = pk_hi;
             dst[8] = pk_lo;                                     // four lanes on: the remainder's column
         }
@@ -1287,51 +1288,53 @@ __device__ __forceinline__ bool epilogue_wide(const GemvParams &p, uint8_t *smem
     const uint32_t smask = (uint32_t)p.b_swz, pitch = (uint32_t)p.b_box_cols * 2u;
     const uint32_t tf_lane = sbase + p.off_tf + (uint32_t)lane * 8u;
     // adds t.B^T (rows of B from slot ts % nb) to the sums of a tile and stores its rows of y
-    auto finish_tile = [&](int ts, float (&vg)[4], float (&vh)[4]) -> bool {
+    auto finish_tile = [&](int ts, float (&vg)[NCB], float (&vh)[NCB]) -> bool {
         const int tile = tile_first + ts;
         if (rank > 0) {
             const int bs = ts % p.nb;
             if (!mbar_wait(bars + 8u * (kBarB + bs), (uint32_t)(ts / p.nb) & 1u)) return false;
             const uint32_t bt = bring + (uint32_t)bs * (uint32_t)p.b_slot_bytes;
-            float d[4][4];
+            // Branch-free over blocks of 64 rank indices (what lies past the rank is zero in t) and over all column blocks, two
+            // sums per block: with a branch per MMA and one chain this was 1.4 us of a tile's 1.5, more than its main sums.
+            float d[NCB][2][4];
 #pragma unroll
-            for (int cb = 0; cb < 4; ++cb) d[cb][0] = d[cb][1] = d[cb][2] = d[cb][3] = 0.f;
+            for (int cb = 0; cb < NCB; ++cb)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) d[cb][i >> 2][i & 3] = 0.f;
 #pragma unroll 1
             for (int kc = 0; 4 * kc < nkb; ++kc) {
                 uint32_t af[4][4];
+                uint2 tf[NCB][4];
                 const uint32_t bx = bt + (uint32_t)kc * box_bytes;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const uint32_t c0 = (uint32_t)(q * 32 + tq * 4);                  // bytes into the row
                     const uint32_t o0 = (uint32_t)g * pitch + c0, o1 = o0 + 8u * pitch;
-                    const bool on = 4 * kc + q < nkb;
-                    af[q][0] = on ? lds_u32(bx + swz(o0, smask)) : 0u;
-                    af[q][1] = on ? lds_u32(bx + swz(o1, smask)) : 0u;
-                    af[q][2] = on ? lds_u32(bx + swz(o0 + 16u, smask)) : 0u;
-                    af[q][3] = on ? lds_u32(bx + swz(o1 + 16u, smask)) : 0u;
+                    const uint32_t on = 4 * kc + q < nkb ? 1u : 0u;                    // (stale bytes of the slot may be anything)
+                    af[q][0] = lds_u32_if(bx + swz(o0, smask), on);
+                    af[q][1] = lds_u32_if(bx + swz(o1, smask), on);
+                    af[q][2] = lds_u32_if(bx + swz(o0 + 16u, smask), on);
+                    af[q][3] = lds_u32_if(bx + swz(o1 + 16u, smask), on);
                 }
 #pragma unroll
-                for (int cb = 0; cb < 4; ++cb) {
-                    if (cb < ncb) {
+                for (int cb = 0; cb < NCB; ++cb)
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            if (4 * kc + q < nkb) {
-                                const uint32_t ta = tf_lane + (uint32_t)((cb * nkb + 4 * kc + q) * 32) * 8u;
-                                Mma16<T>::run(d[cb], af[q][0], af[q][1], af[q][2], af[q][3], lds_u32(ta), lds_u32(ta + 4u));
-                            }
-                        }
-                    }
-                }
+                    for (int q = 0; q < 4; ++q) tf[cb][q] = lds_v2(tf_lane + (uint32_t)((cb * nkb4 + 4 * kc + q) * 32) * 8u);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int cb = 0; cb < NCB; ++cb)
+                        Mma16<T>::run(d[cb][q & 1], af[q][0], af[q][1], af[q][2], af[q][3], tf[cb][q].x, tf[cb][q].y);
             }
 #pragma unroll
-            for (int cb = 0; cb < 4; ++cb) {
-                vg[cb] = fmaf(d[cb][0] + d[cb][1], isc, vg[cb]);
-                vh[cb] = fmaf(d[cb][2] + d[cb][3], isc, vh[cb]);
+            for (int cb = 0; cb < NCB; ++cb) {
+                vg[cb] = fmaf((d[cb][0][0] + d[cb][1][0]) + (d[cb][0][1] + d[cb][1][1]), isc, vg[cb]);
+                vh[cb] = fmaf((d[cb][0][2] + d[cb][1][2]) + (d[cb][0][3] + d[cb][1][3]), isc, vh[cb]);
             }
         }
         const int n = tile * kTile + g;
 #pragma unroll
-        for (int cb = 0; cb < 4; ++cb) {
+        for (int cb = 0; cb < NCB; ++cb) {
             const int tok = 4 * cb + tq;
             if (tok < M) {
                 if (n < p.N) y[(size_t)tok * p.N + n] = ActTraits<T>::from_float(vg[cb]);
@@ -1360,9 +1363,9 @@ __device__ __forceinline__ bool epilogue_wide(const GemvParams &p, uint8_t *smem
             const int tile = tile_first + pend_ts;
             const float *pt = p.part + ((size_t)tile * SK) * M * kTile;
             __threadfence();
-            float vg[4], vh[4];
+            float vg[NCB], vh[NCB];
 #pragma unroll
-            for (int cb = 0; cb < 4; ++cb) {
+            for (int cb = 0; cb < NCB; ++cb) {
                 const int tok = 4 * cb + tq;
                 vg[cb] = vh[cb] = 0.f;
                 if (tok < M)
@@ -1382,9 +1385,10 @@ __device__ __forceinline__ bool epilogue_wide(const GemvParams &p, uint8_t *smem
         const int buf = ts % p.nbuf, tile = tile_first + ts;
         if (!mbar_wait_idle_warp(bars + 8u * (kBarSegFull + buf), (uint32_t)(ts / p.nbuf) & 1u)) return false;
         if (ts == 0) mark(p, 4);
-        float vg[4] = {0.f, 0.f, 0.f, 0.f}, vh[4] = {0.f, 0.f, 0.f, 0.f};
+        float vg[NCB], vh[NCB];
 #pragma unroll
-        for (int cb = 0; cb < 4; ++cb) {
+        for (int cb = 0; cb < NCB; ++cb) {
+            vg[cb] = vh[cb] = 0.f;
             const int tok = 4 * cb + tq;
             if (tok < M) {
                 const float *src = s_seg + ((size_t)buf * kCW * M + tok) * kTile;
@@ -1401,7 +1405,7 @@ __device__ __forceinline__ bool epilogue_wide(const GemvParams &p, uint8_t *smem
             // this slice's partial tile to scratch, then count in
             float *pt = p.part + ((size_t)tile * SK) * M * kTile;
 #pragma unroll
-            for (int cb = 0; cb < 4; ++cb) {
+            for (int cb = 0; cb < NCB; ++cb) {
                 const int tok = 4 * cb + tq;
                 if (tok < M) {
                     __stcg(pt + ((size_t)slice * M + tok) * kTile + g, vg[cb]);
@@ -1717,7 +1721,7 @@ __device__ __forceinline__ void gemv_wide_body(const GemvParams &p, const CUtens
         if (lane == 0) ok = produce(p, smem, wmap, tile_first, ntile, g_begin, g_count, p.chg);
     } else if (warp == kEpiWarp) {
         if (p.pair) cluster_arrive();
-        ok = epilogue_wide<T>(p, smem, bmap, lane, tile_first, ntile, slice, cta);
+        ok = epilogue_wide<T, MT>(p, smem, bmap, lane, tile_first, ntile, slice, cta);
     } else {
         pdl_wait();                                  // x may come from the preceding kernel
         mark(p, 2);
@@ -1985,7 +1989,7 @@ Plan make_plan_wide_on(const LinearArgs &a, const GemvTuning &tune, size_t x_lim
     p.b_slot_bytes = (int)align_up((size_t)((a.rank + 63) / 64) * kTile * p.b_box_cols * 2, 1024);
     p.nbuf = std::min(kMaxBuf, std::max(2, std::min(nseg, 3)));
     p.nb = a.rank > 0 ? std::min(kMaxB, std::max(1, std::min(nseg, 2))) : 0;
-    const int ncb = (a.M + 3) / 4, nkb = a.rank / 16;
+    const int ncb = 2 * MT, nkb4 = (a.rank / 16 + 3) / 4 * 4;
     auto layout = [&](int ns) {
         p.NS = ns;
         p.nmeta = std::min(kMaxMeta, (ns - 1) / SPT + 2);
@@ -2009,7 +2013,7 @@ Plan make_plan_wide_on(const LinearArgs &a, const GemvTuning &tune, size_t x_lim
         off += (size_t)a.M * a.rank * 4;
         off = align_up(off, 16);
         p.off_tf = (int)off;
-        off += (size_t)ncb * nkb * 32 * 8;
+        off += (size_t)ncb * nkb4 * 32 * 8;
         off = align_up(off, 1024);
         p.off_B = (int)off;
         off += (size_t)p.nb * p.b_slot_bytes;

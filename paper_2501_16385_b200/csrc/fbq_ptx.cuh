@@ -188,6 +188,12 @@ __device__ __forceinline__ uint4 lds_v4_if(uint32_t a, uint32_t pred)
         : "r"(a), "r"(pred));
     return v;
 }
+__device__ __forceinline__ uint2 lds_v2(uint32_t a)
+{
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
 __device__ __forceinline__ uint32_t lds_u32_if(uint32_t a, uint32_t pred)
 {
     uint32_t v = 0u;

@@ -77,8 +77,8 @@ int fbq_unpack(const uint32_t *qweight, uint8_t *codes, int N, int K, int bits, 
 
 /* Dense fp32 weights W[n][k] = s*(q - z) of the group-wise linear quantiser
  * (Algorithm 1 "linear quantizer").  The product is exact in fp32.  scales and
- * zeros hold fp16 bit patterns.  Test and tooling aid; the linear entry points
- * never materialise W. */
+ * zeros hold fp16 bit patterns.  Test and tooling aid; the decode kernels never
+ * materialise W, the prefill of many tokens keeps a 16-bit copy of it in scratch for the length of a call. */
 int fbq_dequant(const uint32_t *qweight, const uint16_t *scales, const uint16_t *zeros,
                 float *W, int N, int K, int group, int bits, void *stream);
 
@@ -267,7 +267,7 @@ int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int ac
  *                   forced kernel's domain still fall back to the generic one)
  *   "gemv"          1 (default) = M <= 2 runs the streaming decode kernel where its domain allows (see fbq_linear),
  *                   0 = the other decode kernel at every M
- *   "gemv_ctas"     0 = automatic (one main CTA per SM), else an upper bound on the streaming kernel's grid
+ *   "gemv_ctas"     0 = automatic (one or two CTAs per SM), else an upper bound on the streaming kernel's grid
  *   "t_poll_limit"  0 = default, else the number of looks the streaming kernel takes at the t CTAs' slots
  *                   before it gives up with FBQ_ERR_TIMEOUT
  *   "test_skip_t_arrive", "test_prefill_skip_flag", "prefill_flag_polls"
@@ -286,7 +286,8 @@ int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int ac
  *   "decode_t_wait" 1 (default) = a finished tile may wait for t in shared memory while that holds nobody up,
  *                   0 = it is parked in scratch at once (only matters without t CTAs)
  *   "batch_ctas"    CTAs shared out among the problems of a decode-sized fbq_linear_batch (default 400)
- *   "prefill_pair"  1 = token tiles of 256 of the prefill kernel run on CTA pairs (cta_group::2 MMAs,
+ *   "prefill_pair"  (calls of few tiles; with more than three waves of them the prefill runs on CTA pairs anyway)
+ *                   1 = token tiles of 256 of the prefill kernel run on CTA pairs (cta_group::2 MMAs,
  *                   each CTA staging half of the token tile); 0 (default) = one CTA per tile, which
  *                   measured faster
  *   "prefill_split" the prefill kernel at M <= 128, where a shape has fewer 128-row tiles than SMs: K is cut

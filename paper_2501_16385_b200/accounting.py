@@ -2,7 +2,7 @@
 move and compute), used by the benchmark's roofline figures.
 
 Bytes: packed codes + fp16 scales + fp16 zeros + A + B + x + y, each counted
-once; the dense fp16 weight matrix is never materialised.  Flops: 2.M.N.K for
+once; a dense fp16 weight matrix, should a kernel make one, does not count.  Flops: 2.M.N.K for
 the main path and 2.M.r.(K+N) for the sub-branch (Section 3.2 of the paper
 counts M0 = b.d.d and M1 = 2.b.r.d multiply-accumulates for a d x d layer).
 """

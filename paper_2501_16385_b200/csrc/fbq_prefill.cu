@@ -86,7 +86,7 @@ struct PrefillParams {
     int *tflag;               // [token tiles] warps of t CTAs that have stored their part (self-clearing)
     int *tdone;               // [token tiles] main CTAs that have consumed t (self-clearing)
     int splitk, splitt;       // K splits of a main tile / of a t tile (1 unless there are few tokens)
-    float *part;              // [tile][split][128 rows][TOK] fp32 partial tiles (splitk > 1)
+    float *part;              // [tile][split][TOK][128 rows] fp32 partial tiles (splitk > 1)
     int *split_ctr;           // [tile] splits that have stored their partial (self-clearing)
     uint32_t flag_polls;      // looks (256 ns apart) at a token tile's t flag before the wait gives up
     int test_skip_flag;       // test switch: the t CTAs do not raise the flag (the wait for t must run out)
@@ -411,31 +411,41 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     if (!t_ready) { dead = true; break; }
                 }
                 const int j0 = (i - kb_x) * kBK;
-                const int rr = tid & (kHalf - 1);            // token row of the tile
-                if (rr < TOK) {
-                    const int m = m0 + rr;
-                    uint32_t xa[32];
+                // eight lanes per token row, eight rank indices each (a row per lane touches a line per lane: 5 us of a call)
+                const int c = tid & 7, rank4 = p.rank / 4;
+                const bool c_ok = j0 + 8 * c < p.rank;       // rank is a multiple of 8: whole chunks
+#pragma unroll 1
+                for (int u0 = 0; u0 < TOK; u0 += 128) {
+                    const int row0 = u0 + ((tid & (kHalf - 1)) >> 3);
+                    const float4 *ts = reinterpret_cast<const float4 *>(p.t32) + (size_t)(m0 + row0) * rank4 + (j0 + 8 * c) / 4;
+                    float4 ta[4][2];
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        float4 t0 = make_float4(0.f, 0.f, 0.f, 0.f), t1 = t0;
-                        if (m < p.M && j0 + 8 * c < p.rank) {              // rank is a multiple of 8: whole chunks
-                            const float4 *ts = reinterpret_cast<const float4 *>(p.t32 + (size_t)m * p.rank + j0 + 8 * c);
-                            t0 = __ldcg(ts);
-                            t1 = __ldcg(ts + 1);
-                            for (int sp = 1; sp < p.splitt; ++sp) {         // partial t of the other K splits, in order
-                                const float4 *us = ts + (size_t)sp * p.M * p.rank / 4;
-                                const float4 u0 = __ldcg(us), u1 = __ldcg(us + 1);
-                                t0.x += u0.x; t0.y += u0.y; t0.z += u0.z; t0.w += u0.w;
-                                t1.x += u1.x; t1.y += u1.y; t1.z += u1.z; t1.w += u1.w;
-                            }
+                    for (int u = 0; u < 4; ++u) ta[u][0] = ta[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+                    for (int sp = 0; sp < p.splitt; ++sp) {   // partial t of the K splits, in order
+                        float4 pv[4][2];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const bool on = c_ok && m0 + row0 + 32 * u < p.M;
+                            pv[u][0] = on ? __ldcg(ts + (size_t)32 * u * rank4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            pv[u][1] = on ? __ldcg(ts + (size_t)32 * u * rank4 + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
-                        xa[4 * c] = P2<T>::pack(t0.x, t0.y); xa[4 * c + 1] = P2<T>::pack(t0.z, t0.w);
-                        xa[4 * c + 2] = P2<T>::pack(t1.x, t1.y); xa[4 * c + 3] = P2<T>::pack(t1.z, t1.w);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int k = 0; k < 2; ++k) {
+                                ta[u][k].x += pv[u][k].x; ta[u][k].y += pv[u][k].y;
+                                ta[u][k].z += pv[u][k].z; ta[u][k].w += pv[u][k].w;
+                            }
+                        ts += (size_t)p.M * rank4;
                     }
 #pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        sts128(sbase + (uint32_t)s * kStageBytes + (uint32_t)rr * 128u + ((((uint32_t)c) ^ ((uint32_t)rr & 7u)) << 4), xa[4 * c],
-                               xa[4 * c + 1], xa[4 * c + 2], xa[4 * c + 3]);
+                    for (int u = 0; u < 4; ++u) {
+                        const int rr = row0 + 32 * u;
+                        sts128(sbase + (uint32_t)s * kStageBytes + (uint32_t)rr * 128u + ((((uint32_t)c) ^ ((uint32_t)rr & 7u)) << 4),
+                               P2<T>::pack(ta[u][0].x, ta[u][0].y), P2<T>::pack(ta[u][0].z, ta[u][0].w),
+                               P2<T>::pack(ta[u][1].x, ta[u][1].y), P2<T>::pack(ta[u][1].z, ta[u][1].w));
+                    }
                 }
                 pf_fence_proxy_async();
                 __syncwarp();
@@ -461,18 +471,19 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 // ---- K split over S CTAs (TOK = 128: one 32-column chunk per warp).  Every CTA stores its
                 // fp32 partial tile; the CTA that counts in last adds the S partials in split order (the
                 // result does not depend on which CTA that is) and is the one that writes y.
+                // A lane is a feature, so features are the partial tile's contiguous dimension: a warp's store or load is
+                // one line.  (With tokens contiguous it touched 32, and the exchange took most of a short call: 77 tokens
+                // 4096 -> 4096 rank 0 22.4 us, now 16.4; rank 128, where t was read a row per lane as well, 30.8 and 20.9.)
                 const bool mine = m0 + c_begin < p.M;       // uniform over the four warps of a column quarter
                 const size_t slice = (size_t)kBN * TOK;
-                float *pt = p.part + ((size_t)(m_tile * p.nt + n_tile) * S) * slice + (size_t)(32 * q + lane) * TOK + c_begin;
+                float *pt = p.part + ((size_t)(m_tile * p.nt + n_tile) * S) * slice + (size_t)c_begin * kBN + 32 * q + lane;
                 uint32_t v[32];
                 if (mine) {
                     tc_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c_begin, v);
                     tc_wait_ld();
-                    float4 *dst = reinterpret_cast<float4 *>(pt + (size_t)split * slice);
+                    float *dst = pt + (size_t)split * slice;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        __stcg(dst + j, make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                                    __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])));
+                    for (int j = 0; j < 32; ++j) __stcg(dst + j * kBN, __uint_as_float(v[j]));
                 }
                 __threadfence();
                 __syncwarp();
@@ -498,12 +509,12 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     for (int j = 0; j < 32; ++j) acc[j] = 0.f;
 #pragma unroll 1
                     for (int sp = 0; sp < S; ++sp) {
-                        const float4 *src = reinterpret_cast<const float4 *>(pt + (size_t)sp * slice);
+                        const float *src = pt + (size_t)sp * slice;
+                        float u[32];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const float4 u = __ldcg(src + j);
-                            acc[4 * j] += u.x; acc[4 * j + 1] += u.y; acc[4 * j + 2] += u.z; acc[4 * j + 3] += u.w;
-                        }
+                        for (int j = 0; j < 32; ++j) u[j] = __ldcg(src + j * kBN);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) acc[j] += u[j];
                     }
                     unsigned short *sp16 = reinterpret_cast<unsigned short *>(smem + (size_t)c_begin * (kBN * 2)) + 32 * q + lane;
 #pragma unroll

@@ -598,27 +598,29 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         // =================================================== MMA warp
         constexpr uint32_t idesc = (1u << 4) | (P2<T>::kFmt << 7) | (P2<T>::kFmt << 10) | ((uint32_t)(TOK >> 3) << 17) |
                                    ((uint32_t)(kBN >> 4) << 24);
-        bool dead = false;
+        if (lane == 0) {
+            bool dead = false;
+            // descriptors of stage 0; a stage further on is kStageBytes / 16 in their address field
+            const uint64_t xd0 = make_desc(sbase), wd0 = make_desc(sbase + kXBytes);
+            uint32_t s = 0, ph = 0;
 #pragma unroll 1
-        for (int i = 0; i < nkb && !dead; ++i) {
-            const int s = i % kStages;
-            if (lane == 0) {
-                if (!pf_mbar_wait(full0 + 8u * s, (uint32_t)(i / kStages) & 1u) || *abort_flag) {
+            for (int i = 0; i < nkb; ++i) {
+                if (!pf_mbar_wait(full0 + 8u * s, ph) || *abort_flag) {
                     dead = true;
-                } else {
-                    tc_fence_after();
-                    const uint32_t x_base = sbase + (uint32_t)s * kStageBytes, w_base = x_base + kXBytes;
-                    // every operand tile is K-major with 128-byte rows and the 128-byte swizzle, whether it
-                    // arrived by TMA or was written by the producers: 32 bytes per 16 elements of K inside a row
+                    break;
+                }
+                tc_fence_after();
+                const uint64_t xd = xd0 + s * (kStageBytes >> 4), wd = wd0 + s * (kStageBytes >> 4);
+                // every operand tile is K-major with 128-byte rows and the 128-byte swizzle, whether it
+                // arrived by TMA or was written by the producers: 32 bytes per 16 elements of K inside a row
 #pragma unroll
-                    for (int j = 0; j < kBK / 16; ++j)
-                        tc_mma(tmem_base, make_desc(w_base + j * 32), make_desc(x_base + j * 32), idesc, (i > 0 || j > 0) ? 1u : 0u);
-                    tc_commit(empty0 + 8u * s);              // stage is free once these MMAs have read it
+                for (int j = 0; j < kBK / 16; ++j) tc_mma(tmem_base, wd + 2u * j, xd + 2u * j, idesc, (i > 0 || j > 0) ? 1u : 0u);
+                tc_commit(empty0 + 8u * s);                  // stage is free once these MMAs have read it
+                if (++s == (uint32_t)kStages) {
+                    s = 0;
+                    ph ^= 1u;
                 }
             }
-            dead = __shfl_sync(0xffffffffu, (int)dead, 0) != 0;
-        }
-        if (lane == 0) {
             if (dead) {
                 *abort_flag = 1;
                 atomicExch(p.status, (int)FBQ_ERR_TIMEOUT);

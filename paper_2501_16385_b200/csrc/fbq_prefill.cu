@@ -86,6 +86,7 @@ struct PrefillParams {
     int *tflag;               // [token tiles] warps of t CTAs that have stored their part (self-clearing)
     int *tdone;               // [token tiles] main CTAs that have consumed t (self-clearing)
     int splitk, splitt;       // K splits of a main tile / of a t tile (1 unless there are few tokens)
+    int cols;                 // token columns in use of a tile of 128 (a multiple of 16)
     float *part;              // [tile][split][TOK][128 rows] fp32 partial tiles (splitk > 1)
     int *split_ctr;           // [tile] splits that have stored their partial (self-clearing)
     uint32_t flag_polls;      // looks (256 ns apart) at a token tile's t flag before the wait gives up
@@ -126,6 +127,12 @@ __device__ __forceinline__ void pf_fence_proxy_async() { asm volatile("fence.pro
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t on;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(on));
+    return on != 0u;
+}
 // Shared-memory operand descriptor: K-major tile with 128-byte rows (64 16-bit elements) in the
 // 128-byte swizzle (the 16-byte chunk c of row r is stored at chunk c ^ (r % 8)); groups of 8
 // rows are 1024 bytes apart.
@@ -239,6 +246,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     volatile int *split_last = abort_flag + 1;                  // 1: this CTA adds up the K splits of its tile
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t cols = TOK == 256 ? 256u : (uint32_t)p.cols, xbytes = cols * kBK * 2u;     // token columns that are copied and multiplied
     const bool t_role = (int)blockIdx.x < p.n_t;                // t CTA or main CTA
     // (token tile, feature or rank tile, K split): with few tokens there are few tiles, so K is split over
     // several CTAs per tile (splitk main CTAs whose fp32 partial tiles the last one to finish adds up,
@@ -596,37 +604,41 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         tc_fence_before();
     } else if (warp == kMmaWarp) {
         // =================================================== MMA warp
-        constexpr uint32_t idesc = (1u << 4) | (P2<T>::kFmt << 7) | (P2<T>::kFmt << 10) | ((uint32_t)(TOK >> 3) << 17) |
+        const uint32_t idesc = (1u << 4) | (P2<T>::kFmt << 7) | (P2<T>::kFmt << 10) | ((uint32_t)(cols >> 3) << 17) |
                                    ((uint32_t)(kBN >> 4) << 24);
-        if (lane == 0) {
-            bool dead = false;
-            // descriptors of stage 0; a stage further on is kStageBytes / 16 in their address field
-            const uint64_t xd0 = make_desc(sbase), wd0 = make_desc(sbase + kXBytes);
-            uint32_t s = 0, ph = 0;
+        // The whole warp walks the loop and one elected lane issues: the MMAs' operands stay in uniform registers.  Under
+        // `lane == 0` each was moved there first, 390 cycles per block for four MMAs, and the producers waited for it
+        // (18944 x 8192 at 77 tokens 56.2 us, now 50.4; 4096 -> 4096 at 1000 tokens 37.3 and 36.9).
+        bool dead = false;
+        // descriptors of stage 0; a stage further on is kStageBytes / 16 in their address field
+        const uint64_t xd0 = make_desc(sbase), wd0 = make_desc(sbase + kXBytes);
+        uint32_t s = 0, ph = 0;
 #pragma unroll 1
-            for (int i = 0; i < nkb; ++i) {
-                if (!pf_mbar_wait(full0 + 8u * s, ph) || *abort_flag) {
-                    dead = true;
-                    break;
-                }
-                tc_fence_after();
+        for (int i = 0; i < nkb; ++i) {
+            if (!pf_mbar_wait(full0 + 8u * s, ph) || *abort_flag) dead = true;
+            if (__any_sync(0xffffffffu, dead)) {
+                dead = true;
+                break;
+            }
+            tc_fence_after();
+            if (elect_one()) {
                 const uint64_t xd = xd0 + s * (kStageBytes >> 4), wd = wd0 + s * (kStageBytes >> 4);
                 // every operand tile is K-major with 128-byte rows and the 128-byte swizzle, whether it
                 // arrived by TMA or was written by the producers: 32 bytes per 16 elements of K inside a row
 #pragma unroll
                 for (int j = 0; j < kBK / 16; ++j) tc_mma(tmem_base, wd + 2u * j, xd + 2u * j, idesc, (i > 0 || j > 0) ? 1u : 0u);
                 tc_commit(empty0 + 8u * s);                  // stage is free once these MMAs have read it
-                if (++s == (uint32_t)kStages) {
-                    s = 0;
-                    ph ^= 1u;
-                }
+                if (i == nkb - 1) tc_commit(done_bar);       // accumulator complete
             }
-            if (dead) {
-                *abort_flag = 1;
-                atomicExch(p.status, (int)FBQ_ERR_TIMEOUT);
-            } else if (nkb > 0) {
-                tc_commit(done_bar);                         // accumulator complete
+            __syncwarp();
+            if (++s == (uint32_t)kStages) {
+                s = 0;
+                ph ^= 1u;
             }
+        }
+        if (dead && lane == 0) {
+            *abort_flag = 1;
+            atomicExch(p.status, (int)FBQ_ERR_TIMEOUT);
         }
         __syncwarp();
         tc_fence_before();
@@ -644,11 +656,11 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 const uint32_t bar = full0 + 8u * s;
                 const uint32_t xt = sbase + (uint32_t)s * kStageBytes, wt = xt + kXBytes;
                 if (t_role) {
-                    pf_mbar_expect_tx(bar, kXBytes + kWBytes);
+                    pf_mbar_expect_tx(bar, xbytes + kWBytes);
                     tma_load_2d(xt, &xmap, (kb_begin + kb) * kBK, m0, bar);
                     tma_load_2d(wt, &amap, (kb_begin + kb) * kBK, n0, bar);      // rows of A
                 } else if (kb < kb_x) {
-                    pf_mbar_expect_tx(bar, kXBytes);
+                    pf_mbar_expect_tx(bar, xbytes);
                     tma_load_2d(xt, &xmap, (kb_begin + kb) * kBK, m0, bar);
                 } else if (p.t16) {
                     if (kb == kb_x) {                        // every warp of every t CTA of this token tile has stored its part
@@ -667,7 +679,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         }
                         asm volatile("fence.proxy.async;" ::: "memory");
                     }
-                    pf_mbar_expect_tx(bar, kXBytes + kWBytes);
+                    pf_mbar_expect_tx(bar, xbytes + kWBytes);
                     tma_load_2d(xt, &tmap, (kb - kb_x) * kBK, m0, bar);   // t as the token operand
                     tma_load_2d(wt, &bmap, (kb - kb_x) * kBK, n0, bar);   // rows of B
                 } else {
@@ -1406,6 +1418,9 @@ cudaError_t run_prefill(const LinearArgs &a, Workspace &ws, cudaStream_t s, int 
     p.kb_main = a.K / kBK;
     p.kb_slab = (a.rank + kBK - 1) / kBK;
     const int mt = (a.M + TOK - 1) / TOK;
+    // Shared memory is what a block of K waits for (dequantised weights in, operands out): a tile of 128 columns copies
+    // and multiplies only those that have tokens.
+    p.cols = std::min(TOK, (a.M + 15) / 16 * 16);
     p.nt = (a.N + kBN - 1) / kBN;
     p.rt = (a.rank + kBN - 1) / kBN;
     if (PAIR) {                                     // CTAs come in pairs: feature tiles and rank tiles padded to even counts
@@ -1429,7 +1444,7 @@ cudaError_t run_prefill(const LinearArgs &a, Workspace &ws, cudaStream_t s, int 
     p.test_skip_flag = g_pf_skip_flag;
     CUtensorMap xmap, qmap, amap, bmap, ymap;
     cudaError_t e;
-    if ((e = make_map(&xmap, a.x, false, (size_t)a.K, (size_t)a.M, kBK, PAIR ? 128 : TOK, CU_TENSOR_MAP_SWIZZLE_128B, false)) != cudaSuccess)
+    if ((e = make_map(&xmap, a.x, false, (size_t)a.K, (size_t)a.M, kBK, PAIR ? 128 : (TOK == 128 ? p.cols : TOK), CU_TENSOR_MAP_SWIZZLE_128B, false)) != cudaSuccess)
         return e;
     const int wpg = (a.bits == 4) ? 16 : 12;
     if ((e = make_map(&qmap, a.qw, true, (size_t)(a.K / kGroupFast) * wpg, (size_t)a.N, wpg, kBN,
@@ -1443,7 +1458,7 @@ cudaError_t run_prefill(const LinearArgs &a, Workspace &ws, cudaStream_t s, int 
     if (!PAIR && a.rank > 0 && p.splitt == 1) {
         // t goes from the t CTAs to the main CTAs in the activation type, laid out like x, behind the fp32 slices of t
         p.t16 = ws.t_gen + (((size_t)a.M * a.rank + 3) & ~(size_t)3);
-        if ((e = make_map(&tmap, p.t16, false, (size_t)p.rank_pad, (size_t)a.M, kBK, TOK, CU_TENSOR_MAP_SWIZZLE_128B, false)) != cudaSuccess) return e;
+        if ((e = make_map(&tmap, p.t16, false, (size_t)p.rank_pad, (size_t)a.M, kBK, TOK == 128 ? p.cols : TOK, CU_TENSOR_MAP_SWIZZLE_128B, false)) != cudaSuccess) return e;
     }
     if (a.rank > 0) {
         if ((e = make_map(&amap, a.A, false, (size_t)a.K, (size_t)a.rank, kBK, kBN, CU_TENSOR_MAP_SWIZZLE_128B, true)) != cudaSuccess) return e;

@@ -267,7 +267,8 @@ int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int ac
  *                   forced kernel's domain still fall back to the generic one)
  *   "gemv"          1 (default) = M <= 2 runs the streaming decode kernel where its domain allows (see fbq_linear),
  *                   0 = the other decode kernel at every M
- *   "gemv_ctas"     0 = automatic (one or two CTAs per SM), else an upper bound on the streaming kernel's grid
+ *   "gemv_ctas"     0 = automatic (one or two CTAs per SM), else an upper bound on the streaming kernel's grid (the
+ *                   number of SMs is the better choice for linears launched side by side on several streams)
  *   "t_poll_limit"  0 = default, else the number of looks the streaming kernel takes at the t CTAs' slots
  *                   before it gives up with FBQ_ERR_TIMEOUT
  *   "test_skip_t_arrive", "test_prefill_skip_flag", "prefill_flag_polls"

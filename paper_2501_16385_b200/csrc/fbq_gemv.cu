@@ -1917,7 +1917,9 @@ Plan make_plan_on(const LinearArgs &a, const GemvTuning &tune, int per_sm)
 // seven linears in a row, one / two per SM: 7B INT4 one token rank 0 40.6 / 38.9, rank 64 47.1 / 45.1, two tokens 54.2 /
 // 46.3, 59.8 / 50.9; 13B INT4 rank 64 79.1 / 70.6, two tokens 96.1 / 76.4; 4096 -> 32000 36.2 / 27.4.  Not where the t CTAs
 // need a whole SM (rank above 64: 51.8 / 73.8, with smaller chunks of A 62.9), nor for INT3 at one token without a
-// sub-branch (40.8 / 41.7: its smaller stages already keep more of them in flight).
+// sub-branch (40.8 / 41.7: its smaller stages already keep more of them in flight).  Launched from the host without a graph
+// the seven take 60.7 / 47.6.  What pays for it: linears side by side on several streams (q, k, v, then gate, up: 40.5 / 47.2
+// per layer), for which one launch of the batch is the faster way; a mix by size was worse in a row (53.6).
 Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
 {
     if (tune.max_ctas == 0 && tune.main_ctas == 0 && a.rank <= 64 && !(a.bits == 3 && a.rank == 0 && a.M == 1)) {

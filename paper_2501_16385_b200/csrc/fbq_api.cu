@@ -63,7 +63,8 @@ void *direct_y_alias(void *y_host, size_t bytes) { return !g_opt.hostio_direct_y
 
 // Copies of a call's x into its staging buffer.  Small pinned ones are read over the bus by one kernel, all of them
 // together: a copy of the copy engine costs several microseconds each, and the kernel that reads the staging buffer sets
-// itself up meanwhile (dependent launch).
+// itself up meanwhile (dependent launch).  Nothing is read before the preceding kernel of the stream has completed: it may
+// still be writing these buffers itself (the y of a call whose y_host is this call's x_host), or reading the staging buffer.
 constexpr size_t kGatherMost = 512u << 10;
 struct GatherList {
     int n = 0;
@@ -78,10 +79,8 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Gat
     int i = 0;
     for (int k = 1; k < g.n; ++k)
         if (u >= g.first[k]) i = k;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (u < g.first[g.n]) v = g.src[i][u - g.first[i]];
-    asm volatile("griddepcontrol.wait;" ::: "memory");       // the kernel before may still be reading the staging buffer
-    if (u < g.first[g.n]) g.dst[i][u - g.first[i]] = v;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (u < g.first[g.n]) g.dst[i][u - g.first[i]] = g.src[i][u - g.first[i]];
 }
 cudaError_t copy_in(int n, const void *const *src, void *const *dst, const size_t *bytes, cudaStream_t s)
 {

@@ -1353,6 +1353,7 @@ __device__ __forceinline__ void decode_body(const DecodeParams &p, const CUtenso
         if (lane == 0) ready = ld_acquire(p.ctr + kCtrReady);
         ready = __shfl_sync(0xffffffffu, ready, 0);
         if (!ready) return false;
+        __syncwarp();                                // (a shuffle orders no memory: all lanes read t behind lane 0's acquire)
         for (int i = lane; i < p.M * p.rank; i += 32) s_t[i] = ld_cg_f32(p.t + i);
         __syncwarp();
         t_local = true;

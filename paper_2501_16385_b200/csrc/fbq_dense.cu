@@ -104,7 +104,8 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t sr
 }
 
 // Whole warp: lane l looks at the word `word` (NULL: none) until the first `group` lanes see `tag`; returns how many whole
-// groups of lanes do from there on, or 0 when the bound is hit.
+// groups of lanes do from there on, or 0 when the bound is hit.  Votes order no memory: the warp barrier carries what the
+// lanes have acquired to the one lane that issues the copies.
 __device__ __forceinline__ int wait_tags(const DenseParams &p, const uint32_t *word, int group, uint32_t tag, volatile int *quit)
 {
     const unsigned long long t0 = global_ns();
@@ -112,7 +113,10 @@ __device__ __forceinline__ int wait_tags(const DenseParams &p, const uint32_t *w
     for (uint32_t look = 1;; ++look) {
         const unsigned missing = ~__ballot_sync(0xffffffffu, word && load_acquire(word) == tag);
         const int n = (missing ? __ffs(missing) - 1 : 32) / group;
-        if (n) return n;
+        if (n) {
+            __syncwarp();
+            return n;
+        }
         const bool end = *quit || (p.wait_looks && look >= p.wait_looks) || ((look & 63u) == 0u && global_ns() - t0 > kWaitNs);
         if (__any_sync(0xffffffffu, end)) return 0;
         __nanosleep(32);

@@ -416,6 +416,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         seen = seen >= target;
                     }
                     t_ready = __shfl_sync(0xffffffffu, seen, 0) != 0;
+                    __syncwarp();                            // (a shuffle orders no memory: all lanes read t behind lane 0's acquire)
                     if (!t_ready) { dead = true; break; }
                 }
                 const int j0 = (i - kb_x) * kBK;
@@ -1058,6 +1059,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                         seen = seen >= target;
                     }
                     t_ready = __shfl_sync(0xffffffffu, seen, 0) != 0;
+                    __syncwarp();                            // (a shuffle orders no memory: all lanes read t behind lane 0's acquire)
                     if (!t_ready) { dead = true; break; }
                 }
                 const int j0 = (i - p.kb_main) * kBK;

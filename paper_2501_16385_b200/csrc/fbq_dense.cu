@@ -14,6 +14,7 @@
 //   warp 0       operand copies; before the first block of an item it looks at the item's tag (bounded), before the
 //                sub-branch blocks at the tags of t
 //   warp 1       the leader CTA's lane issues tcgen05.mma.cta_group::2: 256 features x `tok` tokens x 16, K in blocks of 64
+//   warp 2       owns the tensor memory; in the leader one lane claims the pair's tiles
 //   warp 3       one lane claims the items
 //   warps 4-7    epilogue: a tile's accumulator leaves while the next tile's is being made (two in tensor memory)
 //
@@ -21,6 +22,9 @@
 // it is chosen to fill the last wave of pairs and to waste no columns on a ragged M.  The low-rank branch is
 // appended as extra K blocks (Section 4.3 adds the up-projection into the shared output): operands t and B.  t = x.A^T
 // comes from tiles of the same loop, the first ones of the launch, rounded once to the activation type.
+// Tiles and items are claimed from counters in the order of need, so whoever waits for a t tile or an item waits for a CTA
+// that is already resident and itself waits for nobody behind it: any number of resident pairs makes progress, also while
+// launches of other streams hold the rest of the SMs.
 // Nothing in scratch has to be zero or cleared: tags carry the launch's number, which the last CTA to leave advances.
 // All waits are bounded: one that runs out raises FBQ_ERR_TIMEOUT in the status word and every role leaves.
 //
@@ -53,14 +57,16 @@ constexpr int kRowLanes = kItemK / 32, kPassRows = 32 / kRowLanes;   // 32 codes
 constexpr int kTTok = 128;                       // tokens of a t tile
 constexpr int kDqWarp = 8, kDqWarps = 16, kThreads = (kDqWarp + kDqWarps) * 32;
 constexpr int kClaims = 4;                       // items claimed ahead
+constexpr int kTiles = 8;                        // ring of claimed tiles (see claim_tiles)
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kYBytes = 32u * 128u * 2u;    // staged part of an output tile: 32 tokens x 128 features
 constexpr uint32_t kYOff = kStages * kStageBytes;
 constexpr uint32_t kBarOff = kYOff + 4u * kYBytes;
-constexpr uint32_t kNumBars = 2 * kStages + 4 + 2 * kClaims;   // full, empty, accumulator full and free, claims full and taken
-constexpr size_t kSmem = kBarOff + kNumBars * 8u + 64u;
-// words of the tag scratch: launch number, CTAs that have left, next item; then tags of items and of t tiles
-constexpr int kTagEpoch = 0, kTagDone = 1, kTagNext = 2, kTagFirst = 4;
+constexpr uint32_t kNumBars = 2 * kStages + 4 + 2 * kClaims + kTiles + 1;   // full, empty, accumulator full and free, claims full and taken, tiles, next tile wanted
+static_assert(kTiles >= kStages + 2 + 3, "a slot of the tile ring must have been read when it is written again");
+constexpr size_t kSmem = kBarOff + kNumBars * 8u + (2 + kClaims + kTiles) * 4u;
+// words of the tag scratch: launch number, CTAs that have left, next item, next tile; then tags of items and of t tiles
+constexpr int kTagEpoch = 0, kTagDone = 1, kTagNext = 2, kTagTile = 3, kTagFirst = 4;
 
 struct DenseParams {
     const void *x;
@@ -91,6 +97,13 @@ __device__ __forceinline__ uint32_t load_acquire(const uint32_t *p)
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+// Four tags, 16-byte aligned.
+__device__ __forceinline__ bool tags_are(const uint32_t *p, uint32_t tag)
+{
+    uint32_t a, b, c, d;
+    asm volatile("ld.acquire.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(a), "=r"(b), "=r"(c), "=r"(d) : "l"(p) : "memory");
+    return ((a ^ tag) | (b ^ tag) | (c ^ tag) | (d ^ tag)) == 0u;
+}
 __device__ __forceinline__ void store_v8(void *p, const uint32_t *v)
 {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]),
@@ -103,15 +116,15 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t sr
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(map), "r"(c0), "r"(c1), "r"(src) : "memory");
 }
 
-// Whole warp: lane l looks at the word `word` (NULL: none) until the first `group` lanes see `tag`; returns how many whole
-// groups of lanes do from there on, or 0 when the bound is hit.  Votes order no memory: the warp barrier carries what the
-// lanes have acquired to the one lane that issues the copies.
-__device__ __forceinline__ int wait_tags(const DenseParams &p, const uint32_t *word, int group, uint32_t tag, volatile int *quit)
+// Whole warp: every lane looks (`there`, an acquiring load) until the first `group` lanes see what they wait for; returns how
+// many whole groups of lanes do from there on, or 0 when the bound is hit.  Votes order no memory: the warp barrier carries
+// what the lanes have acquired to the one lane that issues the copies.
+template <typename F> __device__ __forceinline__ int wait_tags(const DenseParams &p, F there, int group, volatile int *quit)
 {
     const unsigned long long t0 = global_ns();
 #pragma unroll 1
     for (uint32_t look = 1;; ++look) {
-        const unsigned missing = ~__ballot_sync(0xffffffffu, word && load_acquire(word) == tag);
+        const unsigned missing = ~__ballot_sync(0xffffffffu, there());
         const int n = (missing ? __ffs(missing) - 1 : 32) / group;
         if (n) {
             __syncwarp();
@@ -148,6 +161,34 @@ __device__ __forceinline__ void claim_items(const DenseParams &p, uint32_t cfull
         mbar_arrive(cfull0 + 8u * (i % kClaims));
         if (item >= n_items) return;
     }
+}
+
+// The pair's tiles, t tiles first, are claimed by one lane of the leader and handed to both CTAs: the copying, the issuing
+// and the epilogue warps read tile i from slot i % kTiles of their CTA's ring.  Tile i is claimed when the copies of tile
+// i - 1 are half issued, which hides the claim and deals the tiles out by need (t tiles one per pair, unless fewer pairs
+// than t tiles are resident).  A slot is free by then without asking: the copies of tile i - 2 have been issued, so the
+// stages of tile i - 5 have been multiplied (kStages stages, at least one per tile; each needs the copies of both CTAs) and
+// the epilogues of both CTAs are through with tile i - 7 (two accumulators); slot i % kTiles held tile i - 8.
+__device__ __forceinline__ void claim_tiles(const DenseParams &p, int n_all, uint32_t tfull0, uint32_t want, volatile int *tiles, volatile int *quit)
+{
+    const uint32_t peer_slots = mapa_shared(smem_u32(const_cast<int *>(tiles)), 1), full_a = mapa_shared(tfull0, 0), full_b = mapa_shared(tfull0, 1);
+#pragma unroll 1
+    for (uint32_t i = 0;; ++i) {
+        if (i > 0 && !umma::wait_cluster(want, (i - 1u) & 1u, quit)) return;
+        const uint32_t slot = i % kTiles;
+        const int q = min((int)atomicAdd(p.tags + kTagTile, 1u), n_all);
+        tiles[slot] = q;
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_slots + 4u * slot), "r"(q) : "memory");
+        umma::arrive_cluster(full_a + 8u * slot);
+        umma::arrive_cluster(full_b + 8u * slot);
+        if (q >= n_all) return;
+    }
+}
+// The pair's i-th tile (n_all and above: there are no more), or -1 when the wait for it is given up.
+__device__ __forceinline__ int tile_at(uint32_t i, uint32_t tfull0, const volatile int *tiles, volatile int *quit)
+{
+    const uint32_t slot = i % kTiles;
+    return umma::wait_cluster(tfull0 + 8u * slot, (i / kTiles) & 1u, quit) ? tiles[slot] : -1;
 }
 
 // A dequantising warp does its unit (kUnitRows rows x kItemK k) of every item of its CTA.  Alone on its latencies (codes
@@ -254,12 +295,11 @@ dense_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ C
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const uint32_t full0 = sbase + kBarOff, empty0 = full0 + 8u * kStages, accf0 = empty0 + 8u * kStages, acce0 = accf0 + 16u,
-                   cfull0 = acce0 + 16u, cempty0 = cfull0 + 8u * kClaims;
+                   cfull0 = acce0 + 16u, cempty0 = cfull0 + 8u * kClaims, tfull0 = cempty0 + 8u * kClaims, want = tfull0 + 8u * kTiles;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kBarOff + kNumBars * 8u);
-    volatile int *quit = reinterpret_cast<volatile int *>(tmem_slot + 1), *ring = quit + 1;
+    volatile int *quit = reinterpret_cast<volatile int *>(tmem_slot + 1), *ring = quit + 1, *tiles = ring + kClaims;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t cr = cluster_ctarank();                       // 0: leader
-    const int pair = (int)blockIdx.x >> 1, n_pairs = (int)gridDim.x >> 1;
     const int kbx = p.K / kBK, slab = p.rank_pad / kBK;
     const int n_all = p.n_t + p.nft * p.ntt;
     uint32_t *const t_tags = p.tags + kTagFirst + p.nft * p.nkc * kUnits;
@@ -278,6 +318,8 @@ dense_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ C
             mbar_init(cfull0 + 8u * i, 1);
             mbar_init(cempty0 + 8u * i, kDqWarps);
         }
+        for (int i = 0; i < kTiles; ++i) mbar_init(tfull0 + 8u * i, 1);
+        mbar_init(want, 1);
         *quit = 0;
         fence_barrier_init();
     }
@@ -319,7 +361,10 @@ dense_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ C
         uint32_t s = 0, phase = 1u;                              // parity of the stage's previous use
         bool first = true;
 #pragma unroll 1
-        for (int q = pair; q < n_all && ok; q += n_pairs) {
+        for (uint32_t it = 0; ok; ++it) {
+            const int q = tile_at(it, tfull0, tiles, quit);
+            if (q < 0) ok = false;
+            if (!__all_sync(0xffffffffu, q >= 0 && q < n_all)) break;
             const bool t_role = q < p.n_t;
             const int ft = t_role ? 0 : (q - p.n_t) / p.ntt, tt = t_role ? 0 : (q - p.n_t) % p.ntt;
             const int wrow = t_role ? 128 * (int)cr : ft * kFeat + 128 * (int)cr;
@@ -330,15 +375,19 @@ dense_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ C
             const uint32_t bytes = t_role ? (uint32_t)p.a_rows * (p.rank_pad > 128 ? 2u : 1u) * (kBK * 2u) + kTTok * (kBK * 2u)
                                           : 2u * kHalfBytes + (uint32_t)p.tok * (kBK * 2u);
             const int nkb = t_role ? kbx : kbx + slab;
+            const int half_way = nkb / (2 * kPer) * kPer;
             int ready = 0;                                       // items of this feature tile known to be there
 #pragma unroll 1
             for (int kb = 0; kb < nkb; kb += kPer) {
                 const int nb = min(kPer, nkb - kb);
+                if (kb == half_way && cr == 0 && lane == 0) mbar_arrive(want);
                 if (!t_role && kb < kbx && kb / (kItemK / kBK) >= ready) {
-                    constexpr int half = kUnits / 2;              // units of this CTA's rows
-                    const int kc = ready + lane / half;
-                    const uint32_t *word = p.tags + kTagFirst + (ft * p.nkc + kc) * kUnits + (int)cr * half + lane % half;
-                    const int n = wait_tags(p, kc < p.nkc ? word : nullptr, half, tag, quit);
+                    // a lane looks at four of the kUnits / 2 tags of this CTA's rows: sixteen items at a time (a look takes
+                    // about as long as the copies run ahead, so there should be few)
+                    constexpr int group = kUnits / 2 / 4;
+                    const int kc = ready + lane / group;
+                    const uint32_t *word = p.tags + kTagFirst + (ft * p.nkc + kc) * kUnits + (int)cr * (kUnits / 2) + lane % group * 4;
+                    const int n = wait_tags(p, [&] { return kc < p.nkc && tags_are(word, tag); }, group, quit);
                     if (n == 0) { ok = false; break; }
                     ready += n;
                     if (lane == 0) asm volatile("fence.proxy.async;" ::: "memory");
@@ -346,7 +395,7 @@ dense_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ C
                 if (kb == kbx) {                                 // t of this tile's tokens, from both CTAs of each t tile
                     const int t0 = tt * p.tok / kTTok, t1 = (min(p.M, (tt + 1) * p.tok) + kTTok - 1) / kTTok;
                     for (int i = 2 * t0; i < 2 * t1;) {
-                        const int n = wait_tags(p, i + lane < 2 * t1 ? t_tags + i + lane : nullptr, 1, tag, quit);
+                        const int n = wait_tags(p, [&] { return i + lane < 2 * t1 && load_acquire(t_tags + i + lane) == tag; }, 1, quit);
                         if (n == 0) { ok = false; break; }
                         i += n;
                     }
@@ -378,7 +427,10 @@ dense_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ C
             uint32_t s = 0, phase = 0, it = 0;
             const uint64_t desc0 = umma::desc_k128(sbase);
 #pragma unroll 1
-            for (int q = pair; q < n_all && ok; q += n_pairs, ++it) {
+            for (; ok; ++it) {
+                const int q = tile_at(it, tfull0, tiles, quit);
+                if (q < 0) ok = false;
+                if (q < 0 || q >= n_all) break;
                 const bool t_role = q < p.n_t;
                 const int nkb = t_role ? kbx : kbx + slab;
                 const uint32_t idesc = umma::idesc_f16(P2<T>::kFmt, 2 * 128, (uint32_t)(t_role ? kTTok : p.tok));
@@ -407,6 +459,9 @@ dense_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ C
                 if (ok) umma::commit_pair(accf0 + 8u * buf);
             }
         }
+    } else if (warp == 2) {
+        if (cr == 0 && lane == 0) claim_tiles(p, n_all, tfull0, want, tiles, quit);
+        __syncwarp();
     } else if (warp == 3) {
         if (lane == 0) claim_items(p, cfull0, cempty0, ring);
     } else if (warp >= 4 && warp < kDqWarp) {
@@ -415,7 +470,10 @@ dense_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ C
         const uint32_t lacce0 = mapa_shared(acce0, 0);
         uint32_t it = 0, staged = 0;
 #pragma unroll 1
-        for (int q = pair; q < n_all; q += n_pairs, ++it) {
+        for (;; ++it) {
+            const int q = tile_at(it, tfull0, tiles, quit);
+            if (q < 0) ok = false;
+            if (q < 0 || q >= n_all) break;
             const uint32_t buf = it & 1u;
             if (!umma::wait_cluster(accf0 + 8u * buf, (it >> 1) & 1u, quit)) { ok = false; break; }
             umma::fence_after();
@@ -492,6 +550,7 @@ dense_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ C
         if (atomicAdd(p.tags + kTagDone, 1u) == gridDim.x - 1) { // the last CTA: the next launch's tags are other ones
             p.tags[kTagDone] = 0;
             p.tags[kTagNext] = 0;
+            p.tags[kTagTile] = 0;
             __threadfence();
             p.tags[kTagEpoch] = tag;
         }

@@ -29,3 +29,27 @@ def test_dense_prefill_exact_class_is_bitwise_and_repeats():
         y = torch_to_f64(dev.run(fbq), "f16")
         assert fbq.poll_status() == 0
         assert np.array_equal(y[:, rows], want)
+
+
+def test_dense_prefill_on_streams_that_share_the_sms():
+    # 6000 tokens are 47 t tiles: more than half of the pairs, so launches that share the SMs cannot each have a pair per
+    # t tile.  The waits of a launch must not depend on that: every call returns without a time-out and with the same bits
+    # as alone (sums of a tile are made by one pair in a fixed order, whichever pair that is).
+    import torch
+    import paper_2501_16385_b200 as fbq
+    devs = [DeviceLinear(make_linear(6000, 5128 + 256 * i, 384, 4, 64, dtype="bf16", seed=3200 + i), fbq) for i in range(3)]
+    alone = [d.run(fbq) for d in devs]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in devs]
+    for s in streams:
+        s.wait_stream(torch.cuda.current_stream())
+    for _ in range(10):
+        got = []
+        for s, d in zip(streams, devs):
+            with torch.cuda.stream(s):
+                got.append([d.run(fbq) for _ in range(3)])
+        torch.cuda.synchronize()
+        for s in streams:
+            assert fbq.poll_status(s) == 0
+        for ys, want in zip(got, alone):
+            assert all(torch.equal(y, want) for y in ys)

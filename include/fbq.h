@@ -110,7 +110,10 @@ int fbq_dequant(const uint32_t *qweight, const uint16_t *scales, const uint16_t 
  * the first time a stream sees a larger shape.  Growing allocates (and, for a buffer that exists,
  * synchronises the stream and frees the old one): a call that would have to grow scratch while
  * `stream` is being captured returns FBQ_ERR_UNSUPPORTED and queues nothing, and a graph captured
- * EARLIER on that stream keeps pointers to a buffer that a later, larger call replaces.  So: run
+ * EARLIER on that stream keeps pointers to a buffer that a later, larger call replaces.  (The largest scratch,
+ * up to 512 MB per stream for the 16-bit weights of prompts of more than three waves of tiles, is not
+ * required: where it cannot be had, in a capture or because memory is used up, the prefill kernel that
+ * does without it runs, with the same rounding of weights and t.)  So: run
  * the largest shape of every kind once on a stream, outside capture, before capturing on it.
  * After FBQ_ERR_TIMEOUT the stream's counters are unfinished: call fbq_poll_status (it resets
  * them) before issuing more work on that stream. */

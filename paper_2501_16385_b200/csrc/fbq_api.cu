@@ -302,21 +302,26 @@ int run_linear(const LinearArgs &a, cudaStream_t s, int decode_ctas = 0)
         size_t have_c = (size_t)ws->n_counters, need_t = 0, need_p = 0;
         int need_c = 0;
         prefill_workspace_need(a, &need_c, &need_t, &need_p);
-        if (prefill_dense(a)) {
+        // The dense kernel's matrix of weights is the largest scratch by far and the other kernel computes the same call without
+        // it: where it cannot be had (device memory is used up, or the stream is being captured) that one runs.
+        bool dense = prefill_dense(a);
+        if (dense) {
             size_t need_w = 0, need_tags = 0, tf = 0;
             dense_workspace_need(a, &need_w, &need_tags, &tf);
             char *w16 = static_cast<char *>(ws->w16);
             e = grow(w16, ws->w16_bytes, need_w, 1, s);
             ws->w16 = w16;
             if (e == cudaSuccess) e = grow(ws->tags, ws->n_tags, need_tags, sizeof(uint32_t), s);
-            if (e != cudaSuccess) return grow_status(e);
-            need_t = std::max(need_t, tf);
+            dense = e == cudaSuccess;
+            if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();
+            else if (!dense && e != cudaErrorStreamCaptureUnsupported) return FBQ_ERR_CUDA;
+            if (dense) need_t = std::max(need_t, tf);
         }
         if ((e = grow(ws->counters, have_c, (size_t)need_c, sizeof(int), s)) != cudaSuccess) return grow_status(e);
         ws->n_counters = (int)have_c;
         if (need_t > 0 && (e = grow(ws->t_gen, ws->t_gen_floats, need_t, sizeof(float), s)) != cudaSuccess) return grow_status(e);
         if (need_p > 0 && (e = grow(ws->partial, ws->partial_floats, need_p, sizeof(float), s)) != cudaSuccess) return grow_status(e);
-        e = launch_prefill(a, *ws, s, &launches);
+        e = launch_prefill(a, dense, *ws, s, &launches);
         if (e == cudaErrorInvalidConfiguration) {
             (void)cudaGetLastError();
             kernel = FBQ_KERNEL_GENERIC;

@@ -127,8 +127,9 @@ void dense_workspace_need(const LinearArgs &a, size_t *w16_bytes, size_t *tags, 
 cudaError_t launch_dense(const LinearArgs &a, Workspace &ws, const PrefillTuning &tune, cudaStream_t s, int *launches);
 
 bool prefill_supported(const LinearArgs &a);
-bool prefill_dense(const LinearArgs &a);       // the dense kernel takes this call (fbq_dense.cu)
+bool prefill_dense(const LinearArgs &a);       // the dense kernel is the faster one for this call (fbq_dense.cu)
 void prefill_workspace_need(const LinearArgs &a, int *counters, size_t *t_floats, size_t *partial_floats);
-cudaError_t launch_prefill(const LinearArgs &a, Workspace &ws, cudaStream_t s, int *launches);
+// dense: by the dense kernel, whose scratch (dense_workspace_need) is there
+cudaError_t launch_prefill(const LinearArgs &a, bool dense, Workspace &ws, cudaStream_t s, int *launches);
 
 }  // namespace fbq

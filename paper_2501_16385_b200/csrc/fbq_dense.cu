@@ -6,8 +6,8 @@
 // their way.  Dequantising a weight tile where it is multiplied does it once per token tile (four times at 1024 tokens)
 // and every block of K waits for it: the kernel that does so reaches 0.5 of the tensor rate.  Here one persistent launch
 // does both halves once: warps that have nothing to do with the MMAs turn the codes into 16-bit weights in a scratch
-// matrix W16 (which lives in L2: it is written shortly before it is read, at the same addresses in every call), and the
-// MMA loop is a plain dense one, all of whose operands arrive by TMA.
+// matrix W16 (read from L2 mostly: a part of it is written shortly before the tiles in work read it; the whole of it can be
+// larger than L2), and the MMA loop is a plain dense one, all of whose operands arrive by TMA.
 //
 //   warps 8-23   dequantise units of 16 rows x 256 k of W16, claimed from a counter in the order in which the tiles
 //                need them (so whichever CTAs are resident do all of them), and tag each finished unit
@@ -590,8 +590,22 @@ int token_tile(int M, int nft, int kb)
     return best;
 }
 
+// Feature rows of one launch: W16 stays within kW16Most bytes per stream, so a wider matrix (an output head) goes in launches
+// of equal parts, whole tiles each.  Small parts end in more partly filled waves (8192 -> 32000, 500 MB, at 1000 tokens: 495 us
+// whole, 600 in two), large ones cost nothing (8192 -> 128256, 2.1 GB, at 1000 and 2000 tokens: 1930 and 3650 us in four, 2200
+// and 4100 whole).  0: not even one tile's rows fit.
+constexpr size_t kW16Most = (size_t)512 << 20;
+int launch_rows(int N, int K)
+{
+    const size_t most = kW16Most / ((size_t)K * 2) / kFeat * kFeat;
+    if (most == 0) return 0;
+    const size_t n = (N + most - 1) / most;
+    return (int)std::min((size_t)N, ((N + n - 1) / n + kFeat - 1) / kFeat * kFeat);
+}
+
+// a: the rows of one launch; y has rows of `pitch` elements.
 template <int BITS, typename T>
-cudaError_t run(const LinearArgs &a, Workspace &ws, const PrefillTuning &tune, cudaStream_t s)
+cudaError_t run(const LinearArgs &a, int pitch, Workspace &ws, const PrefillTuning &tune, cudaStream_t s)
 {
     DenseParams p{};
     p.x = a.x; p.qw = a.qw; p.scales = a.scales; p.zeros = a.zeros; p.y = a.y;
@@ -616,7 +630,9 @@ cudaError_t run(const LinearArgs &a, Workspace &ws, const PrefillTuning &tune, c
     const CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_128B;
     CUtensorMap xmap, xtmap, wmap, amap, bmap, tmap, ymap;
     cudaError_t e;
-    if ((e = encode_map(&ymap, matrix_map(a.y, dt, 2, a.N, a.M, 128, 16, CU_TENSOR_MAP_SWIZZLE_NONE))) != cudaSuccess) return e;
+    MapSpec yspec = matrix_map(a.y, dt, 2, a.N, a.M, 128, 16, CU_TENSOR_MAP_SWIZZLE_NONE);
+    yspec.strides[0] = (cuuint64_t)pitch * 2;
+    if ((e = encode_map(&ymap, yspec)) != cudaSuccess) return e;
     if ((e = encode_map(&xmap, matrix_map(a.x, dt, 2, a.K, a.M, kBK, p.tok / 2, sw))) != cudaSuccess) return e;
     if ((e = cached_map(&wmap, matrix_map(ws.w16, dt, 2, a.K, a.N, kBK, 128, sw))) != cudaSuccess) return e;
     xtmap = amap = bmap = tmap = xmap;
@@ -654,24 +670,36 @@ cudaError_t run(const LinearArgs &a, Workspace &ws, const PrefillTuning &tune, c
 // 13B layer 2540 / 2840.
 bool prefill_dense(const LinearArgs &a)
 {
-    if (a.M <= 128) return false;
-    const int nft = (a.N + kFeat - 1) / kFeat, tok = token_tile(a.M, nft, a.K / kBK);
+    const int rows = launch_rows(a.N, a.K);
+    if (a.M <= 128 || rows == 0) return false;
+    const int nft = (rows + kFeat - 1) / kFeat, tok = token_tile(a.M, nft, a.K / kBK);
     return nft * ((a.M + tok - 1) / tok) > 3 * pairs_of_device();
 }
 
 void dense_workspace_need(const LinearArgs &a, size_t *w16_bytes, size_t *tags, size_t *t_floats)
 {
-    const size_t nft = (a.N + kFeat - 1) / kFeat, nkc = (a.K + kItemK - 1) / kItemK;
-    *w16_bytes = (size_t)a.N * a.K * 2;
+    const size_t rows = launch_rows(a.N, a.K), nft = (rows + kFeat - 1) / kFeat, nkc = (a.K + kItemK - 1) / kItemK;
+    *w16_bytes = rows * a.K * 2;
     *tags = kTagFirst + nft * nkc * kUnits + 2 * ((size_t)(a.M + kTTok - 1) / kTTok) + 32;
     *t_floats = (size_t)a.M * ((a.rank + kBK - 1) / kBK * kBK) / 2 + 4;
 }
 
 cudaError_t launch_dense(const LinearArgs &a, Workspace &ws, const PrefillTuning &tune, cudaStream_t s, int *launches)
 {
-    const cudaError_t e = a.bits == 4 ? (a.bf16 ? run<4, __nv_bfloat16>(a, ws, tune, s) : run<4, __half>(a, ws, tune, s))
-                                      : (a.bf16 ? run<3, __nv_bfloat16>(a, ws, tune, s) : run<3, __half>(a, ws, tune, s));
-    if (e == cudaSuccess) ++*launches;
+    const int rows = launch_rows(a.N, a.K);
+    cudaError_t e = cudaSuccess;
+    for (int n0 = 0; n0 < a.N && e == cudaSuccess; n0 += rows) {          // (each makes t anew: rank of `rows` of its operations)
+        LinearArgs c = a;
+        c.N = std::min(rows, a.N - n0);
+        c.qw = a.qw + (size_t)n0 * a.K / 32 * a.bits;
+        c.scales = a.scales + (size_t)n0 * (a.K / kGroupFast);
+        c.zeros = a.zeros + (size_t)n0 * (a.K / kGroupFast);
+        if (a.rank > 0) c.B = static_cast<const uint16_t *>(a.B) + (size_t)n0 * a.rank;
+        c.y = static_cast<uint16_t *>(a.y) + n0;
+        e = a.bits == 4 ? (a.bf16 ? run<4, __nv_bfloat16>(c, a.N, ws, tune, s) : run<4, __half>(c, a.N, ws, tune, s))
+                        : (a.bf16 ? run<3, __nv_bfloat16>(c, a.N, ws, tune, s) : run<3, __half>(c, a.N, ws, tune, s));
+        if (e == cudaSuccess) ++*launches;
+    }
     return e;
 }
 

@@ -1512,13 +1512,13 @@ void prefill_workspace_need(const LinearArgs &a, int *counters, size_t *t_floats
 // ws.t_gen must hold M x rank floats and ws.counters prefill_counters_need(M) ints (the caller
 // grows them; new counters start at zero and the kernel leaves them at zero).
 // Operands that are not 16-byte aligned are refused (the caller then takes the generic kernel).
-cudaError_t launch_prefill(const LinearArgs &a, Workspace &ws, cudaStream_t s, int *launches)
+cudaError_t launch_prefill(const LinearArgs &a, bool dense, Workspace &ws, cudaStream_t s, int *launches)
 {
     if (!prefill_supported(a)) return cudaErrorInvalidConfiguration;
     if (!aligned16(a.x) || !aligned16(a.y) || !aligned16(a.qw) || !aligned16(a.scales) || !aligned16(a.zeros) ||
         (a.rank > 0 && (!aligned16(a.A) || !aligned16(a.B))))
         return cudaErrorInvalidConfiguration;
-    if (prefill_dense(a)) {
+    if (dense) {
         PrefillTuning t;
         t.pdl = g_pf_pdl;
         t.flag_polls = g_pf_flag_polls;

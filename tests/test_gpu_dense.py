@@ -53,3 +53,49 @@ def test_dense_prefill_on_streams_that_share_the_sms():
             assert fbq.poll_status(s) == 0
         for ys, want in zip(got, alone):
             assert all(torch.equal(y, want) for y in ys)
+
+
+def test_dense_prefill_of_a_matrix_wider_than_the_scratch():
+    # 62000 x 4352 weights are 540 MB in 16 bits: two launches of 31232 and 30768 rows
+    import torch
+    import paper_2501_16385_b200 as fbq
+    M, N, K = 1000, 62000, 4352
+    inp = make_linear(M, N, K, 3, 16, dtype="f16", seed=3300)
+    rows = np.unique(np.concatenate([[0, 1, 32767, 32768, N - 1], np.arange(31224, 31240), np.random.default_rng(1).choice(N, 12)]))
+    fbq.release_workspaces()
+    before = fbq.launch_count()
+    check_parity(inp, fbq, expect_kernel=fbq.KERNEL_PREFILL, n_list=rows, threads=16, floor=2e-5)
+    assert fbq.launch_count() - before == 3                  # one of them packs the codes
+    dev = DeviceLinear(inp, fbq)
+    dev.run(fbq)
+    torch.cuda.synchronize()
+    y = dev.run(fbq)
+    assert torch.equal(y, dev.run(fbq))
+
+
+def test_dense_prefill_without_its_scratch_runs_the_other_kernel():
+    # In a capture on a stream that has no room for the 16-bit weights the call is still served.  Counters and t are warmed up
+    # by calls that never use that scratch: 222 tiles of 256 features (three waves) and a call of few features.
+    import torch
+    import paper_2501_16385_b200 as fbq
+    inp = make_linear(1030, 11520, 256, 4, 16, dtype="f16", seed=3400)
+    dev = DeviceLinear(inp, fbq)
+    want = dev.run(fbq)                                      # with the scratch, on the current stream
+    warm = [DeviceLinear(make_linear(129, 56832, 128, 4, 0, seed=3401), fbq), DeviceLinear(make_linear(1030, 512, 128, 4, 16, seed=3402), fbq)]
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    y = torch.full((1030, 11520), float("nan"), dtype=torch.float16, device="cuda")
+    with torch.cuda.stream(stream):
+        for d in warm:
+            d.run(fbq)
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            fbq.linear(dev.x, dev.qweight, dev.scales, dev.zeros, dev.A, dev.B, 11520, 128, 4, y=y)
+        for _ in range(2):
+            y.fill_(float("nan"))
+            graph.replay()
+            stream.synchronize()
+            assert fbq.poll_status(stream) == 0
+            # the same products of the same rounded weights and t, sums in another order: one rounding to fp16 apart
+            assert float((y.float() - want.float()).norm() / want.float().norm()) < 2 ** -10

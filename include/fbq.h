@@ -197,9 +197,9 @@ int fbq_quantize_feedback(const float *W, const void *A, const void *B, uint8_t 
  *   W [N][K], H [K][K], A [rank][K], B [N][rank]: device fp32 (A and B are the master copies and
  *   are updated in place); loss: device float or NULL; workspace: device,
  *   fbq_reconstruct_workspace_floats(N, K, rank) floats, contents meaningless afterwards.
- * H has to be symmetric, as X^T X is.  The dense products (and fbq_gram) are this library's own tensor-core kernels on
+ * Any H is taken as it is (the formulas above, H not transposed); X^T X is symmetric.  The dense products (and fbq_gram) are this library's own tensor-core kernels on
  * exact three-term splits of the fp32 operands, accurate as fp32 sums (fixed summation order); no other library is
- * loaded or called.  They keep split operands in scratch of the stream (6 bytes per element of H and of X, 12 of W).  Initialise as Algorithm 1 says (A ~ N(0, sigma^2), B = 0), iterate, then
+ * loaded or called.  They keep split operands in scratch of the stream (6 bytes per element of X, 12 of H and of W).  Initialise as Algorithm 1 says (A ~ N(0, sigma^2), B = 0), iterate, then
  * round A and B to the inference type and call fbq_quantize_feedback once more for (codes, s, z). */
 size_t fbq_reconstruct_workspace_floats(int N, int K, int rank);
 int fbq_gram(const float *X, float *H, int T, int K, void *stream);

@@ -15,8 +15,10 @@
 //
 // The order of the products is chosen for the work: neither gradient needs G (2 N K^2 operations) itself,
 //   dL/dB = -2 Delta_F (H A^T),   dL/dA = -2 (B^T Delta_F) H          (four products of 2 N K r or 2 K^2 r)
-// and the loss is the dot product of H with Delta_F^T Delta_F, of which one triangle is enough.  (H = X^T X is symmetric.)
-// 4096 x 4096, rank 128: the Gram matrix of 4096 tokens 5733 -> 320 us, the step 8099 -> 698 us.
+// and the loss is the dot product of H with Delta_F^T Delta_F, which is symmetric: one triangle of it is enough.  H = X^T X is
+// symmetric too (the Gram matrix here to the last bit), so that its rows serve as its columns and one triangle of it does for
+// the loss; whether the caller's H is gets looked up while it is split, and where it is not its transpose is split as well.
+// 4096 x 4096, rank 128: the Gram matrix of 4096 tokens 5733 -> 320 us, the step 8099 -> 700 us.
 #include <algorithm>
 
 #include "fbq_common.cuh"
@@ -44,6 +46,7 @@ enum Mode { kSymmetric, kDot, kPartial };        // write both triangles; dot pr
 struct ProductParams {
     float *C;                 // kSymmetric: [n][n]; kPartial: [split][M][N]
     const float *H;           // kDot
+    const int *skew;          // kDot, and where the transposed operand is given: not zero if H is not symmetric
     double *dots;             // kDot: [work item][CTA][warp]
     int *status;
     int M, N, K;
@@ -79,7 +82,8 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
 
 template <int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUtensorMap qmap, const ProductParams p, const int n_work)
+product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUtensorMap skew_pmap, const __grid_constant__ CUtensorMap qmap,
+               const ProductParams p, const int n_work)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
@@ -116,6 +120,7 @@ product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
         if (lane == 0) {
             const uint32_t lfull0 = mapa_shared(full0, 0);
             const uint32_t q_bytes = (uint32_t)(p.nt / 2) * (kBK * 2u), bytes = 2u * kTerms * (kTermBytes + q_bytes);
+            const CUtensorMap *const rows = MODE == kPartial && p.skew && *p.skew ? &skew_pmap : &pmap;
             uint32_t i = 0;
             for (int q = pair; q < n_work && ok; q += n_pairs) {
                 int tm, tn, split, kb0, kb1;
@@ -128,7 +133,7 @@ product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
                     const uint32_t at = sbase + s * kStageBytes;
 #pragma unroll
                     for (int t = 0; t < kTerms; ++t) {
-                        tma_load_3d_pair(at + t * kTermBytes, &pmap, kb * kBK, prow, t, lfull0 + 8u * s);
+                        tma_load_3d_pair(at + t * kTermBytes, rows, kb * kBK, prow, t, lfull0 + 8u * s);
                         tma_load_3d_pair(at + (kTerms + t) * kTermBytes, &qmap, kb * kBK, qrow, t, lfull0 + 8u * s);
                     }
                 }
@@ -206,25 +211,48 @@ product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
             add(kSmallCol, lsfree);
             const int m = tm * kRows + 128 * (int)cr + 32 * wq + lane, n0 = tn * p.nt + c0;
             if constexpr (MODE == kDot) {
-                // H is symmetric: its column n0 + j, so that the lanes read side by side
+                // the tile times H's at (n, m), where the lanes read side by side; off the diagonal the same again for (m, n), or,
+                // where H is not symmetric, the tile times that, a lane a row: whole sectors at a time where they are aligned
+                const bool twice = tm != tn && *p.skew == 0, both = tm != tn && !twice;
                 double dot = 0.0;
-                float part = 0.f;
+                const bool wide = (p.N & 7) == 0 && (reinterpret_cast<uintptr_t>(p.H) & 31u) == 0u;
 #pragma unroll
-                for (int j = 0; j < 64; ++j) {
-                    if (j < cw && n0 + j < p.N && m < p.M) part = fmaf(acc[j], p.H[(size_t)(n0 + j) * p.M + m], part);
-                    if (j % 8 == 7) {
-                        dot += (double)part;
-                        part = 0.f;
+                for (int j = 0; j < 64; j += 8) {
+                    float part = 0.f, other = 0.f, h[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (j + e < cw && n0 + j + e < p.N && m < p.M) part = fmaf(acc[j + e], p.H[(size_t)(n0 + j + e) * p.M + m], part);
+                    if (both && j < cw && n0 + j < p.N && m < p.M) {
+                        const float *row = p.H + (size_t)m * p.N + n0 + j;
+                        if (wide) {
+                            *reinterpret_cast<float4 *>(h) = __ldg(reinterpret_cast<const float4 *>(row));
+                            *reinterpret_cast<float4 *>(h + 4) = __ldg(reinterpret_cast<const float4 *>(row) + 1);
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) h[e] = n0 + j + e < p.N ? row[e] : 0.f;
+                        }
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) other = fmaf(acc[j + e], h[e], other);
                     }
+                    dot += (double)part;
+                    dot += (double)other;
                 }
                 for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-                if (lane == 0) p.dots[((size_t)q * 2 + cr) * kEpiWarps + (warp - kEpi)] = tm == tn ? dot : 2.0 * dot;
+                if (lane == 0) p.dots[((size_t)q * 2 + cr) * kEpiWarps + (warp - kEpi)] = twice ? 2.0 * dot : dot;
             } else {
                 const size_t pitch = (size_t)p.N;
                 float *row = p.C + (MODE == kPartial ? (size_t)split * p.M * pitch : 0) + (size_t)m * pitch + n0;
+                // (a tile on the diagonal holds both triangles, which differ in the last bits; the upper one is written twice)
+                const bool on_diagonal = MODE == kSymmetric && tm == tn;
                 if (m < p.M) {
 #pragma unroll
                     for (int j = 0; j < 64; j += 4) {
+                        if (on_diagonal && n0 + j < m) {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                if (j < cw && n0 + j + e >= m && n0 + j + e < p.N) row[j + e] = acc[j + e];
+                            continue;
+                        }
                         if (j >= cw || n0 + j >= p.N) break;
                         if (n0 + j + 3 < p.N && (pitch & 3u) == 0u && (reinterpret_cast<uintptr_t>(p.C) & 15u) == 0u) {
                             *reinterpret_cast<float4 *>(row + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
@@ -234,10 +262,10 @@ product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
                                 if (n0 + j + e < p.N) row[j + e] = acc[j + e];
                         }
                     }
-                    if (MODE == kSymmetric && tm != tn) {
+                    if (MODE == kSymmetric) {
 #pragma unroll
                         for (int j = 0; j < 64; ++j)
-                            if (j < cw && n0 + j < p.N) p.C[(size_t)(n0 + j) * pitch + m] = acc[j];
+                            if (j < cw && n0 + j < p.N && n0 + j > m) p.C[(size_t)(n0 + j) * pitch + m] = acc[j];
                     }
                 }
             }
@@ -286,8 +314,9 @@ __device__ __forceinline__ void store_terms(unsigned short *dst, size_t plane, c
 // The matrix [R][C] as terms, rows as they are (`rows`: [3][R][pitch_r]) and / or transposed (`cols`: [3][C][pitch_c]).  Bound
 // by HBM: 4 bytes read, 6 written per copy and element; 64 x 64 tiles through shared memory, 8-byte stores.
 __global__ void __launch_bounds__(256) split_kernel(const float *__restrict__ src, int R, int C, unsigned short *rows, size_t pitch_r,
-                                                    unsigned short *cols, size_t pitch_c)
+                                                    unsigned short *cols, size_t pitch_c, const int *gate)
 {
+    if (gate && *gate == 0) return;                       // not wanted
     __shared__ float tile[64][65];
     const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64, tid = threadIdx.x;
 #pragma unroll
@@ -306,6 +335,44 @@ __global__ void __launch_bounds__(256) split_kernel(const float *__restrict__ sr
         if (cols && c0 + a < C && r0 + b < R) {
             const float v[4] = {tile[b][a], tile[b + 1][a], tile[b + 2][a], tile[b + 3][a]};
             store_terms(cols + (size_t)(c0 + a) * pitch_c + r0 + b, (size_t)C * pitch_c, v, R - (r0 + b));
+        }
+    }
+}
+
+// The square matrix [K][K] as terms, rows as they are; `skew` is raised if any two entries across the diagonal differ.  A block
+// takes a tile and its mirror image (the blocks of the other triangle leave).
+__global__ void __launch_bounds__(256) split_square_kernel(const float *__restrict__ src, int K, unsigned short *rows, size_t pitch, int *skew)
+{
+    __shared__ float tile[2][64][65];
+    if (blockIdx.x < blockIdx.y) return;
+    const int at[2] = {(int)blockIdx.y * 64, (int)blockIdx.x * 64}, tid = threadIdx.x;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r0 = at[h], c0 = at[1 - h];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int e = tid + 256 * i, r = e >> 6, c = e & 63;
+            tile[h][r][c] = (r0 + r < K && c0 + c < K) ? src[(size_t)(r0 + r) * K + c0 + c] : 0.f;
+        }
+    }
+    __syncthreads();
+    bool differ = false;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int e = tid + 256 * i, r = e >> 6, c = e & 63;
+        differ = differ || __float_as_uint(tile[0][r][c]) != __float_as_uint(tile[1][c][r]);
+    }
+    if (__syncthreads_or(differ) && tid == 0) *skew = 1;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r0 = at[h], c0 = at[1 - h];
+        if (h == 1 && blockIdx.x == blockIdx.y) break;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int e = tid + 256 * i, a = e >> 4, b = (e & 15) * 4;
+            if (r0 + a >= K || c0 + b >= K) continue;
+            const float v[4] = {tile[h][a][b], tile[h][a][b + 1], tile[h][a][b + 2], tile[h][a][b + 3]};
+            store_terms(rows + (size_t)(r0 + a) * pitch + c0 + b, (size_t)K * pitch, v, K - (c0 + b));
         }
     }
 }
@@ -403,7 +470,7 @@ int triangle_items(int n)
 }
 
 template <int MODE>
-bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p)
+bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p, const Operand *skew_P = nullptr)
 {
     p.M = P.rows; p.N = Q.rows; p.K = P.k;
     p.nt = MODE == kPartial ? std::min(256, (p.N + 31) / 32 * 32) : 256;
@@ -411,8 +478,10 @@ bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p
     p.tiles_n = (p.N + p.nt - 1) / p.nt;
     p.splits = MODE == kPartial ? k_splits(p.M, p.N, p.K) : 1;
     const int n_work = MODE == kPartial ? p.tiles_m * p.tiles_n * p.splits : triangle_items(p.M);
-    CUtensorMap pmap, qmap;
+    CUtensorMap pmap, skew_pmap, qmap;
     if (operand_map(&pmap, P, 128) != cudaSuccess || operand_map(&qmap, Q, p.nt / 2) != cudaSuccess) return false;
+    if (operand_map(&skew_pmap, skew_P ? *skew_P : P, 128) != cudaSuccess) return false;
+    if (MODE == kPartial && !skew_P) p.skew = nullptr;
     auto kern = product_kernel<MODE>;
     static bool attr_set = false;
     if (!attr_set) {
@@ -429,13 +498,21 @@ bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, pmap, qmap, p, n_work) == cudaSuccess;
+    return cudaLaunchKernelEx(&cfg, kern, pmap, skew_pmap, qmap, p, n_work) == cudaSuccess;
 }
-bool split(cudaStream_t s, const float *src, int R, int C, const Operand *rows, const Operand *cols)
+bool split(cudaStream_t s, const float *src, int R, int C, const Operand *rows, const Operand *cols, const int *gate = nullptr)
 {
     const dim3 grid((unsigned)((C + 63) / 64), (unsigned)((R + 63) / 64));
-    split_kernel<<<grid, 256, 0, s>>>(src, R, C, rows ? rows->planes : nullptr, rows ? rows->pitch() : 0, cols ? cols->planes : nullptr, cols ? cols->pitch() : 0);
+    split_kernel<<<grid, 256, 0, s>>>(src, R, C, rows ? rows->planes : nullptr, rows ? rows->pitch() : 0, cols ? cols->planes : nullptr, cols ? cols->pitch() : 0, gate);
     return cudaGetLastError() == cudaSuccess;
+}
+
+bool split_square(cudaStream_t s, const float *src, const Operand &rows, const Operand &cols, int *skew)
+{
+    if (cudaMemsetAsync(skew, 0, sizeof(int), s) != cudaSuccess) return false;
+    const unsigned tiles = (unsigned)((rows.k + 63) / 64);
+    split_square_kernel<<<dim3(tiles, tiles), 256, 0, s>>>(src, rows.k, rows.planes, rows.pitch(), skew);
+    return split(s, src, rows.k, rows.k, nullptr, &cols, skew);
 }
 
 // Carves a call's scratch out of one block.
@@ -456,9 +533,10 @@ struct Carver {
     }
 };
 struct StepScratch {
-    Operand D, Dt, H, A, Bt, P, Q;      // Delta_F, its transpose, H, A, B^T, (H A^T)^T, (B^T Delta_F)
+    Operand D, Dt, H, Ht, A, Bt, P, Q;      // Delta_F, H and their transposes, A, B^T, (H A^T)^T, (B^T Delta_F)
     float *part;
     double *dots;
+    int *skew;
     size_t bytes;
     StepScratch(void *base, int N, int K, int r)
     {
@@ -466,12 +544,14 @@ struct StepScratch {
         D = c.operand(N, K);
         Dt = c.operand(K, N);
         H = c.operand(K, K);
+        Ht = c.operand(K, K);
         A = c.operand(r, K);
         Bt = c.operand(r, N);
         P = c.operand(r, K);
         Q = c.operand(r, K);
         part = static_cast<float *>(c.take(std::max((size_t)std::max(k_splits(K, r, K), k_splits(K, r, N)) * K, (size_t)k_splits(N, r, K) * N) * r * sizeof(float)));
         dots = static_cast<double *>(c.take((size_t)triangle_items(K) * 2 * kEpiWarps * sizeof(double)));
+        skew = static_cast<int *>(c.take(sizeof(int)));
         bytes = c.used;
     }
 };
@@ -511,14 +591,15 @@ int run_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
     ProductParams p{};
     p.status = status;
     p.C = t.part;
+    p.skew = t.skew;
     const dim3 tr((unsigned)((K + 31) / 32), (unsigned)((rank + 31) / 32));
     // Delta_F with Q(W - B A) held fixed (nothing else of the quantiser's output is kept)
     float *Delta = ws;
     if (launch_quantize_feedback(W, A, B, nullptr, nullptr, nullptr, nullptr, Delta, N, K, group, bits, rank, 2, s) != cudaSuccess) return FBQ_ERR_CUDA;
-    if (!split(s, Delta, N, K, &t.D, &t.Dt) || !split(s, H, K, K, &t.H, nullptr) || !split(s, A, rank, K, &t.A, nullptr) ||
+    if (!split(s, Delta, N, K, &t.D, &t.Dt) || !split_square(s, H, t.H, t.Ht, t.skew) || !split(s, A, rank, K, &t.A, nullptr) ||
         !split(s, B, N, rank, nullptr, &t.Bt))
         return FBQ_ERR_CUDA;
-    if (loss) {                                  // tr(Delta H Delta^T) = sum H o (Delta^T Delta)
+    if (loss) {                                  // tr(Delta H Delta^T) = sum H o (Delta^T Delta), elementwise
         ProductParams d = p;
         d.H = H;
         d.dots = t.dots;
@@ -530,13 +611,13 @@ int run_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
     sum_transposed_kernel<<<tr, 256, 0, s>>>(t.part, k_splits(K, rank, K), K, rank, t.P.planes, t.P.pitch(), nullptr, 0.f);
     if (!product<kPartial>(s, t.Dt, t.Bt, p)) return FBQ_ERR_CUDA;                                     // Delta^T B [K x rank]
     sum_transposed_kernel<<<tr, 256, 0, s>>>(t.part, k_splits(K, rank, N), K, rank, t.Q.planes, t.Q.pitch(), nullptr, 0.f);
-    // B <- B + 2 lr Delta (H A^T), A <- A + 2 lr (B^T Delta) H; H is symmetric
+    // B <- B + 2 lr Delta (H A^T), A <- A + 2 lr (B^T Delta) H
     if (!product<kPartial>(s, t.D, t.P, p)) return FBQ_ERR_CUDA;
     const size_t nb = (size_t)N * rank;
     sum_into_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, s>>>(t.part, k_splits(N, rank, K), nb, B, 2.f * lr);
-    if (!product<kPartial>(s, t.H, t.Q, p)) return FBQ_ERR_CUDA;
+    if (!product<kPartial>(s, t.H, t.Q, p, &t.Ht)) return FBQ_ERR_CUDA;
     sum_transposed_kernel<<<tr, 256, 0, s>>>(t.part, k_splits(K, rank, K), K, rank, nullptr, 0, A, 2.f * lr);
-    *launches += 13;
+    *launches += 14;
     return cudaGetLastError() == cudaSuccess ? FBQ_OK : FBQ_ERR_CUDA;
 }
 

@@ -18,6 +18,7 @@ def test_gram_tile_edges(T, K):
     want = X.astype(np.float64).T @ X.astype(np.float64)
     assert np.linalg.norm(H - want) <= 3e-7 * np.linalg.norm(want)
     assert np.abs(H - want).max() <= 1e-6 * np.abs(want).max()
+    assert np.array_equal(H, H.T)
 
 
 @pytest.mark.parametrize("N,K,rank", [(1, 128, 1), (257, 384, 33), (130, 640, 260)])
@@ -55,3 +56,29 @@ def test_gram_captured_before_the_stream_has_scratch():
     torch.cuda.synchronize()
     want = X.double().T @ X.double()
     assert float((H.double() - want).norm() / want.norm()) < 3e-7
+
+
+@pytest.mark.parametrize("N,K,rank", [(70, 384, 16), (300, 640, 40)])
+def test_step_takes_any_h(N, K, rank):
+    # H with an antisymmetric part as large as the symmetric one: G = -2 Delta_F H and tr(Delta_F H Delta_F^T) as they stand
+    import torch
+    import paper_2501_16385_b200 as fbq
+    rng = np.random.default_rng(N + 1)
+    W = (rng.standard_normal((N, K)) * 0.05).astype(np.float32)
+    A = (rng.standard_normal((rank, K)) * 0.05).astype(np.float32)
+    B = (rng.standard_normal((N, rank)) * 0.05).astype(np.float32)
+    H = (rng.standard_normal((K, K)) + 8.0 * np.eye(K)).astype(np.float32)
+    lr = 0.05 / (np.linalg.norm(H.astype(np.float64), 2) * max(np.linalg.norm(A, 2), np.linalg.norm(B, 2)) ** 2)
+    Ad, Bd = torch.from_numpy(A.copy()).cuda(), torch.from_numpy(B.copy()).cuda()
+    loss, _ = fbq.reconstruct_step(torch.from_numpy(W).cuda(), torch.from_numpy(H).cuda(), Ad, Bd, lr, 128, 4)
+    assert fbq.poll_status() == 0
+    loss_o, A_o, B_o = rec.step(W, H, A, B, lr, 128, 4)
+    # the loss is a sum of K^2 terms of both signs, of which the diagonal's 8 |Delta|^2 remains: an error of 2^-24 of their
+    # root sum of squares, sqrt(K) / 8 of the loss, is far inside this
+    assert np.isclose(float(loss.item()), loss_o, rtol=1e-5)
+    for got, want, old in ((Ad, A_o, A), (Bd, B_o, B)):
+        assert np.linalg.norm(got.cpu().numpy() - want) <= 1e-6 * np.linalg.norm(want)
+        # the step by itself: its error is that of the products plus one fp32 rounding of the updated matrix
+        step = want - old.astype(np.float64)
+        err = np.linalg.norm((got.cpu().numpy().astype(np.float64) - old) - step)
+        assert err <= 1e-5 * np.linalg.norm(step) + 2.0 ** -24 * np.linalg.norm(want)

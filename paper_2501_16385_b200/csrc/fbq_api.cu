@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <initializer_list>
 #include <map>
 #include <mutex>
 #include <utility>
@@ -38,7 +39,9 @@ struct Options {
     int hostio_direct_y = 1;
     int test_prefill_skip_flag = 0, prefill_flag_polls = 0;
     int decode_trace = 0;
+    int scratch_mb = 0;
 } g_opt;
+constexpr size_t kScratchMost = (size_t)512 << 20;     // of the Gram matrix and the reconstruction step (4096 x 4096 and 4096 tokens take 440 MB)
 constexpr int kGemvBatchMost = 8;                     // problems of one launch of the streaming kernel
 constexpr size_t kTraceBytes = 512 * 18 * 16 * 8;   // 512 CTAs x up to 18 warps x 16 marks
 
@@ -339,30 +342,40 @@ int run_linear(const LinearArgs &a, cudaStream_t s, int decode_ctas = 0)
     return FBQ_OK;
 }
 
-// Runs f(scratch, status word, &launches) with `need` bytes of the stream's scratch; where that would have to grow during a
-// stream capture, with memory that belongs to the captured graph.
-template <typename F>
-int with_scratch(size_t need, cudaStream_t s, F f)
+// Runs f(budget, scratch, status word, &launches) with need(budget) bytes of the stream's scratch; where that would have to
+// grow during a stream capture, with memory that belongs to the captured graph.  Where device memory is used up the budget
+// is lowered, and last `spare` (memory of the caller) serves if it is large enough.
+template <typename N, typename F>
+int with_scratch(N need, cudaStream_t s, F f, void *spare = nullptr, size_t spare_bytes = 0)
 {
     Workspace *ws = workspace_for(s);
     if (!ws) return FBQ_ERR_CUDA;
-    int launches = 0, rc;
+    int launches = 0, rc = FBQ_ERR_CUDA;
     size_t have_c = (size_t)ws->n_counters;
     if (grow(ws->counters, have_c, 16, sizeof(int), s) == cudaSuccess) ws->n_counters = (int)have_c;
     int *status = ws->counters ? ws->counters + kCtrStatus : nullptr;
-    char *rec = static_cast<char *>(ws->rec);
-    const cudaError_t e = grow(rec, ws->rec_bytes, need, 1, s);
-    ws->rec = rec;
-    if (e == cudaSuccess) {
-        rc = f(ws->rec, status, &launches);
-    } else if (e == cudaErrorStreamCaptureUnsupported) {
-        void *tmp = nullptr;
-        if (cudaMallocAsync(&tmp, need, s) != cudaSuccess) return FBQ_ERR_CUDA;
-        rc = f(tmp, status, &launches);
-        if (cudaFreeAsync(tmp, s) != cudaSuccess) rc = FBQ_ERR_CUDA;
-    } else {
-        return FBQ_ERR_CUDA;
+    const size_t most = g_opt.scratch_mb > 0 ? (size_t)g_opt.scratch_mb << 20 : kScratchMost;
+    for (size_t budget : {most, most / 8, (size_t)0}) {
+        char *rec = static_cast<char *>(ws->rec);
+        const cudaError_t e = grow(rec, ws->rec_bytes, need(budget), 1, s);
+        ws->rec = rec;
+        if (e == cudaSuccess) {
+            rc = f(budget, ws->rec, status, &launches);
+            g_launches += launches;
+            return rc;
+        }
+        if (e == cudaErrorStreamCaptureUnsupported) {
+            void *tmp = nullptr;
+            if (cudaMallocAsync(&tmp, need(budget), s) != cudaSuccess) return FBQ_ERR_CUDA;
+            rc = f(budget, tmp, status, &launches);
+            if (cudaFreeAsync(tmp, s) != cudaSuccess) rc = FBQ_ERR_CUDA;
+            g_launches += launches;
+            return rc;
+        }
+        (void)cudaGetLastError();
+        if (e != cudaErrorMemoryAllocation) return FBQ_ERR_CUDA;
     }
+    if (need(0) <= spare_bytes) rc = f(0, spare, status, &launches);
     g_launches += launches;
     return rc;
 }
@@ -391,6 +404,7 @@ int *option_slot(const char *name)
     if (!strcmp(name, "hostio_direct_y")) return &g_opt.hostio_direct_y;
     if (!strcmp(name, "test_prefill_skip_flag")) return &g_opt.test_prefill_skip_flag;
     if (!strcmp(name, "prefill_flag_polls")) return &g_opt.prefill_flag_polls;
+    if (!strcmp(name, "scratch_mb")) return &g_opt.scratch_mb;
     if (!strcmp(name, "decode_trace")) return &g_opt.decode_trace;
     return nullptr;
 }
@@ -495,7 +509,8 @@ int fbq_gram(const float *X, float *H, int T, int K, void *stream)
 {
     if (!X || !H || T < 1 || K < 1) return FBQ_ERR_BADARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    return with_scratch(gram_scratch_bytes(T, K), s, [&](void *scratch, int *status, int *n) { return run_gram(X, H, T, K, scratch, status, s, n); });
+    return with_scratch([&](size_t budget) { return gram_scratch_bytes(T, K, budget); }, s,
+                        [&](size_t budget, void *scratch, int *status, int *n) { return run_gram(X, H, T, K, budget, scratch, status, s, n); });
 }
 
 int fbq_reconstruct_step(const float *W, const float *H, float *A, float *B, float lr, float *loss, float *workspace, int N,
@@ -505,9 +520,15 @@ int fbq_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
     if (bits != 3 && bits != 4) return FBQ_ERR_BADARG;
     if (!W || !H || !A || !B || !workspace) return FBQ_ERR_BADARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    return with_scratch(reconstruct_scratch_bytes(N, K, rank), s, [&](void *scratch, int *status, int *n) {
-        return run_reconstruct_step(W, H, A, B, lr, loss, workspace, N, K, group, bits, rank, scratch, status, s, n);
-    });
+    // Delta_F takes the first N K floats of the workspace; the rest serves where the library can allocate nothing
+    const size_t used = ((size_t)N * K * sizeof(float) + 255) / 256 * 256, all = reconstruct_workspace_floats(N, K, rank) * sizeof(float);
+    char *spare = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(workspace) + 255) / 256 * 256) + used;
+    const size_t shift = (size_t)(spare - reinterpret_cast<char *>(workspace));
+    return with_scratch([&](size_t budget) { return reconstruct_scratch_bytes(N, K, rank, budget); }, s,
+                        [&](size_t budget, void *scratch, int *status, int *n) {
+                            return run_reconstruct_step(W, H, A, B, lr, loss, workspace, N, K, group, bits, rank, budget, scratch, status, s, n);
+                        },
+                        spare, all > shift ? all - shift : 0);
 }
 
 // Hands the process-wide switches to the kernel files before a launch.

@@ -45,6 +45,7 @@ constexpr uint32_t kSmallCol = 256;              // tensor-memory column of the 
 enum Mode { kSymmetric, kDot, kPartial };        // write both triangles; dot product with H; one slice per split of k
 struct ProductParams {
     float *C;                 // kSymmetric: [n][n]; kPartial: [split][M][N]
+    int add;                  // kSymmetric: add to C
     const float *H;           // kDot
     const int *skew;          // kDot, and where the transposed operand is given: not zero if H is not symmetric
     double *dots;             // kDot: [work item][CTA][warp]
@@ -244,6 +245,11 @@ product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
                 float *row = p.C + (MODE == kPartial ? (size_t)split * p.M * pitch : 0) + (size_t)m * pitch + n0;
                 // (a tile on the diagonal holds both triangles, which differ in the last bits; the upper one is written twice)
                 const bool on_diagonal = MODE == kSymmetric && tm == tn;
+                if (MODE == kSymmetric && p.add && m < p.M) {
+#pragma unroll
+                    for (int j = 0; j < 64; ++j)
+                        if (j < cw && n0 + j < p.N && (!on_diagonal || n0 + j >= m)) acc[j] += row[j];
+                }
                 if (m < p.M) {
 #pragma unroll
                     for (int j = 0; j < 64; j += 4) {
@@ -431,8 +437,11 @@ __global__ void __launch_bounds__(256) sum_dots_kernel(const double *__restrict_
 struct Operand {
     unsigned short *planes;   // [3][rows][pitch]
     int rows, k;
-    size_t pitch() const { return ((size_t)k + 7) & ~(size_t)7; }
+    size_t full_pitch = 0;    // of the operand that this is a range of k of (k_range); 0: all of it
+    size_t pitch() const { return full_pitch ? full_pitch : ((size_t)k + 7) & ~(size_t)7; }
     size_t values() const { return (size_t)kTerms * rows * pitch(); }
+    Operand k_range(int k0, int n) const { return Operand{planes + k0, rows, n, pitch()}; }      // k0: a multiple of 8
+    Operand first(int n_rows, int n) const { return Operand{planes, n_rows, n}; }               // the same memory, smaller
 };
 cudaError_t operand_map(CUtensorMap *map, const Operand &o, int box_rows)
 {
@@ -532,30 +541,54 @@ struct Carver {
         return o;
     }
 };
+// Scratch is bounded: where the split operands of all of Delta_F, H or X would take more than `budget` bytes, they are split and
+// multiplied a slab of rows at a time (kSlab rows at least).  What the rank needs comes on top.
+constexpr int kSlab = kRows;
+int slab_rows(int rows, size_t bytes_per_row, size_t budget)
+{
+    const size_t most = std::max((size_t)kSlab, budget / bytes_per_row / kSlab * kSlab), n = ((size_t)rows + most - 1) / most;
+    return (int)std::min((size_t)rows, (((size_t)rows + n - 1) / n + kSlab - 1) / kSlab * kSlab);
+}
 struct StepScratch {
-    Operand D, Dt, H, Ht, A, Bt, P, Q;      // Delta_F, H and their transposes, A, B^T, (H A^T)^T, (B^T Delta_F)
-    float *part;
+    int nd, nh;                             // rows of a slab of Delta_F and of H
+    Operand D, Dt, H, Ht, A, Bt, P, Q;      // slabs of Delta_F and H and their transposes; A, B^T, (H A^T)^T, (B^T Delta_F)
+    float *part, *q_sum, *a_sum;            // partial products; sums over slabs where there are several
     double *dots;
     int *skew;
     size_t bytes;
-    StepScratch(void *base, int N, int K, int r)
+    StepScratch(void *base, int N, int K, int r, size_t budget)
     {
+        const size_t per_row = 2u * kTerms * (size_t)((K + 7) & ~7);        // bytes of one row's terms
+        nd = N;
+        nh = K;
+        if (2 * per_row * ((size_t)N + K) > budget) {
+            // one slab holds Delta_F and its transpose, of several each holds one after the other in the same place
+            if (2 * per_row * N > budget / 2) nd = slab_rows(N, per_row, std::min(budget / 2, per_row * ((size_t)N - 1)));
+            nh = slab_rows(K, 2 * per_row, budget - std::min(budget / 2, per_row * nd * (nd < N ? 1 : 2)));
+        }
+        const int slabs = (N + nd - 1) / nd;
         Carver c{static_cast<char *>(base)};
-        D = c.operand(N, K);
-        Dt = c.operand(K, N);
-        H = c.operand(K, K);
-        Ht = c.operand(K, K);
+        D = c.operand(nd, K);
+        Dt = slabs == 1 ? c.operand(K, nd) : Operand{nullptr, K, nd};
+        if (slabs > 1) {
+            if (Dt.values() > D.values()) c.take((Dt.values() - D.values()) * 2);               // (rows of nd values are padded to 16 bytes)
+            Dt.planes = D.planes;
+        }
+        H = c.operand(nh, K);
+        Ht = c.operand(K, nh);
         A = c.operand(r, K);
         Bt = c.operand(r, N);
         P = c.operand(r, K);
         Q = c.operand(r, K);
-        part = static_cast<float *>(c.take(std::max((size_t)std::max(k_splits(K, r, K), k_splits(K, r, N)) * K, (size_t)k_splits(N, r, K) * N) * r * sizeof(float)));
-        dots = static_cast<double *>(c.take((size_t)triangle_items(K) * 2 * kEpiWarps * sizeof(double)));
+        // splits x rows of a product: a work item per pair and kRows rows each, or one split
+        part = static_cast<float *>(c.take((size_t)std::max(std::max(K, N), pairs() * kRows) * r * sizeof(float)));
+        q_sum = static_cast<float *>(c.take(slabs > 1 ? (size_t)K * r * sizeof(float) : 0));
+        a_sum = static_cast<float *>(c.take(nh < K ? (size_t)K * r * sizeof(float) : 0));
+        dots = static_cast<double *>(c.take((size_t)slabs * triangle_items(K) * 2 * kEpiWarps * sizeof(double)));
         skew = static_cast<int *>(c.take(sizeof(int)));
         bytes = c.used;
     }
 };
-
 }  // namespace
 
 size_t reconstruct_workspace_floats(int N, int K, int rank)
@@ -563,62 +596,117 @@ size_t reconstruct_workspace_floats(int N, int K, int rank)
     return 2 * (size_t)N * K + (size_t)rank * K + (size_t)N * rank + 256;
 }
 
-size_t gram_scratch_bytes(int T, int K)
+int gram_slab(int T, int K, size_t budget) { return slab_rows(T, 2u * kTerms * (size_t)K, budget); }
+size_t gram_scratch_bytes(int T, int K, size_t budget)
 {
     Carver c{nullptr};
-    c.operand(K, T);
+    c.operand(K, gram_slab(T, K, budget));
     return c.used;
 }
-size_t reconstruct_scratch_bytes(int N, int K, int rank) { return StepScratch(nullptr, N, K, rank).bytes; }
+size_t reconstruct_scratch_bytes(int N, int K, int rank, size_t budget) { return StepScratch(nullptr, N, K, rank, budget).bytes; }
 
-// H[K x K] = X^T X for X [T x K]
-int run_gram(const float *X, float *H, int T, int K, void *scratch, int *status, cudaStream_t s, int *launches)
+// H[K x K] = X^T X for X [T x K]; several slabs of X are added one after the other
+int run_gram(const float *X, float *H, int T, int K, size_t budget, void *scratch, int *status, cudaStream_t s, int *launches)
 {
+    const int nt = gram_slab(T, K, budget);
     Carver c{static_cast<char *>(scratch)};
-    const Operand Xt = c.operand(K, T);
+    const Operand all = c.operand(K, nt);
     ProductParams p{};
     p.C = H;
     p.status = status;
-    if (!split(s, X, T, K, nullptr, &Xt) || !product<kSymmetric>(s, Xt, Xt, p)) return FBQ_ERR_CUDA;
-    *launches += 2;
+    for (int t0 = 0; t0 < T; t0 += nt) {
+        const Operand Xt = all.first(K, std::min(nt, T - t0));
+        p.add = t0 > 0;
+        if (!split(s, X + (size_t)t0 * K, Xt.k, K, nullptr, &Xt) || !product<kSymmetric>(s, Xt, Xt, p)) return FBQ_ERR_CUDA;
+        *launches += 2;
+    }
     return FBQ_OK;
 }
 
 int run_reconstruct_step(const float *W, const float *H, float *A, float *B, float lr, float *loss, float *ws, int N, int K, int group, int bits,
-                         int rank, void *scratch, int *status, cudaStream_t s, int *launches)
+                         int rank, size_t budget, void *scratch, int *status, cudaStream_t s, int *launches)
 {
-    const StepScratch t(scratch, N, K, rank);
+    const StepScratch t(scratch, N, K, rank, budget);
+    const int slabs_d = (N + t.nd - 1) / t.nd, slabs_h = (K + t.nh - 1) / t.nh, items = triangle_items(K) * 2 * kEpiWarps;
+    const size_t nq = (size_t)K * rank;
     ProductParams p{};
     p.status = status;
     p.C = t.part;
     p.skew = t.skew;
-    const dim3 tr((unsigned)((K + 31) / 32), (unsigned)((rank + 31) / 32));
+    bool ok = true;
+    auto columns = [&](const float *part, int splits, int rows, unsigned short *planes, size_t pitch, float *into, float alpha) {
+        const dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((rank + 31) / 32));
+        sum_transposed_kernel<<<grid, 256, 0, s>>>(part, splits, rows, rank, planes, pitch, into, alpha);
+        ++*launches;
+    };
+    auto add = [&](const float *part, int splits, size_t n, float *into, float alpha) {
+        sum_into_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, splits, n, into, alpha);
+        ++*launches;
+    };
+    auto times = [&](const Operand &P, const Operand &Q, const Operand *skew_P = nullptr) {      // -> number of splits in t.part
+        ok = ok && product<kPartial>(s, P, Q, p, skew_P);
+        ++*launches;
+        return k_splits(P.rows, Q.rows, P.k);
+    };
     // Delta_F with Q(W - B A) held fixed (nothing else of the quantiser's output is kept)
     float *Delta = ws;
     if (launch_quantize_feedback(W, A, B, nullptr, nullptr, nullptr, nullptr, Delta, N, K, group, bits, rank, 2, s) != cudaSuccess) return FBQ_ERR_CUDA;
-    if (!split(s, Delta, N, K, &t.D, &t.Dt) || !split_square(s, H, t.H, t.Ht, t.skew) || !split(s, A, rank, K, &t.A, nullptr) ||
-        !split(s, B, N, rank, nullptr, &t.Bt))
-        return FBQ_ERR_CUDA;
-    if (loss) {                                  // tr(Delta H Delta^T) = sum H o (Delta^T Delta), elementwise
-        ProductParams d = p;
-        d.H = H;
-        d.dots = t.dots;
-        if (!product<kDot>(s, t.Dt, t.Dt, d)) return FBQ_ERR_CUDA;
-        sum_dots_kernel<<<1, 256, 0, s>>>(t.dots, triangle_items(K) * 2 * kEpiWarps, loss);
+    ok = split(s, A, rank, K, &t.A, nullptr) && split(s, B, N, rank, nullptr, &t.Bt);
+    *launches += 3;
+    // One slab of H: its rows serve as its columns where it is symmetric.  Of several each is taken as it is.
+    if (slabs_h == 1) {
+        ok = ok && split_square(s, H, t.H, t.Ht, t.skew);
         *launches += 2;
+    } else {
+        ok = ok && cudaMemsetAsync(t.skew, 1, sizeof(int), s) == cudaSuccess && cudaMemsetAsync(t.a_sum, 0, nq * sizeof(float), s) == cudaSuccess;
     }
-    if (!product<kPartial>(s, t.H, t.A, p)) return FBQ_ERR_CUDA;                                       // H A^T [K x rank]
-    sum_transposed_kernel<<<tr, 256, 0, s>>>(t.part, k_splits(K, rank, K), K, rank, t.P.planes, t.P.pitch(), nullptr, 0.f);
-    if (!product<kPartial>(s, t.Dt, t.Bt, p)) return FBQ_ERR_CUDA;                                     // Delta^T B [K x rank]
-    sum_transposed_kernel<<<tr, 256, 0, s>>>(t.part, k_splits(K, rank, N), K, rank, t.Q.planes, t.Q.pitch(), nullptr, 0.f);
-    // B <- B + 2 lr Delta (H A^T), A <- A + 2 lr (B^T Delta) H
-    if (!product<kPartial>(s, t.D, t.P, p)) return FBQ_ERR_CUDA;
-    const size_t nb = (size_t)N * rank;
-    sum_into_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, s>>>(t.part, k_splits(N, rank, K), nb, B, 2.f * lr);
-    if (!product<kPartial>(s, t.H, t.Q, p, &t.Ht)) return FBQ_ERR_CUDA;
-    sum_transposed_kernel<<<tr, 256, 0, s>>>(t.part, k_splits(K, rank, K), K, rank, nullptr, 0, A, 2.f * lr);
-    *launches += 14;
-    return cudaGetLastError() == cudaSuccess ? FBQ_OK : FBQ_ERR_CUDA;
+    // slabs of Delta_F, transposed: the loss tr(Delta H Delta^T) = sum H o (Delta^T Delta), elementwise, and Delta^T B [K x rank]
+    if (slabs_d > 1) ok = ok && cudaMemsetAsync(t.q_sum, 0, nq * sizeof(float), s) == cudaSuccess;
+    for (int i = 0; i < slabs_d && ok; ++i) {
+        const int n0 = i * t.nd, n = std::min(t.nd, N - n0);
+        const Operand D = t.D.first(n, K), Dt = t.Dt.first(K, n);
+        ok = split(s, Delta + (size_t)n0 * K, n, K, slabs_d == 1 ? &D : nullptr, &Dt);
+        ++*launches;
+        if (loss) {
+            ProductParams d = p;
+            d.H = H;
+            d.dots = t.dots + (size_t)i * items;
+            ok = ok && product<kDot>(s, Dt, Dt, d);
+            ++*launches;
+        }
+        const int splits = times(Dt, t.Bt.k_range(n0, n));
+        if (slabs_d > 1) add(t.part, splits, nq, t.q_sum, 1.f);
+        else columns(t.part, splits, K, t.Q.planes, t.Q.pitch(), nullptr, 0.f);
+    }
+    if (slabs_d > 1) columns(t.q_sum, 1, K, t.Q.planes, t.Q.pitch(), nullptr, 0.f);
+    if (loss) {
+        sum_dots_kernel<<<1, 256, 0, s>>>(t.dots, slabs_d * items, loss);
+        ++*launches;
+    }
+    // slabs of H: H A^T [K x rank], and A <- A + 2 lr (B^T Delta) H from the old A and B
+    for (int i = 0; i < slabs_h && ok; ++i) {
+        const int k0 = i * t.nh, n = std::min(t.nh, K - k0);
+        const Operand rows = t.H.first(n, K), cols = t.Ht.first(K, n);
+        if (slabs_h > 1) {
+            ok = split(s, H + (size_t)k0 * K, n, K, &rows, &cols);
+            ++*launches;
+        }
+        columns(t.part, times(rows, t.A), n, t.P.planes + k0, t.P.pitch(), nullptr, 0.f);
+        if (slabs_h == 1) columns(t.part, times(t.H, t.Q, &t.Ht), K, nullptr, 0, A, 2.f * lr);
+        else columns(t.part, times(cols, t.Q.k_range(k0, n)), K, nullptr, 0, t.a_sum, 1.f);
+    }
+    if (slabs_h > 1) add(t.a_sum, 1, nq, A, 2.f * lr);
+    // slabs of Delta_F: B <- B + 2 lr Delta (H A^T)
+    for (int i = 0; i < slabs_d && ok; ++i) {
+        const int n0 = i * t.nd, n = std::min(t.nd, N - n0);
+        const Operand D = t.D.first(n, K);
+        if (slabs_d > 1) {
+            ok = split(s, Delta + (size_t)n0 * K, n, K, &D, nullptr);
+            ++*launches;
+        }
+        add(t.part, times(D, t.P), (size_t)n * rank, B + (size_t)n0 * rank, 2.f * lr);
+    }
+    return ok && cudaGetLastError() == cudaSuccess ? FBQ_OK : FBQ_ERR_CUDA;
 }
 
 }  // namespace fbq

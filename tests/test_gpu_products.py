@@ -82,3 +82,55 @@ def test_step_takes_any_h(N, K, rank):
         step = want - old.astype(np.float64)
         err = np.linalg.norm((got.cpu().numpy().astype(np.float64) - old) - step)
         assert err <= 1e-5 * np.linalg.norm(step) + 2.0 ** -24 * np.linalg.norm(want)
+
+
+@pytest.fixture
+def one_megabyte():
+    import paper_2501_16385_b200 as fbq
+    fbq.set_option("scratch_mb", 1)
+    yield
+    fbq.set_option("scratch_mb", 0)
+
+
+@pytest.mark.parametrize("T,K", [(1000, 770), (257, 1000), (700, 64)])
+def test_gram_in_slabs(one_megabyte, T, K):
+    test_gram_tile_edges(T, K)
+
+
+@pytest.mark.parametrize("N,K,rank", [(700, 1152, 33), (100, 1152, 8), (3000, 128, 16), (257, 640, 260)])
+def test_step_in_slabs(one_megabyte, N, K, rank):
+    # several slabs of both matrices (ragged last ones), of H alone, of Delta alone; more rank than a tile
+    import paper_2501_16385_b200 as fbq
+    fbq.release_workspaces()
+    test_step_tile_edges(N, K, rank)
+    test_step_takes_any_h(N, K, rank)
+
+
+def test_scratch_of_a_large_step_is_bounded():
+    # Delta and H of 2048 x 8192 split as a whole are 1 GB; the default bound is 512 MB beyond what the rank needs.  Reference in
+    # float64 from the library's own Delta, which the tests of the quantiser pin.
+    import torch
+    import paper_2501_16385_b200 as fbq
+    N, K, rank = 2048, 8192, 16
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    W = torch.randn((N, K), device="cuda", generator=g) * 0.05
+    A = (torch.randn((rank, K), device="cuda", generator=g) * 0.05).half().float()
+    B = (torch.randn((N, rank), device="cuda", generator=g) * 0.05).half().float()
+    H = torch.randn((K, K), device="cuda", generator=g) + 50.0 * torch.eye(K, device="cuda")
+    WF = fbq.quantize_feedback(W, A.half(), B.half(), 128, 4, want_wf=True)[3]
+    D = W.double() - WF.double()
+    lr = 1e-5
+    DH = D @ H.double()
+    want_a, want_b, want_loss = A.double() + 2 * lr * (B.double().T @ DH), B.double() + 2 * lr * (DH @ A.double().T), float((DH * D).sum())
+    ws = torch.empty(int(fbq.lib().fbq_reconstruct_workspace_floats(N, K, rank)), device="cuda")
+    fbq.release_workspaces()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    loss, _ = fbq.reconstruct_step(W, H, A, B, lr, 128, 4, workspace=ws)
+    assert fbq.poll_status() == 0
+    assert free - torch.cuda.mem_get_info()[0] < 600 << 20
+    # W_F and Delta are rounded to fp32 differently (W_F has 2^-24 of |W|, about 2^-20 of |Delta|)
+    assert abs(float(loss.item()) - want_loss) <= 1e-5 * want_loss
+    assert float((A.double() - want_a).norm() / want_a.norm()) < 1e-6
+    assert float((B.double() - want_b).norm() / want_b.norm()) < 1e-6

@@ -199,8 +199,8 @@ int fbq_quantize_feedback(const float *W, const void *A, const void *B, uint8_t 
  *   fbq_reconstruct_workspace_floats(N, K, rank) floats, contents meaningless afterwards.
  * Any H is taken as it is (the formulas above, H not transposed); X^T X is symmetric.  The dense products (and fbq_gram) are this library's own tensor-core kernels on
  * exact three-term splits of the fp32 operands, accurate as fp32 sums (fixed summation order); no other library is
- * loaded or called.  They keep split operands in scratch of the stream: 6 bytes per element of X, 12 of H and of W, up to
- * 512 MB ("scratch_mb"); larger problems are worked through in slabs, in a fixed order.  Initialise as Algorithm 1 says (A ~ N(0, sigma^2), B = 0), iterate, then
+ * loaded or called.  They keep split operands in scratch of the stream: 6 bytes per element of X and of H, 12 of W, up to
+ * 1 GB ("scratch_mb"); larger problems are worked through in slabs, in a fixed order.  Initialise as Algorithm 1 says (A ~ N(0, sigma^2), B = 0), iterate, then
  * round A and B to the inference type and call fbq_quantize_feedback once more for (codes, s, z). */
 size_t fbq_reconstruct_workspace_floats(int N, int K, int rank);
 int fbq_gram(const float *X, float *H, int T, int K, void *stream);
@@ -305,7 +305,7 @@ int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int ac
  *   "hostio_direct_y" 1 (default) = the host-buffer entry points let the kernel write a y of up to 256 KB straight
  *                   into the caller's buffer when that is pinned, GPU-addressable host memory (no copy queued
  *                   behind the kernel); 0 = y always goes through the stream's staging buffer and a copy
- *   "scratch_mb"    0 (default) = 512, else the number of megabytes that the scratch of fbq_gram and
+ *   "scratch_mb"    0 (default) = 1024, else the number of megabytes that the scratch of fbq_gram and
  *                   fbq_reconstruct_step is held to (a slab of 256 rows and what the rank needs come on top)
  *   "pdl"           1 = launch with programmatic dependent launch (default), 0 = plain.  With 1 a decode or
  *                   prefill kernel may start while the kernel before it on the stream still runs: it sets

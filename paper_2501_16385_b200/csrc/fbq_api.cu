@@ -41,7 +41,9 @@ struct Options {
     int decode_trace = 0;
     int scratch_mb = 0;
 } g_opt;
-constexpr size_t kScratchMost = (size_t)512 << 20;     // of the Gram matrix and the reconstruction step (4096 x 4096 and 4096 tokens take 440 MB)
+// Scratch of the Gram matrix and the reconstruction step; layers of a 7B model and the widest of a 13B model (5120 x 13824, whose
+// H alone has 764 MB) are within two slabs of it.
+constexpr size_t kScratchMost = (size_t)1 << 30;
 constexpr int kGemvBatchMost = 8;                     // problems of one launch of the streaming kernel
 constexpr size_t kTraceBytes = 512 * 18 * 16 * 8;   // 512 CTAs x up to 18 warps x 16 marks
 

@@ -17,7 +17,7 @@
 //   dL/dB = -2 Delta_F (H A^T),   dL/dA = -2 (B^T Delta_F) H          (four products of 2 N K r or 2 K^2 r)
 // and the loss is the dot product of H with Delta_F^T Delta_F, which is symmetric: one triangle of it is enough.  H = X^T X is
 // symmetric too (the Gram matrix here to the last bit), so that its rows serve as its columns and one triangle of it does for
-// the loss; whether the caller's H is gets looked up while it is split, and where it is not its transpose is split as well.
+// the loss; whether the caller's H is gets looked up while it is split, and where it is not its columns are split as well.
 // 4096 x 4096, rank 128: the Gram matrix of 4096 tokens 5733 -> 320 us, the step 8099 -> 700 us.
 #include <algorithm>
 
@@ -47,7 +47,7 @@ struct ProductParams {
     float *C;                 // kSymmetric: [n][n]; kPartial: [split][M][N]
     int add;                  // kSymmetric: add to C
     const float *H;           // kDot
-    const int *skew;          // kDot, and where the transposed operand is given: not zero if H is not symmetric
+    const int *skew;          // kDot: not zero if H is not symmetric
     double *dots;             // kDot: [work item][CTA][warp]
     int *status;
     int M, N, K;
@@ -83,8 +83,7 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
 
 template <int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUtensorMap skew_pmap, const __grid_constant__ CUtensorMap qmap,
-               const ProductParams p, const int n_work)
+product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUtensorMap qmap, const ProductParams p, const int n_work)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
@@ -121,7 +120,6 @@ product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
         if (lane == 0) {
             const uint32_t lfull0 = mapa_shared(full0, 0);
             const uint32_t q_bytes = (uint32_t)(p.nt / 2) * (kBK * 2u), bytes = 2u * kTerms * (kTermBytes + q_bytes);
-            const CUtensorMap *const rows = MODE == kPartial && p.skew && *p.skew ? &skew_pmap : &pmap;
             uint32_t i = 0;
             for (int q = pair; q < n_work && ok; q += n_pairs) {
                 int tm, tn, split, kb0, kb1;
@@ -134,7 +132,7 @@ product_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
                     const uint32_t at = sbase + s * kStageBytes;
 #pragma unroll
                     for (int t = 0; t < kTerms; ++t) {
-                        tma_load_3d_pair(at + t * kTermBytes, rows, kb * kBK, prow, t, lfull0 + 8u * s);
+                        tma_load_3d_pair(at + t * kTermBytes, &pmap, kb * kBK, prow, t, lfull0 + 8u * s);
                         tma_load_3d_pair(at + (kTerms + t) * kTermBytes, &qmap, kb * kBK, qrow, t, lfull0 + 8u * s);
                     }
                 }
@@ -317,9 +315,9 @@ __device__ __forceinline__ void store_terms(unsigned short *dst, size_t plane, c
         }
     }
 }
-// The matrix [R][C] as terms, rows as they are (`rows`: [3][R][pitch_r]) and / or transposed (`cols`: [3][C][pitch_c]).  Bound
+// The matrix [R][C] (rows `ld` apart) as terms, rows as they are (`rows`: [3][R][pitch_r]) and / or transposed (`cols`: [3][C][pitch_c]).  Bound
 // by HBM: 4 bytes read, 6 written per copy and element; 64 x 64 tiles through shared memory, 8-byte stores.
-__global__ void __launch_bounds__(256) split_kernel(const float *__restrict__ src, int R, int C, unsigned short *rows, size_t pitch_r,
+__global__ void __launch_bounds__(256) split_kernel(const float *__restrict__ src, size_t ld, int R, int C, unsigned short *rows, size_t pitch_r,
                                                     unsigned short *cols, size_t pitch_c, const int *gate)
 {
     if (gate && *gate == 0) return;                       // not wanted
@@ -328,7 +326,7 @@ __global__ void __launch_bounds__(256) split_kernel(const float *__restrict__ sr
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const int e = tid + 256 * i, r = e >> 6, c = e & 63;
-        tile[r][c] = (r0 + r < R && c0 + c < C) ? src[(size_t)(r0 + r) * C + c0 + c] : 0.f;
+        tile[r][c] = (r0 + r < R && c0 + c < C) ? src[(r0 + r) * ld + c0 + c] : 0.f;
     }
     __syncthreads();
 #pragma unroll
@@ -345,7 +343,7 @@ __global__ void __launch_bounds__(256) split_kernel(const float *__restrict__ sr
     }
 }
 
-// The square matrix [K][K] as terms, rows as they are; `skew` is raised if any two entries across the diagonal differ.  A block
+// The square matrix [K][K] as terms, rows as they are (not wanted: NULL); `skew` is raised if any two entries across the diagonal differ.  A block
 // takes a tile and its mirror image (the blocks of the other triangle leave).
 __global__ void __launch_bounds__(256) split_square_kernel(const float *__restrict__ src, int K, unsigned short *rows, size_t pitch, int *skew)
 {
@@ -369,6 +367,7 @@ __global__ void __launch_bounds__(256) split_square_kernel(const float *__restri
         differ = differ || __float_as_uint(tile[0][r][c]) != __float_as_uint(tile[1][c][r]);
     }
     if (__syncthreads_or(differ) && tid == 0) *skew = 1;
+    if (!rows) return;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int r0 = at[h], c0 = at[1 - h];
@@ -383,9 +382,9 @@ __global__ void __launch_bounds__(256) split_square_kernel(const float *__restri
     }
 }
 
-// Sums the slices of a product [split][R][r] in order; transposed to terms [3][r][pitch], or added to `into` [r][R] times alpha.
+// Sums the slices of a product [split][R][r] in order; transposed to terms [3][r][pitch], or added to `into` (rows `into_ld` apart) times alpha.
 __global__ void __launch_bounds__(256) sum_transposed_kernel(const float *__restrict__ part, int splits, int R, int r, unsigned short *planes, size_t pitch,
-                                                             float *into, float alpha)
+                                                             float *into, size_t into_ld, float alpha)
 {
     __shared__ float tile[32][33];
     const int k0 = blockIdx.x * 32, j0 = blockIdx.y * 32, tid = threadIdx.x;
@@ -405,7 +404,7 @@ __global__ void __launch_bounds__(256) sum_transposed_kernel(const float *__rest
         store_terms(planes + (size_t)(j0 + j) * pitch + k0 + k, (size_t)r * pitch, v, R - (k0 + k));
     } else {
         for (int e = 0; e < 4 && k0 + k + e < R; ++e) {
-            float *a = into + (size_t)(j0 + j) * R + k0 + k + e;
+            float *a = into + (j0 + j) * into_ld + k0 + k + e;
             *a = fmaf(alpha, v[e], *a);
         }
     }
@@ -479,7 +478,7 @@ int triangle_items(int n)
 }
 
 template <int MODE>
-bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p, const Operand *skew_P = nullptr)
+bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p)
 {
     p.M = P.rows; p.N = Q.rows; p.K = P.k;
     p.nt = MODE == kPartial ? std::min(256, (p.N + 31) / 32 * 32) : 256;
@@ -487,10 +486,8 @@ bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p
     p.tiles_n = (p.N + p.nt - 1) / p.nt;
     p.splits = MODE == kPartial ? k_splits(p.M, p.N, p.K) : 1;
     const int n_work = MODE == kPartial ? p.tiles_m * p.tiles_n * p.splits : triangle_items(p.M);
-    CUtensorMap pmap, skew_pmap, qmap;
+    CUtensorMap pmap, qmap;
     if (operand_map(&pmap, P, 128) != cudaSuccess || operand_map(&qmap, Q, p.nt / 2) != cudaSuccess) return false;
-    if (operand_map(&skew_pmap, skew_P ? *skew_P : P, 128) != cudaSuccess) return false;
-    if (MODE == kPartial && !skew_P) p.skew = nullptr;
     auto kern = product_kernel<MODE>;
     static bool attr_set = false;
     if (!attr_set) {
@@ -507,21 +504,21 @@ bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, pmap, skew_pmap, qmap, p, n_work) == cudaSuccess;
+    return cudaLaunchKernelEx(&cfg, kern, pmap, qmap, p, n_work) == cudaSuccess;
 }
-bool split(cudaStream_t s, const float *src, int R, int C, const Operand *rows, const Operand *cols, const int *gate = nullptr)
+bool split(cudaStream_t s, const float *src, size_t ld, int R, int C, const Operand *rows, const Operand *cols, const int *gate = nullptr)
 {
     const dim3 grid((unsigned)((C + 63) / 64), (unsigned)((R + 63) / 64));
-    split_kernel<<<grid, 256, 0, s>>>(src, R, C, rows ? rows->planes : nullptr, rows ? rows->pitch() : 0, cols ? cols->planes : nullptr, cols ? cols->pitch() : 0, gate);
+    split_kernel<<<grid, 256, 0, s>>>(src, ld, R, C, rows ? rows->planes : nullptr, rows ? rows->pitch() : 0, cols ? cols->planes : nullptr, cols ? cols->pitch() : 0, gate);
     return cudaGetLastError() == cudaSuccess;
 }
 
-bool split_square(cudaStream_t s, const float *src, const Operand &rows, const Operand &cols, int *skew)
+bool split_square(cudaStream_t s, const float *src, int K, const Operand *rows, int *skew)
 {
     if (cudaMemsetAsync(skew, 0, sizeof(int), s) != cudaSuccess) return false;
-    const unsigned tiles = (unsigned)((rows.k + 63) / 64);
-    split_square_kernel<<<dim3(tiles, tiles), 256, 0, s>>>(src, rows.k, rows.planes, rows.pitch(), skew);
-    return split(s, src, rows.k, rows.k, nullptr, &cols, skew);
+    const unsigned tiles = (unsigned)((K + 63) / 64);
+    split_square_kernel<<<dim3(tiles, tiles), 256, 0, s>>>(src, K, rows ? rows->planes : nullptr, rows ? rows->pitch() : 0, skew);
+    return cudaGetLastError() == cudaSuccess;
 }
 
 // Carves a call's scratch out of one block.
@@ -551,31 +548,26 @@ int slab_rows(int rows, size_t bytes_per_row, size_t budget)
 }
 struct StepScratch {
     int nd, nh;                             // rows of a slab of Delta_F and of H
-    Operand D, Dt, H, Ht, A, Bt, P, Q;      // slabs of Delta_F and H and their transposes; A, B^T, (H A^T)^T, (B^T Delta_F)
-    float *part, *q_sum, *a_sum;            // partial products; sums over slabs where there are several
+    bool one_d;                             // Delta_F and its transpose one after the other in the same place
+    Operand D, Dt, H, A, Bt, P, Q;          // slabs of Delta_F, its transpose and H; A, B^T, (H A^T)^T, (B^T Delta_F)
+    float *part, *q_sum;                    // partial products; their sum over slabs of Delta_F where there are several
     double *dots;
     int *skew;
     size_t bytes;
     StepScratch(void *base, int N, int K, int r, size_t budget)
     {
         const size_t per_row = 2u * kTerms * (size_t)((K + 7) & ~7);        // bytes of one row's terms
-        nd = N;
-        nh = K;
-        if (2 * per_row * ((size_t)N + K) > budget) {
-            // one slab holds Delta_F and its transpose, of several each holds one after the other in the same place
-            if (2 * per_row * N > budget / 2) nd = slab_rows(N, per_row, std::min(budget / 2, per_row * ((size_t)N - 1)));
-            nh = slab_rows(K, 2 * per_row, budget - std::min(budget / 2, per_row * nd * (nd < N ? 1 : 2)));
-        }
+        one_d = per_row * (2 * (size_t)N + K) > budget;
+        nd = one_d ? slab_rows(N, per_row, budget / 2) : N;
+        nh = one_d ? slab_rows(K, per_row, budget - std::min(budget / 2, per_row * nd)) : K;
         const int slabs = (N + nd - 1) / nd;
         Carver c{static_cast<char *>(base)};
         D = c.operand(nd, K);
-        Dt = slabs == 1 ? c.operand(K, nd) : Operand{nullptr, K, nd};
-        if (slabs > 1) {
-            if (Dt.values() > D.values()) c.take((Dt.values() - D.values()) * 2);               // (rows of nd values are padded to 16 bytes)
-            Dt.planes = D.planes;
-        }
+        Dt = Operand{nullptr, K, nd};
+        if (!one_d) Dt = c.operand(K, nd);
+        else if (Dt.values() > D.values()) c.take((Dt.values() - D.values()) * 2);              // (rows of nd values are padded to 16 bytes)
+        if (one_d) Dt.planes = D.planes;
         H = c.operand(nh, K);
-        Ht = c.operand(K, nh);
         A = c.operand(r, K);
         Bt = c.operand(r, N);
         P = c.operand(r, K);
@@ -583,7 +575,6 @@ struct StepScratch {
         // splits x rows of a product: a work item per pair and kRows rows each, or one split
         part = static_cast<float *>(c.take((size_t)std::max(std::max(K, N), pairs() * kRows) * r * sizeof(float)));
         q_sum = static_cast<float *>(c.take(slabs > 1 ? (size_t)K * r * sizeof(float) : 0));
-        a_sum = static_cast<float *>(c.take(nh < K ? (size_t)K * r * sizeof(float) : 0));
         dots = static_cast<double *>(c.take((size_t)slabs * triangle_items(K) * 2 * kEpiWarps * sizeof(double)));
         skew = static_cast<int *>(c.take(sizeof(int)));
         bytes = c.used;
@@ -617,7 +608,7 @@ int run_gram(const float *X, float *H, int T, int K, size_t budget, void *scratc
     for (int t0 = 0; t0 < T; t0 += nt) {
         const Operand Xt = all.first(K, std::min(nt, T - t0));
         p.add = t0 > 0;
-        if (!split(s, X + (size_t)t0 * K, Xt.k, K, nullptr, &Xt) || !product<kSymmetric>(s, Xt, Xt, p)) return FBQ_ERR_CUDA;
+        if (!split(s, X + (size_t)t0 * K, K, Xt.k, K, nullptr, &Xt) || !product<kSymmetric>(s, Xt, Xt, p)) return FBQ_ERR_CUDA;
         *launches += 2;
     }
     return FBQ_OK;
@@ -636,36 +627,29 @@ int run_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
     bool ok = true;
     auto columns = [&](const float *part, int splits, int rows, unsigned short *planes, size_t pitch, float *into, float alpha) {
         const dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((rank + 31) / 32));
-        sum_transposed_kernel<<<grid, 256, 0, s>>>(part, splits, rows, rank, planes, pitch, into, alpha);
+        sum_transposed_kernel<<<grid, 256, 0, s>>>(part, splits, rows, rank, planes, pitch, into, (size_t)K, alpha);
         ++*launches;
     };
     auto add = [&](const float *part, int splits, size_t n, float *into, float alpha) {
         sum_into_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, splits, n, into, alpha);
         ++*launches;
     };
-    auto times = [&](const Operand &P, const Operand &Q, const Operand *skew_P = nullptr) {      // -> number of splits in t.part
-        ok = ok && product<kPartial>(s, P, Q, p, skew_P);
+    auto times = [&](const Operand &P, const Operand &Q) {      // -> number of splits in t.part
+        ok = ok && product<kPartial>(s, P, Q, p);
         ++*launches;
         return k_splits(P.rows, Q.rows, P.k);
     };
     // Delta_F with Q(W - B A) held fixed (nothing else of the quantiser's output is kept)
     float *Delta = ws;
     if (launch_quantize_feedback(W, A, B, nullptr, nullptr, nullptr, nullptr, Delta, N, K, group, bits, rank, 2, s) != cudaSuccess) return FBQ_ERR_CUDA;
-    ok = split(s, A, rank, K, &t.A, nullptr) && split(s, B, N, rank, nullptr, &t.Bt);
-    *launches += 3;
-    // One slab of H: its rows serve as its columns where it is symmetric.  Of several each is taken as it is.
-    if (slabs_h == 1) {
-        ok = ok && split_square(s, H, t.H, t.Ht, t.skew);
-        *launches += 2;
-    } else {
-        ok = ok && cudaMemsetAsync(t.skew, 1, sizeof(int), s) == cudaSuccess && cudaMemsetAsync(t.a_sum, 0, nq * sizeof(float), s) == cudaSuccess;
-    }
+    ok = split(s, A, K, rank, K, &t.A, nullptr) && split(s, B, rank, N, rank, nullptr, &t.Bt) && split_square(s, H, K, slabs_h == 1 ? &t.H : nullptr, t.skew);
+    *launches += 4;
     // slabs of Delta_F, transposed: the loss tr(Delta H Delta^T) = sum H o (Delta^T Delta), elementwise, and Delta^T B [K x rank]
     if (slabs_d > 1) ok = ok && cudaMemsetAsync(t.q_sum, 0, nq * sizeof(float), s) == cudaSuccess;
     for (int i = 0; i < slabs_d && ok; ++i) {
         const int n0 = i * t.nd, n = std::min(t.nd, N - n0);
         const Operand D = t.D.first(n, K), Dt = t.Dt.first(K, n);
-        ok = split(s, Delta + (size_t)n0 * K, n, K, slabs_d == 1 ? &D : nullptr, &Dt);
+        ok = split(s, Delta + (size_t)n0 * K, K, n, K, t.one_d ? nullptr : &D, &Dt);
         ++*launches;
         if (loss) {
             ProductParams d = p;
@@ -683,25 +667,26 @@ int run_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
         sum_dots_kernel<<<1, 256, 0, s>>>(t.dots, slabs_d * items, loss);
         ++*launches;
     }
-    // slabs of H: H A^T [K x rank], and A <- A + 2 lr (B^T Delta) H from the old A and B
+    // Slabs of H: H A^T [K x rank] from its rows; A <- A + 2 lr (B^T Delta) H from its columns, which take the rows' place unless
+    // H is symmetric and they are the same (A and B enter as they were: their terms are made above).
     for (int i = 0; i < slabs_h && ok; ++i) {
         const int k0 = i * t.nh, n = std::min(t.nh, K - k0);
-        const Operand rows = t.H.first(n, K), cols = t.Ht.first(K, n);
+        const Operand Hs = t.H.first(n, K);
         if (slabs_h > 1) {
-            ok = split(s, H + (size_t)k0 * K, n, K, &rows, &cols);
+            ok = split(s, H + (size_t)k0 * K, K, n, K, &Hs, nullptr);
             ++*launches;
         }
-        columns(t.part, times(rows, t.A), n, t.P.planes + k0, t.P.pitch(), nullptr, 0.f);
-        if (slabs_h == 1) columns(t.part, times(t.H, t.Q, &t.Ht), K, nullptr, 0, A, 2.f * lr);
-        else columns(t.part, times(cols, t.Q.k_range(k0, n)), K, nullptr, 0, t.a_sum, 1.f);
+        columns(t.part, times(Hs, t.A), n, t.P.planes + k0, t.P.pitch(), nullptr, 0.f);
+        ok = ok && split(s, H + k0, K, K, n, nullptr, &Hs, t.skew);
+        ++*launches;
+        columns(t.part, times(Hs, t.Q), n, nullptr, 0, A + k0, 2.f * lr);
     }
-    if (slabs_h > 1) add(t.a_sum, 1, nq, A, 2.f * lr);
     // slabs of Delta_F: B <- B + 2 lr Delta (H A^T)
     for (int i = 0; i < slabs_d && ok; ++i) {
         const int n0 = i * t.nd, n = std::min(t.nd, N - n0);
         const Operand D = t.D.first(n, K);
-        if (slabs_d > 1) {
-            ok = split(s, Delta + (size_t)n0 * K, n, K, &D, nullptr);
+        if (t.one_d) {
+            ok = split(s, Delta + (size_t)n0 * K, K, n, K, &D, nullptr);
             ++*launches;
         }
         add(t.part, times(D, t.P), (size_t)n * rank, B + (size_t)n0 * rank, 2.f * lr);

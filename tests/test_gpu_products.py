@@ -107,11 +107,11 @@ def test_step_in_slabs(one_megabyte, N, K, rank):
 
 
 def test_scratch_of_a_large_step_is_bounded():
-    # Delta and H of 2048 x 8192 split as a whole are 1 GB; the default bound is 512 MB beyond what the rank needs.  Reference in
-    # float64 from the library's own Delta, which the tests of the quantiser pin.
+    # Delta, its transpose and H of 3072 x 12288 split as a whole are 1.36 GB; the default bound is 1 GB beyond what the rank needs.
+    # Reference in float64 from the library's own Delta, which the tests of the quantiser pin.
     import torch
     import paper_2501_16385_b200 as fbq
-    N, K, rank = 2048, 8192, 16
+    N, K, rank = 3072, 12288, 16
     g = torch.Generator(device="cuda")
     g.manual_seed(5)
     W = torch.randn((N, K), device="cuda", generator=g) * 0.05
@@ -129,7 +129,7 @@ def test_scratch_of_a_large_step_is_bounded():
     free = torch.cuda.mem_get_info()[0]
     loss, _ = fbq.reconstruct_step(W, H, A, B, lr, 128, 4, workspace=ws)
     assert fbq.poll_status() == 0
-    assert free - torch.cuda.mem_get_info()[0] < 600 << 20
+    assert free - torch.cuda.mem_get_info()[0] < 1100 << 20
     # W_F and Delta are rounded to fp32 differently (W_F has 2^-24 of |W|, about 2^-20 of |Delta|)
     assert abs(float(loss.item()) - want_loss) <= 1e-5 * want_loss
     assert float((A.double() - want_a).norm() / want_a.norm()) < 1e-6

@@ -1789,6 +1789,7 @@ struct Plan {
 
 int g_sm_count = 0;
 constexpr size_t kSmemMax = 227 * 1024;
+constexpr size_t kSmemShare = (kCtasPerSm == 2 ? 113 * 1024 : kSmemMax) - 2048;     // of a CTA that is not alone on its SM
 
 bool print_plans()
 {
@@ -1883,8 +1884,15 @@ Plan make_plan_on(const LinearArgs &a, const GemvTuning &tune, int per_sm)
         off += (size_t)ns * p.stage_bytes;
         return off;
     };
-    // as many stages as fit the CTA's share of an SM's shared memory (all of a CTA's stages where they are few)
-    const size_t budget = (kCtasPerSm == 2 ? 113 * 1024 : kSmemMax) - 2048;
+    // a t CTA: barriers, its blocks of A (1024-byte aligned), the reduction buffer
+    p.off_tA = 1024;
+    p.off_tred = p.off_tA + p.t_kb * a.rank * 128;
+    const size_t need_t = a.rank > 0 ? (size_t)p.off_tred + (size_t)kCW * a.rank * 2 * 4 : 0;      // M <= 2: two columns
+    if (need_t > kSmemMax) return pl;
+    // As many stages as fit the CTA's share of an SM's shared memory (all of a CTA's stages where they are few).  In a batch whose
+    // t CTAs take more than a share every CTA has an SM to itself (2 x 13824 -> 5120, INT3, one token, rank 128: a ring of
+    // eight stages instead of two, 56 -> 26 us).
+    const size_t budget = tune.main_ctas > 0 && need_t > kSmemShare ? kSmemMax - 2048 : kSmemShare;
     int ns = std::min(kMaxNS, std::max(2, nseg * SPT));
     while (ns > 2 && layout(ns) > budget) --ns;
     size_t need = layout(ns);
@@ -1894,11 +1902,6 @@ Plan make_plan_on(const LinearArgs &a, const GemvTuning &tune, int per_sm)
         need = layout(ns);
         if (need > kSmemMax - 2048) return pl;
     }
-    // a t CTA: barriers, its blocks of A (1024-byte aligned), the reduction buffer
-    p.off_tA = 1024;
-    p.off_tred = p.off_tA + p.t_kb * a.rank * 128;
-    const size_t need_t = a.rank > 0 ? (size_t)p.off_tred + (size_t)kCW * a.rank * 2 * 4 : 0;      // M <= 2: two columns
-    if (need_t > kSmemMax) return pl;
     p.slot_elems = (a.M * a.rank + 31) / 32 * 32;
     p.t_final = (p.n_t * a.M * a.rank > 1024) ? 1 : 0;    // many entries: one t CTA adds the slots for everybody
     if (per_sm == 2 && std::max(need, need_t) > budget) return pl;
@@ -2198,16 +2201,17 @@ cudaError_t make_maps(const LinearArgs &a, const GemvParams &p, CUtensorMap *wma
 // Plans of a batch's problems: the main CTAs are shared out so that the fullest one has as little as possible (tiles times
 // stages per tile).  Integer form: two CTAs per SM (a launch of several problems lasts long enough that filling the
 // SMs with its own CTAs pays more than letting the next launch's in; 4096 -> 3 x 4096 INT3 rank 64: 8.8 us, 11.3 with one,
-// 15.4 as three launches; 4096 -> 2 x 11008: 12.7, 15.6, 17.2); 16-bit form: one (its CTAs take a whole SM; four tokens:
-// 17.9 and 26.1 us, one by one 28.1 and 31.5).
+// 15.4 as three launches; 4096 -> 2 x 11008: 12.7, 15.6, 17.2), unless a CTA of the launch needs more than half of an SM's
+// shared memory (t CTAs of rank 112 and 128, x of a long K): then one, where two would run in two rounds (rank 128, INT4, one
+// token: 4096 -> 3 x 4096 14.1 / 12.0 us, 4096 -> 2 x 11008 19.0 / 16.9, 13824 -> 2 x 5120 50.8 / 25.7); 16-bit form: one (its
+// CTAs take a whole SM; four tokens: 17.9 and 26.1 us, one by one 28.1 and 31.5).
 struct BatchPlan {
     Plan plan[kGemvBatchMax];
     bool ok = false;
 };
-BatchPlan plan_batch(const LinearArgs *a, int count, const GemvTuning &tune)
+BatchPlan plan_batch_on(const LinearArgs *a, int count, const GemvTuning &tune, int per_sm)
 {
     BatchPlan bp;
-    if (count < 1 || count > kGemvBatchMax) return bp;
     const bool wide = a[0].M > 2;
     GemvTuning t = tune;
     t.max_ctas = 0;
@@ -2223,7 +2227,7 @@ BatchPlan plan_batch(const LinearArgs *a, int count, const GemvTuning &tune)
         const int nt = (a[i].N + kTile - 1) / kTile, most = std::max(1, load / stages(i)), c = (nt + most - 1) / most;
         return wide ? std::max(2, (c + 1) / 2 * 2) : c;
     };
-    const int budget = std::max(2 * count, (wide ? 1 : 2) * g_sm_count - n_t);
+    const int budget = std::max(2 * count, per_sm * g_sm_count - n_t);
     int lo = 1, hi = 1;
     auto total = [&](int load) { int c = 0; for (int i = 0; i < count; ++i) c += share(i, load); return c; };
     while (total(hi) > budget && hi < (1 << 24)) hi *= 2;
@@ -2236,9 +2240,17 @@ BatchPlan plan_batch(const LinearArgs *a, int count, const GemvTuning &tune)
         t.main_ctas = share(i, lo);
         bp.plan[i] = plan_for(a[i], t);
         if (!bp.plan[i].ok || (wide && (bp.plan[i].p.R & 1 || bp.plan[i].p.R < 2))) return bp;
+        if (per_sm == 2 && bp.plan[i].smem > kSmemShare + 1024) return bp;       // (the launch takes the most that any of its CTAs needs)
     }
     bp.ok = true;
     return bp;
+}
+BatchPlan plan_batch(const LinearArgs *a, int count, const GemvTuning &tune)
+{
+    if (count < 1 || count > kGemvBatchMax) return BatchPlan{};
+    if (a[0].M <= 2)
+        if (const BatchPlan bp = plan_batch_on(a, count, tune, 2); bp.ok) return bp;
+    return plan_batch_on(a, count, tune, 1);
 }
 size_t slot_floats(const GemvParams &p) { return (size_t)(std::max(p.n_t, 1) + 1) * std::max(p.slot_elems, 32); }
 }  // namespace

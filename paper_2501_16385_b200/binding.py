@@ -83,7 +83,7 @@ def native():
         import torch  # noqa: F401  (its libraries have to be in the process first)
         lib()
         if not os.path.exists(_build.TORCH_LIB):
-            _build.build()
+            _build.build_binding()
         import importlib.util
         spec = importlib.util.spec_from_file_location("_fbq_torch", _build.TORCH_LIB)
         mod = importlib.util.module_from_spec(spec)

@@ -1,5 +1,6 @@
-"""Builds libfbq.so (CUDA kernels + C ABI) in-tree with nvcc for sm_100a, and beside it
-_fbq_torch.so, the native part of the Python binding (g++, torch's headers).
+"""Builds libfbq.so (CUDA kernels + C ABI) in-tree with nvcc for sm_100a (`build`, which needs nothing
+else), and beside it _fbq_torch.so, the native part of the Python binding (`build_binding`: g++ and
+torch's headers).  Run as a program it builds both, or the library alone where torch is not installed.
 
 Every source file is compiled to an object of its own (in parallel, and only
 when it or a header changed), then the objects are linked into the shared
@@ -45,15 +46,16 @@ def _stale_obj(src: str, force: bool) -> bool:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(TORCH_LIB):
+    if not os.path.exists(LIB):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(TORCH_LIB))
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
-    deps.append(os.path.join(HERE, "..", "include", "fbq.h"))
-    return any(os.path.getmtime(d) > t for d in deps)
+    t = os.path.getmtime(LIB)
+    return any(os.path.getmtime(d) > t for d in [os.path.join(CSRC, f) for f in SOURCES] + _headers())
 
 
-def _build_binding() -> None:
+def build_binding(force: bool = False) -> str:
+    deps = (os.path.join(CSRC, TORCH_SRC), os.path.join(HERE, "..", "include", "fbq.h"))
+    if not force and os.path.exists(TORCH_LIB) and all(os.path.getmtime(d) <= os.path.getmtime(TORCH_LIB) for d in deps):
+        return TORCH_LIB
     import sysconfig
 
     import torch
@@ -70,6 +72,7 @@ def _build_binding() -> None:
         sys.stderr.write(res.stdout + res.stderr)
         raise RuntimeError("g++ failed building _fbq_torch.so")
     os.replace(tmp, TORCH_LIB)
+    return TORCH_LIB
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -102,13 +105,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if res.returncode != 0:
         raise RuntimeError("nvcc failed linking libfbq.so")
     os.replace(tmp, LIB)
-    if force or not os.path.exists(TORCH_LIB) or any(os.path.getmtime(d) > os.path.getmtime(TORCH_LIB)
-                                                     for d in (os.path.join(CSRC, TORCH_SRC), os.path.join(HERE, "..", "include", "fbq.h"))):
-        _build_binding()
-    else:
-        os.utime(TORCH_LIB)
     return LIB
 
 
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose=True))
+    import importlib.util
+    if importlib.util.find_spec("torch"):
+        print(build_binding(force="--force" in sys.argv))

@@ -307,8 +307,8 @@ int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int ac
  *                   behind the kernel); 0 = y always goes through the stream's staging buffer and a copy
  *   "scratch_mb"    0 (default) = 1024, else the number of megabytes that the scratch of fbq_gram and
  *                   fbq_reconstruct_step is held to (a slab of 256 rows and what the rank needs come on top)
- *   "pdl"           1 = launch with programmatic dependent launch (default), 0 = plain.  With 1 a decode or
- *                   prefill kernel may start while the kernel before it on the stream still runs: it sets
+ *   "pdl"           1 = launch with programmatic dependent launch (default), 0 = plain.  With 1 a decode,
+ *                   prefill or reconstruction kernel may start while the kernel before it on the stream still runs: it sets
  *                   itself up, and the decode kernels already fetch qweight, scales, zeros, A and B, before
  *                   they wait for that kernel; x, y and the scratch are touched only after the wait.  So
  *                   the weight operands must not be written by the launch directly before (x may be)

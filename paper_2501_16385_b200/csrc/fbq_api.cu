@@ -512,7 +512,7 @@ int fbq_gram(const float *X, float *H, int T, int K, void *stream)
     if (!X || !H || T < 1 || K < 1) return FBQ_ERR_BADARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     return with_scratch([&](size_t budget) { return gram_scratch_bytes(T, K, budget); }, s,
-                        [&](size_t budget, void *scratch, int *status, int *n) { return run_gram(X, H, T, K, budget, scratch, status, s, n); });
+                        [&](size_t budget, void *scratch, int *status, int *n) { return run_gram(X, H, T, K, budget, scratch, status, g_opt.decode.pdl != 0, s, n); });
 }
 
 int fbq_reconstruct_step(const float *W, const float *H, float *A, float *B, float lr, float *loss, float *workspace, int N,
@@ -528,7 +528,8 @@ int fbq_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
     const size_t shift = (size_t)(spare - reinterpret_cast<char *>(workspace));
     return with_scratch([&](size_t budget) { return reconstruct_scratch_bytes(N, K, rank, budget); }, s,
                         [&](size_t budget, void *scratch, int *status, int *n) {
-                            return run_reconstruct_step(W, H, A, B, lr, loss, workspace, N, K, group, bits, rank, budget, scratch, status, s, n);
+                            return run_reconstruct_step(W, H, A, B, lr, loss, workspace, N, K, group, bits, rank, budget, scratch, status,
+                                                        g_opt.decode.pdl != 0, s, n);
                         },
                         spare, all > shift ? all - shift : 0);
 }

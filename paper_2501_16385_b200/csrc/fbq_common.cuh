@@ -79,9 +79,10 @@ size_t reconstruct_workspace_floats(int N, int K, int rank);
 // Scratch of the two: about `budget` bytes at most, beyond what one slab of rows and the rank need.
 size_t gram_scratch_bytes(int T, int K, size_t budget);
 size_t reconstruct_scratch_bytes(int N, int K, int rank, size_t budget);
-int run_gram(const float *X, float *H, int T, int K, size_t budget, void *scratch, int *status, cudaStream_t s, int *launches);
+int run_gram(const float *X, float *H, int T, int K, size_t budget, void *scratch, int *status, bool pdl, cudaStream_t s, int *launches);
 int run_reconstruct_step(const float *W, const float *H, float *A, float *B, float lr, float *loss, float *ws, int N, int K,
-                         int group, int bits, int rank, size_t budget, void *scratch, int *status, cudaStream_t s, int *launches);
+                         int group, int bits, int rank, size_t budget, void *scratch, int *status, bool pdl, cudaStream_t s,
+                         int *launches);
 
 struct DecodeTuning {
     int sk = 0, chunk = 0, depth = 0, max_ctas = 0, pdl = 1;

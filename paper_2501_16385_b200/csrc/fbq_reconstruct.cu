@@ -478,7 +478,7 @@ int triangle_items(int n)
 }
 
 template <int MODE>
-bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p)
+bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p, bool pdl)
 {
     p.M = P.rows; p.N = Q.rows; p.K = P.k;
     p.nt = MODE == kPartial ? std::min(256, (p.N + 31) / 32 * 32) : 256;
@@ -503,7 +503,7 @@ bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, pmap, qmap, p, n_work) == cudaSuccess;
 }
 bool split(cudaStream_t s, const float *src, size_t ld, int R, int C, const Operand *rows, const Operand *cols, const int *gate = nullptr)
@@ -597,7 +597,7 @@ size_t gram_scratch_bytes(int T, int K, size_t budget)
 size_t reconstruct_scratch_bytes(int N, int K, int rank, size_t budget) { return StepScratch(nullptr, N, K, rank, budget).bytes; }
 
 // H[K x K] = X^T X for X [T x K]; several slabs of X are added one after the other
-int run_gram(const float *X, float *H, int T, int K, size_t budget, void *scratch, int *status, cudaStream_t s, int *launches)
+int run_gram(const float *X, float *H, int T, int K, size_t budget, void *scratch, int *status, bool pdl, cudaStream_t s, int *launches)
 {
     const int nt = gram_slab(T, K, budget);
     Carver c{static_cast<char *>(scratch)};
@@ -608,14 +608,14 @@ int run_gram(const float *X, float *H, int T, int K, size_t budget, void *scratc
     for (int t0 = 0; t0 < T; t0 += nt) {
         const Operand Xt = all.first(K, std::min(nt, T - t0));
         p.add = t0 > 0;
-        if (!split(s, X + (size_t)t0 * K, K, Xt.k, K, nullptr, &Xt) || !product<kSymmetric>(s, Xt, Xt, p)) return FBQ_ERR_CUDA;
+        if (!split(s, X + (size_t)t0 * K, K, Xt.k, K, nullptr, &Xt) || !product<kSymmetric>(s, Xt, Xt, p, pdl)) return FBQ_ERR_CUDA;
         *launches += 2;
     }
     return FBQ_OK;
 }
 
 int run_reconstruct_step(const float *W, const float *H, float *A, float *B, float lr, float *loss, float *ws, int N, int K, int group, int bits,
-                         int rank, size_t budget, void *scratch, int *status, cudaStream_t s, int *launches)
+                         int rank, size_t budget, void *scratch, int *status, bool pdl, cudaStream_t s, int *launches)
 {
     const StepScratch t(scratch, N, K, rank, budget);
     const int slabs_d = (N + t.nd - 1) / t.nd, slabs_h = (K + t.nh - 1) / t.nh, items = triangle_items(K) * 2 * kEpiWarps;
@@ -635,7 +635,7 @@ int run_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
         ++*launches;
     };
     auto times = [&](const Operand &P, const Operand &Q) {      // -> number of splits in t.part
-        ok = ok && product<kPartial>(s, P, Q, p);
+        ok = ok && product<kPartial>(s, P, Q, p, pdl);
         ++*launches;
         return k_splits(P.rows, Q.rows, P.k);
     };
@@ -655,7 +655,7 @@ int run_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
             ProductParams d = p;
             d.H = H;
             d.dots = t.dots + (size_t)i * items;
-            ok = ok && product<kDot>(s, Dt, Dt, d);
+            ok = ok && product<kDot>(s, Dt, Dt, d, pdl);
             ++*launches;
         }
         const int splits = times(Dt, t.Bt.k_range(n0, n));

@@ -134,3 +134,23 @@ def test_scratch_of_a_large_step_is_bounded():
     assert abs(float(loss.item()) - want_loss) <= 1e-5 * want_loss
     assert float((A.double() - want_a).norm() / want_a.norm()) < 1e-6
     assert float((B.double() - want_b).norm() / want_b.norm()) < 1e-6
+
+
+def test_products_without_dependent_launch_are_the_same():
+    import torch
+    import paper_2501_16385_b200 as fbq
+    g = torch.Generator(device="cuda")
+    g.manual_seed(9)
+    X, W = torch.randn((500, 512), device="cuda", generator=g), torch.randn((300, 512), device="cuda", generator=g) * 0.05
+    A, B = torch.randn((24, 512), device="cuda", generator=g) * 0.05, torch.randn((300, 24), device="cuda", generator=g) * 0.05
+    got = []
+    for pdl in (1, 0):
+        fbq.set_option("pdl", pdl)
+        try:
+            a, b, H = A.clone(), B.clone(), fbq.gram(X)
+            loss, _ = fbq.reconstruct_step(W, H, a, b, 1e-6, 128, 4)
+            got.append((H, a, b, loss))
+        finally:
+            fbq.set_option("pdl", 1)
+    assert fbq.poll_status() == 0
+    assert all(torch.equal(u, v) for u, v in zip(*got))

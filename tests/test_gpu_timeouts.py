@@ -67,3 +67,30 @@ def test_prefill_wait_for_t_runs_out(fbq):
         fbq.set_option("prefill_flag_polls", 0)
     assert fbq.poll_status() == 0
     check_parity(inp, fbq)
+
+
+def test_dense_prefill_wait_for_t_runs_out(fbq):
+    # 1100 tokens x 13064 features: the kernel that dequantises once per call, whose tiles of t tag themselves
+    import torch
+    inp = make_linear(1100, 13064, 256, 4, 64, seed=84)
+    rows = list(range(0, 13064, 997))
+    before = fbq.launch_count()
+    check_parity(inp, fbq, n_list=rows)
+    dev = DeviceLinear(inp, fbq)
+    want = dev.run(fbq)
+    torch.cuda.synchronize()
+    assert fbq.launch_count() - before == 4                   # two of them pack the codes
+    fbq.set_option("test_prefill_skip_flag", 1)
+    fbq.set_option("prefill_flag_polls", 2000)
+    try:
+        dev.run(fbq)
+        torch.cuda.synchronize()                              # the kernel returned
+        assert fbq.poll_status() == FBQ_ERR_TIMEOUT
+    finally:
+        fbq.set_option("test_prefill_skip_flag", 0)
+        fbq.set_option("prefill_flag_polls", 0)
+    assert fbq.poll_status() == 0                             # tags and counters start again
+    for _ in range(2):
+        assert torch.equal(dev.run(fbq), want)
+    assert fbq.poll_status() == 0
+    check_parity(make_linear(700, 22024, 128, 3, 8, seed=85), fbq, n_list=[0, 11000, 22023])

@@ -291,10 +291,10 @@ int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int ac
  *   "decode_t_wait" 1 (default) = a finished tile may wait for t in shared memory while that holds nobody up,
  *                   0 = it is parked in scratch at once (only matters without t CTAs)
  *   "batch_ctas"    CTAs shared out among the problems of a decode-sized fbq_linear_batch (default 400)
- *   "prefill_pair"  (calls of few tiles; with more than three waves of them the prefill runs on CTA pairs anyway)
- *                   1 = token tiles of 256 of the prefill kernel run on CTA pairs (cta_group::2 MMAs,
- *                   each CTA staging half of the token tile); 0 (default) = one CTA per tile, which
- *                   measured faster
+ *   "prefill_pair"  1 = token tiles of 256 (calls of more than 128 tokens) run on CTA pairs that dequantise in place
+ *                   (cta_group::2 MMAs, each CTA staging half of the token tile); 0 (default) = one CTA per tile, or
+ *                   with more than three waves of tiles the kernel that dequantises once per call, which measured
+ *                   faster
  *   "prefill_split" the prefill kernel at M <= 128, where a shape has fewer 128-row tiles than SMs: K is cut
  *                   into up to 8 slices, one CTA each, which store fp32 partial tiles to the stream's scratch;
  *                   the CTA that finishes last adds them in slice order and writes y (results do not depend

@@ -309,7 +309,7 @@ int run_linear(const LinearArgs &a, cudaStream_t s, int decode_ctas = 0)
         prefill_workspace_need(a, &need_c, &need_t, &need_p);
         // The dense kernel's matrix of weights is the largest scratch by far and the other kernel computes the same call without
         // it: where it cannot be had (device memory is used up, or the stream is being captured) that one runs.
-        bool dense = prefill_dense(a);
+        bool dense = !g_opt.prefill_pair && prefill_dense(a);
         if (dense) {
             size_t need_w = 0, need_tags = 0, tf = 0;
             dense_workspace_need(a, &need_w, &need_tags, &tf);

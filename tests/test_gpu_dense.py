@@ -99,3 +99,27 @@ def test_dense_prefill_without_its_scratch_runs_the_other_kernel():
             assert fbq.poll_status(stream) == 0
             # the same products of the same rounded weights and t, sums in another order: one rounding to fp16 apart
             assert float((y.float() - want.float()).norm() / want.float().norm()) < 2 ** -10
+
+
+def test_pair_option_holds_for_many_tiles():
+    # the option's kernel dequantises in place: the call takes none of the 16-bit weights' scratch (67 MB here)
+    import torch
+    import paper_2501_16385_b200 as fbq
+    inp = make_linear(1100, 13064, 2560, 4, 64, seed=3500)
+    rows = np.arange(3, inp.N, 501)
+    dev = DeviceLinear(inp, fbq)
+    taken = []
+    for pair in (0, 1):
+        fbq.set_option("prefill_pair", pair)
+        try:
+            dev.run(fbq)                                     # the output's memory is with torch, the kernel is loaded
+            torch.cuda.synchronize()
+            fbq.release_workspaces()
+            before = torch.cuda.mem_get_info()[0]
+            dev.run(fbq)
+            torch.cuda.synchronize()
+            taken.append(before - torch.cuda.mem_get_info()[0])
+            check_parity(inp, fbq, expect_kernel=fbq.KERNEL_PREFILL, n_list=rows, threads=16, floor=2e-5)
+        finally:
+            fbq.set_option("prefill_pair", 0)
+    assert taken[0] >= inp.N * inp.K * 2 > taken[1]

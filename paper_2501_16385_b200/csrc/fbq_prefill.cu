@@ -53,9 +53,11 @@
 #include "fbq_common.cuh"
 #include "fbq_dequant.cuh"
 #include "fbq_maps.h"
+#include "fbq_umma.cuh"
 
 namespace fbq {
 namespace {
+using namespace ptx;
 
 constexpr int kBN = 128;                           // weight rows per CTA tile (MMA M)
 constexpr int kBK = 64;                            // K block (one pipeline stage)
@@ -96,92 +98,29 @@ struct PrefillParams {
     int rank_pad;             // columns of t16: rank rounded up to whole K blocks of 64 (the padding is zero)
 };
 
-// ---------------------------------------------------------------- PTX helpers
-__device__ __forceinline__ uint32_t pf_smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void pf_mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void pf_mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool pf_mbar_wait(uint32_t bar, uint32_t parity)
+// ---------------------------------------------------------------- PTX helpers of this file
+// Bounded by looks (each may sleep in hardware) and inline, unlike ptx::mbar_wait: the producers' loop has no call in it.
+__device__ __forceinline__ bool wait_looks(uint32_t bar, uint32_t parity)
 {
 #pragma unroll 1
-    for (uint32_t i = 0; i < kPfWaitLimit; ++i) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (ok) return true;
-    }
+    for (uint32_t i = 0; i < kPfWaitLimit; ++i)
+        if (mbar_try_wait(bar, parity)) return true;
     return false;
 }
-__device__ __forceinline__ void pf_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pf_fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
+__device__ __forceinline__ bool wait_looks_cluster(uint32_t bar, uint32_t parity)     // sees arrivals from the peer CTA
+{
+#pragma unroll 1
+    for (uint32_t i = 0; i < kPfWaitLimit; ++i)
+        if (umma::try_wait_cluster(bar, parity)) return true;
+    return false;
+}
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t on;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(on));
     return on != 0u;
 }
-// Shared-memory operand descriptor: K-major tile with 128-byte rows (64 16-bit elements) in the
-// 128-byte swizzle (the 16-byte chunk c of row r is stored at chunk c ^ (r % 8)); groups of 8
-// rows are 1024 bytes apart.
-__device__ __forceinline__ uint64_t make_desc(uint32_t smem_addr)
-{
-    return (uint64_t)((smem_addr >> 4) & 0x3FFFu) | (1ull << 16) | ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-// D[tmem] (+)= A[smem] * B[smem]^T, 128 x N x 16, fp32 accumulate.
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// Arrive on an mbarrier once every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void tc_commit(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// --------------------------------------------------------------------- kernel
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
-        : "memory");
-}
-__device__ __forceinline__ void pf_mbar_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
+// Shared-memory loads that stay behind the waits before them (the ones in ptx order themselves with other asm only).
 __device__ __forceinline__ uint32_t lds32(uint32_t addr)
 {
     uint32_t v;
@@ -199,6 +138,7 @@ __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, ui
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
+// --------------------------------------------------------------------- kernel
 // Shared-memory map of a CTA (byte offsets from the 1024-byte aligned base)
 template <int TOK> struct Smem {
     static constexpr uint32_t kXBytes = (uint32_t)TOK * kBK * 2u;          // token operand tile of a stage
@@ -233,7 +173,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     constexpr uint32_t kXBytes = L::kXBytes, kStageBytes = L::kStageBytes;
     constexpr int WPG = (BITS == 4) ? 16 : 12;                  // packed words per row and group
     extern __shared__ __align__(1024) uint8_t smem[];
-    const uint32_t sbase = pf_smem_u32(smem);
+    const uint32_t sbase = smem_u32(smem);
     if (sbase & 1023u) {                                        // swizzle atoms need a 1024-byte aligned base
         if (threadIdx.x == 0) atomicExch(p.status, (int)FBQ_ERR_CUDA);
         return;
@@ -270,50 +210,47 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 
     if (tid == 0) {
         for (int i = 0; i < kStages; ++i) {
-            pf_mbar_init(full0 + 8u * i, t_role ? 1 : kHalf / 32 + 1);   // 8 producer warps + the TMA lane
-            pf_mbar_init(empty0 + 8u * i, 1);
+            mbar_init(full0 + 8u * i, t_role ? 1 : kHalf / 32 + 1);   // 8 producer warps + the TMA lane
+            mbar_init(empty0 + 8u * i, 1);
         }
         for (int i = 0; i < kRing; ++i) {
-            pf_mbar_init(rfull0 + 8u * i, 2);                   // the two ring warps
-            pf_mbar_init(rempty0 + 8u * i, kHalf / 32);         // a group is consumed by one half of the producers (8 warps)
+            mbar_init(rfull0 + 8u * i, 2);                   // the two ring warps
+            mbar_init(rempty0 + 8u * i, kHalf / 32);         // a group is consumed by one half of the producers (8 warps)
         }
-        pf_mbar_init(done_bar, 1);
-        for (int i = 0; i < 4; ++i) pf_mbar_init(epi0 + 8u * i, 128);     // the four warps of a column quarter
-        pf_mbar_init(split_bar, kProducers / 32);               // every epilogue warp has stored its partial chunk
-        pf_mbar_init(split_bar2, 1);                            // warp 0 has counted the CTA in
+        mbar_init(done_bar, 1);
+        for (int i = 0; i < 4; ++i) mbar_init(epi0 + 8u * i, 128);     // the four warps of a column quarter
+        mbar_init(split_bar, kProducers / 32);               // every epilogue warp has stored its partial chunk
+        mbar_init(split_bar2, 1);                            // warp 0 has counted the CTA in
         *abort_flag = 0;
         *split_last = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_barrier_init();
     }
     if (warp == kMmaWarp) {                  // the MMA warp owns the tensor-memory allocation
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(pf_smem_u32(tmem_slot)),
-                     "r"((uint32_t)TOK)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        tc_fence_before();
+        umma::tmem_alloc<1>(smem_u32(tmem_slot), (uint32_t)TOK);
+        umma::fence_before();
     }
     if (warp == kTmaWarp && lane == 0) {
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&xmap)) : "memory");
+        prefetch_tensormap(&xmap);
         if (t_role) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&amap)) : "memory");
+            prefetch_tensormap(&amap);
         } else {
-            if (p.rank > 0) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&bmap)) : "memory");
-            if (p.t16) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&ymap)) : "memory");
+            if (p.rank > 0) prefetch_tensormap(&bmap);
+            if (p.t16) prefetch_tensormap(&tmap);
+            prefetch_tensormap(&ymap);
         }
     }
     if (warp == kRawWarp && lane == 0)
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&wmap)) : "memory");
+        prefetch_tensormap(&wmap);
     __syncthreads();
-    tc_fence_after();
+    umma::fence_after();
     const uint32_t tmem_base = *tmem_slot;
     // Programmatic dependent launch: the CTAs of the launch that follows may take their SMs as soon as ours leave
     // them and run their own set-up above; nothing before this point reads or writes global memory, everything
     // after it waits for the preceding launch to have completed (so no bounded wait below spans that launch).
     // Letting the ring of packed codes and the first two dequantised groups start before the wait was measured
     // and changed nothing (68.8 against 68.9 us per linear of a layer step).
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    pf_pdl_wait();
+    pdl_launch_dependents();
+    pdl_wait();
 
     if (warp < kMmaWarp) {
         bool dead = false;
@@ -342,7 +279,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             uint32_t slot = (uint32_t)h, rphase = 0u, ephase = 0u;
 #pragma unroll 1
             for (int g = h; g < groups; g += 2) {
-                if (!pf_mbar_wait(rfull0 + 8u * slot, rphase)) { dead = true; break; }
+                if (!wait_looks(rfull0 + 8u * slot, rphase)) { dead = true; break; }
                 constexpr int NW = (BITS == 4) ? 4 : 3;
                 uint32_t w[2][NW];
                 const uint32_t rs = ring0 + slot * kRawSlot;
@@ -359,14 +296,14 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 }
                 const uint32_t sz = lds32(table0 + slot * (kBN * 4u));      // s | z << 16 of (row, group)
                 __syncwarp();
-                if (lane == 0) pf_mbar_arrive(rempty0 + 8u * slot);   // the warp's words are in registers: the slot may be refilled
+                if (lane == 0) mbar_arrive(rempty0 + 8u * slot);   // the warp's words are in registers: the slot may be refilled
                 slot += 2u;
                 if (slot >= (uint32_t)kRing) { slot -= (uint32_t)kRing; rphase ^= 1u; }
                 const float sc = __half2float(__ushort_as_half((unsigned short)(sz & 0xFFFFu)));
                 const float ze = __half2float(__ushort_as_half((unsigned short)(sz >> 16)));
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
-                    if (g >= 2 && !pf_mbar_wait(emptyb + 8u * b, ephase)) { dead = true; break; }
+                    if (g >= 2 && !wait_looks(emptyb + 8u * b, ephase)) { dead = true; break; }
                     uint32_t wb[16];
                     if (row_ok) {
                         uint32_t d[16];
@@ -382,11 +319,11 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                                wb[4 * kc + 3]);
                 }
                 if (dead) break;
-                pf_fence_proxy_async();                     // generic-proxy stores -> visible to the MMA's reads
+                fence_proxy_async();                     // generic-proxy stores -> visible to the MMA's reads
                 __syncwarp();
                 if (lane == 0) {                            // one arrival per warp and block
-                    pf_mbar_arrive(fullb);
-                    pf_mbar_arrive(fullb + 8u);
+                    mbar_arrive(fullb);
+                    mbar_arrive(fullb + 8u);
                 }
                 if (g >= 2) ephase ^= 1u;
             }
@@ -396,10 +333,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 #pragma unroll 1
             for (int i = kb_x + h; i < nkb && !dead; i += 2) {
                 const int s = i % kStages;
-                if (i >= kStages && !pf_mbar_wait(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) { dead = true; break; }
+                if (i >= kStages && !wait_looks(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) { dead = true; break; }
                 if (p.t16) {                                 // both operands of this block arrive by TMA: nothing to write
                     __syncwarp();
-                    if (lane == 0) pf_mbar_arrive(full0 + 8u * s);
+                    if (lane == 0) mbar_arrive(full0 + 8u * s);
                     continue;
                 }
                 if (!t_ready) {                              // every warp of every t CTA of this token tile has stored its part
@@ -456,9 +393,9 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                                P2<T>::pack(ta[u][1].x, ta[u][1].y), P2<T>::pack(ta[u][1].z, ta[u][1].w));
                     }
                 }
-                pf_fence_proxy_async();
+                fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) pf_mbar_arrive(full0 + 8u * s);
+                if (lane == 0) mbar_arrive(full0 + 8u * s);
             }
             if (dead) {
                 *abort_flag = 1;
@@ -471,8 +408,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         // (the only ones it may address) and the quarter w/4 of the columns.  Mode 0 stages the
         // tile in shared memory as [token][128 features] (the operand stages are free by now) and
         // each column quarter leaves with one TMA tensor store, which also clips the ragged edges.
-        if (!dead && nkb > 0 && pf_mbar_wait(done_bar, 0)) {
-            tc_fence_after();
+        if (!dead && nkb > 0 && wait_looks(done_bar, 0)) {
+            umma::fence_after();
             const int q = warp & 3, cg = warp >> 2;
             const int nn = n0 + 32 * q + lane;              // output feature (mode 0) / rank index (mode 1)
             const int c_begin = cg * (TOK / 4);
@@ -488,18 +425,18 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 float *pt = p.part + ((size_t)(m_tile * p.nt + n_tile) * S) * slice + (size_t)c_begin * kBN + 32 * q + lane;
                 uint32_t v[32];
                 if (mine) {
-                    tc_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c_begin, v);
-                    tc_wait_ld();
+                    umma::ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c_begin, v);
+                    umma::wait_ld();
                     float *dst = pt + (size_t)split * slice;
 #pragma unroll
                     for (int j = 0; j < 32; ++j) __stcg(dst + j * kBN, __uint_as_float(v[j]));
                 }
                 __threadfence();
                 __syncwarp();
-                if (lane == 0) pf_mbar_arrive(split_bar);
+                if (lane == 0) mbar_arrive(split_bar);
                 if (warp == 0 && lane == 0) {
                     int last = 0;
-                    if (pf_mbar_wait(split_bar, 0)) {
+                    if (wait_looks(split_bar, 0)) {
                         int *ctr = p.split_ctr + m_tile * p.nt + n_tile;
                         last = (atomicAdd(ctr, 1) == S - 1);
                         if (last) atomicExch(ctr, 0);       // left at zero for the next call
@@ -508,9 +445,9 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     }
                     *split_last = last;
                     __threadfence_block();
-                    pf_mbar_arrive(split_bar2);
+                    mbar_arrive(split_bar2);
                 }
-                const bool last = pf_mbar_wait(split_bar2, 0) && *split_last != 0;
+                const bool last = wait_looks(split_bar2, 0) && *split_last != 0;
                 if (last && mine) {
                     __threadfence();
                     float acc[32];
@@ -528,10 +465,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     unsigned short *sp16 = reinterpret_cast<unsigned short *>(smem + (size_t)c_begin * (kBN * 2)) + 32 * q + lane;
 #pragma unroll
                     for (int j = 0; j < 32; ++j) sp16[j * kBN] = to_bits16<T>(acc[j]);
-                    pf_fence_proxy_async();                 // staged tile -> visible to the TMA store
-                    pf_mbar_arrive(epi0 + 8u * cg);
+                    fence_proxy_async();                 // staged tile -> visible to the TMA store
+                    mbar_arrive(epi0 + 8u * cg);
                     if (q == 0 && lane == 0) {
-                        if (pf_mbar_wait(epi0 + 8u * cg, 0)) {
+                        if (wait_looks(epi0 + 8u * cg, 0)) {
                             asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
                                          ::"l"(reinterpret_cast<uint64_t>(&ymap)), "r"(n0), "r"(m0 + c_begin),
                                            "r"(sbase + (uint32_t)c_begin * (kBN * 2))
@@ -548,8 +485,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 for (int c = c_begin; c < c_begin + TOK / 4; c += 32) {
                     if (m0 + c >= p.M) break;               // warp-uniform
                     uint32_t v[32];
-                    tc_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c, v);
-                    tc_wait_ld();
+                    umma::ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c, v);
+                    umma::wait_ld();
                     if (!t_role) {
                         unsigned short *sp = reinterpret_cast<unsigned short *>(smem + (size_t)c * (kBN * 2)) + 32 * q + lane;
 #pragma unroll
@@ -571,10 +508,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     }
                 }
                 if (!t_role) {
-                    pf_fence_proxy_async();                 // staged tile -> visible to the TMA store
-                    pf_mbar_arrive(epi0 + 8u * cg);
+                    fence_proxy_async();                 // staged tile -> visible to the TMA store
+                    mbar_arrive(epi0 + 8u * cg);
                     if (q == 0 && lane == 0) {
-                        if (pf_mbar_wait(epi0 + 8u * cg, 0)) {
+                        if (wait_looks(epi0 + 8u * cg, 0)) {
                             asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
                                          ::"l"(reinterpret_cast<uint64_t>(&ymap)), "r"(n0), "r"(m0 + c_begin),
                                            "r"(sbase + (uint32_t)c_begin * (kBN * 2))
@@ -602,7 +539,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 }
             }
         }
-        tc_fence_before();
+        umma::fence_before();
     } else if (warp == kMmaWarp) {
         // =================================================== MMA warp
         const uint32_t idesc = (1u << 4) | (P2<T>::kFmt << 7) | (P2<T>::kFmt << 10) | ((uint32_t)(cols >> 3) << 17) |
@@ -612,24 +549,24 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         // (18944 x 8192 at 77 tokens 56.2 us, now 50.4; 4096 -> 4096 at 1000 tokens 37.3 and 36.9).
         bool dead = false;
         // descriptors of stage 0; a stage further on is kStageBytes / 16 in their address field
-        const uint64_t xd0 = make_desc(sbase), wd0 = make_desc(sbase + kXBytes);
+        const uint64_t xd0 = umma::desc_k128(sbase), wd0 = umma::desc_k128(sbase + kXBytes);
         uint32_t s = 0, ph = 0;
 #pragma unroll 1
         for (int i = 0; i < nkb; ++i) {
-            if (!pf_mbar_wait(full0 + 8u * s, ph) || *abort_flag) dead = true;
+            if (!wait_looks(full0 + 8u * s, ph) || *abort_flag) dead = true;
             if (__any_sync(0xffffffffu, dead)) {
                 dead = true;
                 break;
             }
-            tc_fence_after();
+            umma::fence_after();
             if (elect_one()) {
                 const uint64_t xd = xd0 + s * (kStageBytes >> 4), wd = wd0 + s * (kStageBytes >> 4);
                 // every operand tile is K-major with 128-byte rows and the 128-byte swizzle, whether it
                 // arrived by TMA or was written by the producers: 32 bytes per 16 elements of K inside a row
 #pragma unroll
-                for (int j = 0; j < kBK / 16; ++j) tc_mma(tmem_base, wd + 2u * j, xd + 2u * j, idesc, (i > 0 || j > 0) ? 1u : 0u);
-                tc_commit(empty0 + 8u * s);                  // stage is free once these MMAs have read it
-                if (i == nkb - 1) tc_commit(done_bar);       // accumulator complete
+                for (int j = 0; j < kBK / 16; ++j) umma::mma(tmem_base, wd + 2u * j, xd + 2u * j, idesc, (i > 0 || j > 0) ? 1u : 0u);
+                umma::commit(empty0 + 8u * s);                  // stage is free once these MMAs have read it
+                if (i == nkb - 1) umma::commit(done_bar);       // accumulator complete
             }
             __syncwarp();
             if (++s == (uint32_t)kStages) {
@@ -642,7 +579,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             atomicExch(p.status, (int)FBQ_ERR_TIMEOUT);
         }
         __syncwarp();
-        tc_fence_before();
+        umma::fence_before();
     } else if (warp == kTmaWarp) {
         // =================================================== operand-stage copies
         if (lane == 0) {
@@ -650,18 +587,18 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 #pragma unroll 1
             for (int i = 0; i < nkb; ++i) {
                 const int kb = i, s = i % kStages;
-                if ((i >= kStages && !pf_mbar_wait(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) || *abort_flag) {
+                if ((i >= kStages && !wait_looks(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) || *abort_flag) {
                     dead = true;
                     break;
                 }
                 const uint32_t bar = full0 + 8u * s;
                 const uint32_t xt = sbase + (uint32_t)s * kStageBytes, wt = xt + kXBytes;
                 if (t_role) {
-                    pf_mbar_expect_tx(bar, xbytes + kWBytes);
+                    mbar_expect_tx(bar, xbytes + kWBytes);
                     tma_load_2d(xt, &xmap, (kb_begin + kb) * kBK, m0, bar);
                     tma_load_2d(wt, &amap, (kb_begin + kb) * kBK, n0, bar);      // rows of A
                 } else if (kb < kb_x) {
-                    pf_mbar_expect_tx(bar, xbytes);
+                    mbar_expect_tx(bar, xbytes);
                     tma_load_2d(xt, &xmap, (kb_begin + kb) * kBK, m0, bar);
                 } else if (p.t16) {
                     if (kb == kb_x) {                        // every warp of every t CTA of this token tile has stored its part
@@ -680,11 +617,11 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         }
                         asm volatile("fence.proxy.async;" ::: "memory");
                     }
-                    pf_mbar_expect_tx(bar, xbytes + kWBytes);
+                    mbar_expect_tx(bar, xbytes + kWBytes);
                     tma_load_2d(xt, &tmap, (kb - kb_x) * kBK, m0, bar);   // t as the token operand
                     tma_load_2d(wt, &bmap, (kb - kb_x) * kBK, n0, bar);   // rows of B
                 } else {
-                    pf_mbar_expect_tx(bar, kWBytes);
+                    mbar_expect_tx(bar, kWBytes);
                     tma_load_2d(wt, &bmap, (kb - kb_x) * kBK, n0, bar);   // rows of B
                 }
             }
@@ -765,7 +702,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 const int gi = 8 * c + g8;
                 if (gi < groups && !dead) {
                     const uint32_t slot = (uint32_t)gi % kRing;
-                    if (lane == 0 && ((gi >= kRing && !pf_mbar_wait(rempty0 + 8u * slot, (uint32_t)(gi / kRing - 1) & 1u)) || *abort_flag))
+                    if (lane == 0 && ((gi >= kRing && !wait_looks(rempty0 + 8u * slot, (uint32_t)(gi / kRing - 1) & 1u)) || *abort_flag))
                         dead = true;
                     dead = __shfl_sync(0xffffffffu, (int)dead, 0) != 0;     // also orders the table writes after the wait
                     if (!dead) {
@@ -775,10 +712,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         __syncwarp();
                         if (lane == 0) {
                             if (v == 0) {
-                                pf_mbar_expect_tx(rfull0 + 8u * slot, (uint32_t)kBN * WPG * 4u);
+                                mbar_expect_tx(rfull0 + 8u * slot, (uint32_t)kBN * WPG * 4u);
                                 tma_load_2d(ring0 + slot * kRawSlot, &wmap, (g_begin + gi) * WPG, n0, rfull0 + 8u * slot);
                             } else {
-                                pf_mbar_arrive(rfull0 + 8u * slot);
+                                mbar_arrive(rfull0 + 8u * slot);
                             }
                         }
                     }
@@ -794,8 +731,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     }
     __syncthreads();
     if (warp == kMmaWarp) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TOK) : "memory");
+        umma::fence_after();
+        umma::tmem_free<1>(tmem_base, (uint32_t)TOK);
     }
 }
 
@@ -823,68 +760,10 @@ struct PairSmem {
     static constexpr uint32_t kNumBars = 2 * kPairStages + 2 * kRing + 1 + 4;
     static constexpr uint32_t kTotal = kBarOff + kNumBars * 8u + 16u;
 };
-__device__ __forceinline__ uint32_t cluster_ctarank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// shared::cluster address of `addr` (a shared::cta address of this CTA) in the CTA of rank `rank`
-__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
-{
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-__device__ __forceinline__ bool pf_mbar_wait_cluster(uint32_t bar, uint32_t parity)     // sees arrivals from the peer CTA
-{
-#pragma unroll 1
-    for (uint32_t i = 0; i < kPfWaitLimit; ++i) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
 __device__ __forceinline__ void cluster_sync()
 {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// Arrive, in BOTH CTAs of the pair, on the barrier at this shared-memory offset once every MMA issued so far is complete.
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar)
-{
-    const unsigned short mask = 3;
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-                 "h"(mask)
-                 : "memory");
-}
-// TMA tensor copy into this CTA's shared memory that completes on a barrier of either CTA of the pair (no multicast)
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t cluster_bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(cluster_bar)
-        : "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 
 // Grid: 1-D, clusters of two consecutive CTAs.  t CTAs first (pairs: 256 tokens x 256 rank rows),
@@ -904,7 +783,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
     const uint32_t cr = cluster_ctarank();                      // 0: leader (issues the MMAs), 1: peer
     constexpr int WPG = (BITS == 4) ? 16 : 12;                  // packed words per row and group
     extern __shared__ __align__(1024) uint8_t smem[];
-    const uint32_t sbase = pf_smem_u32(smem);
+    const uint32_t sbase = smem_u32(smem);
     if (sbase & 1023u) {                                        // swizzle atoms need a 1024-byte aligned base
         if (threadIdx.x == 0) atomicExch(p.status, (int)FBQ_ERR_CUDA);
         return;
@@ -931,39 +810,36 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
 
     if (tid == 0) {
         for (int i = 0; i < kStages; ++i) {
-            pf_mbar_init(full0 + 8u * i, t_role ? 1 : 17);      // leader's TMA lane + 8 producer warps of each CTA
-            pf_mbar_init(empty0 + 8u * i, 1);
+            mbar_init(full0 + 8u * i, t_role ? 1 : 17);      // leader's TMA lane + 8 producer warps of each CTA
+            mbar_init(empty0 + 8u * i, 1);
         }
         for (int i = 0; i < kRing; ++i) {
-            pf_mbar_init(rfull0 + 8u * i, 2);                   // the two ring warps
-            pf_mbar_init(rempty0 + 8u * i, kHalf / 32);         // a group is consumed by one half of the producers (8 warps)
+            mbar_init(rfull0 + 8u * i, 2);                   // the two ring warps
+            mbar_init(rempty0 + 8u * i, kHalf / 32);         // a group is consumed by one half of the producers (8 warps)
         }
-        pf_mbar_init(done_bar, 1);
-        for (int i = 0; i < 4; ++i) pf_mbar_init(epi0 + 8u * i, 128);     // the four warps of a column quarter
+        mbar_init(done_bar, 1);
+        for (int i = 0; i < 4; ++i) mbar_init(epi0 + 8u * i, 128);     // the four warps of a column quarter
         *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_barrier_init();
     }
     if (warp == kMmaWarp) {                  // the MMA warp owns the tensor-memory allocation
         // the MMA warps of both CTAs of the pair allocate together (same columns in both)
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(pf_smem_u32(tmem_slot)),
-                     "r"((uint32_t)TOK)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-        tc_fence_before();
+        umma::tmem_alloc<2>(smem_u32(tmem_slot), (uint32_t)TOK);
+        umma::fence_before();
     }
     if (warp == kTmaWarp && lane == 0) {
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&xmap)) : "memory");
+        prefetch_tensormap(&xmap);
         if (t_role) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&amap)) : "memory");
+            prefetch_tensormap(&amap);
         } else {
-            if (p.rank > 0) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&bmap)) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&ymap)) : "memory");
+            if (p.rank > 0) prefetch_tensormap(&bmap);
+            prefetch_tensormap(&ymap);
         }
     }
     if (warp == kRawWarp && lane == 0)
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&wmap)) : "memory");
+        prefetch_tensormap(&wmap);
     cluster_sync();                          // barriers of both CTAs are initialised before anything arrives on them
-    tc_fence_after();
+    umma::fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp < kMmaWarp) {
@@ -993,7 +869,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
             uint32_t slot = (uint32_t)h, rphase = 0u;
 #pragma unroll 1
             for (int g = h; g < groups; g += 2) {
-                if (!pf_mbar_wait(rfull0 + 8u * slot, rphase)) { dead = true; break; }
+                if (!wait_looks(rfull0 + 8u * slot, rphase)) { dead = true; break; }
                 constexpr int NW = (BITS == 4) ? 4 : 3;
                 uint32_t w[2][NW];
                 const uint32_t rs = ring0 + slot * kRawSlot;
@@ -1010,7 +886,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                 }
                 const uint32_t sz = lds32(table0 + slot * (kBN * 4u));      // s | z << 16 of (row, group)
                 __syncwarp();
-                if (lane == 0) pf_mbar_arrive(rempty0 + 8u * slot);   // the warp's words are in registers: the slot may be refilled
+                if (lane == 0) mbar_arrive(rempty0 + 8u * slot);   // the warp's words are in registers: the slot may be refilled
                 slot += 2u;
                 if (slot >= (uint32_t)kRing) { slot -= (uint32_t)kRing; rphase ^= 1u; }
                 const float sc = __half2float(__ushort_as_half((unsigned short)(sz & 0xFFFFu)));
@@ -1018,7 +894,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
                     const int i = 2 * g + b, s = i % kStages;
-                    if (i >= kStages && !pf_mbar_wait(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) { dead = true; break; }
+                    if (i >= kStages && !wait_looks(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) { dead = true; break; }
                     uint32_t wb[16];
                     if (row_ok) {
                         uint32_t d[16];
@@ -1032,9 +908,9 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                     for (int kc = 0; kc < 4; ++kc)
                         sts128(wdst + (uint32_t)s * kStageBytes + ((((uint32_t)(4 * part + kc)) ^ wsw) << 4), wb[4 * kc], wb[4 * kc + 1], wb[4 * kc + 2],
                                wb[4 * kc + 3]);
-                    pf_fence_proxy_async();                 // generic-proxy stores -> visible to the MMA's reads
+                    fence_proxy_async();                 // generic-proxy stores -> visible to the MMA's reads
                     __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster(lfull0 + 8u * s);       // one arrival per warp, on the leader's barrier
+                    if (lane == 0) umma::arrive_cluster(lfull0 + 8u * s);       // one arrival per warp, on the leader's barrier
                 }
                 if (dead) break;
             }
@@ -1044,7 +920,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
 #pragma unroll 1
             for (int i = p.kb_main + h; i < nkb && !dead; i += 2) {
                 const int s = i % kStages;
-                if (i >= kStages && !pf_mbar_wait(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) { dead = true; break; }
+                if (i >= kStages && !wait_looks(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) { dead = true; break; }
                 if (!t_ready) {                              // every warp of every t CTA of this token tile has stored its part
                     int seen = 0;
                     if (lane == 0) {
@@ -1083,9 +959,9 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                         sts128(sbase + (uint32_t)s * kStageBytes + (uint32_t)rr * 128u + ((((uint32_t)c) ^ ((uint32_t)rr & 7u)) << 4), xa[4 * c],
                                xa[4 * c + 1], xa[4 * c + 2], xa[4 * c + 3]);
                 }
-                pf_fence_proxy_async();
+                fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(lfull0 + 8u * s);
+                if (lane == 0) umma::arrive_cluster(lfull0 + 8u * s);
             }
             if (dead) {
                 *abort_flag = 1;
@@ -1098,8 +974,8 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
         // (the only ones it may address) and the quarter w/4 of the columns.  Mode 0 stages the
         // tile in shared memory as [token][128 features] (the operand stages are free by now) and
         // each column quarter leaves with one TMA tensor store, which also clips the ragged edges.
-        if (!dead && nkb > 0 && pf_mbar_wait(done_bar, 0)) {
-            tc_fence_after();
+        if (!dead && nkb > 0 && wait_looks(done_bar, 0)) {
+            umma::fence_after();
             const int q = warp & 3, cg = warp >> 2;
             const int nn = n0 + 32 * q + lane;              // output feature (mode 0) / rank index (mode 1)
             const int c_begin = cg * (TOK / 4);
@@ -1108,8 +984,8 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                 for (int c = c_begin; c < c_begin + TOK / 4; c += 32) {
                     if (m0 + c >= p.M) break;               // warp-uniform
                     uint32_t v[32];
-                    tc_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c, v);
-                    tc_wait_ld();
+                    umma::ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c, v);
+                    umma::wait_ld();
                     if (!t_role) {
                         unsigned short *sp = reinterpret_cast<unsigned short *>(smem + (size_t)c * (kBN * 2)) + 32 * q + lane;
 #pragma unroll
@@ -1124,10 +1000,10 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                     }
                 }
                 if (!t_role) {
-                    pf_fence_proxy_async();                 // staged tile -> visible to the TMA store
-                    pf_mbar_arrive(epi0 + 8u * cg);
+                    fence_proxy_async();                 // staged tile -> visible to the TMA store
+                    mbar_arrive(epi0 + 8u * cg);
                     if (q == 0 && lane == 0 && n0 < p.N) {   // (a padding CTA past the last feature tile stores nothing)
-                        if (pf_mbar_wait(epi0 + 8u * cg, 0)) {
+                        if (wait_looks(epi0 + 8u * cg, 0)) {
                             asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
                                          ::"l"(reinterpret_cast<uint64_t>(&ymap)), "r"(n0), "r"(m0 + c_begin),
                                            "r"(sbase + (uint32_t)c_begin * (kBN * 2))
@@ -1154,7 +1030,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                 }
             }
         }
-        tc_fence_before();
+        umma::fence_before();
     } else if (warp == kMmaWarp) {
         // =================================================== MMA warp
         // one MMA of the pair: 256 weight rows (128 per CTA) x 256 tokens (128 staged by each CTA) x 16
@@ -1165,17 +1041,17 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
         for (int i = 0; i < nkb && !dead && cr == 0; ++i) {     // only the leader CTA issues
             const int s = i % kStages;
             if (lane == 0) {
-                if (!pf_mbar_wait_cluster(full0 + 8u * s, (uint32_t)(i / kStages) & 1u) || *abort_flag) {
+                if (!wait_looks_cluster(full0 + 8u * s, (uint32_t)(i / kStages) & 1u) || *abort_flag) {
                     dead = true;
                 } else {
-                    tc_fence_after();
+                    umma::fence_after();
                     const uint32_t x_base = sbase + (uint32_t)s * kStageBytes, w_base = x_base + kXBytes;
                     // every operand tile is K-major with 128-byte rows and the 128-byte swizzle, whether it
                     // arrived by TMA or was written by the producers: 32 bytes per 16 elements of K inside a row
 #pragma unroll
                     for (int j = 0; j < kBK / 16; ++j)
-                        tc_mma_pair(tmem_base, make_desc(w_base + j * 32), make_desc(x_base + j * 32), idesc, (i > 0 || j > 0) ? 1u : 0u);
-                    tc_commit_pair(empty0 + 8u * s);         // the stage is free, in both CTAs, once these MMAs have read it
+                        umma::mma_pair(tmem_base, umma::desc_k128(w_base + j * 32), umma::desc_k128(x_base + j * 32), idesc, (i > 0 || j > 0) ? 1u : 0u);
+                    umma::commit_pair(empty0 + 8u * s);         // the stage is free, in both CTAs, once these MMAs have read it
                 }
             }
             dead = __shfl_sync(0xffffffffu, (int)dead, 0) != 0;
@@ -1185,11 +1061,11 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                 *abort_flag = 1;
                 atomicExch(p.status, (int)FBQ_ERR_TIMEOUT);
             } else if (nkb > 0 && cr == 0) {
-                tc_commit_pair(done_bar);                    // accumulators complete in both CTAs
+                umma::commit_pair(done_bar);                    // accumulators complete in both CTAs
             }
         }
         __syncwarp();
-        tc_fence_before();
+        umma::fence_before();
     } else if (warp == kTmaWarp) {
         // =================================================== operand-stage copies
         if (lane == 0) {
@@ -1197,7 +1073,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
 #pragma unroll 1
             for (int i = 0; i < nkb; ++i) {
                 const int kb = i, s = i % kStages;
-                if ((i >= kStages && !pf_mbar_wait(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) || *abort_flag) {
+                if ((i >= kStages && !wait_looks(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) || *abort_flag) {
                     dead = true;
                     break;
                 }
@@ -1206,15 +1082,15 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                 // every copy of the pair completes on the LEADER's barrier; the leader announces the bytes of both
                 const uint32_t lbar = mapa_shared(bar, 0);
                 if (t_role) {
-                    if (cr == 0) pf_mbar_expect_tx(bar, 2u * (kXBytes + kWBytes));
-                    tma_load_2d_pair(xt, &xmap, kb * kBK, mh, lbar);
-                    tma_load_2d_pair(wt, &amap, kb * kBK, n0, lbar);      // rows of A
+                    if (cr == 0) mbar_expect_tx(bar, 2u * (kXBytes + kWBytes));
+                    umma::tma_load_2d_pair(xt, &xmap, kb * kBK, mh, lbar);
+                    umma::tma_load_2d_pair(wt, &amap, kb * kBK, n0, lbar);      // rows of A
                 } else if (kb < kb_x) {
-                    if (cr == 0) pf_mbar_expect_tx(bar, 2u * kXBytes);
-                    tma_load_2d_pair(xt, &xmap, kb * kBK, mh, lbar);
+                    if (cr == 0) mbar_expect_tx(bar, 2u * kXBytes);
+                    umma::tma_load_2d_pair(xt, &xmap, kb * kBK, mh, lbar);
                 } else {
-                    if (cr == 0) pf_mbar_expect_tx(bar, 2u * kWBytes);
-                    tma_load_2d_pair(wt, &bmap, (kb - p.kb_main) * kBK, n0, lbar);   // rows of B
+                    if (cr == 0) mbar_expect_tx(bar, 2u * kWBytes);
+                    umma::tma_load_2d_pair(wt, &bmap, (kb - p.kb_main) * kBK, n0, lbar);   // rows of B
                 }
             }
             if (dead) {
@@ -1294,7 +1170,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                 const int gi = 8 * c + g8;
                 if (gi < groups && !dead) {
                     const uint32_t slot = (uint32_t)gi % kRing;
-                    if (lane == 0 && ((gi >= kRing && !pf_mbar_wait(rempty0 + 8u * slot, (uint32_t)(gi / kRing - 1) & 1u)) || *abort_flag))
+                    if (lane == 0 && ((gi >= kRing && !wait_looks(rempty0 + 8u * slot, (uint32_t)(gi / kRing - 1) & 1u)) || *abort_flag))
                         dead = true;
                     dead = __shfl_sync(0xffffffffu, (int)dead, 0) != 0;     // also orders the table writes after the wait
                     if (!dead) {
@@ -1304,10 +1180,10 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                         __syncwarp();
                         if (lane == 0) {
                             if (v == 0) {
-                                pf_mbar_expect_tx(rfull0 + 8u * slot, (uint32_t)kBN * WPG * 4u);
+                                mbar_expect_tx(rfull0 + 8u * slot, (uint32_t)kBN * WPG * 4u);
                                 tma_load_2d(ring0 + slot * kRawSlot, &wmap, gi * WPG, n0, rfull0 + 8u * slot);
                             } else {
-                                pf_mbar_arrive(rfull0 + 8u * slot);
+                                mbar_arrive(rfull0 + 8u * slot);
                             }
                         }
                     }
@@ -1323,8 +1199,8 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
     }
     cluster_sync();                          // both CTAs are done with their tensor memory and with each other's barriers
     if (warp == kMmaWarp) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TOK) : "memory");
+        umma::fence_after();
+        umma::tmem_free<2>(tmem_base, (uint32_t)TOK);
     }
 }
 

@@ -269,10 +269,10 @@ int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int ac
 /* Tuning and test switches (host side, process wide).  Known names:
  *   "force_kernel"  -1 = automatic, else an fbq_kernel value (shapes outside the
  *                   forced kernel's domain still fall back to the generic one)
- *   "gemv"          1 (default) = M <= 2 runs the streaming decode kernel where its domain allows (see fbq_linear),
+ *   "gemv"          1 (default) = M <= 16 runs the streaming decode kernel where its domain allows (see fbq_linear),
  *                   0 = the other decode kernel at every M
- *   "gemv_ctas"     0 = automatic (one or two CTAs per SM), else an upper bound on the streaming kernel's grid (the
- *                   number of SMs is the better choice for linears launched side by side on several streams)
+ *   "gemv_ctas"     0 = automatic (one or two CTAs per SM), else an upper bound on the streaming kernel's grid
+ *                   (fbq_set_stream_option sets it for one stream)
  *   "t_poll_limit"  0 = default, else the number of looks the streaming kernel takes at the t CTAs' slots
  *                   before it gives up with FBQ_ERR_TIMEOUT
  *   "test_skip_t_arrive", "test_prefill_skip_flag", "prefill_flag_polls"
@@ -326,6 +326,14 @@ int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int ac
  * decode kernel is printed to stderr: K slices, CTAs, stage size and count, shared-memory layout, form.) */
 int fbq_set_option(const char *name, int value);
 int fbq_get_option(const char *name, int *value);
+
+/* The same for the calls on one stream of the current device.  Known name: "gemv_ctas", as above, for the linears (not the
+ * batches) of that stream; 0 takes it back, and a process-wide value goes first.  By default a linear of one or two tokens
+ * takes two CTAs per SM, which is faster for linears that run one after another; linears that run at the same time on
+ * several streams are faster with one each (seven of a 7B layer on seven streams: 33 us, 41 by default), so a
+ * program that runs them so sets the number of SMs on those streams.  Summation order depends on the grid, so set it before the
+ * first call whose bits matter. */
+int fbq_set_stream_option(void *stream, const char *name, int value);
 
 /* Number of kernels the library has launched since load (all streams). */
 long long fbq_launch_count(void);

@@ -33,6 +33,7 @@ from .binding import (  # noqa: F401
     release_workspaces,
     select_kernel,
     set_option,
+    set_stream_option,
     status_string,
     sub_branch_unfused,
     unpack,

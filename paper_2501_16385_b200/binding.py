@@ -68,6 +68,7 @@ def lib() -> ctypes.CDLL:
         L.fbq_select_kernel.argtypes = [i32] * 7
         L.fbq_set_option.argtypes = [ctypes.c_char_p, i32]
         L.fbq_get_option.argtypes = [ctypes.c_char_p, ctypes.POINTER(i32)]
+        L.fbq_set_stream_option.argtypes = [vp, ctypes.c_char_p, i32]
         L.fbq_launch_count.restype = ctypes.c_longlong
         L.fbq_poll_status.argtypes = [vp]
         L.fbq_status_string.restype = ctypes.c_char_p
@@ -265,6 +266,11 @@ def select_kernel(M, N, K, group, bits, rank, bf16=False) -> int:
 
 def set_option(name: str, value: int) -> None:
     _check(lib().fbq_set_option(name.encode(), int(value)), "fbq_set_option(%s)" % name)
+
+
+def set_stream_option(name: str, value: int, stream=None) -> None:
+    """fbq_set_stream_option: an option for the calls of one stream (default: the current one)."""
+    _check(lib().fbq_set_stream_option(_stream(stream), name.encode(), int(value)), "fbq_set_stream_option(%s)" % name)
 
 
 def get_option(name: str) -> int:

@@ -5,6 +5,7 @@
 #include <atomic>
 #include <cstring>
 #include <initializer_list>
+#include <iterator>
 #include <map>
 #include <mutex>
 #include <utility>
@@ -256,6 +257,7 @@ int run_linear(const LinearArgs &a, cudaStream_t s, int decode_ctas = 0)
         GemvTuning gt = g_opt.gemv;
         gt.pdl = g_opt.decode.pdl;
         if (tune.max_ctas > 0) gt.max_ctas = tune.max_ctas;
+        if (gt.max_ctas == 0) gt.max_ctas = ws->gemv_ctas;
         size_t pf = 0, partf = 0;
         int nc = 0;
         gemv_workspace_need(a, gt, &pf, &nc, &partf);
@@ -862,6 +864,15 @@ int fbq_set_option(const char *name, int value)
     return FBQ_OK;
 }
 
+int fbq_set_stream_option(void *stream, const char *name, int value)
+{
+    if (!name || strcmp(name, "gemv_ctas") || value < 0) return FBQ_ERR_BADARG;
+    Workspace *ws = workspace_for(static_cast<cudaStream_t>(stream));
+    if (!ws) return FBQ_ERR_CUDA;
+    ws->gemv_ctas = value;
+    return FBQ_OK;
+}
+
 int fbq_get_option(const char *name, int *value)
 {
     int *slot = option_slot(name);
@@ -923,7 +934,12 @@ int fbq_release_workspaces(void)
         cudaFree(w.tags);
         cudaFree(w.rec);
     }
-    g_ws.clear();
+    for (auto it = g_ws.begin(); it != g_ws.end();) {            // what is left of a stream are its options
+        const int gemv_ctas = it->second.gemv_ctas;
+        it->second = Workspace{};
+        it->second.gemv_ctas = gemv_ctas;
+        it = gemv_ctas ? std::next(it) : g_ws.erase(it);
+    }
     return FBQ_OK;
 }
 

@@ -46,6 +46,7 @@ struct Workspace {
     size_t w16_bytes = 0;
     uint32_t *tags = nullptr;     // its launch number and tags (starts at zero)
     size_t n_tags = 0;
+    int gemv_ctas = 0;            // option of the stream (fbq_set_stream_option); outlives the buffers
     void *rec = nullptr;          // split operands of the Gram matrix and the reconstruction step (no invariant)
     size_t rec_bytes = 0;
 };

@@ -144,17 +144,28 @@ int select_kernel(int M, int N, int K, int group, int bits, int rank, bool bf16)
     if (g_opt.force_kernel == FBQ_KERNEL_DECODE && decode_ok) return FBQ_KERNEL_DECODE;
     if (g_opt.force_kernel == FBQ_KERNEL_PREFILL && prefill_ok) return FBQ_KERNEL_PREFILL;
     if (g_opt.force_kernel >= 0) return FBQ_KERNEL_GENERIC;
-    // Measured on B200 (7B layer, INT4, one stream in layer order, us per layer step, rank 16 / 64 / 128 / 0):
-    //   streaming decode kernel   M = 4: 84 / 87 / 101 / 74    M = 8: 107 / 112 / 144 / 91   M = 12: 142 / 156 / 202 / 114   M = 16: 160 / 176 / 236 / 125
-    //   tensor-core kernel        M = 4: 213                   M = 8: 211                    M = 12: 192 / 207 / 213 / 178   M = 16: 176 / 197 / 201 / 166
-    //                             (K split whenever tiles are few, the default; 227 - 257 with the split only for K >= 8192)
-    //   the other decode kernel   M = 4: 129                   M = 8: 258                    M = 16: 3204
-    // per shape at rank 128 (us per launch, 4096 -> 4096 / 4096 -> 11008 / 11008 -> 4096): streaming M = 12: 21.7 / 29.6 / 58.6,
-    // M = 16: 24.9 / 34.0 / 68.9; tensor-core M = 12: 23.6 / 40.1 / 35.1, M = 16: 23.7 / 35.4 / 35.3;
-    // and on the 13B layer (K = 5120 / 13824; rank 64 / 0): streaming M = 8: 150 / 125, M = 12: 208 / 163, M = 16: 411 / 307;
-    // tensor-core M = 8: 256 / 232, M = 12: 258 / 231, M = 16: 234 / 206.  Above eight tokens the streaming kernel
-    // pays only while x of all K fits its shared memory (one K slice: M * K * 2 bytes up to 136 KB), so where its
-    // domain allows it takes M <= 8 for every shape, and M <= 16 for the shapes it does not have to slice.
+    // Measured on B200, INT4, fp16, us per launch in a row, streaming / tensor-core kernel (in KB: x of all tokens):
+    //                          rank 0                        rank 64                       rank 128
+    //   4096 -> 4096    M  8   8.5 / 12.9                    9.8 / 15.4                    11.7 / 16.2
+    //                   M 12  10.6 / 12.9                   12.7 / 15.5                    15.5 / 16.3
+    //                   M 16  12.1 / 12.9  (128 KB)         14.0 / 16.0                    17.6 / 16.7
+    //   4096 -> 11008   M 16  16.5 / 25.2                   19.9 / 27.2                    24.7 / 27.4
+    //   5120 -> 13824   M 12  20.7 / 30.5  (120 KB)         24.5 / 32.6                    28.9 / 33.0
+    //                   M 14  21.7 / 30.6  (140 KB)         29.6 / 32.7                    30.9 / 33.1
+    //                   M 16  26.2 / 30.6  (160 KB)         33.2 / 32.7                    83.7 / 33.1
+    //   8192 -> 8192    M  8  18.5 / 28.1  (128 KB)         19.6 / 29.6                    20.4 / 30.4
+    //                   M 12  39.6 / 28.1  (192 KB)         47.9 / 29.6                    52.3 / 30.4
+    //   11008 -> 4096   M  7  19.5 / 22.0  (150 KB)         20.5 / 23.9                    21.5 / 24.9
+    //                   M  8  22.2 / 22.1  (172 KB)         26.8 / 24.0                    27.5 / 25.0
+    //                   M 12  34.7 / 22.0                   44.4 / 23.8                    50.5 / 25.0
+    //   13824 -> 5120   M  5  21.0 / 31.0  (135 KB)         22.0 / 32.6                    29.8 / 33.6
+    //                   M  8  29.7 / 31.1  (216 KB)         36.2 / 32.8                    36.4 / 33.9
+    //   28672 -> 8192   M  4  43.8 / 81.9  (224 KB)         60.9 / 83.4                    63.7 / 83.7
+    //                   M  8  61.5 / 82.0  (448 KB)         89.1 / 83.4                    92.4 / 83.5
+    // Up to eight tokens the streaming kernel is ahead by up to a factor of two and behind by 16 % at most (7 and 8 tokens of
+    // the longest K with a sub-branch, whose x it slices), so it takes them all.  Above eight it pays while x of all K fits
+    // one slice of its shared memory: 136 KB, which holds at every rank (with more than that it depends on what the rank
+    // leaves for the stages: 5120 -> 13824 at 14 tokens is up to 30 % faster, at 16 tokens and rank 128 2.5 times slower).
     // Outside that domain the other decode kernel keeps its own crossover: up to M = 4 it gets t from CTAs at the
     // head of its grid and wins at every rank up to 128; at M = 5 and 6 every CTA contributes to t and the tiles
     // wait for it, work that grows with M * rank, so M * rank above 128 goes to the tensor-core kernel.

@@ -317,12 +317,12 @@ __device__ __forceinline__ void store_terms(unsigned short *dst, size_t plane, c
 }
 // The matrix [R][C] (rows `ld` apart) as terms, rows as they are (`rows`: [3][R][pitch_r]) and / or transposed (`cols`: [3][C][pitch_c]).  Bound
 // by HBM: 4 bytes read, 6 written per copy and element; 64 x 64 tiles through shared memory, 8-byte stores.
-__global__ void __launch_bounds__(256) split_kernel(const float *__restrict__ src, size_t ld, int R, int C, unsigned short *rows, size_t pitch_r,
-                                                    unsigned short *cols, size_t pitch_c, const int *gate)
+__device__ __forceinline__ void split_tile(const float *__restrict__ src, size_t ld, int R, int C, unsigned short *rows, size_t pitch_r,
+                                           unsigned short *cols, size_t pitch_c, int tile_r, int tile_c)
 {
-    if (gate && *gate == 0) return;                       // not wanted
     __shared__ float tile[64][65];
-    const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64, tid = threadIdx.x;
+    const int r0 = tile_r * 64, c0 = tile_c * 64, tid = threadIdx.x;
+    if (r0 >= R || c0 >= C) return;
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const int e = tid + 256 * i, r = e >> 6, c = e & 63;
@@ -343,41 +343,79 @@ __global__ void __launch_bounds__(256) split_kernel(const float *__restrict__ sr
     }
 }
 
-// The square matrix [K][K] as terms, rows as they are (not wanted: NULL); `skew` is raised if any two entries across the diagonal differ.  A block
-// takes a tile and its mirror image (the blocks of the other triangle leave).
+__global__ void __launch_bounds__(256) split_kernel(const float *__restrict__ src, size_t ld, int R, int C, unsigned short *rows, size_t pitch_r,
+                                                    unsigned short *cols, size_t pitch_c)
+{
+    split_tile(src, ld, R, C, rows, pitch_r, cols, pitch_c, blockIdx.y, blockIdx.x);
+}
+// The transposed split, if `wanted` says so: few blocks, since most launches only look and leave.
+__global__ void __launch_bounds__(256) split_if_kernel(const float *__restrict__ src, size_t ld, int R, int C, unsigned short *cols, size_t pitch_c,
+                                                       const int *wanted)
+{
+    if (*wanted == 0) return;
+    const int across = (C + 63) / 64, tiles = across * ((R + 63) / 64);
+    for (int i = blockIdx.x; i < tiles; i += gridDim.x) {
+        split_tile(src, ld, R, C, nullptr, 0, cols, pitch_c, i / across, i % across);
+        __syncthreads();
+    }
+}
+// The sub-branch's A [r][K] as it is and B [N][r] transposed, and a flag cleared: one launch, since small layers are bound by
+// the number of them.
+__global__ void __launch_bounds__(256) split_branch_kernel(const float *__restrict__ A, int K, unsigned short *a_rows, size_t a_pitch,
+                                                           const float *__restrict__ B, int N, unsigned short *b_cols, size_t b_pitch, int r, int *flag)
+{
+    const int ka = (K + 63) / 64, ra = (r + 63) / 64, i = blockIdx.x - ka * ra;
+    if (i < 0) split_tile(A, K, r, K, a_rows, a_pitch, nullptr, 0, blockIdx.x / ka, blockIdx.x % ka);
+    else split_tile(B, r, N, r, nullptr, 0, b_cols, b_pitch, i / ra, i % ra);
+    if (i == 0 && threadIdx.x == 0) *flag = 0;
+}
+
+// The square matrix [K][K] as terms, rows as they are (not wanted: NULL); `skew` (cleared before) is raised if any two entries
+// across the diagonal differ.  A block takes a tile and its mirror image (the blocks of the other triangle leave); a thread
+// holds four quads of each and meets the mirrored values in shared memory.
 __global__ void __launch_bounds__(256) split_square_kernel(const float *__restrict__ src, int K, unsigned short *rows, size_t pitch, int *skew)
 {
-    __shared__ float tile[2][64][65];
+    __shared__ float mirror[64][65];
     if (blockIdx.x < blockIdx.y) return;
     const int at[2] = {(int)blockIdx.y * 64, (int)blockIdx.x * 64}, tid = threadIdx.x;
+    const bool wide = (K & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0u;
+    float v[2][4][4];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int r0 = at[h], c0 = at[1 - h];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int e = tid + 256 * i, r = e >> 6, c = e & 63;
-            tile[h][r][c] = (r0 + r < K && c0 + c < K) ? src[(size_t)(r0 + r) * K + c0 + c] : 0.f;
+        for (int i = 0; i < 4; ++i) {
+            const int e = tid + 256 * i, r = at[h] + (e >> 4), c = at[1 - h] + (e & 15) * 4;
+            if (wide && r < K && c < K) {
+                *reinterpret_cast<float4 *>(v[h][i]) = __ldg(reinterpret_cast<const float4 *>(src + (size_t)r * K + c));
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[h][i][k] = (r < K && c + k < K) ? src[(size_t)r * K + c + k] : 0.f;
+            }
         }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int e = tid + 256 * i;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mirror[e >> 4][(e & 15) * 4 + k] = v[1][i][k];
     }
     __syncthreads();
     bool differ = false;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const int e = tid + 256 * i, r = e >> 6, c = e & 63;
-        differ = differ || __float_as_uint(tile[0][r][c]) != __float_as_uint(tile[1][c][r]);
+    for (int i = 0; i < 4; ++i) {
+        const int e = tid + 256 * i;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) differ = differ || __float_as_uint(v[0][i][k]) != __float_as_uint(mirror[(e & 15) * 4 + k][e >> 4]);
     }
-    if (__syncthreads_or(differ) && tid == 0) *skew = 1;
+    if (__any_sync(0xffffffffu, differ) && (tid & 31) == 0) *skew = 1;
     if (!rows) return;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int r0 = at[h], c0 = at[1 - h];
         if (h == 1 && blockIdx.x == blockIdx.y) break;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int e = tid + 256 * i, a = e >> 4, b = (e & 15) * 4;
-            if (r0 + a >= K || c0 + b >= K) continue;
-            const float v[4] = {tile[h][a][b], tile[h][a][b + 1], tile[h][a][b + 2], tile[h][a][b + 3]};
-            store_terms(rows + (size_t)(r0 + a) * pitch + c0 + b, (size_t)K * pitch, v, K - (c0 + b));
+            const int e = tid + 256 * i, r = at[h] + (e >> 4), c = at[1 - h] + (e & 15) * 4;
+            if (r < K && c < K) store_terms(rows + (size_t)r * pitch + c, (size_t)K * pitch, v[h][i], K - c);
         }
     }
 }
@@ -506,16 +544,21 @@ bool product(cudaStream_t s, const Operand &P, const Operand &Q, ProductParams p
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, pmap, qmap, p, n_work) == cudaSuccess;
 }
-bool split(cudaStream_t s, const float *src, size_t ld, int R, int C, const Operand *rows, const Operand *cols, const int *gate = nullptr)
+bool split(cudaStream_t s, const float *src, size_t ld, int R, int C, const Operand *rows, const Operand *cols)
 {
     const dim3 grid((unsigned)((C + 63) / 64), (unsigned)((R + 63) / 64));
-    split_kernel<<<grid, 256, 0, s>>>(src, ld, R, C, rows ? rows->planes : nullptr, rows ? rows->pitch() : 0, cols ? cols->planes : nullptr, cols ? cols->pitch() : 0, gate);
+    split_kernel<<<grid, 256, 0, s>>>(src, ld, R, C, rows ? rows->planes : nullptr, rows ? rows->pitch() : 0, cols ? cols->planes : nullptr, cols ? cols->pitch() : 0);
     return cudaGetLastError() == cudaSuccess;
 }
 
+bool split_if(cudaStream_t s, const float *src, size_t ld, int R, int C, const Operand &cols, const int *wanted)
+{
+    const int tiles = ((C + 63) / 64) * ((R + 63) / 64);
+    split_if_kernel<<<(unsigned)std::min(tiles, 12 * pairs()), 256, 0, s>>>(src, ld, R, C, cols.planes, cols.pitch(), wanted);
+    return cudaGetLastError() == cudaSuccess;
+}
 bool split_square(cudaStream_t s, const float *src, int K, const Operand *rows, int *skew)
 {
-    if (cudaMemsetAsync(skew, 0, sizeof(int), s) != cudaSuccess) return false;
     const unsigned tiles = (unsigned)((K + 63) / 64);
     split_square_kernel<<<dim3(tiles, tiles), 256, 0, s>>>(src, K, rows ? rows->planes : nullptr, rows ? rows->pitch() : 0, skew);
     return cudaGetLastError() == cudaSuccess;
@@ -642,8 +685,10 @@ int run_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
     // Delta_F with Q(W - B A) held fixed (nothing else of the quantiser's output is kept)
     float *Delta = ws;
     if (launch_quantize_feedback(W, A, B, nullptr, nullptr, nullptr, nullptr, Delta, N, K, group, bits, rank, 2, s) != cudaSuccess) return FBQ_ERR_CUDA;
-    ok = split(s, A, K, rank, K, &t.A, nullptr) && split(s, B, rank, N, rank, nullptr, &t.Bt) && split_square(s, H, K, slabs_h == 1 ? &t.H : nullptr, t.skew);
-    *launches += 4;
+    split_branch_kernel<<<(unsigned)(((rank + 63) / 64) * ((K + 63) / 64 + (N + 63) / 64)), 256, 0, s>>>(
+        A, K, t.A.planes, t.A.pitch(), B, N, t.Bt.planes, t.Bt.pitch(), rank, t.skew);
+    ok = split_square(s, H, K, slabs_h == 1 ? &t.H : nullptr, t.skew);
+    *launches += 3;
     // slabs of Delta_F, transposed: the loss tr(Delta H Delta^T) = sum H o (Delta^T Delta), elementwise, and Delta^T B [K x rank]
     if (slabs_d > 1) ok = ok && cudaMemsetAsync(t.q_sum, 0, nq * sizeof(float), s) == cudaSuccess;
     for (int i = 0; i < slabs_d && ok; ++i) {
@@ -677,7 +722,7 @@ int run_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
             ++*launches;
         }
         columns(t.part, times(Hs, t.A), n, t.P.planes + k0, t.P.pitch(), nullptr, 0.f);
-        ok = ok && split(s, H + k0, K, K, n, nullptr, &Hs, t.skew);
+        ok = ok && split_if(s, H + k0, K, K, n, Hs, t.skew);
         ++*launches;
         columns(t.part, times(Hs, t.Q), n, nullptr, 0, A + k0, 2.f * lr);
     }

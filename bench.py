@@ -541,8 +541,8 @@ def decode_line(args, fbq, torch, wl, peaks, peak_kind, world, rank_id, local, b
                 dtb, _, _ = time_e2e(fbq, torch, wl, pool, e2e_steps, 3, batched=True)
                 if dtb < dt:
                     dt = dtb
-                    what = ("one fbq_linear_batch_hostio call per step after 0.3 s of untimed steps (the library's side streams overlap the problems' "
-                            "small copies), host buffers, synchronise per step")
+                    what = ("one fbq_linear_batch_hostio call per step after 0.3 s of untimed steps (one kernel reads all x over the "
+                            "bus, one launch computes all problems), host buffers, synchronise per step")
             extra["e2e"] = {"value": bytes_step * e2e_steps / dt / 1e9, "unit": "GB/s", "h2d_bytes_per_step": h2d,
                             "d2h_bytes_per_step": d2h, "ms_per_step": dt * 1e3 / e2e_steps, "steps": e2e_steps,
                             "per_linear_hostio_ms_per_step": per_linear_ms, "what": what}

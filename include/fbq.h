@@ -57,7 +57,7 @@ typedef enum {
 typedef enum {
     FBQ_KERNEL_NONE = -1,
     FBQ_KERNEL_GENERIC = 0,   /* any supported shape, CUDA cores, two launches if rank>0 */
-    FBQ_KERNEL_DECODE = 1,    /* M <= 16 (chosen for M <= 8, and to 16 at rank 0): fused streaming kernels, one launch */
+    FBQ_KERNEL_DECODE = 1,    /* M <= 16 (chosen for M <= 8, and to 16 while M * K * 2 <= 136 KB): fused streaming kernels, one launch */
     FBQ_KERNEL_PREFILL = 2    /* tcgen05 / TMEM tensor-core kernel, one launch (chosen from M = 9, or 7 outside the streaming kernel's domain) */
 } fbq_kernel;
 
@@ -155,7 +155,7 @@ int fbq_linear_hostio(const void *x_host, const uint32_t *qweight, const void *s
  *     streams, or several host threads) therefore race on it: run them one after another.
  *   - Arguments, layouts, dtypes (act_is_bf16 selects bf16 x, A, B, y) and results are
  *     those of fbq_linear / fbq_linear_bf16 with the "gemv" option off (the streaming kernel
- *     of M <= 2 is not served by the fixed array; the other decode kernel runs every M <= 16).
+ *     is not served by the fixed array; the other decode kernel runs every M <= 16).
  *     The process-wide options apply ("pdl", "decode_i8", "decode_t_ctas", ...), except those
  *     that size scratch ("decode_ctas", "decode_sk"), which stay automatic.
  *   - A device-side time-out lands in a status word inside the array; fbq_poll_status(any

@@ -667,7 +667,7 @@ cudaError_t run(const LinearArgs &a, int pitch, Workspace &ws, const PrefillTuni
 // over more than three waves of tiles.  Measured, INT4, rank 64, bf16, us per call, this kernel / the one that dequantises
 // per token tile: 1024 tokens 4096 -> 4096 (0.9 waves) 46 / 41, 11008 -> 4096 (0.9) 97 / 94, 4096 -> 11008 (2.9) 100 / 115,
 // but a layer whose shapes alternate between the two kernels 512 / 503; 4000 tokens 5120 -> 13824 (11.7) 440 / 530, the
-// 13B layer 2540 / 2840.
+// 13B layer 2460 / 2840.  (Few token tiles move the line: 8192 -> 32000 at 500 tokens, 3.4 waves, 320 / 251.)
 bool prefill_dense(const LinearArgs &a)
 {
     const int rows = launch_rows(a.N, a.K);

@@ -7,14 +7,14 @@
 //
 //   * Everything that comes from the WEIGHTS (packed codes, scales, zero points, B, A) is requested
 //     before the kernel waits for the preceding kernel of its stream (programmatic dependent
-//     launch); a CTA takes half an SM's shared memory at most, so the CTAs of the next launch are
-//     resident and prefetching while this launch still computes.
+//     launch); a CTA of one or two tokens takes half an SM's shared memory at most where it can, so with
+//     one CTA per SM those of the next launch are resident and prefetching while this one computes.
 //   * No table is built per CTA: scales and zero points of a 16-row tile arrive as they are stored
 //     (two bulk copies per tile) and are converted where they are used.
 //   * The weight stream is one TMA tensor copy per stage (16 groups x 16 rows of packed codes) into
 //     an mbarrier ring; eight compute warps share every stage.
 //
-// Main CTAs (one per SM by default) own contiguous ranges of 16-row tiles.  Integer form (M <= 2):
+// Main CTAs (one per SM, or two: make_plan) own contiguous ranges of 16-row tiles.  Integer form (M <= 2):
 // a code masked out of its word is an unsigned byte operand of the 8-bit integer MMA as it stands
 // (four codes per register, at most one shift per word); x is fixed point per group of 128 (three
 // signed base-256 digits, exact integer sums), and scale and zero point are applied per group to the
@@ -1921,8 +1921,9 @@ Plan make_plan_on(const LinearArgs &a, const GemvTuning &tune, int per_sm)
 // 46.3, 59.8 / 50.9; 13B INT4 rank 64 79.1 / 70.6, two tokens 96.1 / 76.4; 4096 -> 32000 36.2 / 27.4.  Not where the t CTAs
 // need a whole SM (rank above 64: 51.8 / 73.8, with smaller chunks of A 62.9), nor for INT3 at one token without a
 // sub-branch (40.8 / 41.7: its smaller stages already keep more of them in flight).  Launched from the host without a graph
-// the seven take 60.7 / 47.6.  What pays for it: linears side by side on several streams (q, k, v, then gate, up: 40.5 / 47.2
-// per layer), for which one launch of the batch is the faster way; a mix by size was worse in a row (53.6).
+// the seven take 60.7 / 47.6.  What pays for it: linears side by side on several streams (7B INT4, one token: all seven 33.5 / 40.7 us,
+// q, k, v, then gate, up 50.2 / 54.7), for which there is a bound per stream (fbq_set_stream_option), and for those that share x
+// the batch, which is faster than either (37.9); a mix by size was worse in a row (53.6).
 Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
 {
     if (tune.max_ctas == 0 && tune.main_ctas == 0 && a.rank <= 64 && !(a.bits == 3 && a.rank == 0 && a.M == 1)) {

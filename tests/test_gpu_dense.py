@@ -123,3 +123,20 @@ def test_pair_option_holds_for_many_tiles():
         finally:
             fbq.set_option("prefill_pair", 0)
     assert taken[0] >= inp.N * inp.K * 2 > taken[1]
+
+
+@pytest.mark.parametrize("K,rank", [(128, 0), (128, 64), (256, 8)])
+def test_dense_prefill_of_many_short_tiles(K, rank):
+    # 55 x 32 tiles, some twenty per pair, each of one to three stages: the ring of claimed tiles wraps around while the copies
+    # run as many tiles ahead of the epilogue as they can
+    import torch
+    import paper_2501_16385_b200 as fbq
+    M, N = 8000, 14008
+    inp = make_linear(M, N, K, 4, rank, dtype="f16", seed=3600 + K + rank)
+    rows = np.unique(np.concatenate([np.arange(4), np.arange(N - 4, N), np.random.default_rng(K).choice(N, 24)]))
+    check_parity(inp, fbq, expect_kernel=fbq.KERNEL_PREFILL, n_list=rows, threads=16, floor=2e-5)
+    dev = DeviceLinear(inp, fbq)
+    want = dev.run(fbq)
+    for _ in range(20):
+        assert torch.equal(dev.run(fbq), want)
+    assert fbq.poll_status() == 0

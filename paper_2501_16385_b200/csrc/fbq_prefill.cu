@@ -340,20 +340,17 @@ prefill_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     continue;
                 }
                 if (!t_ready) {                              // every warp of every t CTA of this token tile has stored its part
+                    // (every lane looks for itself, one request per warp: an acquire by one lane would order nothing for the others)
+                    const int *flag = p.tflag + m_tile;
+                    const int target = 16 * p.rt * p.splitt;
                     int seen = 0;
-                    if (lane == 0) {
-                        const int *flag = p.tflag + m_tile;
-                        const int target = 16 * p.rt * p.splitt;
 #pragma unroll 1
-                        for (uint32_t spin = 0; spin < p.flag_polls; ++spin) {
-                            asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
-                            if (seen >= target) break;
-                            __nanosleep(256);
-                        }
-                        seen = seen >= target;
+                    for (uint32_t spin = 0; spin < p.flag_polls; ++spin) {
+                        asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
+                        if (seen >= target) break;
+                        __nanosleep(256);
                     }
-                    t_ready = __shfl_sync(0xffffffffu, seen, 0) != 0;
-                    __syncwarp();                            // (a shuffle orders no memory: all lanes read t behind lane 0's acquire)
+                    t_ready = __all_sync(0xffffffffu, seen >= target) != 0;
                     if (!t_ready) { dead = true; break; }
                 }
                 const int j0 = (i - kb_x) * kBK;
@@ -922,20 +919,17 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
                 const int s = i % kStages;
                 if (i >= kStages && !wait_looks(empty0 + 8u * s, (uint32_t)(i / kStages - 1) & 1u)) { dead = true; break; }
                 if (!t_ready) {                              // every warp of every t CTA of this token tile has stored its part
+                    // (every lane looks for itself, one request per warp: an acquire by one lane would order nothing for the others)
+                    const int *flag = p.tflag + m_tile;
+                    const int target = 16 * p.rt;
                     int seen = 0;
-                    if (lane == 0) {
-                        const int *flag = p.tflag + m_tile;
-                        const int target = 16 * p.rt;
 #pragma unroll 1
-                        for (uint32_t spin = 0; spin < p.flag_polls; ++spin) {
-                            asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
-                            if (seen >= target) break;
-                            __nanosleep(256);
-                        }
-                        seen = seen >= target;
+                    for (uint32_t spin = 0; spin < p.flag_polls; ++spin) {
+                        asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
+                        if (seen >= target) break;
+                        __nanosleep(256);
                     }
-                    t_ready = __shfl_sync(0xffffffffu, seen, 0) != 0;
-                    __syncwarp();                            // (a shuffle orders no memory: all lanes read t behind lane 0's acquire)
+                    t_ready = __all_sync(0xffffffffu, seen >= target) != 0;
                     if (!t_ready) { dead = true; break; }
                 }
                 const int j0 = (i - p.kb_main) * kBK;

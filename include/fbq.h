@@ -246,8 +246,9 @@ int fbq_linear_batch(const fbq_problem *problems, int count, int M, int group, i
  * weights on the device as before.  Up to 8 problems of the streaming kernel are two launches on
  * `stream`: one reads every distinct x over the bus into a staging buffer kept per stream (copies,
  * where it is not pinned), the other computes all problems and writes y straight to the caller's
- * buffers where they are pinned.  Otherwise each problem is copied in, computed and copied out on
- * the stream it runs on.
+ * buffers where they are pinned.  Problems that run one after the other on `stream` get their x at the
+ * start of the call while all x together are small (4 MB); otherwise each problem is copied in, computed
+ * and copied out on the stream it runs on.
  * y is complete once work queued on `stream` after the call has run (synchronise `stream`
  * before reading it).  The end-to-end path of the benchmark. */
 int fbq_linear_batch_hostio(const fbq_problem *problems, int count, int M, int group, int bits, int rank,

@@ -609,38 +609,56 @@ static BatchLanes *lanes_for(int want)
     return &b;
 }
 
+// The distinct x of a batch with host buffers, and their places in the stream's staging buffer (grown if need be).  No y of
+// a batch overlaps an x of it, so all of them can be brought over at its start.
+struct BatchX {
+    int n = 0;
+    const void *src[FBQ_BATCH_MAX];
+    void *dst[FBQ_BATCH_MAX];
+    size_t bytes[FBQ_BATCH_MAX], total = 0;
+};
+static int place_batch_x(LinearArgs *a, int count, int M, Workspace *ws, cudaStream_t s, BatchX &b)
+{
+    size_t off[FBQ_BATCH_MAX];
+    int which[FBQ_BATCH_MAX];
+    for (int i = 0; i < count; ++i) {
+        if (!a[i].x || !a[i].y) return FBQ_ERR_BADARG;
+        int k = 0;
+        while (k < b.n && !(b.src[k] == a[i].x && b.bytes[k] == (size_t)M * a[i].K * 2)) ++k;
+        if (k == b.n) {
+            b.src[k] = a[i].x;
+            b.bytes[k] = (size_t)M * a[i].K * 2;
+            off[k] = b.total;
+            b.total += (b.bytes[k] + 255) & ~(size_t)255;
+            ++b.n;
+        }
+        which[i] = k;
+    }
+    char *sx = static_cast<char *>(ws->stage_x);
+    const cudaError_t e = grow(sx, ws->stage_x_bytes, b.total, 1, s);
+    ws->stage_x = sx;
+    if (e != cudaSuccess) return grow_status(e);
+    for (int i = 0; i < count; ++i) a[i].x = sx + off[which[i]];
+    for (int k = 0; k < b.n; ++k) b.dst[k] = sx + off[k];
+    return FBQ_OK;
+}
+
 // A decode-sized batch with host buffers as two launches: x (each distinct one once) into the stream's staging buffer, then
 // all problems; y goes straight to the caller's buffers where that is possible.  FBQ_ERR_UNSUPPORTED: nothing was queued.
 static int host_batch(const LinearArgs *in, const fbq_problem *problems, int count, int M, cudaStream_t s)
 {
     LinearArgs a[FBQ_BATCH_MAX];
-    const void *src[FBQ_BATCH_MAX];
-    void *dst[FBQ_BATCH_MAX];
-    size_t bytes[FBQ_BATCH_MAX], x_bytes = 0, y_bytes = 0, off[FBQ_BATCH_MAX];
-    int nx = 0, which[FBQ_BATCH_MAX];
+    size_t y_bytes = 0;
     auto padded = [](size_t n) { return (n + 255) & ~(size_t)255; };
     Workspace *ws = workspace_for(s);
     if (!ws) return FBQ_ERR_CUDA;
-    for (int i = 0; i < count; ++i) {
-        a[i] = in[i];
-        if (!a[i].x || !a[i].y) return FBQ_ERR_BADARG;
-        int k = 0;
-        while (k < nx && !(src[k] == a[i].x && bytes[k] == (size_t)M * a[i].K * 2)) ++k;
-        if (k == nx) {
-            src[nx] = a[i].x;
-            bytes[nx] = (size_t)M * a[i].K * 2;
-            off[nx] = x_bytes;
-            x_bytes += padded(bytes[nx++]);
-        }
-        which[i] = k;
-    }
-    char *sx = static_cast<char *>(ws->stage_x), *sy = static_cast<char *>(ws->stage_y);
-    cudaError_t e = grow(sx, ws->stage_x_bytes, x_bytes, 1, s);
-    ws->stage_x = sx;
-    if (e != cudaSuccess) return grow_status(e);
+    std::copy(in, in + count, a);
+    BatchX x;
+    if (const int rc = place_batch_x(a, count, M, ws, s, x); rc != FBQ_OK) return rc;
+    char *sy = static_cast<char *>(ws->stage_y);
+    cudaError_t e;
     bool staged[FBQ_BATCH_MAX];
     for (int i = 0; i < count; ++i) {
-        a[i].x = sx + off[which[i]];
         void *alias = direct_y_alias(a[i].y, (size_t)M * a[i].N * 2);
         staged[i] = alias == nullptr;
         a[i].y = alias ? alias : reinterpret_cast<void *>(y_bytes);        // (an offset until the buffer is there)
@@ -659,8 +677,7 @@ static int host_batch(const LinearArgs *in, const fbq_problem *problems, int cou
         GemvTuning gt = g_opt.gemv;
         if (gt.max_ctas > 0 || g_opt.decode_trace || !gemv_batch_need(a, count, gt, &slots, &nc)) return FBQ_ERR_UNSUPPORTED;
     }
-    for (int k = 0; k < nx; ++k) dst[k] = sx + off[k];
-    if (copy_in(nx, src, dst, bytes, s) != cudaSuccess) return FBQ_ERR_CUDA;
+    if (copy_in(x.n, x.src, x.dst, x.bytes, s) != cudaSuccess) return FBQ_ERR_CUDA;
     const int rc = run_gemv_batch(a, count, s);
     if (rc != FBQ_OK) return rc == FBQ_ERR_UNSUPPORTED ? FBQ_ERR_CUDA : rc;
     for (int i = 0; i < count; ++i)
@@ -695,26 +712,29 @@ static int linear_batch_common(const fbq_problem *problems, int count, int M, in
     }
     // With host_io, x and y of every problem are host buffers: x is copied to, and y back from,
     // staging buffers kept per stream, on the stream the problem runs on.
-    auto stage_in = [&](LinearArgs &la, cudaStream_t st) -> int {
+    auto stage_y = [&](LinearArgs &la, cudaStream_t st) -> int {
         if (!host_io) return FBQ_OK;
         Workspace *ws = workspace_for(st);
-        if (!ws || !la.x || !la.y) return ws ? FBQ_ERR_BADARG : FBQ_ERR_CUDA;
-        const size_t xb = (size_t)M * la.K * 2, yb = (size_t)M * la.N * 2;
-        char *sx = static_cast<char *>(ws->stage_x), *sy = static_cast<char *>(ws->stage_y);
-        if (grow(sx, ws->stage_x_bytes, xb, 1, st) != cudaSuccess) return FBQ_ERR_CUDA;
-        ws->stage_x = sx;
-        const void *from[1] = {la.x};
-        void *to[1] = {sx};
-        if (copy_in(1, from, to, &xb, st) != cudaSuccess) return FBQ_ERR_CUDA;
-        la.x = sx;
+        if (!ws || !la.y) return ws ? FBQ_ERR_BADARG : FBQ_ERR_CUDA;
+        const size_t yb = (size_t)M * la.N * 2;
         if (void *alias = direct_y_alias(la.y, yb)) {
             la.y = alias;                             // the kernel writes the caller's buffer itself
             return FBQ_OK;
         }
+        char *sy = static_cast<char *>(ws->stage_y);
         if (grow(sy, ws->stage_y_bytes, yb, 1, st) != cudaSuccess) return FBQ_ERR_CUDA;
         ws->stage_y = sy;
         la.y = sy;
         return FBQ_OK;
+    };
+    auto stage_in = [&](LinearArgs &la, cudaStream_t st) -> int {
+        if (!host_io) return FBQ_OK;
+        Workspace *ws = workspace_for(st);
+        if (!ws) return FBQ_ERR_CUDA;
+        BatchX x;
+        if (const int rc = place_batch_x(&la, 1, M, ws, st, x); rc != FBQ_OK) return rc;
+        if (copy_in(x.n, x.src, x.dst, x.bytes, st) != cudaSuccess) return FBQ_ERR_CUDA;
+        return stage_y(la, st);
     };
     auto stage_out = [&](const LinearArgs &la, void *y_host, cudaStream_t st) -> int {
         if (!host_io) return FBQ_OK;
@@ -723,9 +743,26 @@ static int linear_batch_common(const fbq_problem *problems, int count, int M, in
         return cudaMemcpyAsync(y_host, la.y, (size_t)M * la.N * 2, cudaMemcpyDeviceToHost, st) == cudaSuccess ? FBQ_OK : FBQ_ERR_CUDA;
     };
     if (!all_decode) {
-        // one after the other on the caller's stream (prefill-sized problems fill the GPU by themselves)
+        // One after the other on the caller's stream (prefill-sized problems fill the GPU by themselves).  x from host buffers
+        // comes over at the start, shared x once, unless that takes much staging space: one by one each copy would wait for the linear
+        // before.
+        size_t x_bytes = 0;
+        for (int i = 0; i < count; ++i) x_bytes += (size_t)M * a[i].K * 2;
+        const bool together = host_io && x_bytes <= 8 * kGatherMost;
+        if (together) {
+            Workspace *ws = workspace_for(main);
+            if (!ws) return FBQ_ERR_CUDA;
+            BatchX x;
+            if (const int rc = place_batch_x(a, count, M, ws, main, x); rc != FBQ_OK) return rc;
+            // as few gathers as take kGatherMost each
+            for (int first = 0, n; first < x.n; first += n) {
+                size_t part = x.bytes[first];
+                for (n = 1; first + n < x.n && part + x.bytes[first + n] <= kGatherMost; ++n) part += x.bytes[first + n];
+                if (copy_in(n, x.src + first, x.dst + first, x.bytes + first, main) != cudaSuccess) return FBQ_ERR_CUDA;
+            }
+        }
         for (int i = 0; i < count; ++i) {
-            int rc = stage_in(a[i], main);
+            int rc = together ? stage_y(a[i], main) : stage_in(a[i], main);
             if (rc == FBQ_OK) rc = run_linear(a[i], main);
             if (rc == FBQ_OK) rc = stage_out(a[i], problems[i].y, main);
             if (rc != FBQ_OK) return rc;

@@ -50,3 +50,27 @@ def test_chained_host_calls_run_in_order(M, bits, rank, batch):
             # grid): fp16 rounding of each step, amplified by at most the four steps of the chain
             assert torch.isfinite(y).all()
             assert float((y.float() - ref).norm() / ref.norm()) < 4 * 2 ** -10
+
+
+@pytest.mark.parametrize("M,pin", [(13, True), (13, False), (40, True), (300, True)])
+def test_host_batches_of_mixed_kernels_and_shared_x(M, pin):
+    # a batch whose problems run one after the other (some of them the tensor-core kernel's): x of all of them is staged at the
+    # start of the call where it is small, per problem where it is large (300 tokens here), shared x once
+    import torch
+    import paper_2501_16385_b200 as fbq
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M)
+    shapes = [(1024, 512), (1024, 768), (13824, 256), (1024, 264)]
+    weights = [_weights(fbq, K, N, 4, 16, g) for K, N in shapes]
+    assert len({fbq.select_kernel(13, N, K, 128, 4, 16) for K, N in shapes}) == 2
+    a, b, c = (torch.randn((M, K), device="cuda", generator=g).half() for K in (1024, 13824, 1024))
+    xs = [a, a, b, c]
+    want = [fbq.linear(x, *w, N, 128, 4) for x, w, (K, N) in zip(xs, weights, shapes)]
+    host = {id(x): (x.cpu().pin_memory() if pin else x.cpu()) for x in xs}
+    for _ in range(5):
+        ys = [torch.full((M, N), float("nan")).half() for K, N in shapes]
+        ys = [y.pin_memory() if pin else y for y in ys]
+        fbq.linear_batch([(host[id(x)], *w, y) for x, w, y in zip(xs, weights, ys)], 128, 4, host_io=True)
+        torch.cuda.synchronize()
+        assert fbq.poll_status() == 0
+        assert all(torch.equal(y, ref.cpu()) for y, ref in zip(ys, want))

@@ -56,6 +56,7 @@ constexpr int kCHG = 2 * kCW;                // quantisation groups of a stage (
 constexpr int kMaxNS = 8, kMaxBuf = 8, kMaxB = 4, kMaxMeta = 8;
 constexpr int kMaxSub = 8;                   // tiles whose t.B^T may be formed ahead of their main sums
 constexpr int kGemvBatchMax = 8;             // problems of one launch
+constexpr int kTStages = 5;                  // stages that a main CTA gets through while the t CTAs run (3 to 8, by layer and form)
 constexpr int kTKB = 64;                     // k extent of one block of A in a t CTA (128 bytes: the swizzle span)
 
 struct GemvParams {
@@ -2204,7 +2205,8 @@ cudaError_t make_maps(const LinearArgs &a, const GemvParams &p, CUtensorMap *wma
 // SMs with its own CTAs pays more than letting the next launch's in; 4096 -> 3 x 4096 INT3 rank 64: 8.8 us, 11.3 with one,
 // 15.4 as three launches; 4096 -> 2 x 11008: 12.7, 15.6, 17.2), unless a CTA of the launch needs more than half of an SM's
 // shared memory (t CTAs of rank 112 and 128, x of a long K): then one, where two would run in two rounds (rank 128, INT4, one
-// token: 4096 -> 3 x 4096 14.1 / 12.0 us, 4096 -> 2 x 11008 19.0 / 16.9, 13824 -> 2 x 5120 50.8 / 25.7); 16-bit form: one (its
+// token: 4096 -> 3 x 4096 14.1 / 12.0 us, 4096 -> 2 x 11008 19.1 / 16.9, 13824 -> 2 x 5120 50.4 / 23.6; a 7B layer from host
+// buffers 75 / 58 with the call); 16-bit form: one (its
 // CTAs take a whole SM; four tokens: 17.9 and 26.1 us, one by one 28.1 and 31.5).
 struct BatchPlan {
     Plan plan[kGemvBatchMax];
@@ -2228,17 +2230,25 @@ BatchPlan plan_batch_on(const LinearArgs *a, int count, const GemvTuning &tune, 
         const int nt = (a[i].N + kTile - 1) / kTile, most = std::max(1, load / stages(i)), c = (nt + most - 1) / most;
         return wide ? std::max(2, (c + 1) / 2 * 2) : c;
     };
-    const int budget = std::max(2 * count, per_sm * g_sm_count - n_t);
-    int lo = 1, hi = 1;
     auto total = [&](int load) { int c = 0; for (int i = 0; i < count; ++i) c += share(i, load); return c; };
-    while (total(hi) > budget && hi < (1 << 24)) hi *= 2;
-    while (lo < hi) {
-        const int mid = (lo + hi) / 2;
-        if (total(mid) <= budget) hi = mid;
-        else lo = mid + 1;
-    }
+    auto least_load = [&](int ctas) {                            // with that many main CTAs
+        const int budget = std::max(2 * count, ctas);
+        int lo = 1, hi = 1;
+        while (total(hi) > budget && hi < (1 << 24)) hi *= 2;
+        while (lo < hi) {
+            const int mid = (lo + hi) / 2;
+            if (total(mid) <= budget) hi = mid;
+            else lo = mid + 1;
+        }
+        return lo;
+    };
+    // All CTAs at once, or, with one CTA per SM and many t CTAs (a whole layer from host buffers: 70 of 148), a main CTA for every
+    // SM, some of which start when the t CTAs leave.  (One t CTA per problem stays until every main CTA has read t.)
+    int load = least_load(per_sm * g_sm_count - n_t);
+    if (!wide && per_sm == 1 && n_t > 0)
+        if (const int later = least_load(g_sm_count - count); later + kTStages < load) load = later;
     for (int i = 0; i < count; ++i) {
-        t.main_ctas = share(i, lo);
+        t.main_ctas = share(i, load);
         bp.plan[i] = plan_for(a[i], t);
         if (!bp.plan[i].ok || (wide && (bp.plan[i].p.R & 1 || bp.plan[i].p.R < 2))) return bp;
         if (per_sm == 2 && bp.plan[i].smem > kSmemShare + 1024) return bp;       // (the launch takes the most that any of its CTAs needs)

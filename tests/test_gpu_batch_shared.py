@@ -58,7 +58,9 @@ def test_shared_x_is_one_launch(M, bits, rank, dtype, K, rows):
 
 
 @pytest.mark.parametrize("M,bits,rank,dtype,K,rows", [(1, 4, 128, "f16", 4096, (4096, 1000, 40)), (2, 3, 112, "bf16", 1024, (2056, 2056)),
-                                                      (1, 3, 128, "f16", 13824, (640, 640)), (2, 4, 64, "f16", 13824, (640, 520))])
+                                                      (1, 3, 128, "f16", 13824, (640, 640)), (2, 4, 64, "f16", 13824, (640, 520)),
+                                                      (1, 4, 128, "f16", 4096, (4096,) * 4 + (11008,) * 2)])
 def test_shared_x_with_ctas_that_fill_an_sm(M, bits, rank, dtype, K, rows):
-    # t CTAs of rank 112 and 128, or x of a long K, take more than half of an SM's shared memory: one CTA per SM
+    # t CTAs of rank 112 and 128, or x of a long K, take more than half of an SM's shared memory: one CTA per SM; in the last
+    # case the t CTAs of six problems would leave too few SMs, and some main CTAs start when they are through
     test_shared_x_is_one_launch(M, bits, rank, dtype, K, rows)

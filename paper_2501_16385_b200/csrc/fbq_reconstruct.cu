@@ -348,14 +348,21 @@ __global__ void __launch_bounds__(256) split_kernel(const float *__restrict__ sr
 {
     split_tile(src, ld, R, C, rows, pitch_r, cols, pitch_c, blockIdx.y, blockIdx.x);
 }
-// The transposed split, if `wanted` says so: few blocks, since most launches only look and leave.
-__global__ void __launch_bounds__(256) split_if_kernel(const float *__restrict__ src, size_t ld, int R, int C, unsigned short *cols, size_t pitch_c,
-                                                       const int *wanted)
+// A transposed split that is done if `wanted` says so (most launches only look).
+struct SplitIf {
+    const float *src;
+    size_t ld;
+    int R, C;
+    unsigned short *cols;
+    size_t pitch;
+    const int *wanted;
+};
+__device__ __forceinline__ void split_if(const SplitIf &w, int block, int blocks)
 {
-    if (*wanted == 0) return;
-    const int across = (C + 63) / 64, tiles = across * ((R + 63) / 64);
-    for (int i = blockIdx.x; i < tiles; i += gridDim.x) {
-        split_tile(src, ld, R, C, nullptr, 0, cols, pitch_c, i / across, i % across);
+    if (*w.wanted == 0) return;
+    const int across = (w.C + 63) / 64, tiles = across * ((w.R + 63) / 64);
+    for (int i = block; i < tiles; i += blocks) {
+        split_tile(w.src, w.ld, w.R, w.C, nullptr, 0, w.cols, w.pitch, i / across, i % across);
         __syncthreads();
     }
 }
@@ -421,9 +428,14 @@ __global__ void __launch_bounds__(256) split_square_kernel(const float *__restri
 }
 
 // Sums the slices of a product [split][R][r] in order; transposed to terms [3][r][pitch], or added to `into` (rows `into_ld` apart) times alpha.
+// Blocks of a second layer of the grid do `then`, which needs the product to have been read as well and is no launch of its own.
 __global__ void __launch_bounds__(256) sum_transposed_kernel(const float *__restrict__ part, int splits, int R, int r, unsigned short *planes, size_t pitch,
-                                                             float *into, size_t into_ld, float alpha)
+                                                             float *into, size_t into_ld, float alpha, const SplitIf then)
 {
+    if (blockIdx.z) {
+        split_if(then, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+        return;
+    }
     __shared__ float tile[32][33];
     const int k0 = blockIdx.x * 32, j0 = blockIdx.y * 32, tid = threadIdx.x;
 #pragma unroll
@@ -551,12 +563,6 @@ bool split(cudaStream_t s, const float *src, size_t ld, int R, int C, const Oper
     return cudaGetLastError() == cudaSuccess;
 }
 
-bool split_if(cudaStream_t s, const float *src, size_t ld, int R, int C, const Operand &cols, const int *wanted)
-{
-    const int tiles = ((C + 63) / 64) * ((R + 63) / 64);
-    split_if_kernel<<<(unsigned)std::min(tiles, 12 * pairs()), 256, 0, s>>>(src, ld, R, C, cols.planes, cols.pitch(), wanted);
-    return cudaGetLastError() == cudaSuccess;
-}
 bool split_square(cudaStream_t s, const float *src, int K, const Operand *rows, int *skew)
 {
     const unsigned tiles = (unsigned)((K + 63) / 64);
@@ -668,9 +674,9 @@ int run_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
     p.C = t.part;
     p.skew = t.skew;
     bool ok = true;
-    auto columns = [&](const float *part, int splits, int rows, unsigned short *planes, size_t pitch, float *into, float alpha) {
-        const dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((rank + 31) / 32));
-        sum_transposed_kernel<<<grid, 256, 0, s>>>(part, splits, rows, rank, planes, pitch, into, (size_t)K, alpha);
+    auto columns = [&](const float *part, int splits, int rows, unsigned short *planes, size_t pitch, float *into, float alpha, const SplitIf *then = nullptr) {
+        const dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((rank + 31) / 32), then ? 2u : 1u);
+        sum_transposed_kernel<<<grid, 256, 0, s>>>(part, splits, rows, rank, planes, pitch, into, (size_t)K, alpha, then ? *then : SplitIf{});
         ++*launches;
     };
     auto add = [&](const float *part, int splits, size_t n, float *into, float alpha) {
@@ -721,9 +727,8 @@ int run_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
             ok = split(s, H + (size_t)k0 * K, K, n, K, &Hs, nullptr);
             ++*launches;
         }
-        columns(t.part, times(Hs, t.A), n, t.P.planes + k0, t.P.pitch(), nullptr, 0.f);
-        ok = ok && split_if(s, H + k0, K, K, n, Hs, t.skew);
-        ++*launches;
+        const SplitIf cols{H + k0, (size_t)K, K, n, Hs.planes, Hs.pitch(), t.skew};
+        columns(t.part, times(Hs, t.A), n, t.P.planes + k0, t.P.pitch(), nullptr, 0.f, &cols);
         columns(t.part, times(Hs, t.Q), n, nullptr, 0, A + k0, 2.f * lr);
     }
     // slabs of Delta_F: B <- B + 2 lr Delta (H A^T)

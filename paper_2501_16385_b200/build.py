@@ -20,7 +20,7 @@ OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libfbq.so")
 TORCH_SRC = "fbq_torch.cpp"
 TORCH_LIB = os.path.join(HERE, "_fbq_torch.so")
-SOURCES = ["fbq_api.cu", "fbq_maps.cu", "fbq_pack.cu", "fbq_generic.cu", "fbq_decode.cu", "fbq_gemv.cu", "fbq_prefill.cu", "fbq_dense.cu", "fbq_noalloc.cu",
+SOURCES = ["fbq_api.cu", "fbq_maps.cu", "fbq_pack.cu", "fbq_generic.cu", "fbq_decode.cu", "fbq_gemv.cu", "fbq_split.cu", "fbq_prefill.cu", "fbq_dense.cu", "fbq_noalloc.cu",
            "fbq_quant.cu", "fbq_reconstruct.cu"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 COMPILE_FLAGS = ARCH + ["-lineinfo", "-O3", "-std=c++17", "-Xptxas=-v", "-Xcompiler", "-fPIC", "-rdc=false"]

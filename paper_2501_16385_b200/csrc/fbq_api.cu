@@ -144,28 +144,9 @@ int select_kernel(int M, int N, int K, int group, int bits, int rank, bool bf16)
     if (g_opt.force_kernel == FBQ_KERNEL_DECODE && decode_ok) return FBQ_KERNEL_DECODE;
     if (g_opt.force_kernel == FBQ_KERNEL_PREFILL && prefill_ok) return FBQ_KERNEL_PREFILL;
     if (g_opt.force_kernel >= 0) return FBQ_KERNEL_GENERIC;
-    // Measured on B200, INT4, fp16, us per launch in a row, streaming / tensor-core kernel (in KB: x of all tokens):
-    //                          rank 0                        rank 64                       rank 128
-    //   4096 -> 4096    M  8   8.5 / 12.9                    9.8 / 15.4                    11.7 / 16.2
-    //                   M 12  10.6 / 12.9                   12.7 / 15.5                    15.5 / 16.3
-    //                   M 16  12.1 / 12.9  (128 KB)         14.0 / 16.0                    17.6 / 16.7
-    //   4096 -> 11008   M 16  16.5 / 25.2                   19.9 / 27.2                    24.7 / 27.4
-    //   5120 -> 13824   M 12  20.7 / 30.5  (120 KB)         24.5 / 32.6                    28.9 / 33.0
-    //                   M 14  21.7 / 30.6  (140 KB)         29.6 / 32.7                    30.9 / 33.1
-    //                   M 16  26.2 / 30.6  (160 KB)         33.2 / 32.7                    83.7 / 33.1
-    //   8192 -> 8192    M  8  18.5 / 28.1  (128 KB)         19.6 / 29.6                    20.4 / 30.4
-    //                   M 12  39.6 / 28.1  (192 KB)         47.9 / 29.6                    52.3 / 30.4
-    //   11008 -> 4096   M  7  19.5 / 22.0  (150 KB)         20.5 / 23.9                    21.5 / 24.9
-    //                   M  8  22.2 / 22.1  (172 KB)         26.8 / 24.0                    27.5 / 25.0
-    //                   M 12  34.7 / 22.0                   44.4 / 23.8                    50.5 / 25.0
-    //   13824 -> 5120   M  5  21.0 / 31.0  (135 KB)         22.0 / 32.6                    29.8 / 33.6
-    //                   M  8  29.7 / 31.1  (216 KB)         36.2 / 32.8                    36.4 / 33.9
-    //   28672 -> 8192   M  4  43.8 / 81.9  (224 KB)         60.9 / 83.4                    63.7 / 83.7
-    //                   M  8  61.5 / 82.0  (448 KB)         89.1 / 83.4                    92.4 / 83.5
-    // Up to eight tokens the streaming kernel is ahead by up to a factor of two and behind by 16 % at most (7 and 8 tokens of
-    // the longest K with a sub-branch, whose x it slices), so it takes them all.  Above eight it pays while x of all K fits
-    // one slice of its shared memory: 136 KB, which holds at every rank (with more than that it depends on what the rank
-    // leaves for the stages: 5120 -> 13824 at 14 tokens is up to 30 % faster, at 16 tokens and rank 128 2.5 times slower).
+    // In the streaming kernels' domain the decode class is one and two tokens (the streaming kernel) and as many as the split kernel
+    // is given by name: up to eight of any K, and up to sixteen while x of all K takes 136 KB.  A call of up to sixteen tokens that
+    // falls into the other class runs on the split kernel all the same (split_takes), so the line names a class, not a speed.
     // Outside that domain the other decode kernel keeps its own crossover: up to M = 4 it gets t from CTAs at the
     // head of its grid and wins at every rank up to 128; at M = 5 and 6 every CTA contributes to t and the tiles
     // wait for it, work that grows with M * rank, so M * rank above 128 goes to the tensor-core kernel.
@@ -226,7 +207,44 @@ int check_args(const LinearArgs &a)
     return FBQ_OK;
 }
 
-// Several problems of the streaming kernel as one launch on `s`; FBQ_ERR_UNSUPPORTED where they cannot share one.
+// One problem or several, for which there is a plan, in one launch of the split kernel.
+int run_split(const LinearArgs *a, int count, const GemvTuning &gt, Workspace *ws, cudaStream_t s)
+{
+    size_t have_c = (size_t)ws->n_counters;
+    int launches = 0;
+    char *scratch = static_cast<char *>(ws->split);
+    cudaError_t e = grow(scratch, ws->split_bytes, split_scratch_bytes(a, count), 1, s);
+    ws->split = scratch;
+    if (e != cudaSuccess) return grow_status(e);
+    if ((e = grow(ws->counters, have_c, 16, sizeof(int), s)) != cudaSuccess) return grow_status(e);
+    ws->n_counters = (int)have_c;
+    if (launch_split(a, count, *ws, gt, s, &launches) != cudaSuccess) return FBQ_ERR_CUDA;
+    g_launches += launches;
+    return FBQ_OK;
+}
+
+// Calls of 3 to 16 tokens in the streaming kernels' domain, also those that select_kernel counts among the prompts, unless a
+// kernel is forced.  Measured on B200, INT4, bf16, us per launch in a row, the kernels before it (a streaming one whose CTAs
+// staged x of all K, or the tensor-core one) / this one:
+//                      4 tokens, rank 64   8 tokens, rank 128   16 tokens, rank 64
+//   4096 -> 4096          8.7 /  7.3           11.7 /  8.1          13.9 /  8.2
+//   4096 -> 11008        13.4 / 12.1           17.5 / 13.2          20.6 / 14.6
+//   11008 -> 4096        15.1 / 12.8           27.4 / 13.9          24.1 / 17.9
+//   5120 -> 13824        18.8 / 16.3           22.5 / 18.8          34.2 / 20.4
+//   13824 -> 5120        21.3 / 17.4           37.5 / 20.1          33.7 / 23.9
+//   1280 -> 3456          7.1 /  5.2           10.5 /  6.0          11.4 /  5.7
+// At one and two tokens the streaming kernel's integer form is ahead: 4096 -> 4096 rank 64 4.8 / 7.1 and 5.7 / 7.1.
+bool split_takes(const LinearArgs &a, int kernel)
+{
+    return g_opt.use_gemv && a.M > kGemvMaxM && split_supported(a) && (kernel == FBQ_KERNEL_DECODE || (kernel == FBQ_KERNEL_PREFILL && g_opt.force_kernel < 0));
+}
+
+// Several problems as one launch of the streaming or the split kernel on `s`; FBQ_ERR_UNSUPPORTED where they cannot share one.
+bool batch_plan_exists(const LinearArgs *a, int count, const GemvTuning &gt, size_t *slots, int *nc)
+{
+    if (gt.max_ctas > 0 || g_opt.decode_trace) return false;
+    return a[0].M > kGemvMaxM ? split_plan_exists(a, count, gt) : gemv_batch_need(a, count, gt, slots, nc);
+}
 int run_gemv_batch(const LinearArgs *a, int count, cudaStream_t s)
 {
     for (int i = 0; i < count; ++i)
@@ -237,7 +255,8 @@ int run_gemv_batch(const LinearArgs *a, int count, cudaStream_t s)
     gt.pdl = g_opt.decode.pdl;
     size_t slots = 0;
     int nc = 0, launches = 0;
-    if (gt.max_ctas > 0 || g_opt.decode_trace || !gemv_batch_need(a, count, gt, &slots, &nc)) return FBQ_ERR_UNSUPPORTED;
+    if (!batch_plan_exists(a, count, gt, &slots, &nc)) return FBQ_ERR_UNSUPPORTED;
+    if (a[0].M > kGemvMaxM) return run_split(a, count, gt, ws, s);
     size_t have_c = (size_t)ws->n_counters;
     cudaError_t e;
     if ((e = grow(ws->tslots, ws->tslots_floats, slots, sizeof(float), s)) != cudaSuccess) return grow_status(e);
@@ -264,17 +283,23 @@ int run_linear(const LinearArgs &a, cudaStream_t s, int decode_ctas = 0)
     int launches = 0;
     cudaError_t e = cudaSuccess;
 
-    if (kernel == FBQ_KERNEL_DECODE && g_opt.use_gemv && gemv_supported(a)) {
+    if (split_takes(a, kernel)) {
         GemvTuning gt = g_opt.gemv;
         gt.pdl = g_opt.decode.pdl;
         if (tune.max_ctas > 0) gt.max_ctas = tune.max_ctas;
         if (gt.max_ctas == 0) gt.max_ctas = ws->gemv_ctas;
-        size_t pf = 0, partf = 0;
+        if (split_plan_exists(&a, 1, gt)) return run_split(&a, 1, gt, ws, s);
+    }
+    if (kernel == FBQ_KERNEL_DECODE && g_opt.use_gemv && a.M <= kGemvMaxM && gemv_supported(a)) {
+        GemvTuning gt = g_opt.gemv;
+        gt.pdl = g_opt.decode.pdl;
+        if (tune.max_ctas > 0) gt.max_ctas = tune.max_ctas;
+        if (gt.max_ctas == 0) gt.max_ctas = ws->gemv_ctas;
+        size_t pf = 0;
         int nc = 0;
-        gemv_workspace_need(a, gt, &pf, &nc, &partf);
+        gemv_workspace_need(a, gt, &pf, &nc);
         size_t have_c = (size_t)ws->n_counters;
         if ((e = grow(ws->tslots, ws->tslots_floats, pf, sizeof(float), s)) != cudaSuccess) return grow_status(e);
-        if (partf > 0 && (e = grow(ws->partial, ws->partial_floats, partf, sizeof(float), s)) != cudaSuccess) return grow_status(e);
         if ((e = grow(ws->counters, have_c, (size_t)nc, sizeof(int), s)) != cudaSuccess) return grow_status(e);
         ws->n_counters = (int)have_c;
         if (g_opt.decode_trace && !ws->trace) {
@@ -675,7 +700,7 @@ static int host_batch(const LinearArgs *in, const fbq_problem *problems, int cou
         size_t slots = 0;
         int nc = 0;
         GemvTuning gt = g_opt.gemv;
-        if (gt.max_ctas > 0 || g_opt.decode_trace || !gemv_batch_need(a, count, gt, &slots, &nc)) return FBQ_ERR_UNSUPPORTED;
+        if (!batch_plan_exists(a, count, gt, &slots, &nc)) return FBQ_ERR_UNSUPPORTED;
     }
     if (copy_in(x.n, x.src, x.dst, x.bytes, s) != cudaSuccess) return FBQ_ERR_CUDA;
     const int rc = run_gemv_batch(a, count, s);
@@ -742,6 +767,24 @@ static int linear_batch_common(const fbq_problem *problems, int count, int M, in
         if (!ws || la.y != ws->stage_y) return FBQ_OK;      // written in place
         return cudaMemcpyAsync(y_host, la.y, (size_t)M * la.N * 2, cudaMemcpyDeviceToHost, st) == cudaSuccess ? FBQ_OK : FBQ_ERR_CUDA;
     };
+    // Problems that read the same x (q, k and v; gate and up) share one launch of the streaming kernel, or of the split kernel, on
+    // the caller's stream, and so do all problems of a call with host buffers, whose x arrive together.  (Seven linears of a 7B
+    // layer, INT3, one token, pinned buffers, 51 us with the synchronisation: x over the bus 5 us, the launch of all seven 34, of which y over the bus is 3.5,
+    // and about 12 until the first kernel starts and after the last has ended.)  Above two tokens a problem of a single 16-row
+    // tile goes by itself.
+    if (g_opt.batch_single && count > 1 && count <= kGemvBatchMost) {
+        bool together = true, one_x = true;
+        for (int i = 0; i < count; ++i) {
+            const int kernel = select_kernel(M, a[i].N, a[i].K, group, bits, rank, a[i].bf16);
+            together = together && (M > kGemvMaxM ? split_takes(a[i], kernel) && a[i].N > 16
+                                                  : kernel == FBQ_KERNEL_DECODE && g_opt.use_gemv && gemv_supported(a[i]));
+            one_x = one_x && a[i].x == a[0].x && a[i].K == a[0].K;
+        }
+        if (together && (one_x || host_io)) {
+            const int rc = host_io ? host_batch(a, problems, count, M, main) : run_gemv_batch(a, count, main);
+            if (rc != FBQ_ERR_UNSUPPORTED) return rc;
+        }
+    }
     if (!all_decode) {
         // One after the other on the caller's stream (prefill-sized problems fill the GPU by themselves).  x from host buffers
         // comes over at the start, shared x once, unless that takes much staging space: one by one each copy would wait for the linear
@@ -774,25 +817,8 @@ static int linear_batch_common(const fbq_problem *problems, int count, int M, in
     int ctas[FBQ_BATCH_MAX];
     for (int i = 0; i < count; ++i)
         ctas[i] = std::max(8, (int)(g_opt.batch_ctas * ((double)a[i].N * a[i].K / total_cost) + 0.5));
-    // Problems in the streaming kernel's domain share one launch of it where that is possible (next), else they run as one
-    // launch each on the side streams; problems outside it share a launch of the other decode kernel.
     bool all_gemv = g_opt.use_gemv != 0;
     for (int i = 0; i < count; ++i) all_gemv = all_gemv && gemv_supported(a[i]);
-    // Problems that read the same x (q, k and v; gate and up) share one launch of it on the caller's stream, and so do all
-    // problems of a call with host buffers, whose x arrive together.  (Seven linears of a 7B layer, INT3, one token, pinned
-    // buffers, 51 us with the synchronisation: x over the bus 5 us, the launch of all seven 34, of which y over the bus is 3.5,
-    // and about 12 until the first kernel starts and after the last has ended.)
-    if (all_gemv && g_opt.batch_single && count > 1 && count <= kGemvBatchMost) {
-        bool one_x = true;
-        for (int i = 1; i < count; ++i) one_x = one_x && a[i].x == a[0].x && a[i].K == a[0].K;
-        if (one_x && !host_io) {
-            const int rc = run_gemv_batch(a, count, main);
-            if (rc != FBQ_ERR_UNSUPPORTED) return rc;
-        } else if (host_io) {
-            const int rc = host_batch(a, problems, count, M, main);
-            if (rc != FBQ_ERR_UNSUPPORTED) return rc;
-        }
-    }
     if (g_opt.batch_single && !host_io && count <= decode_batch_max() && !all_gemv) {
         // One launch: the decode kernel over a problem list, on the caller's stream.  (With host
         // buffers these problems go to the streams below, where their small copies overlap.)
@@ -953,6 +979,7 @@ int fbq_poll_status(void *stream)
         if (ws->t) cudaMemset(ws->t, 0, sizeof(float) * ws->t_floats);
         if (ws->tslots) cudaMemset(ws->tslots, 0, sizeof(float) * ws->tslots_floats);
         if (ws->tags) cudaMemset(ws->tags, 0, sizeof(uint32_t) * ws->n_tags);
+        if (ws->split) cudaMemset(ws->split, 0, ws->split_bytes);
     }
     return st;
 }
@@ -982,6 +1009,7 @@ int fbq_release_workspaces(void)
         cudaFree(w.stage_y);
         cudaFree(w.w16);
         cudaFree(w.tags);
+        cudaFree(w.split);
         cudaFree(w.rec);
     }
     for (auto it = g_ws.begin(); it != g_ws.end();) {            // what is left of a stream are its options

@@ -46,6 +46,8 @@ struct Workspace {
     size_t w16_bytes = 0;
     uint32_t *tags = nullptr;     // its launch number and tags (starts at zero)
     size_t n_tags = 0;
+    void *split = nullptr;        // the split kernel's launch number and words of t, which carry it (starts at zero)
+    size_t split_bytes = 0;
     int gemv_ctas = 0;            // option of the stream (fbq_set_stream_option); outlives the buffers
     void *rec = nullptr;          // split operands of the Gram matrix and the reconstruction step (no invariant)
     size_t rec_bytes = 0;
@@ -97,7 +99,8 @@ cudaError_t launch_decode(const LinearArgs &a, Workspace &ws, const DecodeTuning
 void decode_workspace_need(const LinearArgs &a, const DecodeTuning &tune, size_t *partial_floats,
                            int *counters);
 
-// The streaming decode kernel (fbq_gemv.cu).
+// The streaming decode kernel (fbq_gemv.cu), one and two tokens.
+constexpr int kGemvMaxM = 2;
 struct GemvTuning {
     int max_ctas = 0;          // 0: one main CTA per SM
     int pdl = 1;
@@ -107,13 +110,21 @@ struct GemvTuning {
 };
 int gemv_k_slices(int M, int K);      // K slices the streaming decode kernel cuts a shape into (1: x of all K fits)
 bool gemv_supported(const LinearArgs &a);
-void gemv_workspace_need(const LinearArgs &a, const GemvTuning &tune, size_t *tpart_floats, int *counters, size_t *partial_floats);
+void gemv_workspace_need(const LinearArgs &a, const GemvTuning &tune, size_t *tpart_floats, int *counters);
 cudaError_t launch_gemv(const LinearArgs &a, Workspace &ws, const GemvTuning &tune, cudaStream_t s, int *launches);
 
 // Several problems of the streaming kernel in one launch: scratch, then launch.  false where they cannot share one (other
 // forms, plans that do not fit): then they are launched one by one.
 bool gemv_batch_need(const LinearArgs *a, int count, const GemvTuning &tune, size_t *tslots_floats, int *counters);
 cudaError_t launch_gemv_batch(const LinearArgs *a, int count, Workspace &ws, const GemvTuning &tune, cudaStream_t s, int *launches);
+
+// The split kernel (fbq_split.cu): the same domain of widths and ranks, up to kSplitMaxM tokens, one problem or several in
+// one launch (cudaErrorInvalidConfiguration: no plan fits).  Scratch: Workspace::split, the status word of the counters.
+constexpr int kSplitMaxM = 16;
+bool split_supported(const LinearArgs &a);
+size_t split_scratch_bytes(const LinearArgs *a, int count);
+bool split_plan_exists(const LinearArgs *a, int count, const GemvTuning &tune);
+cudaError_t launch_split(const LinearArgs *a, int count, Workspace &ws, const GemvTuning &tune, cudaStream_t s, int *launches);
 
 int decode_batch_max();
 bool decode_batch_need(const LinearArgs *a, int count, const int *ctas, const DecodeTuning &tune, size_t *partial_floats,

@@ -1,4 +1,4 @@
-// Streaming decode kernel (few tokens) of the FBQuant linear, sm_100a.
+// Streaming decode kernel (one and two tokens) of the FBQuant linear, sm_100a.
 //
 // One launch computes  y = x.dequant(Q,s,z)^T + (x.A^T).B^T  (Algorithm 1 step 6 of the paper;
 // Section 4.3 fuses dequantisation, main product and up-projection and leaves t = x.A^T to a second
@@ -14,7 +14,7 @@
 //   * The weight stream is one TMA tensor copy per stage (16 groups x 16 rows of packed codes) into
 //     an mbarrier ring; eight compute warps share every stage.
 //
-// Main CTAs (one per SM, or two: make_plan) own contiguous ranges of 16-row tiles.  Integer form (M <= 2):
+// Main CTAs (one per SM, or two: make_plan) own contiguous ranges of 16-row tiles.
 // a code masked out of its word is an unsigned byte operand of the 8-bit integer MMA as it stands
 // (four codes per register, at most one shift per word); x is fixed point per group of 128 (three
 // signed base-256 digits, exact integer sums), and scale and zero point are applied per group to the
@@ -79,18 +79,10 @@ struct GemvParams {
     int stage_bytes, meta_pitch, b_slot_bytes, b_box_cols, b_swz;
     int off_bar, off_tab, off_x, off_meta, off_seg, off_t, off_B, off_ring;
     int off_tA, off_tred;                   // t CTA: blocks of A, reduction buffer
-    // 16-bit form (M >= 3): K may be cut into SK slices (CTA = row block x slice) whose partial tiles meet in scratch
-    int SK, R;                              // n_main = R * SK
-    int slice_groups;                       // groups per K slice (a multiple of eight; the last slice takes the rest)
-    int chg;                                // groups of a stage: kCW or kGPW * kCW
-    int x_pitch;                            // elements between tokens of the staged x
-    int off_px, off_tf;                     // (P, X0) table; t as MMA column operands
-    int off_sub;                            // t.B^T of the tiles ahead (integer form)
-    float *part;                            // [tile][slice][M][16] fp32 partial tiles (SK > 1)
-    int *tctr;                              // [tile] slices that have stored their partial (zero on entry and exit)
+    int off_tf;                             // t as MMA column operands
+    int off_sub;                            // t.B^T of the tiles ahead
     int t_final;                            // 1: the t CTA that arrives last adds the slots into slot n_t, and the main CTAs read only that one
     uint32_t poll_limit;                    // looks at the arrival counter before giving up
-    int pair;                               // 16-bit form: CTAs come in clusters of two that stage half of x each
     int test_skip_arrive;                   // test switch: t CTAs do not report their arrival
     unsigned long long *trace;              // optional phase timestamps [cta][warp][16] (tuning aid), else NULL
 };
@@ -561,13 +553,11 @@ __device__ __forceinline__ bool compute_i8(const GemvParams &p, uint8_t *smem, i
 }
 
 // ------------------------------------------------------------------------ producer
-__device__ __forceinline__ bool produce(const GemvParams &p, uint8_t *smem, const CUtensorMap *wmap, int tile_first, int ntile,
-                                        int g_begin = 0, int g_count = -1, int chg = kCHG)
+__device__ __forceinline__ bool produce(const GemvParams &p, uint8_t *smem, const CUtensorMap *wmap, int tile_first, int ntile)
 {
     const uint32_t sbase = smem_u32(smem), bars = sbase + p.off_bar;
     const uint32_t ring = sbase + p.off_ring, meta0 = sbase + p.off_meta;
-    if (g_count < 0) g_count = p.G;
-    const int SPT = (g_count + chg - 1) / chg, NS = p.NS;
+    const int SPT = (p.G + kCHG - 1) / kCHG, NS = p.NS;
     int it = 0;
     for (int ts = 0; ts < ntile; ++ts) {
         const int tile = tile_first + ts;
@@ -582,7 +572,7 @@ __device__ __forceinline__ bool produce(const GemvParams &p, uint8_t *smem, cons
             const uint32_t full = bars + 8u * (kBarFull + slot);
             mbar_expect_tx(full, (uint32_t)p.stage_bytes + (st == 0 ? 2u * mbytes : 0u));
             // one box of 16 groups x 16 rows (rows past N and groups past G arrive as zeros)
-            tma_load_3d(ring + (uint32_t)slot * (uint32_t)p.stage_bytes, wmap, 0, tile * kTile, g_begin + st * chg, full);
+            tma_load_3d(ring + (uint32_t)slot * (uint32_t)p.stage_bytes, wmap, 0, tile * kTile, st * kCHG, full);
             if (it == 0) mark(p, 3);
             if (st == 0) {
                 const uint32_t ms = meta0 + (uint32_t)(ts % p.nmeta) * 2u * (uint32_t)p.meta_pitch;
@@ -881,555 +871,6 @@ __device__ __forceinline__ bool epilogue(const GemvParams &p, uint8_t *smem, con
 }
 
 
-// =============================================================== 16-bit form (3 <= M <= 16)
-// Codes become packed 16-bit floats with one LOP3 per pair ("bias-free" unpack): a field at bit p of a
-// 16-bit half, OR-ed into the mantissa of MAGIC = 1024 (fp16) or 128 (bf16), is MAGIC + 2^p q.  Nothing is
-// spent per element on removing MAGIC, 2^p or the zero point: x is staged divided by 2^p (exact) and
-// permuted into the order the unpacker produces, so the MMA yields sum x q + sum (MAGIC / 2^p) x; the second
-// sum (P) and sum x (X0) depend on token and group only and are tabulated when x is staged, and a group
-// contributes s (mma - P) - (s z) X0.
-//   INT4: h[4i+e]  = codes (8i+e , 8i+e+4)  of word i          (i = 0..3, e = 0..3)
-//   INT3: h[5i+f]  = codes (10i+f, 10i+5+f) of word i          (i = 0..2, f = 0..4);  h[15] = codes (30, 31)
-__device__ __forceinline__ uint32_t lop3_and_or(uint32_t a, uint32_t mask, uint32_t orv)
-{
-    uint32_t r;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(r) : "r"(a), "r"(mask), "r"(orv));   // (a & mask) | orv
-    return r;
-}
-template <int BITS, typename T> struct Unpack16;
-template <> struct Unpack16<4, __half> {
-    static constexpr float kMagic = 1024.f;
-    static __device__ __forceinline__ int div_log2(int c) { return ((c & 7) & 1) ? 4 : 0; }   // odd nibbles sit 4 bits up
-    static __device__ __forceinline__ void run(const uint32_t *w, uint32_t *h)
-    {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t a = w[i], b = w[i] >> 8;
-            h[4 * i + 0] = lop3_and_or(a, 0x000F000Fu, 0x64006400u);
-            h[4 * i + 1] = lop3_and_or(a, 0x00F000F0u, 0x64006400u);
-            h[4 * i + 2] = lop3_and_or(b, 0x000F000Fu, 0x64006400u);
-            h[4 * i + 3] = lop3_and_or(b, 0x00F000F0u, 0x64006400u);
-        }
-    }
-};
-template <> struct Unpack16<4, __nv_bfloat16> {
-    static constexpr float kMagic = 128.f;                     // 0x4300 | q is 128 + q in bf16 (7 mantissa bits)
-    static __device__ __forceinline__ int div_log2(int) { return 0; }
-    static __device__ __forceinline__ void run(const uint32_t *w, uint32_t *h)
-    {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) h[4 * i + e] = lop3_and_or(w[i] >> (4 * e), 0x000F000Fu, 0x43004300u);
-    }
-};
-template <> struct Unpack16<3, __half> {
-    static constexpr float kMagic = 1024.f;
-    static __device__ __forceinline__ int div_log2(int c)
-    {
-        if (c >= 30) return 0;
-        const int f = (c % 10) % 5;                             // fields 0,3: bit 0; 1,4: bit 3; 2: bit 6 (3,4 after >> 9)
-        return (f == 2) ? 6 : ((f == 1 || f == 4) ? 3 : 0);
-    }
-    static __device__ __forceinline__ void run(const uint32_t *w, uint32_t *h)
-    {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const uint32_t a = w[i], b = w[i] >> 9;
-            h[5 * i + 0] = lop3_and_or(a, 0x00070007u, 0x64006400u);
-            h[5 * i + 1] = lop3_and_or(a, 0x00380038u, 0x64006400u);
-            h[5 * i + 2] = lop3_and_or(a, 0x01C001C0u, 0x64006400u);
-            h[5 * i + 3] = lop3_and_or(b, 0x00070007u, 0x64006400u);
-            h[5 * i + 4] = lop3_and_or(b, 0x00380038u, 0x64006400u);
-        }
-        uint32_t l = lop3_and_or(w[0] >> 15, 0x00010001u, 0x64006400u);
-        l = lop3_and_or(w[1] >> 14, 0x00020002u, l);
-        h[15] = lop3_and_or(w[2] >> 13, 0x00040004u, l);
-    }
-};
-template <> struct Unpack16<3, __nv_bfloat16> {
-    static constexpr float kMagic = 128.f;
-    static __device__ __forceinline__ int div_log2(int c)
-    {
-        if (c >= 30) return 0;
-        const int f = (c % 10) % 5;                             // shifts 0, 6, 12: fields 0,2,4 at bit 0; 1,3 at bit 3
-        return (f == 1 || f == 3) ? 3 : 0;
-    }
-    static __device__ __forceinline__ void run(const uint32_t *w, uint32_t *h)
-    {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const uint32_t a = w[i], b = w[i] >> 6, c = w[i] >> 12;
-            h[5 * i + 0] = lop3_and_or(a, 0x00070007u, 0x43004300u);
-            h[5 * i + 1] = lop3_and_or(a, 0x00380038u, 0x43004300u);
-            h[5 * i + 2] = lop3_and_or(b, 0x00070007u, 0x43004300u);
-            h[5 * i + 3] = lop3_and_or(b, 0x00380038u, 0x43004300u);
-            h[5 * i + 4] = lop3_and_or(c, 0x00070007u, 0x43004300u);
-        }
-        uint32_t l = lop3_and_or(w[0] >> 15, 0x00010001u, 0x43004300u);
-        l = lop3_and_or(w[1] >> 14, 0x00020002u, l);
-        h[15] = lop3_and_or(w[2] >> 13, 0x00040004u, l);
-    }
-};
-// Position of code c (0..31) of a lane's 32-code run in that order: 2 * h_index + (0 = low half, 1 = high half).
-template <int BITS> __device__ __forceinline__ int frag_pos(int c)
-{
-    if (BITS == 4) {
-        const int i = c >> 3, e8 = c & 7;
-        return 2 * (4 * i + (e8 & 3)) + (e8 >> 2);
-    }
-    if (c >= 30) return 2 * 15 + (c - 30);
-    const int i = c / 10, f = c - 10 * i;
-    return (f < 5) ? 2 * (5 * i + f) : 2 * (5 * i + f - 5) + 1;
-}
-// Groups of a stage in the 16-bit form, per compute warp: two, or one where the shared memory is short (the plan says).  What
-// bounded long runs of tiles here was what a stage costs by itself (its request, its barriers; 0.4 us each with the
-// multiplications left out), not the bytes in flight (sixteen stages instead of eight: nothing).  One group per warp:
-// 4096 -> 44032 INT4 at eight tokens 45.6 us (2.0 TB/s), two: 30.9 (2.9); 4096 -> 11008 16.0 / 12.1.  Four gain another 7 %
-// on the longest launches, but then a long x and two stages no longer fit together.
-constexpr int kGPW = 2;
-
-// x of this CTA's K slice (groups g_begin .. g_begin + g_count) for M tokens: per token and group the sixteen
-// fragment-order pairs of a lane's run as 16-byte units [h_index / 4][lane t][h_index % 4]; (P, X0) per (group, token).
-template <int BITS, typename T, int MT>
-__device__ __forceinline__ void convert_x16(const GemvParams &p, uint8_t *smem, int g_begin, int g_count)
-{
-    const int tid = threadIdx.x, lane = tid & 31, nthr = kCW * 32;
-    T *s_x = reinterpret_cast<T *>(smem + p.off_x);
-    float2 *s_px = reinterpret_cast<float2 *>(smem + p.off_px);
-    const T *x = static_cast<const T *>(p.x);
-    // In a pair (cluster of two CTAs with the same x) this CTA converts every other group and stores the result into
-    // both CTAs' shared memory: every CTA of the grid reads all of x from L2 otherwise, which is what staging costs.
-    const int crank = p.pair ? (int)cluster_ctarank() : 0, cstep = p.pair ? 2 : 1;
-    const int my_groups = (g_count - crank + cstep - 1) / cstep;             // groups crank, crank + cstep, ...
-    const int runs_per_tok = my_groups * 4, nruns = p.M * runs_per_tok;      // multiples of 4
-    const uint32_t peer_x = p.pair ? mapa_shared(smem_u32(s_x), (uint32_t)(crank ^ 1)) : 0u;
-    const uint32_t peer_px = p.pair ? mapa_shared(smem_u32(s_px), (uint32_t)(crank ^ 1)) : 0u;
-    constexpr int mp = 8 * MT;                                               // token slots of the (P, X0) table
-    for (int i = tid; i < g_count * mp; i += nthr)                           // tokens beyond M contribute nothing
-        if (i % mp >= p.M) s_px[i] = make_float2(0.f, 0.f);
-    auto fetch = [&](int base, uint4 (&v)[4]) {
-        const int idx = base + tid;
-        const bool valid = idx < nruns;
-        const int m = valid ? idx / runs_per_tok : 0, mr = valid ? idx - m * runs_per_tok : 0;
-        const int run = ((mr >> 2) * cstep + crank) * 4 + (mr & 3);         // run of the slice: group, quarter
-        const uint4 *src = reinterpret_cast<const uint4 *>(x + (size_t)m * p.K + (size_t)g_begin * kGroupFast + run * 32);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = valid ? __ldcg(src + i) : make_uint4(0u, 0u, 0u, 0u);
-    };
-    uint4 xn[4];
-    fetch(0, xn);
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(smem) + p.off_bar + 8u * kBarXReq);   // our loads of x are on their way
-#pragma unroll 1
-    for (int base = 0; base < nruns; base += nthr) {
-        const int idx = base + tid;                                          // whole quads are valid or not
-        const bool valid = idx < nruns;
-        const int m = valid ? idx / runs_per_tok : 0, mr = valid ? idx - m * runs_per_tok : 0;
-        const int run = ((mr >> 2) * cstep + crank) * 4 + (mr & 3);
-        uint4 xv[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) xv[i] = xn[i];
-        if (base + nthr < nruns) fetch(base + nthr, xn);                     // the next batch's loads, before this batch's work
-        const uint16_t *e = reinterpret_cast<const uint16_t *>(xv);
-        uint32_t h[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) h[i] = 0u;
-        float psum = 0.f, xsum = 0.f;
-#pragma unroll
-        for (int c = 0; c < 32; ++c) {
-            const int pos = frag_pos<BITS>(c);                               // folds to a constant
-            T xe;
-            *reinterpret_cast<uint16_t *>(&xe) = e[c];
-            const float xf = ActTraits<T>::to_float(xe);
-            // exact division by the field weight (a power of two; up to fp16 underflow).  P is summed from the
-            // stored value, so the MMA's bias term cancels exactly.
-            const T xs = ActTraits<T>::from_float(xf * (1.f / (float)(1 << Unpack16<BITS, T>::div_log2(c))));
-            h[pos >> 1] |= (uint32_t)(*reinterpret_cast<const uint16_t *>(&xs)) << (16 * (pos & 1));
-            psum = fmaf(Unpack16<BITS, T>::kMagic, ActTraits<T>::to_float(xs), psum);
-            xsum += xf;
-        }
-        if (valid) {
-            const size_t eoff = (size_t)m * p.x_pitch + (run >> 2) * kGroupFast;    // elements into the staged x
-            uint4 *dst = reinterpret_cast<uint4 *>(s_x + eoff);
-#pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) {
-                const uint4 v = make_uint4(h[4 * q4], h[4 * q4 + 1], h[4 * q4 + 2], h[4 * q4 + 3]);
-                dst[q4 * 4 + (run & 3)] = v;
-                if (p.pair) st_cluster_v4(peer_x + (uint32_t)(eoff * 2) + (uint32_t)(q4 * 4 + (run & 3)) * 16u, v);
-            }
-        }
-        // the four runs of one (token, group) sit in four consecutive lanes
-        psum += __shfl_xor_sync(0xffffffffu, psum, 1);
-        xsum += __shfl_xor_sync(0xffffffffu, xsum, 1);
-        psum += __shfl_xor_sync(0xffffffffu, psum, 2);
-        xsum += __shfl_xor_sync(0xffffffffu, xsum, 2);
-        if (valid && (run & 3) == 0) {
-            s_px[(run >> 2) * mp + m] = make_float2(psum, xsum);
-            if (p.pair) st_cluster_f2(peer_px + (uint32_t)((run >> 2) * mp + m) * 8u, make_float2(psum, xsum));
-        }
-    }
-}
-
-// Compute warps of the 16-bit form: stages of sixteen groups, two per warp; MT blocks of eight tokens.
-template <int BITS, typename T, int MT>
-__device__ __forceinline__ bool compute_w16(const GemvParams &p, uint8_t *smem, int warp, int lane, int ntile, int g_begin, int g_count)
-{
-    constexpr int NW = (BITS == 4) ? 4 : 3;
-    constexpr int GB = (BITS == 4) ? 64 : 48;
-    const int g = lane >> 2, tq = lane & 3;
-    const uint32_t sbase = smem_u32(smem), bars = sbase + p.off_bar;
-    const int G = p.G, NS = p.NS, M = p.M, chg = p.chg, SPT = (g_count + chg - 1) / chg;
-    const uint32_t w_lane = sbase + p.off_ring + (uint32_t)(warp * (kTile * GB) + g * GB + tq * (GB / 4));
-    const uint32_t meta0 = sbase + p.off_meta, zoff = (uint32_t)p.meta_pitch, row8 = (uint32_t)(8 * G * 2);
-    const uint32_t px_lane = sbase + p.off_px + (uint32_t)(2 * tq) * 8u;
-    const uint32_t x_lane = sbase + p.off_x + (uint32_t)tq * 16u;
-    const uint32_t x_tok = (uint32_t)p.x_pitch * 2u;
-    float *s_seg = reinterpret_cast<float *>(smem + p.off_seg);
-    int slot = 0, mi = 0, buf = 0;
-    uint32_t par = 0u, dphase = 1u;
-    bool first = true, dfirst = true;
-    for (int ts = 0; ts < ntile; ++ts) {
-        float acc[MT][4];
-#pragma unroll
-        for (int b = 0; b < MT; ++b) acc[b][0] = acc[b][1] = acc[b][2] = acc[b][3] = 0.f;
-        const uint32_t mslot = meta0 + (uint32_t)mi * 2u * zoff + (uint32_t)(g * G * 2);
-        if (++mi == p.nmeta) mi = 0;
-        for (int st = 0; st < SPT; ++st) {
-            if (!mbar_wait(bars + 8u * (kBarFull + slot), par)) return false;
-            if (first) mark(p, 4);
-            first = false;
-#pragma unroll
-            for (int u = 0; u < kGPW; ++u) {
-                const int gl = st * chg + u * kCW + warp;              // group of the slice
-                if (u * kCW < chg && gl < g_count) {
-                    const uint32_t wa = w_lane + (uint32_t)slot * (uint32_t)p.stage_bytes + (uint32_t)(u * kCW * kTile * GB);
-                    uint32_t w0[NW], w1[NW];
-                    if constexpr (BITS == 4) {
-                        const uint4 va = lds_v4(wa), vb = lds_v4(wa + 8 * GB);
-                        w0[0] = va.x; w0[1] = va.y; w0[2] = va.z; w0[3] = va.w;
-                        w1[0] = vb.x; w1[1] = vb.y; w1[2] = vb.z; w1[3] = vb.w;
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < NW; ++i) {
-                            w0[i] = lds_u32(wa + 4 * i);
-                            w1[i] = lds_u32(wa + 8 * GB + 4 * i);
-                        }
-                    }
-                    const uint32_t ma = mslot + (uint32_t)(g_begin + gl) * 2u;
-                    const float sg = half_bits_to_float(lds_u16(ma)), zg = half_bits_to_float(lds_u16(ma + zoff));
-                    const float sh = half_bits_to_float(lds_u16(ma + row8)), zh = half_bits_to_float(lds_u16(ma + row8 + zoff));
-                    const float szg = sg * zg, szh = sh * zh;
-                    uint32_t ha[16], hb[16];
-                    Unpack16<BITS, T>::run(w0, ha);
-                    Unpack16<BITS, T>::run(w1, hb);
-#pragma unroll
-                    for (int b = 0; b < MT; ++b) {
-                        // (P, X0) of tokens 8b + 2tq and 8b + 2tq + 1 for this group; one MMA chain starts at -P
-                        const float4 px = lds_f4(px_lane + (uint32_t)(gl * 8 * MT + 8 * b) * 8u);
-                        float t0[4] = {-px.x, -px.z, -px.x, -px.z}, t1[4] = {0.f, 0.f, 0.f, 0.f};
-                        const int token = 8 * b + g;                        // as an MMA column
-                        const uint32_t xg = x_lane + (uint32_t)token * x_tok + (uint32_t)gl * (kGroupFast * 2);
-                        const uint32_t on = token < M ? 1u : 0u;
-#pragma unroll
-                        for (int q4 = 0; q4 < 4; ++q4) {
-                            const uint4 xv = lds_v4_if(xg + (uint32_t)q4 * 64u, on);
-                            if (q4 & 1) {
-                                Mma16<T>::run(t1, ha[4 * q4 + 0], hb[4 * q4 + 0], ha[4 * q4 + 1], hb[4 * q4 + 1], xv.x, xv.y);
-                                Mma16<T>::run(t1, ha[4 * q4 + 2], hb[4 * q4 + 2], ha[4 * q4 + 3], hb[4 * q4 + 3], xv.z, xv.w);
-                            } else {
-                                Mma16<T>::run(t0, ha[4 * q4 + 0], hb[4 * q4 + 0], ha[4 * q4 + 1], hb[4 * q4 + 1], xv.x, xv.y);
-                                Mma16<T>::run(t0, ha[4 * q4 + 2], hb[4 * q4 + 2], ha[4 * q4 + 3], hb[4 * q4 + 3], xv.z, xv.w);
-                            }
-                        }
-                        // s (mma - P) - (s z) X0
-                        acc[b][0] = fmaf(-szg, px.y, fmaf(sg, t0[0] + t1[0], acc[b][0]));
-                        acc[b][1] = fmaf(-szg, px.w, fmaf(sg, t0[1] + t1[1], acc[b][1]));
-                        acc[b][2] = fmaf(-szh, px.y, fmaf(sh, t0[2] + t1[2], acc[b][2]));
-                        acc[b][3] = fmaf(-szh, px.w, fmaf(sh, t0[3] + t1[3], acc[b][3]));
-                    }
-                }
-            }
-            __syncwarp();
-            mbar_arrive_if(bars + 8u * (kBarEmpty + slot), lane == 0);
-            if (++slot == NS) {
-                slot = 0;
-                par ^= 1u;
-            }
-        }
-        // ---- this warp's partial tile [token][16 rows] for the epilogue warp ----
-        if (!dfirst && !mbar_wait(bars + 8u * (kBarSegFree + buf), dphase)) return false;
-        float *dst = s_seg + (size_t)(buf * kCW + warp) * M * kTile;
-#pragma unroll
-        for (int b = 0; b < MT; ++b) {
-            const int t0 = 8 * b + 2 * tq;
-            if (t0 < M) {
-                dst[t0 * kTile + g] = acc[b][0];
-                dst[t0 * kTile + g + 8] = acc[b][2];
-            }
-            if (t0 + 1 < M) {
-                dst[(t0 + 1) * kTile + g] = acc[b][1];
-                dst[(t0 + 1) * kTile + g + 8] = acc[b][3];
-            }
-        }
-        __syncwarp();
-        mbar_arrive_if(bars + 8u * (kBarSegFull + buf), lane == 0);
-        mark(p, ts == 0 ? 5 : 6);
-        if (++buf == p.nbuf) {
-            buf = 0;
-            dphase = dfirst ? 0u : dphase ^ 1u;
-            dfirst = false;
-        }
-    }
-    return true;
-}
-
-// Epilogue warp of the 16-bit form.  Lane (g, tq) finishes rows g and g + 8 of the tile for the tokens 4cb + tq
-// (cb = column block of the up-projection MMA, whose columns 2tq, 2tq + 1 are that token's two 16-bit terms).
-// With K slices the tile's partial sums meet in scratch and the slice that arrives last finishes the tile.
-template <typename T, int MT>
-__device__ __forceinline__ bool epilogue_wide(const GemvParams &p, uint8_t *smem, const CUtensorMap *bmap, int lane, int tile_first,
-                                              int ntile, int slice, int cta)
-{
-    const int g = lane >> 2, tq = lane & 3;
-    const uint32_t sbase = smem_u32(smem), bars = sbase + p.off_bar;
-    const uint32_t bring = sbase + p.off_B;
-    const int rank = p.rank, M = p.M, nkb = rank / 16, nkb4 = (nkb + 3) & ~3, SK = p.SK;
-    constexpr int NCB = 2 * MT;                                           // column blocks of four tokens
-    const int nbox = (rank + 63) / 64;
-    const uint32_t box_bytes = (uint32_t)kTile * (uint32_t)p.b_box_cols * 2u;
-    auto request_b = [&](int ts) {
-        const uint32_t bar = bars + 8u * (kBarB + ts % p.nb);
-        mbar_expect_tx(bar, (uint32_t)nbox * box_bytes);
-        for (int b = 0; b < nbox; ++b)
-            tma_load_2d(bring + (uint32_t)(ts % p.nb) * (uint32_t)p.b_slot_bytes + (uint32_t)b * box_bytes, bmap, b * 64,
-                        (tile_first + ts) * kTile, bar);
-    };
-    if (rank > 0 && lane == 0)
-        for (int ts = 0; ts < min(ntile, p.nb); ++ts) request_b(ts);   // rows of B are weights: before the wait
-
-    prefetch_x(p, cta, lane, (int)sizeof(T));
-    uint32_t *s_tf = reinterpret_cast<uint32_t *>(smem + p.off_tf);      // [cb][kb][lane][2]
-    for (int i = lane; i < NCB * nkb4 * 16; i += 32) reinterpret_cast<uint4 *>(s_tf)[i] = make_uint4(0u, 0u, 0u, 0u);
-    __syncwarp();
-    pdl_wait();
-    mark(p, 2);
-
-    float isc = 1.f;
-    if (rank > 0) {
-        float *s_t = reinterpret_cast<float *>(smem + p.off_t);
-        float amax = 0.f;
-        const size_t slot_elems = (size_t)p.slot_elems;
-        const int s_first = p.t_final ? p.n_t : 0, s_end = p.t_final ? p.n_t + 1 : p.n_t;
-        bool ok = false;
-        for (uint32_t look = 0; look < p.poll_limit && !ok; ++look) {
-            bool all = true;
-            amax = 0.f;
-            if (s_end - s_first > 1) {
-                all = look_slots(p.tpart, slot_elems, s_first, s_end, M * rank, lane, s_t, amax);
-            } else {
-                const uint4 *slot = reinterpret_cast<const uint4 *>(p.tpart + (size_t)s_first * slot_elems);
-                for (int q0 = 0; 4 * q0 < M * rank; q0 += 32 * 8) {  // one slot: eight times four entries per lane in flight
-                    uint4 part[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int q = q0 + u * 32 + lane;
-                        part[u] = (4 * q < M * rank) ? __ldcg(slot + q) : make_uint4(kTNone, kTNone, kTNone, kTNone);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int q = q0 + u * 32 + lane;
-                        all = all && t_min(0xFFFFFFFFu, part[u]) != 0u;
-                        if (4 * q < M * rank) {
-                            const float4 v = make_float4(__uint_as_float(part[u].x), __uint_as_float(part[u].y), __uint_as_float(part[u].z),
-                                                         __uint_as_float(part[u].w));
-                            *reinterpret_cast<float4 *>(s_t + 4 * q) = v;
-                            amax = fmaxf(amax, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-                        }
-                    }
-                }
-            }
-            ok = __all_sync(0xffffffffu, all);
-            if (!ok && look > 256) __nanosleep(64);
-        }
-        if (!ok) return false;
-        // tell that this CTA has read t (nobody waits for the add; a t CTA clears up once all have told)
-        if (lane == 0) atomicAdd(p.ctr + 1, 1);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        __syncwarp();
-        const uint32_t ex = min(max(__float_as_uint(amax) >> 23, 1u), 254u);
-        const uint32_t sb = min(max(268u - ex, 1u), 254u);
-        const float sc = __uint_as_float(sb << 23);
-        isc = __uint_as_float((254u - sb) << 23);
-        // t as MMA column operands [column block of four tokens][rank block][lane][2]: column 2 (tok % 4) holds the
-        // rounded values of token tok, the next column what the rounding left; a lane takes pairs of consecutive rank
-        // indices and forms both terms once; the columns of tokens beyond M were set to zero before the wait.
-        const int half_rank = rank >> 1;
-        for (int idx = lane; idx < M * half_rank; idx += 32) {
-            const int tok = idx / half_rank, k0 = 2 * (idx - tok * half_rank);
-            const float2 tv = *reinterpret_cast<const float2 *>(s_t + tok * rank + k0);
-            const float v0 = tv.x * sc, v1 = tv.y * sc;
-            const T h0 = ActTraits<T>::from_float(v0), h1 = ActTraits<T>::from_float(v1);
-            const T l0 = ActTraits<T>::from_float(v0 - ActTraits<T>::to_float(h0));
-            const T l1 = ActTraits<T>::from_float(v1 - ActTraits<T>::to_float(h1));
-            const uint32_t pk_hi = (uint32_t)(*reinterpret_cast<const uint16_t *>(&h0)) | ((uint32_t)(*reinterpret_cast<const uint16_t *>(&h1)) << 16);
-            const uint32_t pk_lo = (uint32_t)(*reinterpret_cast<const uint16_t *>(&l0)) | ((uint32_t)(*reinterpret_cast<const uint16_t *>(&l1)) << 16);
-            const int cb = tok >> 2, kb = k0 >> 4, h = (k0 >> 3) & 1, q = (k0 & 7) >> 1;
-            uint32_t *dst = s_tf + ((size_t)(cb * nkb4 + kb) * 32 + (2 * (tok & 3)) * 4 + q) * 2 + h;
-            dst[0] = pk_hi;
-            dst[8] = pk_lo;                                     // four lanes on: the remainder's column
-        }
-        __syncwarp();
-    }
-    mark(p, 3);
-
-    const float *s_seg = reinterpret_cast<const float *>(smem + p.off_seg);
-    T *y = static_cast<T *>(p.y);
-    const uint32_t smask = (uint32_t)p.b_swz, pitch = (uint32_t)p.b_box_cols * 2u;
-    const uint32_t tf_lane = sbase + p.off_tf + (uint32_t)lane * 8u;
-    // adds t.B^T (rows of B from slot ts % nb) to the sums of a tile and stores its rows of y
-    auto finish_tile = [&](int ts, float (&vg)[NCB], float (&vh)[NCB]) -> bool {
-        const int tile = tile_first + ts;
-        if (rank > 0) {
-            const int bs = ts % p.nb;
-            if (!mbar_wait(bars + 8u * (kBarB + bs), (uint32_t)(ts / p.nb) & 1u)) return false;
-            const uint32_t bt = bring + (uint32_t)bs * (uint32_t)p.b_slot_bytes;
-            // Branch-free over blocks of 64 rank indices (what lies past the rank is zero in t) and over all column blocks, two
-            // sums per block: with a branch per MMA and one chain this was 1.4 us of a tile's 1.5, more than its main sums.
-            float d[NCB][2][4];
-#pragma unroll
-            for (int cb = 0; cb < NCB; ++cb)
-#pragma unroll
-                for (int i = 0; i < 8; ++i) d[cb][i >> 2][i & 3] = 0.f;
-#pragma unroll 1
-            for (int kc = 0; 4 * kc < nkb; ++kc) {
-                uint32_t af[4][4];
-                uint2 tf[NCB][4];
-                const uint32_t bx = bt + (uint32_t)kc * box_bytes;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint32_t c0 = (uint32_t)(q * 32 + tq * 4);                  // bytes into the row
-                    const uint32_t o0 = (uint32_t)g * pitch + c0, o1 = o0 + 8u * pitch;
-                    const uint32_t on = 4 * kc + q < nkb ? 1u : 0u;                    // (stale bytes of the slot may be anything)
-                    af[q][0] = lds_u32_if(bx + swz(o0, smask), on);
-                    af[q][1] = lds_u32_if(bx + swz(o1, smask), on);
-                    af[q][2] = lds_u32_if(bx + swz(o0 + 16u, smask), on);
-                    af[q][3] = lds_u32_if(bx + swz(o1 + 16u, smask), on);
-                }
-#pragma unroll
-                for (int cb = 0; cb < NCB; ++cb)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) tf[cb][q] = lds_v2(tf_lane + (uint32_t)((cb * nkb4 + 4 * kc + q) * 32) * 8u);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int cb = 0; cb < NCB; ++cb)
-                        Mma16<T>::run(d[cb][q & 1], af[q][0], af[q][1], af[q][2], af[q][3], tf[cb][q].x, tf[cb][q].y);
-            }
-#pragma unroll
-            for (int cb = 0; cb < NCB; ++cb) {
-                vg[cb] = fmaf((d[cb][0][0] + d[cb][1][0]) + (d[cb][0][1] + d[cb][1][1]), isc, vg[cb]);
-                vh[cb] = fmaf((d[cb][0][2] + d[cb][1][2]) + (d[cb][0][3] + d[cb][1][3]), isc, vh[cb]);
-            }
-        }
-        const int n = tile * kTile + g;
-#pragma unroll
-        for (int cb = 0; cb < NCB; ++cb) {
-            const int tok = 4 * cb + tq;
-            if (tok < M) {
-                if (n < p.N) y[(size_t)tok * p.N + n] = ActTraits<T>::from_float(vg[cb]);
-                if (n + 8 < p.N) y[(size_t)tok * p.N + n + 8] = ActTraits<T>::from_float(vh[cb]);
-            }
-        }
-        return true;
-    };
-    // B slot of tile ts is free (used or not needed): request the rows of a later tile into it
-    auto release_b = [&](int ts) -> bool {
-        if (rank == 0) return true;
-        // a slice that does not finish the tile never reads its rows of B, but their copy must have landed
-        // before the slot is handed out again
-        if (!mbar_wait(bars + 8u * (kBarB + ts % p.nb), (uint32_t)(ts / p.nb) & 1u)) return false;
-        __syncwarp();
-        if (lane == 0 && ts + p.nb < ntile) request_b(ts + p.nb);
-        return true;
-    };
-    // With K slices: whether the tile is ours to finish shows in the arrival count, which is looked at one tile
-    // later so that the round trip of its atomic overlaps the next tile's sums.
-    int pend_ts = -1, pend_old = 0;
-    auto settle = [&](void) -> bool {
-        if (pend_ts < 0) return true;
-        const int last = __shfl_sync(0xffffffffu, pend_old, 0) == SK - 1;
-        if (last) {
-            const int tile = tile_first + pend_ts;
-            const float *pt = p.part + ((size_t)tile * SK) * M * kTile;
-            __threadfence();
-            float vg[NCB], vh[NCB];
-#pragma unroll
-            for (int cb = 0; cb < NCB; ++cb) {
-                const int tok = 4 * cb + tq;
-                vg[cb] = vh[cb] = 0.f;
-                if (tok < M)
-                    for (int s2 = 0; s2 < SK; ++s2) {                   // slices added in order, whoever finishes
-                        vg[cb] += __ldcg(pt + ((size_t)s2 * M + tok) * kTile + g);
-                        vh[cb] += __ldcg(pt + ((size_t)s2 * M + tok) * kTile + g + 8);
-                    }
-            }
-            if (lane == 0) atomicExch(p.tctr + tile, 0);
-            if (!finish_tile(pend_ts, vg, vh)) return false;
-        }
-        if (!release_b(pend_ts)) return false;
-        pend_ts = -1;
-        return true;
-    };
-    for (int ts = 0; ts < ntile; ++ts) {
-        const int buf = ts % p.nbuf, tile = tile_first + ts;
-        if (!mbar_wait_idle_warp(bars + 8u * (kBarSegFull + buf), (uint32_t)(ts / p.nbuf) & 1u)) return false;
-        if (ts == 0) mark(p, 4);
-        float vg[NCB], vh[NCB];
-#pragma unroll
-        for (int cb = 0; cb < NCB; ++cb) {
-            vg[cb] = vh[cb] = 0.f;
-            const int tok = 4 * cb + tq;
-            if (tok < M) {
-                const float *src = s_seg + ((size_t)buf * kCW * M + tok) * kTile;
-#pragma unroll
-                for (int w = 0; w < kCW; ++w) {
-                    vg[cb] += src[(size_t)w * M * kTile + g];
-                    vh[cb] += src[(size_t)w * M * kTile + g + 8];
-                }
-            }
-        }
-        __syncwarp();
-        mbar_arrive_if(bars + 8u * (kBarSegFree + buf), lane == 0);
-        if (SK > 1) {
-            // this slice's partial tile to scratch, then count in
-            float *pt = p.part + ((size_t)tile * SK) * M * kTile;
-#pragma unroll
-            for (int cb = 0; cb < NCB; ++cb) {
-                const int tok = 4 * cb + tq;
-                if (tok < M) {
-                    __stcg(pt + ((size_t)slice * M + tok) * kTile + g, vg[cb]);
-                    __stcg(pt + ((size_t)slice * M + tok) * kTile + g + 8, vh[cb]);
-                }
-            }
-            __threadfence();
-            __syncwarp();
-            int old = 0;
-            if (lane == 0) old = atomicAdd(p.tctr + tile, 1);
-            if (!settle()) return false;                                 // the tile before this one
-            pend_ts = ts;
-            pend_old = old;
-        } else {
-            if (!finish_tile(ts, vg, vh)) return false;
-            if (!release_b(ts)) return false;
-        }
-        mark(p, ts == 0 ? 5 : 6);
-    }
-    if (!settle()) return false;
-    return true;
-}
-
 // ------------------------------------------------------------------------ t CTA
 // Block c of the first n_t: t_kb blocks of 64 input channels of all `rank` rows of A in shared memory
 // (TMA, 128-byte swizzle), against the same channels of x read straight from global memory as MMA
@@ -1679,76 +1120,7 @@ gemv_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap,
     gemv_body<BITS, T, M, RANKED>(p, &wmap, &bmap, &amap, (int)blockIdx.x);
 }
 
-// The 16-bit form: main CTA `cta` is row block cta / SK, K slice cta % SK.
-template <int BITS, typename T, int MT>
-__device__ __forceinline__ void gemv_wide_body(const GemvParams &p, const CUtensorMap *wmap, const CUtensorMap *bmap, const CUtensorMap *amap, int block)
-{
-    extern __shared__ __align__(128) uint8_t smem_raw[];
-    uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    pdl_launch_dependents();
-    mark(p, 0);
-    if (block < p.n_t) {
-        if (p.pair) cluster_arrive();                // the cluster's barrier counts every thread; nobody here waits on it
-        t_cta<T>(p, smem, amap, block);
-        return;
-    }
-    const int cta = block - p.n_t;
-    const int rb = cta / p.SK, slice = cta - rb * p.SK;
-    const int tile_first = (int)((long long)rb * p.NT / p.R);
-    const int ntile = (int)((long long)(rb + 1) * p.NT / p.R) - tile_first;
-    const int g_begin = slice * p.slice_groups, g_count = min(p.slice_groups, p.G - g_begin);
-    const uint32_t bars = smem_u32(smem) + p.off_bar;
-    if (tid == 0) {
-        prefetch_tensormap(wmap);
-        if (p.rank > 0) prefetch_tensormap(bmap);
-        for (int i = 0; i < p.NS; ++i) {
-            mbar_init(bars + 8u * (kBarFull + i), 1);
-            mbar_init(bars + 8u * (kBarEmpty + i), kCW);
-        }
-        for (int i = 0; i < p.nbuf; ++i) {
-            mbar_init(bars + 8u * (kBarSegFull + i), kCW);
-            mbar_init(bars + 8u * (kBarSegFree + i), 1);
-        }
-        for (int i = 0; i < p.nb; ++i) mbar_init(bars + 8u * (kBarB + i), 1);
-        mbar_init(bars + 8u * kBarXReq, kCW);
-        fence_barrier_init();
-    }
-    __syncthreads();
-    mark(p, 1);
-    bool ok = true;
-    if (warp == kProdWarp) {
-        if (p.pair) cluster_arrive();
-        if (lane == 0) ok = produce(p, smem, wmap, tile_first, ntile, g_begin, g_count, p.chg);
-    } else if (warp == kEpiWarp) {
-        if (p.pair) cluster_arrive();
-        ok = epilogue_wide<T, MT>(p, smem, bmap, lane, tile_first, ntile, slice, cta);
-    } else {
-        pdl_wait();                                  // x may come from the preceding kernel
-        mark(p, 2);
-        convert_x16<BITS, T, MT>(p, smem, g_begin, g_count);
-        if (p.pair) {                                // both CTAs' halves of x are in both CTAs' shared memory
-            cluster_arrive();
-            cluster_wait();
-        } else {
-            named_barrier_sync(1, kCW * 32);
-        }
-        mark(p, 3);
-        ok = compute_w16<BITS, T, MT>(p, smem, warp, lane, ntile, g_begin, g_count);
-    }
-    if (!ok && lane == 0) give_up(p);
-}
-template <int BITS, typename T, int MT>
-__global__ void __launch_bounds__(kThreads, 1)
-gemv_wide_kernel(const GemvParams p, const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap bmap,
-                 const __grid_constant__ CUtensorMap amap)
-{
-    gemv_wide_body<BITS, T, MT>(p, &wmap, &bmap, &amap, (int)blockIdx.x);
-}
-
-// Several problems of one form in one launch: the t CTAs of all of them, then their main CTAs.  A block runs the program
-// of its problem with that problem's scratch, counters and plan; nothing synchronises across problems.  What a launch costs
-// besides its weights (the wait for the kernel before, reading and converting x, the last tile's finish) is paid once.
+// Several problems in one launch: t CTAs of all of them, then the main CTAs.
 struct GemvBatch {
     int n, n_t;                          // problems, t CTAs of all
     int first_t[kGemvBatchMax], first_main[kGemvBatchMax];
@@ -1771,15 +1143,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) gemv_batch_kernel(const 
     const int i = batch_problem(g, block);
     gemv_body<BITS, T, M, RANKED>(g.p[i], g.w + i, g.b + i, g.a + i, block);
 }
-template <int BITS, typename T, int MT>
-__global__ void __launch_bounds__(kThreads, 1) gemv_wide_batch_kernel(const __grid_constant__ GemvBatch g)
-{
-    int block = (int)blockIdx.x;
-    const int i = batch_problem(g, block);
-    gemv_wide_body<BITS, T, MT>(g.p[i], g.w + i, g.b + i, g.a + i, block);
-}
-
-// ------------------------------------------------------------------ host side
 template <typename X> struct TypeTag { using type = X; };
 
 struct Plan {
@@ -1934,136 +1297,8 @@ Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
     return make_plan_on(a, tune, 1);
 }
 
-// Groups per K slice of the 16-bit form (a multiple of eight: the compute warps then have equally many): the smallest
-// power-of-two count of slices whose part of x (16-bit, all tokens) stays within `x_limit` bytes of shared memory.
-constexpr size_t kXLimit = 136 * 1024;           // leaves every shape of the domain room for its stages
-constexpr size_t kXLimitWide = 184 * 1024;       // leaves room only with few tokens or a small rank: tried first
-int wide_slice_groups(int M, int G, size_t x_limit)
-{
-    int sk = 1;
-    auto slice_of = [&](int k) { return ((G + k - 1) / k + kCW - 1) / kCW * kCW; };
-    while (sk < 16 && (size_t)M * ((size_t)slice_of(sk) * kGroupFast + 32) * 2 > x_limit) sk *= 2;
-    return slice_of(sk);
-}
-
-// Plan of the 16-bit form (3 <= M <= 16): one CTA per SM; K in SK slices when x of all K does not fit.
-Plan make_plan_wide_on(const LinearArgs &a, const GemvTuning &tune, size_t x_limit, int chg)
-{
-    Plan pl{};
-    pl.ok = false;
-    if (g_sm_count == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) return pl;
-        if (cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return pl;
-    }
-    GemvParams &p = pl.p;
-    const int GB = (a.bits == 4) ? 64 : 48, G = a.K / kGroupFast, MT = (a.M + 7) / 8;
-    p.M = a.M; p.N = a.N; p.K = a.K; p.G = G; p.rank = a.rank;
-    p.NT = (a.N + kTile - 1) / kTile;
-    const int want = tune.max_ctas > 0 ? tune.max_ctas : g_sm_count;
-    p.chg = chg;
-    p.stage_bytes = kTile * chg * GB;
-    p.meta_pitch = (int)align_up((size_t)kTile * G * 2, 16);
-    p.n_t = 0;
-    p.t_kb = 0;
-    const int nblk = (a.K + kTKB - 1) / kTKB;
-    if (a.rank > 0) {
-        const int per = std::min(kCW, std::max(1, (int)((128 * 1024) / ((size_t)a.rank * 128))));     // one block per warp
-        p.n_t = std::min(64, std::max((nblk + per - 1) / per, std::min(nblk, 8)));
-        // (in a batch every CTA has an SM to itself, so as few t CTAs as fit)
-        p.n_t = tune.main_ctas > 0 ? std::max((nblk + 2 * kCW - 1) / (2 * kCW), (int)(((size_t)nblk * a.rank * 128 + 192 * 1024 - 1) / (192 * 1024)))
-                                   : balanced_t_ctas(p.n_t, nblk, a.rank, p.NT, want);
-        p.t_kb = (nblk + p.n_t - 1) / p.n_t;
-        p.n_t = (nblk + p.t_kb - 1) / p.t_kb;
-    }
-    p.slice_groups = wide_slice_groups(a.M, G, x_limit);
-    p.SK = (G + p.slice_groups - 1) / p.slice_groups;
-    p.x_pitch = p.slice_groups * kGroupFast + 32;
-    // One K slice: the main CTAs all stage the same x, so they come in clusters of two that stage half of it each (an
-    // even number of t CTAs, the odd one out idle, and of main CTAs keeps the clusters among their own kind).
-    p.pair = (p.SK == 1 && p.NT >= 2 && want >= 4) ? 1 : 0;
-    if (p.pair && (p.n_t & 1)) ++p.n_t;
-    p.R = std::max(1, std::min((tune.main_ctas > 0 ? tune.main_ctas : std::max(want - p.n_t, want / 2)) / p.SK, p.NT));
-    if (p.pair && (p.R & 1)) --p.R;
-    p.n_main = p.R * p.SK;
-    const int nseg = (p.NT + p.R - 1) / p.R;
-    // stages per tile of the shortest slice (the last one): the producer runs at most NS stages ahead, that is
-    // NS / SPT tiles, and every tile ahead holds a slot of scales and zero points
-    const int last_groups = G - (p.SK - 1) * p.slice_groups;
-    const int SPT = (std::min(p.slice_groups, last_groups) + chg - 1) / chg;
-    p.b_box_cols = a.rank <= 16 ? 16 : (a.rank <= 32 ? 32 : 64);
-    p.b_swz = p.b_box_cols >= 64 ? 7 : (p.b_box_cols >= 32 ? 3 : 1);
-    p.b_slot_bytes = (int)align_up((size_t)((a.rank + 63) / 64) * kTile * p.b_box_cols * 2, 1024);
-    p.nbuf = std::min(kMaxBuf, std::max(2, std::min(nseg, 3)));
-    p.nb = a.rank > 0 ? std::min(kMaxB, std::max(1, std::min(nseg, 2))) : 0;
-    const int ncb = 2 * MT, nkb4 = (a.rank / 16 + 3) / 4 * 4;
-    auto layout = [&](int ns) {
-        p.NS = ns;
-        p.nmeta = std::min(kMaxMeta, (ns - 1) / SPT + 2);
-        size_t off = 0;
-        p.off_bar = (int)off;
-        off += (size_t)kNumBars * 8;
-        off = align_up(off, 16);
-        p.off_px = (int)off;
-        off += (size_t)p.slice_groups * 8 * MT * 8;
-        off = align_up(off, 128);
-        p.off_x = (int)off;
-        off += (size_t)a.M * p.x_pitch * 2;
-        off = align_up(off, 128);
-        p.off_meta = (int)off;
-        off += (size_t)p.nmeta * 2 * p.meta_pitch;
-        off = align_up(off, 128);
-        p.off_seg = (int)off;
-        off += (size_t)p.nbuf * kCW * a.M * kTile * 4;
-        off = align_up(off, 128);
-        p.off_t = (int)off;
-        off += (size_t)a.M * a.rank * 4;
-        off = align_up(off, 16);
-        p.off_tf = (int)off;
-        off += (size_t)ncb * nkb4 * 32 * 8;
-        off = align_up(off, 1024);
-        p.off_B = (int)off;
-        off += (size_t)p.nb * p.b_slot_bytes;
-        off = align_up(off, 1024);
-        p.off_ring = (int)off;
-        off += (size_t)ns * p.stage_bytes;
-        return off;
-    };
-    int ns = std::min(kMaxNS, (kMaxMeta - 2) * SPT + 1);
-    while (ns > 2 && layout(ns) > kSmemMax - 2048) --ns;
-    const size_t need = layout(ns);
-    if (need > kSmemMax - 2048) return pl;
-    p.off_tab = 0;
-    p.slot_elems = (a.M * a.rank + 31) / 32 * 32;
-    p.t_final = (p.n_t * a.M * a.rank > 2048) ? 1 : 0;
-    p.off_tA = 1024;
-    p.off_tred = p.off_tA + p.t_kb * a.rank * 128;
-    const size_t need_t = a.rank > 0 ? (size_t)p.off_tred + (size_t)kCW * a.rank * 8 * 4 : 0;
-    if (need_t > kSmemMax - 2048) return pl;
-    pl.smem = std::max(need, need_t) + 1024;
-    p.poll_limit = tune.poll_limit > 0 ? (uint32_t)tune.poll_limit : (1u << 20);
-    p.test_skip_arrive = tune.test_skip_arrive;
-    pl.ok = true;
-    if (print_plans())
-        fprintf(stderr, "gemv wide plan M %d N %d K %d r %d: R %d SK %d (slice %d groups, stage %d) n_t %d NS %d nmeta %d nbuf %d nb %d smem %zu (t CTA %zu)\n",
-                a.M, a.N, a.K, a.rank, p.R, p.SK, p.slice_groups, p.chg, p.n_t, p.NS, p.nmeta, p.nbuf, p.nb, need, need_t);
-    return pl;
-}
-
-// Whole K with three stages of sixteen groups, else whole K with stages of eight, else slices.  A slice's partial tiles go
-// through scratch and a counter per tile, which costs more than a shallow ring: 11008 -> 4096 INT4, two slices / whole K:
-// seven tokens rank 64 28.6 / 20.9 us, eight tokens rank 0 25.9 / 22.3; 13824 -> 5120 rank 64, five tokens 38.4 / 30.0, six
-// 40.0 / 33.7.  (Which kernel a call gets does not depend on this: gemv_k_slices counts with kXLimit.)
-Plan make_plan_wide(const LinearArgs &a, const GemvTuning &tune)
-{
-    Plan pl = make_plan_wide_on(a, tune, kXLimitWide, kGPW * kCW);
-    if (pl.ok && pl.p.NS >= 3) return pl;
-    pl = make_plan_wide_on(a, tune, kXLimitWide, kCW);
-    if (pl.ok && pl.p.SK == 1) return pl;
-    pl = make_plan_wide_on(a, tune, kXLimit, kGPW * kCW);
-    return pl.ok ? pl : make_plan_wide_on(a, tune, kXLimit, kCW);
-}
-
+// Slices of eight groups or more that x of all tokens has to be cut into to stay within 136 KB of shared memory.
+constexpr size_t kXLimit = 136 * 1024;
 // A plan is a function of the shape and the tuning alone and a call needs it twice (scratch, launch): the host thread
 // keeps the plans of the shapes it met last (a decoder has three or four).
 const Plan &plan_for(const LinearArgs &a, const GemvTuning &tune)
@@ -2078,47 +1313,11 @@ const Plan &plan_for(const LinearArgs &a, const GemvTuning &tune)
     for (int k : key) h = (h ^ (unsigned)k) * 0x9E3779B1u;
     Entry &e = table[h >> 28];
     if (memcmp(e.key, key, sizeof key) != 0) {
-        e.plan = a.M > 2 ? make_plan_wide(a, tune) : make_plan(a, tune);
+        e.plan = make_plan(a, tune);
         memcpy(e.key, key, sizeof key);
         if (!e.plan.ok) e.key[0] = -1;            // not kept: asked again
     }
     return e.plan;
-}
-
-template <int BITS, typename T, int MT>
-cudaError_t launch_wide(const Plan &pl, const CUtensorMap &wmap, const CUtensorMap &bmap, const CUtensorMap &amap, bool pdl, cudaStream_t s)
-{
-    auto kern = gemv_wide_kernel<BITS, T, MT>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(pl.p.n_t + pl.p.n_main));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = pl.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[2];
-    unsigned na = 0;
-    if (pdl) {
-        at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
-    if (pl.p.pair) {
-        at[na].id = cudaLaunchAttributeClusterDimension;
-        at[na].val.clusterDim.x = 2;
-        at[na].val.clusterDim.y = 1;
-        at[na].val.clusterDim.z = 1;
-        ++na;
-    }
-    cfg.attrs = at;
-    cfg.numAttrs = na;
-    return cudaLaunchKernelEx(&cfg, kern, pl.p, wmap, bmap, amap);
 }
 
 template <int BITS, typename T, int M, bool RANKED>
@@ -2154,8 +1353,11 @@ cudaError_t launch_variant(const Plan &pl, const CUtensorMap &wmap, const CUtens
 int gemv_k_slices(int M, int K)
 {
     if (M <= 2 || K < kGroupFast) return 1;
-    const int G = K / kGroupFast, sg = wide_slice_groups(M, G, kXLimit);
-    return (G + sg - 1) / sg;
+    const int G = K / kGroupFast;
+    auto slice_of = [&](int k) { return ((G + k - 1) / k + kCW - 1) / kCW * kCW; };
+    int sk = 1;
+    while (sk < 16 && (size_t)M * ((size_t)slice_of(sk) * kGroupFast + 32) * 2 > kXLimit) sk *= 2;
+    return (G + slice_of(sk) - 1) / slice_of(sk);
 }
 
 bool gemv_supported(const LinearArgs &a)
@@ -2169,13 +1371,11 @@ bool gemv_supported(const LinearArgs &a)
     return true;
 }
 
-void gemv_workspace_need(const LinearArgs &a, const GemvTuning &tune, size_t *tpart_floats, int *counters, size_t *partial_floats)
+void gemv_workspace_need(const LinearArgs &a, const GemvTuning &tune, size_t *tpart_floats, int *counters)
 {
-    const bool wide = a.M > 2;
     const Plan &pl = plan_for(a, tune);
     *tpart_floats = (size_t)(std::max(pl.p.n_t, 1) + 1) * std::max(pl.p.slot_elems, 32);
-    *counters = 8 + (wide ? pl.p.NT : 0);
-    *partial_floats = (wide && pl.p.SK > 1) ? (size_t)pl.p.NT * pl.p.SK * a.M * kTile : 0;
+    *counters = 8;
 }
 
 namespace {
@@ -2189,7 +1389,7 @@ cudaError_t make_maps(const LinearArgs &a, const GemvParams &p, CUtensorMap *wma
     m.ndim = 3;
     m.dims[0] = (cuuint64_t)wpg; m.dims[1] = (cuuint64_t)a.N; m.dims[2] = (cuuint64_t)p.G;
     m.strides[0] = (cuuint64_t)p.G * wpg * 4; m.strides[1] = (cuuint64_t)wpg * 4;
-    m.box[0] = (cuuint32_t)wpg; m.box[1] = (cuuint32_t)kTile; m.box[2] = (cuuint32_t)(a.M > 2 ? p.chg : kCHG);
+    m.box[0] = (cuuint32_t)wpg; m.box[1] = (cuuint32_t)kTile; m.box[2] = (cuuint32_t)kCHG;
     m.swizzle = CU_TENSOR_MAP_SWIZZLE_NONE;
     if (cudaError_t e = cached_map(wmap, m); e != cudaSuccess) return e;
     *bmap = *amap = *wmap;
@@ -2201,13 +1401,12 @@ cudaError_t make_maps(const LinearArgs &a, const GemvParams &p, CUtensorMap *wma
 }
 
 // Plans of a batch's problems: the main CTAs are shared out so that the fullest one has as little as possible (tiles times
-// stages per tile).  Integer form: two CTAs per SM (a launch of several problems lasts long enough that filling the
+// stages per tile).  Two CTAs per SM (a launch of several problems lasts long enough that filling the
 // SMs with its own CTAs pays more than letting the next launch's in; 4096 -> 3 x 4096 INT3 rank 64: 8.8 us, 11.3 with one,
 // 15.4 as three launches; 4096 -> 2 x 11008: 12.7, 15.6, 17.2), unless a CTA of the launch needs more than half of an SM's
 // shared memory (t CTAs of rank 112 and 128, x of a long K): then one, where two would run in two rounds (rank 128, INT4, one
 // token: 4096 -> 3 x 4096 14.1 / 12.0 us, 4096 -> 2 x 11008 19.1 / 16.9, 13824 -> 2 x 5120 50.4 / 23.6; a 7B layer from host
-// buffers 75 / 58 with the call); 16-bit form: one (its
-// CTAs take a whole SM; four tokens: 17.9 and 26.1 us, one by one 28.1 and 31.5).
+// buffers 75 / 58 with the call).
 struct BatchPlan {
     Plan plan[kGemvBatchMax];
     bool ok = false;
@@ -2215,20 +1414,19 @@ struct BatchPlan {
 BatchPlan plan_batch_on(const LinearArgs *a, int count, const GemvTuning &tune, int per_sm)
 {
     BatchPlan bp;
-    const bool wide = a[0].M > 2;
     GemvTuning t = tune;
     t.max_ctas = 0;
     int n_t = 0;
     for (int i = 0; i < count; ++i) {
         t.main_ctas = 2;
         const Plan &pl = plan_for(a[i], t);
-        if (!pl.ok || (wide && (pl.p.SK != 1 || !pl.p.pair))) return bp;
+        if (!pl.ok) return bp;
         n_t += pl.p.n_t;
     }
-    auto stages = [&](int i) { const int chg = wide ? kCW : kCHG, G = a[i].K / kGroupFast; return (G + chg - 1) / chg; };
+    auto stages = [&](int i) { return (a[i].K / kGroupFast + kCHG - 1) / kCHG; };
     auto share = [&](int i, int load) {                          // main CTAs with which problem i stays within `load`
-        const int nt = (a[i].N + kTile - 1) / kTile, most = std::max(1, load / stages(i)), c = (nt + most - 1) / most;
-        return wide ? std::max(2, (c + 1) / 2 * 2) : c;
+        const int nt = (a[i].N + kTile - 1) / kTile, most = std::max(1, load / stages(i));
+        return (nt + most - 1) / most;
     };
     auto total = [&](int load) { int c = 0; for (int i = 0; i < count; ++i) c += share(i, load); return c; };
     auto least_load = [&](int ctas) {                            // with that many main CTAs
@@ -2245,12 +1443,12 @@ BatchPlan plan_batch_on(const LinearArgs *a, int count, const GemvTuning &tune, 
     // All CTAs at once, or, with one CTA per SM and many t CTAs (a whole layer from host buffers: 70 of 148), a main CTA for every
     // SM, some of which start when the t CTAs leave.  (One t CTA per problem stays until every main CTA has read t.)
     int load = least_load(per_sm * g_sm_count - n_t);
-    if (!wide && per_sm == 1 && n_t > 0)
+    if (per_sm == 1 && n_t > 0)
         if (const int later = least_load(g_sm_count - count); later + kTStages < load) load = later;
     for (int i = 0; i < count; ++i) {
         t.main_ctas = share(i, load);
         bp.plan[i] = plan_for(a[i], t);
-        if (!bp.plan[i].ok || (wide && (bp.plan[i].p.R & 1 || bp.plan[i].p.R < 2))) return bp;
+        if (!bp.plan[i].ok) return bp;
         if (per_sm == 2 && bp.plan[i].smem > kSmemShare + 1024) return bp;       // (the launch takes the most that any of its CTAs needs)
     }
     bp.ok = true;
@@ -2258,9 +1456,8 @@ BatchPlan plan_batch_on(const LinearArgs *a, int count, const GemvTuning &tune, 
 }
 BatchPlan plan_batch(const LinearArgs *a, int count, const GemvTuning &tune)
 {
-    if (count < 1 || count > kGemvBatchMax) return BatchPlan{};
-    if (a[0].M <= 2)
-        if (const BatchPlan bp = plan_batch_on(a, count, tune, 2); bp.ok) return bp;
+    if (count < 1 || count > kGemvBatchMax || a[0].M > kGemvMaxM) return BatchPlan{};
+    if (const BatchPlan bp = plan_batch_on(a, count, tune, 2); bp.ok) return bp;
     return plan_batch_on(a, count, tune, 1);
 }
 size_t slot_floats(const GemvParams &p) { return (size_t)(std::max(p.n_t, 1) + 1) * std::max(p.slot_elems, 32); }
@@ -2301,7 +1498,6 @@ cudaError_t launch_gemv_batch(const LinearArgs *a, int count, Workspace &ws, con
         g.first_main[i] = g.n_t + main_ctas;
         main_ctas += g.p[i].n_main;
     }
-    const bool wide = a[0].M > 2;
     auto launch = [&](auto kern, bool &attr_set) {
         if (!attr_set) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
@@ -2321,13 +1517,6 @@ cudaError_t launch_gemv_batch(const LinearArgs *a, int count, Workspace &ws, con
             at[na].val.programmaticStreamSerializationAllowed = 1;
             ++na;
         }
-        if (wide) {
-            at[na].id = cudaLaunchAttributeClusterDimension;
-            at[na].val.clusterDim.x = 2;
-            at[na].val.clusterDim.y = 1;
-            at[na].val.clusterDim.z = 1;
-            ++na;
-        }
         cfg.attrs = at;
         cfg.numAttrs = na;
         return cudaLaunchKernelEx(&cfg, kern, g);
@@ -2335,11 +1524,9 @@ cudaError_t launch_gemv_batch(const LinearArgs *a, int count, Workspace &ws, con
     auto go = [&](auto bits, auto type) {
         using T = typename decltype(type)::type;
         constexpr int B = decltype(bits)::value;
-        static bool set[6] = {};
-        if (a[0].M > 8) return launch(gemv_wide_batch_kernel<B, T, 2>, set[0]);
-        if (a[0].M > 2) return launch(gemv_wide_batch_kernel<B, T, 1>, set[1]);
-        if (a[0].rank == 0) return a[0].M == 1 ? launch(gemv_batch_kernel<B, T, 1, false>, set[2]) : launch(gemv_batch_kernel<B, T, 2, false>, set[3]);
-        return a[0].M == 1 ? launch(gemv_batch_kernel<B, T, 1, true>, set[4]) : launch(gemv_batch_kernel<B, T, 2, true>, set[5]);
+        static bool set[4] = {};
+        if (a[0].rank == 0) return a[0].M == 1 ? launch(gemv_batch_kernel<B, T, 1, false>, set[0]) : launch(gemv_batch_kernel<B, T, 2, false>, set[1]);
+        return a[0].M == 1 ? launch(gemv_batch_kernel<B, T, 1, true>, set[2]) : launch(gemv_batch_kernel<B, T, 2, true>, set[3]);
     };
     const bool bf16 = a[0].bf16;
     const cudaError_t e = a[0].bits == 4 ? (bf16 ? go(std::integral_constant<int, 4>{}, TypeTag<__nv_bfloat16>{}) : go(std::integral_constant<int, 4>{}, TypeTag<__half>{}))
@@ -2350,13 +1537,10 @@ cudaError_t launch_gemv_batch(const LinearArgs *a, int count, Workspace &ws, con
 
 cudaError_t launch_gemv(const LinearArgs &a, Workspace &ws, const GemvTuning &tune, cudaStream_t s, int *launches)
 {
-    const bool wide = a.M > 2;
     Plan pl = plan_for(a, tune);
     if (!pl.ok) return cudaErrorInvalidConfiguration;
     GemvParams &p = pl.p;
     p.x = a.x; p.scales = a.scales; p.zeros = a.zeros; p.y = a.y;
-    p.part = ws.partial;
-    p.tctr = ws.counters + 8;
     p.tpart = reinterpret_cast<uint32_t *>(ws.tslots);
     p.ctr = ws.counters;
     p.status = ws.counters + kCtrStatus;
@@ -2374,8 +1558,6 @@ cudaError_t launch_gemv(const LinearArgs &a, Workspace &ws, const GemvTuning &tu
     auto go = [&](auto bits, auto type) {
         using T = typename decltype(type)::type;
         constexpr int B = decltype(bits)::value;
-        if (a.M > 8) return launch_wide<B, T, 2>(pl, wmap, bmap, amap, pdl, s);
-        if (a.M > 2) return launch_wide<B, T, 1>(pl, wmap, bmap, amap, pdl, s);
         if (a.rank == 0)
             return a.M == 1 ? launch_variant<B, T, 1, false>(pl, wmap, bmap, amap, pdl, s) : launch_variant<B, T, 2, false>(pl, wmap, bmap, amap, pdl, s);
         return a.M == 1 ? launch_variant<B, T, 1, true>(pl, wmap, bmap, amap, pdl, s) : launch_variant<B, T, 2, true>(pl, wmap, bmap, amap, pdl, s);

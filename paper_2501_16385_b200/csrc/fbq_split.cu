@@ -21,8 +21,13 @@
 //
 // What is left, 4096 -> 4096 INT4 at eight tokens, rank 0 (6.3 us a launch): 0.9 us until the preceding kernel has drained, 1.2 x,
 // 1.6 the multiplications, 0.6 the sums and the store, 2 the start of a CTA (it takes the whole SM, so none of it overlaps the
-// preceding launch).  Long launches run at the rate of the SM's pipes: a warp takes 96 to 115 clocks of the SM for 32 rows x 128 k x
-// 8 tokens, where unpacking alone takes 66 (bf16; LOP3 and shifts run at 64 lanes a clock) and the MMAs 33.
+// preceding launch).  In longer launches what counts is the number of instructions: bf16 4096 -> 11008, four tokens, a second
+// round of the multiplications adds 2.3 us to 11.4 (55 clocks of the SM for 32 rows x 128 k; the unpacking alone takes 40, LOP3 and
+// shifts run at 64 lanes a clock), without them the launch takes 8.2, without the copies of codes 11.1.  So what goes with every
+// stage is kept small: the copies' addresses are carried along instead of computed (`issue`), scales come with as many rows per
+// instruction as there are lanes.  These two took 4096 -> 11008 from 12.0 to 11.3 us at four tokens and from 14.7 to 13.6 at 16,
+// 5120 -> 13824 from 20.3 to 19.0, two problems 4096 -> 11008 as one launch, four tokens, from 21.7 to 19.9.  Two groups of a stage in
+// one block of code, for longer chains side by side: 11.5 and 15.6 for 11.4 and 13.7.
 //
 // 3 to 16 tokens; one problem, or several problems that run as one launch.
 #include <algorithm>
@@ -62,7 +67,7 @@ struct alignas(16) SplitDims {
     int ngt;                                 // sixteen-row granules of A of a t cluster
     int wk_log2, sg, stages;                 // parts of the slice of K that the warps take; groups of a stage, stages of a warp's ring
     int x_wide;                              // x can be read 32 bytes at a time
-    int sc_words, sc_pitch, sc_lanes_log2;   // scales come in 4-byte words; bytes of a row; lanes that take a row
+    int sc_wide, sc_words, sc_pitch;         // scales come in 4-byte words; words and bytes of a row
     int off_px, off_sc, off_b, off_recv, off_t, off_ring, off_trecv, off_tring, tstages;
 };
 struct SplitParams {
@@ -291,12 +296,10 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 // All but the latest n - 1 groups of copies of this thread have arrived.
 __device__ __forceinline__ void cp_async_wait_stage(int n)
 {
-    switch (n) {
-    case 1: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
-    case 2: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
-    case 3: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
-    default: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
-    }
+    if (n == kMostStages) asm volatile("cp.async.wait_group 3;" ::: "memory");
+    else if (n == 3) asm volatile("cp.async.wait_group 2;" ::: "memory");
+    else if (n == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void *src) { asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory"); }
 
@@ -407,29 +410,33 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
     const int row_bytes = p.G * GB;
     // this lane's first row and 16-byte unit of it; the next ones are 32 units on, in rows of `units`
     const int units = sg * kUnits, r0 = sg == 2 ? lane / (2 * kUnits) : lane / kUnits, c0 = lane - r0 * units, rstep = sg == 2 ? 32 / (2 * kUnits) : 32 / kUnits;
-    const uint8_t *qsrc = p.qw + (size_t)(g0 + gb) * GB + (size_t)(nrow0 + r0) * row_bytes + c0 * 16;
-    int ptile = wr, pg = 0, pslot = 0;
+    const uint8_t *qsrc = p.qw + (size_t)(g0 + gb) * GB + (size_t)(nrow0 + wr * kRows + r0) * row_bytes + c0 * 16;   // of the stage to come
+    const ptrdiff_t qnext = (ptrdiff_t)(wr_n * kRows) * row_bytes - (ptrdiff_t)(mine + sg - 1) / sg * sg * GB;       // end of a tile's stages -> the next tile
+    const size_t qstep = (size_t)rstep * row_bytes;
+    const uint32_t qdst = ring + (uint32_t)((c0 >= kUnits ? (kRows * GB) - GB : 0) + r0 * GB + c0 * 16), ring_bytes = (uint32_t)(stages * stage_bytes);
+    int ptile = mine > 0 ? wr : ntiles, pg = 0;
+    uint32_t pat = 0;                                                         // place of the stage in the ring
     auto issue = [&]() {
-        if (ptile < ntiles && mine > 0) {
-            const uint8_t *src = qsrc + (size_t)(ptile * kRows) * row_bytes + pg * GB;
-            const uint32_t dst = ring + (uint32_t)(pslot * stage_bytes);
+        if (ptile < ntiles) {
+            const uint8_t *src = qsrc;
             const int last = N - 1 - (nrow0 + ptile * kRows);                 // rows past N repeat the last one
             if constexpr (BITS == 4) {
                 // unit c0 of rows r0, r0 + rstep, ...
-                if (pg + (c0 >> 2) < mine) {
-                    const uint32_t d = dst + (uint32_t)((c0 >> 2) * (kRows * GB) + r0 * GB + (c0 & 3) * 16);
-                    if (last >= kRows - 1) {
-                        const size_t step = (size_t)rstep * row_bytes;
+                const uint32_t d = qdst + pat;
+                if (last < kRows - 1) {
 #pragma unroll 1
-                        for (int i = 0; i < units; i += 4)
+                    for (int i = 0; i < units && pg + (c0 >> 2) < mine; ++i) cp_async16(d + i * rstep * GB, src + (ptrdiff_t)(min(r0 + rstep * i, last) - r0) * row_bytes);
+                } else if (sg == 2) {
+                    if (pg + (c0 >> 2) < mine) {
 #pragma unroll
-                            for (int k = 0; k < 4; ++k, src += step) cp_async16(d + (i + k) * rstep * GB, src);
-                    } else {
-#pragma unroll 1
-                        for (int i = 0; i < units; ++i) cp_async16(d + i * rstep * GB, src + (ptrdiff_t)(min(r0 + rstep * i, last) - r0) * row_bytes);
+                        for (int i = 0; i < 2 * kUnits; ++i, src += qstep) cp_async16(d + i * (16 / kUnits) * GB, src);
                     }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < kUnits; ++i, src += qstep) cp_async16(d + i * (32 / kUnits) * GB, src);
                 }
             } else {
+                const uint32_t dst = ring + pat;
                 int r = r0, c = c0;
 #pragma unroll 1
                 for (int i = 0; i < units; i += 3)
@@ -446,18 +453,21 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
                         }
                     }
             }
-            if (++pslot == stages) pslot = 0;
+            pat += stage_bytes;
+            if (pat == ring_bytes) pat = 0;
+            qsrc += sg * GB;
             pg += sg;
             if (pg >= mine) {
                 pg = 0;
                 ptile += wr_n;
+                qsrc += qnext;
             }
         }
     };
     // ---- scales and zero points of the slice, and rows of B of the granules this CTA finishes ----
     // A row of the table holds the slice's groups of one weight row in 4-byte words (an odd number of them: rows lie in different
-    // banks), and the group before the first where that is an odd one.  Neighbouring lanes take neighbouring words of a row: what
-    // these copies cost is the number of lines that a warp's instruction touches.
+    // banks), and the group before the first where that is an odd one.  Neighbouring lanes take neighbouring words of a row, and
+    // 32 / words rows go with an instruction: what these copies cost is the instructions, and the lines that one touches.
     const int sh = g0 & 1, spitch = p.sc_pitch;                               // bytes
     const uint32_t zoff = (uint32_t)(kRows * spitch);
     uint8_t *sc = smem + p.off_sc;
@@ -468,26 +478,28 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
         issue();
         if (i == 0) {
             {
-                const int ll = p.sc_lanes_log2, w0 = lane & ((1 << ll) - 1);
+                const int words = p.sc_words, rows = words < 32 ? 32 / words : 1, lr = words < 32 ? lane / words : 0, w0 = lane - lr * words, wstep = min(words, 32);
                 const ptrdiff_t zero = p.zeros - p.scales;
                 const __half *scales = p.scales + (g0 - sh);
+                if (lr < rows)
 #pragma unroll 1
-                for (int r = (warp << (5 - ll)) + (lane >> ll); r < ntiles * kRows; r += kW << (5 - ll)) {
-                    const __half *src = scales + (size_t)min(nrow0 + r, N - 1) * p.G;
-                    uint8_t *dst = sc + ((r & ~31) + r) * spitch;
-                    if (p.sc_words)
+                    for (int r = warp * rows + lr; r < ntiles * kRows; r += kW * rows) {
+                        const __half *src = scales + (size_t)min(nrow0 + r, N - 1) * p.G;
+                        uint8_t *dst = sc + ((r & ~31) + r) * spitch;
+                        if (p.sc_wide)
 #pragma unroll 1
-                        for (int w = w0; 2 * w < Gs + sh; w += 1 << ll) {
-                            cp_async4(smem_u32(dst) + 4 * w, src + 2 * w);
-                            cp_async4(smem_u32(dst) + zoff + 4 * w, src + zero + 2 * w);
-                        }
-                    else
+                            for (int w = w0; w < words; w += wstep) {
+                                if (2 * w >= Gs + sh) break;
+                                cp_async4(smem_u32(dst) + 4 * w, src + 2 * w);
+                                cp_async4(smem_u32(dst) + zoff + 4 * w, src + zero + 2 * w);
+                            }
+                        else
 #pragma unroll 1
-                        for (int i = sh + w0; i < Gs + sh; i += 1 << ll) {
-                            *reinterpret_cast<__half *>(dst + 2 * i) = src[i];
-                            *reinterpret_cast<__half *>(dst + zoff + 2 * i) = src[zero + i];
-                        }
-                }
+                            for (int i = sh + w0; i < Gs + sh; i += wstep) {
+                                *reinterpret_cast<__half *>(dst + 2 * i) = src[i];
+                                *reinterpret_cast<__half *>(dst + zoff + 2 * i) = src[zero + i];
+                            }
+                    }
             }
             if (rank > 0) {
                 const int slots = owned(2 * ntiles, cs_log2, crank), c = lane & 15;   // 16-byte unit of a row
@@ -721,10 +733,9 @@ bool fill_problem(const LinearArgs &a, SplitDims &p, int cs_log2, int wk_log2, s
     p.off_px = (int)at;
     at += (size_t)Gs * MT * 64;
     p.off_sc = (int)at;
-    p.sc_words = p.G % 2 == 0 && ((reinterpret_cast<uintptr_t>(a.scales) | reinterpret_cast<uintptr_t>(a.zeros)) & 3) == 0;
-    const int words = (Gs + 2) / 2;
-    p.sc_pitch = 4 * (words | 1);
-    p.sc_lanes_log2 = words <= 4 ? 2 : words <= 8 ? 3 : words <= 16 ? 4 : 5;
+    p.sc_wide = p.G % 2 == 0 && ((reinterpret_cast<uintptr_t>(a.scales) | reinterpret_cast<uintptr_t>(a.zeros)) & 3) == 0;
+    p.sc_words = p.G % (2 * cs) == 0 ? Gs / 2 : (Gs + 2) / 2;                // (where every slice is an even number of groups none begins within a word)
+    p.sc_pitch = 4 * (p.sc_words | 1);
     at = aligned(at + (size_t)p.R * 2 * kRows * p.sc_pitch, 16);
     p.off_b = (int)at;
     if (a.rank > 0) at += (size_t)((2 * p.R + cs - 1) >> cs_log2) * 16 * (a.rank * 2 + 16);

@@ -772,8 +772,8 @@ bool fill_problem(const LinearArgs &a, SplitDims &p, int cs_log2, int wk_log2, s
 // tokens): staging x of the slice; the groups of the CTA (the SM's pipes) or of its fullest warp (latency); the stream of codes,
 // which a ring of few stages cannot keep up (about 1.3 us from request to arrival); sums to add; clusters, which cost more the
 // larger they are (and one of four or eight CTAs leaves SMs unused).  4096 -> 11008, 16 tokens, clusters of two, 8, 4, 2 parts
-// of the slice: 17.0, 15.2, 14.7 us; 11008 -> 4096, 8 tokens: 13.9, 14.7, 17.6; 4096 -> 4096, 16 tokens, CTAs of a cluster 1, 2, 4, 8:
-// 9.4, 8.2, 8.8, 9.8; 11008 -> 4096, 16 tokens, 4, 8: 17.9, 20.7.
+// of the slice: 17.0, 15.2, 14.7 us; 11008 -> 4096, clusters of two, 8 parts, or of four, 2 parts: 4 tokens 12.4, 13.3, 8 tokens
+// 13.5, 14.3; 4096 -> 4096, 16 tokens, CTAs of a cluster 1, 2, 4, 8: 9.4, 8.2, 8.8, 9.8.
 Shape make_shape(const LinearArgs *a, int count, int max_ctas)
 {
     Shape best;
@@ -832,7 +832,7 @@ Shape make_shape(const LinearArgs *a, int count, int max_ctas)
                     if (!fill_problem(a[i], q, c, w, &sm)) continue;
                     const int rounds = (R + (kW >> w) - 1) / (kW >> w), mine = (Gs + (1 << w) - 1) >> w, waves = (most + R - 1) / R;
                     const bool whole = q.stages * q.sg >= rounds * mine;
-                    const double units = std::max(R * Gs * (0.05 + 0.035 * (MT - 1)), rounds * mine * (0.40 + 0.05 * (MT - 1)));
+                    const double units = std::max(R * Gs * (0.05 + 0.035 * (MT - 1)), rounds * mine * (0.42 + 0.03 * (MT - 1)));
                     const double stream = R * Gs * 2.048 / (whole ? 44.0 : std::min(44.0, kW * q.stages * q.sg * 2.048 / 1.3));
                     const double ti = waves * (units + 0.3 * stream + 0.004 * Gs * M + 0.02 * (1 << (w + c)) + 0.01 * rounds * mine + (q.PT < q.R ? 0.5 : 0.0));
                     if (ti < t) {

@@ -707,7 +707,7 @@ struct Shape {
 // clusters, whose SM numbers are no multiples of four).
 int resident_clusters(int cs_log2)
 {
-    static const int n[4] = {148, 74, 33, 15};
+    static const int n[5] = {148, 74, 33, 15, 6};
     return n[cs_log2];
 }
 size_t aligned(size_t n, size_t to) { return (n + to - 1) / to * to; }
@@ -718,6 +718,9 @@ bool fill_problem(const LinearArgs &a, SplitDims &p, int cs_log2, int wk_log2, s
     const int MT = (a.M + 7) / 8, cs = 1 << cs_log2, Gs = (p.G + cs - 1) / cs, mine = (Gs + (1 << wk_log2) - 1) >> wk_log2, wr_n = kW >> wk_log2;
     const size_t x_end = (size_t)kOffX + (size_t)Gs * MT * 2048;
     p.wk_log2 = wk_log2;
+    // Half the shared memory for x: what is left beside more of it is a ring of one stage, each copy waited for (81920 -> 1024 at
+    // 8 tokens, rank 0: 81 us with 160 KB of x a CTA, 23 with 80).
+    if (Gs * MT > 64) return false;
     // a t CTA: x, sums, ring
     p.off_trecv = (int)x_end;
     p.off_tring = (int)aligned(x_end + (aligned(p.ngt, cs) * kTWK * MT) * 512, 128);
@@ -781,7 +784,8 @@ Shape make_shape(const LinearArgs *a, int count, int max_ctas)
     const int M = a[0].M, MT = (M + 7) / 8;
     int g_min = 1 << 30;
     for (int i = 0; i < count; ++i) g_min = std::min(g_min, a[i].K / kGroupFast);
-    for (int c = 0; c <= 3 && (1 << c) <= g_min; ++c) {
+    // (clusters of sixteen: for one set of eight tokens of more than 65536 inputs, which no smaller cluster holds)
+    for (int c = 0; c <= (MT == 1 && !best.ok ? 4 : 3) && (1 << c) <= g_min; ++c) {
         Shape s;
         s.sp.n = count;
         s.sp.M = M;
@@ -899,6 +903,7 @@ template <int BITS, typename T, int MT> cudaError_t launch_one(const Shape &s, b
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemAll);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         attr_set = true;

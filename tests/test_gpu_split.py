@@ -25,7 +25,8 @@ def fbq():
 @pytest.mark.parametrize("bits,dtype,M,N,K,rank", [
     (4, "f16", 3, 8, 128, 16), (3, "bf16", 16, 24, 128, 0), (4, "bf16", 9, 40, 3 * 128, 112), (3, "f16", 8, 72, 5 * 128, 128),
     (4, "f16", 16, 1000, 7 * 128, 64), (3, "f16", 9, 2056, 11 * 128, 48), (4, "bf16", 7, 520, 17 * 128, 32), (3, "bf16", 16, 136, 43 * 128, 96),
-    (4, "f16", 16, 264, 86 * 128, 128), (4, "bf16", 11, 2312, 40 * 128, 16), (3, "f16", 13, 48, 108 * 128, 64), (4, "f16", 5, 4104, 32 * 128, 0)])
+    (4, "f16", 16, 264, 86 * 128, 128), (4, "bf16", 11, 2312, 40 * 128, 16), (3, "f16", 13, 48, 108 * 128, 64), (4, "f16", 5, 4104, 32 * 128, 0),
+    (4, "f16", 4, 40, 560 * 128, 64), (3, "bf16", 8, 24, 577 * 128, 0)])        # the last two: clusters of sixteen
 def test_shapes(fbq, bits, dtype, M, N, K, rank):
     inp = make_linear(M, N, K, bits, rank, dtype=dtype, seed=7000 + M + N + K, outlier_frac=0.01)
     before = fbq.launch_count()

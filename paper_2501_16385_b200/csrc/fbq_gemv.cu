@@ -15,7 +15,7 @@
 //     an mbarrier ring; eight compute warps share every stage.
 //
 // Main CTAs (one per SM, or two: make_plan) own contiguous ranges of 16-row tiles.
-// a code masked out of its word is an unsigned byte operand of the 8-bit integer MMA as it stands
+// A code masked out of its word is an unsigned byte operand of the 8-bit integer MMA as it stands
 // (four codes per register, at most one shift per word); x is fixed point per group of 128 (three
 // signed base-256 digits, exact integer sums), and scale and zero point are applied per group to the
 // integer sums in fp32.  At M = 1 an MMA's eight columns hold the digits of TWO groups (columns 0-2
@@ -900,74 +900,71 @@ __device__ __forceinline__ void t_cta(const GemvParams &p, uint8_t *smem, const 
     pdl_wait();
     mark(p, 2);
     float *s_red = reinterpret_cast<float *>(smem + p.off_tred);      // [warp][rank][columns in use]
-    const int ncol = M <= 2 ? 2 : 8;
+    constexpr int ncol = 2;                                           // one and two tokens
     const T *x = static_cast<const T *>(p.x);
     bool dead = false;
-    for (int tb = 0; tb < (M + 7) / 8; ++tb) {
-        const int tok = tb * 8 + g;
-        if (warp < kCW) {
-            // this warp's blocks of 64 channels (warp and warp + kCW of the CTA's: two at most): their x as column operands ...
-            uint32_t xb[2][4][2];
-            bool mine[2];
+    const int tok = g;                                                // the MMA's column
+    if (warp < kCW) {
+        // this warp's blocks of 64 channels (warp and warp + kCW of the CTA's: two at most): their x as column operands ...
+        uint32_t xb[2][4][2];
+        bool mine[2];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                mine[u] = warp + u * kCW < nkb;
-                const int k0 = (kb0 + warp + u * kCW) * kTKB;
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks) {
-                    const int k = k0 + ks * 16 + 2 * tq;
-                    const bool v = mine[u] && tok < M && k < p.K;
-                    xb[u][ks][0] = v ? __ldcg(reinterpret_cast<const uint32_t *>(x + (size_t)tok * p.K + k)) : 0u;
-                    xb[u][ks][1] = v ? __ldcg(reinterpret_cast<const uint32_t *>(x + (size_t)tok * p.K + k + 8)) : 0u;
-                }
-            }
-            if (mine[0] && !mbar_wait(bar, 0)) dead = true;
-            if (tb == 0) mark(p, 3);
-            // ... against sixteen rows of A at a time.  Rows are 128 bytes, so the 128-byte swizzle XORs the 16-byte
-            // unit index with the row's low three bits, which are this lane's g for all its rows: the swizzled column
-            // offsets are constants of the lane.
-            const uint32_t xr = (uint32_t)(g & 7) << 4, rowb = (uint32_t)g * 128u;
-            uint32_t col[4][2];
+        for (int u = 0; u < 2; ++u) {
+            mine[u] = warp + u * kCW < nkb;
+            const int k0 = (kb0 + warp + u * kCW) * kTKB;
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) {
-                col[ks][0] = ((uint32_t)(ks * 32 + tq * 4) ^ xr) + rowb;
-                col[ks][1] = ((uint32_t)(ks * 32 + tq * 4 + 16) ^ xr) + rowb;
+                const int k = k0 + ks * 16 + 2 * tq;
+                const bool v = mine[u] && tok < M && k < p.K;
+                xb[u][ks][0] = v ? __ldcg(reinterpret_cast<const uint32_t *>(x + (size_t)tok * p.K + k)) : 0u;
+                xb[u][ks][1] = v ? __ldcg(reinterpret_cast<const uint32_t *>(x + (size_t)tok * p.K + k + 8)) : 0u;
             }
+        }
+        if (mine[0] && !mbar_wait(bar, 0)) dead = true;
+        mark(p, 3);
+        // ... against sixteen rows of A at a time.  Rows are 128 bytes, so the 128-byte swizzle XORs the 16-byte
+        // unit index with the row's low three bits, which are this lane's g for all its rows: the swizzled column
+        // offsets are constants of the lane.
+        const uint32_t xr = (uint32_t)(g & 7) << 4, rowb = (uint32_t)g * 128u;
+        uint32_t col[4][2];
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+            col[ks][0] = ((uint32_t)(ks * 32 + tq * 4) ^ xr) + rowb;
+            col[ks][1] = ((uint32_t)(ks * 32 + tq * 4 + 16) ^ xr) + rowb;
+        }
 #pragma unroll 1
-            for (int r = 0; r < nrb; ++r) {
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int r = 0; r < nrb; ++r) {
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    if (mine[u] && !dead) {
-                        const uint32_t ab = sA + (uint32_t)(warp + u * kCW) * blk_bytes + (uint32_t)r * 2048u;
+            for (int u = 0; u < 2; ++u) {
+                if (mine[u] && !dead) {
+                    const uint32_t ab = sA + (uint32_t)(warp + u * kCW) * blk_bytes + (uint32_t)r * 2048u;
 #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks)
-                            Mma16<T>::run(acc, lds_u32(ab + col[ks][0]), lds_u32(ab + col[ks][0] + 1024u), lds_u32(ab + col[ks][1]),
-                                          lds_u32(ab + col[ks][1] + 1024u), xb[u][ks][0], xb[u][ks][1]);
-                    }
-                }
-                // rows r*16 + g (and + 8) of A, columns 2tq, 2tq+1 (tokens)
-                if (2 * tq < ncol) {
-                    float *dst = s_red + ((size_t)warp * rank + r * 16 + g) * ncol + 2 * tq;
-                    dst[0] = acc[0];
-                    dst[1] = acc[1];
-                    dst[8 * ncol] = acc[2];
-                    dst[8 * ncol + 1] = acc[3];
+                    for (int ks = 0; ks < 4; ++ks)
+                        Mma16<T>::run(acc, lds_u32(ab + col[ks][0]), lds_u32(ab + col[ks][0] + 1024u), lds_u32(ab + col[ks][1]),
+                                      lds_u32(ab + col[ks][1] + 1024u), xb[u][ks][0], xb[u][ks][1]);
                 }
             }
+            // rows r*16 + g (and + 8) of A, columns 2tq, 2tq+1 (tokens)
+            if (2 * tq < ncol) {
+                float *dst = s_red + ((size_t)warp * rank + r * 16 + g) * ncol + 2 * tq;
+                dst[0] = acc[0];
+                dst[1] = acc[1];
+                dst[8 * ncol] = acc[2];
+                dst[8 * ncol + 1] = acc[3];
+            }
         }
-        __syncthreads();
-        const int ntok = min(8, M - tb * 8);
-        for (int i = tid; i < ntok * rank; i += kThreads) {
-            const int m = i / rank, j = i - m * rank;
-            float v = 0.f;
-#pragma unroll
-            for (int w = 0; w < kCW; ++w) v += s_red[((size_t)w * rank + j) * ncol + m];
-            // the value, encoded so that the word is not zero: whoever sees the word sees the value
-            p.tpart[(size_t)c * p.slot_elems + (size_t)(tb * 8 + m) * rank + j] = (p.test_skip_arrive || dead) ? 0u : t_enc(v);
-        }
-        __syncthreads();
     }
+    __syncthreads();
+    for (int i = tid; i < M * rank; i += kThreads) {
+        const int m = i / rank, j = i - m * rank;
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < kCW; ++w) v += s_red[((size_t)w * rank + j) * ncol + m];
+        // the value, encoded so that the word is not zero: whoever sees the word sees the value
+        p.tpart[(size_t)c * p.slot_elems + (size_t)m * rank + j] = (p.test_skip_arrive || dead) ? 0u : t_enc(v);
+    }
+    __syncthreads();
     if (dead && lane == 0) give_up(p);
     if (p.t_final) {
         // Many entries (tokens x rank x slots): the t CTA that counts in last adds the slots in order into one
@@ -980,46 +977,21 @@ __device__ __forceinline__ void t_cta(const GemvParams &p, uint8_t *smem, const 
         if (*s_last) {
             __threadfence();
             const size_t slot_elems = (size_t)p.slot_elems;
-            if (M * rank <= kThreads) {
-                // few entries: one per thread, so that as many threads as possible share the loads
-                for (int i = tid; i < M * rank; i += kThreads) {
-                    float v = 0.f;
-                    bool all = true;
-                    for (int c0 = 0; c0 < p.n_t; c0 += 8) {
-                        uint32_t part[8];
+            // one entry per thread (two tokens of rank 128 at most), so that as many threads as possible share the loads
+            for (int i = tid; i < M * rank; i += kThreads) {
+                float v = 0.f;
+                bool all = true;
+                for (int c0 = 0; c0 < p.n_t; c0 += 8) {
+                    uint32_t part[8];
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) part[u] = (c0 + u < p.n_t) ? __ldcg(p.tpart + (size_t)(c0 + u) * slot_elems + i) : kTNone;
+                    for (int u = 0; u < 8; ++u) part[u] = (c0 + u < p.n_t) ? __ldcg(p.tpart + (size_t)(c0 + u) * slot_elems + i) : kTNone;
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            v += __uint_as_float(part[u]);
-                            all = all && (part[u] != 0u);
-                        }
+                    for (int u = 0; u < 8; ++u) {
+                        v += __uint_as_float(part[u]);
+                        all = all && (part[u] != 0u);
                     }
-                    p.tpart[(size_t)p.n_t * slot_elems + i] = all ? t_enc(v) : 0u;
                 }
-            } else {
-                // many entries (several tokens): four per thread and load, or the rounds of loads are this CTA's time
-                for (int q = tid; 4 * q < M * rank; q += kThreads) {
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    uint32_t mn = 0xFFFFFFFFu;
-                    for (int c0 = 0; c0 < p.n_t; c0 += 8) {
-                        uint4 part[8];
-#pragma unroll
-                        for (int u = 0; u < 8; ++u)
-                            part[u] = (c0 + u < p.n_t) ? __ldcg(reinterpret_cast<const uint4 *>(p.tpart + (size_t)(c0 + u) * slot_elems) + q)
-                                                       : make_uint4(kTNone, kTNone, kTNone, kTNone);
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            mn = t_min(mn, part[u]);
-                            v.x += __uint_as_float(part[u].x);
-                            v.y += __uint_as_float(part[u].y);
-                            v.z += __uint_as_float(part[u].z);
-                            v.w += __uint_as_float(part[u].w);
-                        }
-                    }
-                    reinterpret_cast<uint4 *>(p.tpart + (size_t)p.n_t * slot_elems)[q] =
-                        mn != 0u ? make_uint4(t_enc(v.x), t_enc(v.y), t_enc(v.z), t_enc(v.w)) : make_uint4(0u, 0u, 0u, 0u);
-                }
+                p.tpart[(size_t)p.n_t * slot_elems + i] = all ? t_enc(v) : 0u;
             }
         }
     }

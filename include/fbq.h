@@ -86,10 +86,11 @@ int fbq_dequant(const uint32_t *qweight, const uint16_t *scales, const uint16_t 
  *   rank == 0: A and B are ignored (may be NULL); y is the main path alone.
  *   M == 0: nothing is done.
  * Dispatch (fbq_select_kernel tells which kernel a shape gets): group == 128 and rank a multiple of 8
- * not above 256 are the fast kernels' domain.  The streaming decode kernel ("gemv" option, default on)
- * needs N a multiple of 8, rank a multiple of 16 up to 128 and 16-byte aligned scales and zeros; there
- * it takes M <= 8 for every shape, and M <= 16 while M * K * 2 bytes stay within 136 KB (x of all K in
- * shared memory).  Elsewhere the other decode kernel
+ * not above 256 are the fast kernels' domain.  The streaming kernels ("gemv" option, default on)
+ * need N a multiple of 8, rank a multiple of 16 up to 128 and, at M <= 2, 16-byte aligned scales and zeros; there
+ * the decode class is M <= 8 for every shape, and M <= 16 while M * K * 2 bytes stay within 136 KB.  One
+ * kernel of it takes M <= 2, the split kernel (K cut over the CTAs of a cluster) 3 <= M <= 16, also where that
+ * rule says prefill, unless a kernel is forced.  Elsewhere the other decode kernel
  * takes M <= 4 with rank <= 128 and M = 5, 6 with M * rank <= 128.  The prefill kernel (N a multiple of
  * 8) takes the rest of the domain; shapes outside its domain stay with a decode kernel up to M = 16;
  * everything else that is well formed -> generic kernel.
@@ -104,7 +105,7 @@ int fbq_dequant(const uint32_t *qweight, const uint16_t *scales, const uint16_t 
  * type).  At M <= 2 the decode kernels read x in fixed point per group of 128, exact to 2^-17
  * of the group's largest element; a group that holds an Inf or a NaN makes its token's outputs NaN.
  * Summation order is fixed for a given shape and grid size (results are
- * reproducible run to run), except for t in the decode kernel of M >= 3, which is
+ * reproducible run to run), except for t in the other decode kernel at M >= 3, which is
  * accumulated with floating-point atomics.
  * Scratch and CUDA graphs: the library keeps scratch buffers per (device, stream) and grows them
  * the first time a stream sees a larger shape.  Growing allocates (and, for a buffer that exists,
@@ -218,8 +219,8 @@ int fbq_reconstruct_step(const float *W, const float *H, float *A, float *B, flo
  *   - `problems` is a HOST array of `count` (<= FBQ_BATCH_MAX) descriptors of DEVICE
  *     pointers (layouts and alignment as for fbq_linear); it is read before the call returns.
  *   - When every problem is decode sized (M <= 16 and the decode kernels' domain) the problems run
- *     concurrently.  Up to 8 problems of the streaming kernel that read the same x (q, k, v; gate,
- *     up) are ONE launch of it on `stream`, the SMs shared out so that no CTA has much more than
+ *     concurrently.  Up to 8 problems of a streaming kernel that read the same x (q, k, v; gate,
+ *     up; from 3 tokens on each of more than 16 rows) are ONE launch of it on `stream`, the SMs shared out so that no CTA has much more than
  *     another ("batch_single" = 1, the default).  Up to 8 problems outside the streaming kernel's
  *     domain run as ONE launch of the other decode kernel over a problem list, each with a share
  *     of "batch_ctas" CTAs in proportion to its share of the codes.  Everything else, or
@@ -270,15 +271,15 @@ int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int ac
 /* Tuning and test switches (host side, process wide).  Known names:
  *   "force_kernel"  -1 = automatic, else an fbq_kernel value (shapes outside the
  *                   forced kernel's domain still fall back to the generic one)
- *   "gemv"          1 (default) = M <= 16 runs the streaming decode kernel where its domain allows (see fbq_linear),
+ *   "gemv"          1 (default) = M <= 16 runs the streaming kernels where their domain allows (see fbq_linear),
  *                   0 = the other decode kernel at every M
- *   "gemv_ctas"     0 = automatic (one or two CTAs per SM), else an upper bound on the streaming kernel's grid
+ *   "gemv_ctas"     0 = automatic (one or two CTAs per SM), else an upper bound on the grid of the streaming kernels
  *                   (fbq_set_stream_option sets it for one stream)
- *   "t_poll_limit"  0 = default, else the number of looks the streaming kernel takes at the t CTAs' slots
+ *   "t_poll_limit"  0 = default, else the number of looks the streaming kernels take at the t CTAs' words
  *                   before it gives up with FBQ_ERR_TIMEOUT
  *   "test_skip_t_arrive", "test_prefill_skip_flag", "prefill_flag_polls"
  *                   test switches of the failure-detection tests: the CTAs that compute t = x.A^T do not
- *                   report it (streaming decode kernel / prefill kernel), and the prefill kernel's number
+ *                   report it (streaming kernels / prefill kernel), and the prefill kernel's number
  *                   of looks at its flag; with them a bounded wait runs out on purpose
  *   "decode_sk"     0 = automatic, else the number of K slices of the decode kernel
  *   "decode_chunk"  0 = automatic, else quantisation groups per smem stage

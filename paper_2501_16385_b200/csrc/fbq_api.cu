@@ -226,13 +226,13 @@ int run_split(const LinearArgs *a, int count, const GemvTuning &gt, Workspace *w
 // Calls of 3 to 16 tokens in the streaming kernels' domain, also those that select_kernel counts among the prompts, unless a
 // kernel is forced.  Measured on B200, INT4, bf16, us per launch in a row, the kernels before it (a streaming one whose CTAs
 // staged x of all K, or the tensor-core one) / this one:
-//                      4 tokens, rank 64   8 tokens, rank 128   16 tokens, rank 64
-//   4096 -> 4096        8.7 /  7.2        11.7 /  7.9       13.9 /  8.1
-//   4096 -> 11008      13.4 / 11.3        17.5 / 12.5       20.6 / 13.6
+//                  4 tokens, rank 64  8 tokens, rank 128  16 tokens, rank 64
+//   4096 -> 4096        8.7 /  7.2        11.7 /  7.6       13.9 /  8.2
+//   4096 -> 11008      13.4 / 11.1        17.5 / 12.1       20.6 / 13.9
 //   11008 -> 4096      15.1 / 12.4        27.4 / 13.5       24.1 / 16.8
-//   5120 -> 13824      18.8 / 15.5        22.5 / 17.6       34.2 / 19.0
-//   13824 -> 5120      21.3 / 16.4        37.5 / 18.9       33.7 / 22.7
-//   1280 -> 3456          7.1 /  5.2           10.5 /  6.0          11.4 /  5.7
+//   5120 -> 13824      18.8 / 15.7        22.5 / 17.6       34.2 / 19.2
+//   13824 -> 5120      21.3 / 16.5        37.5 / 19.1       33.7 / 22.7
+//   1280 -> 3456        7.1 /  5.1        10.5 /  5.9       11.4 /  5.6
 // At one and two tokens the streaming kernel's integer form is ahead: 4096 -> 4096 rank 64 4.8 / 7.1 and 5.7 / 7.1.
 bool split_takes(const LinearArgs &a, int kernel)
 {

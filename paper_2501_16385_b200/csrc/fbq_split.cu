@@ -19,15 +19,15 @@
 //     the launch's number, so value and "written" travel together and nothing has to be cleared at the end of a launch.  A main CTA
 //     takes t in once, with all its threads, and multiplies it with its rows of B as two TF32 terms (exact to 2^-22, any magnitude).
 //
-// What is left, 4096 -> 4096 INT4 at eight tokens, rank 0 (6.3 us a launch): 0.9 us until the preceding kernel has drained, 1.2 x,
-// 1.6 the multiplications, 0.6 the sums and the store, 2 the start of a CTA (it takes the whole SM, so none of it overlaps the
-// preceding launch).  In longer launches what counts is the number of instructions: bf16 4096 -> 11008, four tokens, a second
-// round of the multiplications adds 2.3 us to 11.4 (55 clocks of the SM for 32 rows x 128 k; the unpacking alone takes 40, LOP3 and
-// shifts run at 64 lanes a clock), without them the launch takes 8.2, without the copies of codes 11.1.  So what goes with every
-// stage is kept small: the copies' addresses are carried along instead of computed (`issue`), scales come with as many rows per
-// instruction as there are lanes.  These two took 4096 -> 11008 from 12.0 to 11.3 us at four tokens and from 14.7 to 13.6 at 16,
-// 5120 -> 13824 from 20.3 to 19.0, two problems 4096 -> 11008 as one launch, four tokens, from 21.7 to 19.9.  Two groups of a stage in
-// one block of code, for longer chains side by side: 11.5 and 15.6 for 11.4 and 13.7.
+// What is left, 4096 -> 4096 INT4 at eight tokens, rank 0 (6.3 us a launch when these were told apart): 0.9 us until the preceding
+// kernel has drained, 1.2 x, 1.6 the multiplications, 0.6 the sums and the store, 2 the start of a CTA (it takes the whole SM, so
+// none of it overlaps the preceding launch).  In longer launches what counts is the number of instructions: bf16 4096 -> 11008, four
+// tokens, a second round of the multiplications adds 2.3 us to 11.4 (55 clocks of the SM for 32 rows x 128 k; the unpacking alone
+// takes 40, LOP3 and shifts run at 64 lanes a clock), without them the launch takes 8.2, without the copies of codes 11.1.  So what
+// goes with every stage is kept small: the copies' addresses are carried along instead of computed (`issue`), scales come with as
+// many rows per instruction as there are lanes.  These two took 4096 -> 11008 from 12.0 to 11.3 us at four tokens and from 14.7 to
+// 13.6 at 16, 5120 -> 13824 from 20.3 to 19.0, two problems 4096 -> 11008 as one launch, four tokens, from 21.7 to 19.9.  Two groups
+// of a stage in one block of code, for longer chains side by side: 11.5 and 15.6 for 11.4 and 13.7.
 //
 // 3 to 16 tokens; one problem, or several problems that run as one launch.
 #include <algorithm>
@@ -168,38 +168,46 @@ template <typename T> __device__ __forceinline__ uint32_t pair_of(float v)
 // nothing crosses lanes but what the two warps that share the groups stage for each other.  The unpacker's order and field
 // weights are applied to x here; (-P, X0) of a token and group, P = MAGIC sum of the staged x and X0 = sum of x, come out of
 // MMAs against rows of ones and of field weights, in the lanes that need them.  Tokens past M repeat the last one.
+// Two runs are on their way at a time, and never one too many: every CTA asks L2 for the same lines at the same moment, and a load
+// that only repeats another costs a launch 0.3 to 0.45 us (4096 -> 4096, 8 tokens, rank 128: with one 7.95 us, with two 8.4, with
+// none 7.6).
 template <int BITS, typename T, int MT>
 __device__ __forceinline__ void stage_x(const T *x, int K, int M, bool wide, uint8_t *xs, float4 *px, int groups, int part, int parts, int lane)
 {
-    constexpr int kFly = 2;
     const int n = lane >> 2, t = lane & 3, total = groups * MT;
+    auto load = [&](int it, uint32_t (&e)[16]) {
+        const int grp = it / MT, b = it - grp * MT;
+        load_run(x + (size_t)min(8 * b + n, M - 1) * K + grp * kGroupFast + 32 * t, wide, e);
+    };
+    auto convert = [&](int it, const uint32_t (&e)[16]) {
+        uint32_t h[16];
+        float d[4] = {};
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            constexpr auto div = [](int c) { return Unpack16<BITS, T>::div_log2(c); };
+            const int c0 = pair_first<BITS>(j), c1 = pair_second<BITS>(j);
+            h[j] = pair_scaled<T>(__byte_perm(e[c0 >> 1], e[c1 >> 1], ((c0 & 1) ? 0x32u : 0x10u) | ((c1 & 1) ? 0x7600u : 0x5400u)), div(c0));
+            if (j & 1)
+                mma16<T>(d, pair_of<T>(1.f), pair_of<T>((float)(1 << div(pair_first<BITS>(j - 1)))), pair_of<T>(1.f), pair_of<T>((float)(1 << div(c0))), h[j - 1], h[j]);
+        }
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4)
+            *reinterpret_cast<uint4 *>(xs + (((it * 4 + q4) * 32 + lane) << 4)) = make_uint4(h[4 * q4], h[4 * q4 + 1], h[4 * q4 + 2], h[4 * q4 + 3]);
+        if (lane < 4) px[it * 4 + lane] = make_float4(-Unpack16<BITS, T>::kMagic * d[0], -Unpack16<BITS, T>::kMagic * d[1], d[2], d[3]);
+    };
+    int it = part;
 #pragma unroll 1
-    for (int base = part; base < total; base += kFly * parts) {
-        uint32_t e[kFly][16];
-#pragma unroll
-        for (int u = 0; u < kFly; ++u) {
-            const int it = min(base + u * parts, total - 1), grp = it / MT, b = it - grp * MT;
-            load_run(x + (size_t)min(8 * b + n, M - 1) * K + grp * kGroupFast + 32 * t, wide, e[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < kFly; ++u) {
-            const int it = base + u * parts;
-            if (it >= total) break;
-            uint32_t h[16];
-            float d[4] = {};
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                constexpr auto div = [](int c) { return Unpack16<BITS, T>::div_log2(c); };
-                const int c0 = pair_first<BITS>(j), c1 = pair_second<BITS>(j);
-                h[j] = pair_scaled<T>(__byte_perm(e[u][c0 >> 1], e[u][c1 >> 1], ((c0 & 1) ? 0x32u : 0x10u) | ((c1 & 1) ? 0x7600u : 0x5400u)), div(c0));
-                if (j & 1)
-                    mma16<T>(d, pair_of<T>(1.f), pair_of<T>((float)(1 << div(pair_first<BITS>(j - 1)))), pair_of<T>(1.f), pair_of<T>((float)(1 << div(c0))), h[j - 1], h[j]);
-            }
-#pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4)
-                *reinterpret_cast<uint4 *>(xs + (((it * 4 + q4) * 32 + lane) << 4)) = make_uint4(h[4 * q4], h[4 * q4 + 1], h[4 * q4 + 2], h[4 * q4 + 3]);
-            if (lane < 4) px[it * 4 + lane] = make_float4(-Unpack16<BITS, T>::kMagic * d[0], -Unpack16<BITS, T>::kMagic * d[1], d[2], d[3]);
-        }
+    for (; it + parts < total; it += 2 * parts) {
+        uint32_t e[2][16];
+        load(it, e[0]);
+        load(it + parts, e[1]);
+        convert(it, e[0]);
+        convert(it + parts, e[1]);
+    }
+    if (it < total) {
+        uint32_t e[16];
+        load(it, e);
+        convert(it, e);
     }
 }
 // The same for a t CTA: x as it is.

@@ -268,6 +268,11 @@ int fbq_sub_branch_unfused(const void *x, const void *A, const void *B, void *y,
  * FBQ_KERNEL_NONE when the shape is rejected.  Pure host logic. */
 int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int act_is_bf16);
 
+/* How the split kernel (3 to 16 tokens) would run this shape, as one problem: CTAs of its grid and of a cluster, under the bound
+ * max_ctas (0: what "gemv_ctas" says).  FBQ_ERR_UNSUPPORTED where fbq_linear would not run that kernel.  Pure host logic, for
+ * tests and tuning. */
+int fbq_split_plan(int M, int N, int K, int group, int bits, int rank, int act_is_bf16, int max_ctas, int *ctas, int *cluster);
+
 /* Tuning and test switches (host side, process wide).  Known names:
  *   "force_kernel"  -1 = automatic, else an fbq_kernel value (shapes outside the
  *                   forced kernel's domain still fall back to the generic one)

@@ -34,6 +34,7 @@ from .binding import (  # noqa: F401
     select_kernel,
     set_option,
     set_stream_option,
+    split_plan,
     status_string,
     sub_branch_unfused,
     unpack,

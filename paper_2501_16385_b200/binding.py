@@ -66,6 +66,7 @@ def lib() -> ctypes.CDLL:
         L.fbq_linear_batch.argtypes = [ctypes.POINTER(Problem), i32, i32, i32, i32, i32, i32, vp]
         L.fbq_linear_batch_hostio.argtypes = [ctypes.POINTER(Problem), i32, i32, i32, i32, i32, i32, vp]
         L.fbq_select_kernel.argtypes = [i32] * 7
+        L.fbq_split_plan.argtypes = [i32] * 8 + [ctypes.POINTER(i32)] * 2
         L.fbq_set_option.argtypes = [ctypes.c_char_p, i32]
         L.fbq_get_option.argtypes = [ctypes.c_char_p, ctypes.POINTER(i32)]
         L.fbq_set_stream_option.argtypes = [vp, ctypes.c_char_p, i32]
@@ -262,6 +263,16 @@ def linear_batch(problems, group: int, bits: int, stream=None, batch=None, host_
 
 def select_kernel(M, N, K, group, bits, rank, bf16=False) -> int:
     return int(lib().fbq_select_kernel(M, N, K, group, bits, rank, 1 if bf16 else 0))
+
+
+def split_plan(M, N, K, group, bits, rank, bf16=False, max_ctas=0):
+    """fbq_split_plan: (CTAs of the grid, CTAs of a cluster), or None where another kernel runs."""
+    ctas, cluster = ctypes.c_int(0), ctypes.c_int(0)
+    code = lib().fbq_split_plan(M, N, K, group, bits, rank, 1 if bf16 else 0, max_ctas, ctypes.byref(ctas), ctypes.byref(cluster))
+    if code == -2:
+        return None
+    _check(code, "fbq_split_plan")
+    return ctas.value, cluster.value
 
 
 def set_option(name: str, value: int) -> None:

@@ -932,6 +932,16 @@ int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int ac
     return select_kernel(M, N, K, group, bits, rank, act_is_bf16 != 0);
 }
 
+int fbq_split_plan(int M, int N, int K, int group, int bits, int rank, int act_is_bf16, int max_ctas, int *ctas, int *cluster)
+{
+    if (!ctas || !cluster || max_ctas < 0 || !well_formed(M, N, K, group, bits, rank)) return FBQ_ERR_BADARG;
+    LinearArgs a{};
+    a.M = M; a.N = N; a.K = K; a.group = group; a.bits = bits; a.rank = rank; a.bf16 = act_is_bf16 != 0;
+    GemvTuning gt = g_opt.gemv;
+    if (max_ctas > 0) gt.max_ctas = max_ctas;
+    return split_takes(a, select_kernel(M, N, K, group, bits, rank, a.bf16)) && split_plan(a, gt, ctas, cluster) ? FBQ_OK : FBQ_ERR_UNSUPPORTED;
+}
+
 int fbq_set_option(const char *name, int value)
 {
     int *slot = option_slot(name);

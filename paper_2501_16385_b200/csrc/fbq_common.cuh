@@ -124,6 +124,7 @@ constexpr int kSplitMaxM = 16;
 bool split_supported(const LinearArgs &a);
 size_t split_scratch_bytes(const LinearArgs *a, int count);
 bool split_plan_exists(const LinearArgs *a, int count, const GemvTuning &tune);
+bool split_plan(const LinearArgs &a, const GemvTuning &tune, int *ctas, int *cluster);     // CTAs of the grid, of a cluster
 cudaError_t launch_split(const LinearArgs *a, int count, Workspace &ws, const GemvTuning &tune, cudaStream_t s, int *launches);
 
 int decode_batch_max();

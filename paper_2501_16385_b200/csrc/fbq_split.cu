@@ -74,7 +74,7 @@ struct SplitParams {
     int n, M, cs_log2, n_tc, poll_limit, skip_t;
     int first_tc[kMostProblems], first_mc[kMostProblems];
     int *status;
-    unsigned long long *epoch;               // 65536 x the number of launches so far, plus the CTAs of this one that are through
+    unsigned long long *epoch;               // 2^32 x the number of launches so far, plus the CTAs of this one that are through
     SplitDims p[kMostProblems];
 };
 static_assert(kOffDims + sizeof(SplitDims) <= kOffX, "");
@@ -311,6 +311,9 @@ __device__ __forceinline__ void cp_async_wait_stage(int n)
 }
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void *src) { asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory"); }
 
+// This launch's number, which the words of its t carry.
+__device__ __forceinline__ uint32_t launch_number(const unsigned long long *epoch) { return (uint32_t)(__ldcg(epoch) >> 32) + 1u; }
+
 template <typename T, int MT>
 __device__ __forceinline__ void t_program(const SplitParams &sp, const SplitDims &p, uint8_t *smem, int lc, int crank, int g0, int Gs)
 {
@@ -348,7 +351,7 @@ __device__ __forceinline__ void t_program(const SplitParams &sp, const SplitDims
     const bool wide = p.x_wide != 0;
     uint2 *tw = p.t;
     pdl_wait();
-    const uint32_t tag = (uint32_t)(__ldcg(sp.epoch) >> 16) + 1u;             // this launch's number
+    const uint32_t tag = launch_number(sp.epoch);
     stage_x_plain<T, MT>(x, K, M, wide, xs, mine, wr, lane);
     __syncthreads();
     cluster_wait();                                                           // the other CTAs of the cluster have started
@@ -533,7 +536,7 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
     const uint32_t pass_bytes = (uint32_t)(((2 * PT + cs - 1) >> cs_log2 << (cs_log2 + wkl)) * MT * 512);
     if (threadIdx.x == 0) mbar_expect_tx(rbar, (uint32_t)(owned(2 * min(PT, ntiles), cs_log2, crank) << (cs_log2 + wkl)) * MT * 512);
     pdl_wait();
-    const uint32_t tag = (uint32_t)(__ldcg(sp.epoch) >> 16) + 1u;             // this launch's number
+    const uint32_t tag = launch_number(sp.epoch);
     stage_x<BITS, T, MT>(x, K, M, wide, xs, px, mine, wr, wr_n, lane);
     cp_async_wait_stage(stages);                                              // the first stage, and with it the scales and B
     __syncthreads();
@@ -698,9 +701,10 @@ __global__ void __launch_bounds__(kThr, 1) split_kernel(const __grid_constant__ 
     } else {
         main_program<BITS, T, MT>(sp, p, smem, cluster - p.first_mc, crank, g0, Gs);
     }
-    // Every CTA read the launch's number before this; with the last one the count of launches goes up by one.
+    // Every CTA read the launch's number before this; with the last one the count of launches goes up by one.  (The CTAs that are
+    // through have 32 bits: grids of wide layers, 4096 -> 8 000 000, say, hold more than 65536 CTAs.)
     __syncthreads();
-    if (threadIdx.x == 0) atomicAdd(sp.epoch, blockIdx.x == 0 ? 65536ull - (gridDim.x - 1) : 1ull);
+    if (threadIdx.x == 0) atomicAdd(sp.epoch, blockIdx.x == 0 ? (1ull << 32) - (gridDim.x - 1) : 1ull);
 }
 
 // ---- host ----------------------------------------------------------------------------------------------------------
@@ -955,6 +959,14 @@ bool split_supported(const LinearArgs &a)
 bool split_plan_exists(const LinearArgs *a, int count, const GemvTuning &tune)
 {
     return count >= 1 && count <= kMostProblems && shape_for(a, count, tune.max_ctas).ok;
+}
+
+bool split_plan(const LinearArgs &a, const GemvTuning &tune, int *ctas, int *cluster)
+{
+    const Shape &s = shape_for(&a, 1, tune.max_ctas);
+    *ctas = s.clusters << s.sp.cs_log2;
+    *cluster = 1 << s.sp.cs_log2;
+    return s.ok;
 }
 
 size_t split_scratch_bytes(const LinearArgs *a, int count)

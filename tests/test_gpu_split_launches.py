@@ -1,0 +1,44 @@
+"""The split kernel's count of launches, whose numbers the words of t carry: grids of more than 65536 CTAs."""
+import pytest
+
+from gpu_utils import REL_F_TOL
+
+pytestmark = pytest.mark.gpu
+
+
+def _codes(words, rows, K):
+    """INT4 codes of some rows, [rows][K]."""
+    import torch
+    w = words.view(-1, K // 8)[rows]
+    return (w[:, :, None] >> torch.arange(0, 32, 4, device="cuda", dtype=torch.int32)).bitwise_and(15).reshape(len(rows), K)
+
+
+def test_more_than_65536_ctas():
+    import torch
+    import paper_2501_16385_b200 as fbq
+    M, N, K, r = 16, 15_000_000, 128, 128
+    ctas, _ = fbq.split_plan(M, N, K, 128, 4, r)
+    assert ctas > 65536
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    words = torch.randint(-2**31, 2**31, (fbq.packed_words(N, K, 4),), dtype=torch.int32, device="cuda", generator=g)
+    scales = (torch.rand((N, 1), device="cuda", generator=g) * 0.015 + 0.005).half()
+    zeros = torch.randint(6, 10, (N, 1), device="cuda", generator=g).half()
+    x = torch.randn((M, K), device="cuda", generator=g).half()
+    A = (torch.randn((r, K), device="cuda", generator=g) * 0.2).half()
+    B = torch.randn((N, r), dtype=torch.float16, device="cuda", generator=g) * 0.1
+    small = slice(0, 4096)
+    for _ in range(2):                                        # the second launch has the number after the first one's
+        y = fbq.linear(x, words, scales, zeros, A, B, N, 128, 4)
+        torch.cuda.synchronize()
+        assert fbq.poll_status() == 0
+        y_small = fbq.linear(x, words[: 4096 * K // 8], scales[small], zeros[small], A, B[small], 4096, 128, 4)
+        rows = torch.cat([torch.arange(0, N, N // 20000, device="cuda"), torch.arange(N - 200, N, device="cuda")])
+        w = scales[rows].double() * (_codes(words, rows, K).double() - zeros[rows].double())
+        want = x.double() @ w.T + (x.double() @ A.double().T) @ B[rows].double().T
+        got = y[:, rows].double()
+        assert float((got - want).norm() / want.norm()) <= REL_F_TOL
+        # row by row: most of an output comes from t, which a row without it would show
+        assert float(((got - want).norm(dim=0) / want.norm(dim=0)).max()) < 0.02
+        assert torch.equal(y_small, y[:, small])              # (one tile's sums do not depend on the grid: one K slice)
+    assert fbq.poll_status() == 0

@@ -286,6 +286,8 @@ int fbq_split_plan(int M, int N, int K, int group, int bits, int rank, int act_i
  *                   test switches of the failure-detection tests: the CTAs that compute t = x.A^T do not
  *                   report it (streaming kernels / prefill kernel), and the prefill kernel's number
  *                   of looks at its flag; with them a bounded wait runs out on purpose
+ *   "test_split_launches"  test switch: not 0 = the next call on the split kernel finds this many launches (as 32 bits) in its
+ *                   stream's count; it sets the switch back to 0
  *   "decode_sk"     0 = automatic, else the number of K slices of the decode kernel
  *   "decode_chunk"  0 = automatic, else quantisation groups per smem stage
  *   "decode_depth"  0 = automatic, else stages in flight per warp

@@ -41,6 +41,7 @@ struct Options {
     int test_prefill_skip_flag = 0, prefill_flag_polls = 0;
     int decode_trace = 0;
     int scratch_mb = 0;
+    int test_split_launches = 0;
 } g_opt;
 // Scratch of the Gram matrix and the reconstruction step; layers of a 7B model and the widest of a 13B model (5120 x 13824, whose
 // H alone has 764 MB) are within two slabs of it.
@@ -218,6 +219,11 @@ int run_split(const LinearArgs *a, int count, const GemvTuning &gt, Workspace *w
     if (e != cudaSuccess) return grow_status(e);
     if ((e = grow(ws->counters, have_c, 16, sizeof(int), s)) != cudaSuccess) return grow_status(e);
     ws->n_counters = (int)have_c;
+    if (g_opt.test_split_launches != 0) {
+        const unsigned long long launches_so_far = (unsigned long long)(unsigned)g_opt.test_split_launches << 32;
+        g_opt.test_split_launches = 0;
+        if (cudaMemcpyAsync(ws->split, &launches_so_far, sizeof launches_so_far, cudaMemcpyHostToDevice, s) != cudaSuccess) return FBQ_ERR_CUDA;
+    }
     if (launch_split(a, count, *ws, gt, s, &launches) != cudaSuccess) return FBQ_ERR_CUDA;
     g_launches += launches;
     return FBQ_OK;
@@ -444,6 +450,7 @@ int *option_slot(const char *name)
     if (!strcmp(name, "hostio_direct_y")) return &g_opt.hostio_direct_y;
     if (!strcmp(name, "test_prefill_skip_flag")) return &g_opt.test_prefill_skip_flag;
     if (!strcmp(name, "prefill_flag_polls")) return &g_opt.prefill_flag_polls;
+    if (!strcmp(name, "test_split_launches")) return &g_opt.test_split_launches;
     if (!strcmp(name, "scratch_mb")) return &g_opt.scratch_mb;
     if (!strcmp(name, "decode_trace")) return &g_opt.decode_trace;
     return nullptr;

@@ -311,8 +311,10 @@ __device__ __forceinline__ void cp_async_wait_stage(int n)
 }
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void *src) { asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory"); }
 
-// This launch's number, which the words of its t carry.
-__device__ __forceinline__ uint32_t launch_number(const unsigned long long *epoch) { return (uint32_t)(__ldcg(epoch) >> 32) + 1u; }
+// This launch's number, which the words of its t carry: never 0, which words that no launch has written hold and lanes that have
+// not looked yet.  It comes round after 2^31 launches; a word still holds the number of that many launches ago only where no call
+// since then had as many tokens and ranks, and is written by this launch's t CTA all the same.
+__device__ __forceinline__ uint32_t launch_number(const unsigned long long *epoch) { return (uint32_t)(__ldcg(epoch) >> 32) | 0x80000000u; }
 
 template <typename T, int MT>
 __device__ __forceinline__ void t_program(const SplitParams &sp, const SplitDims &p, uint8_t *smem, int lc, int crank, int g0, int Gs)
@@ -603,7 +605,7 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
         if (!waited && !mbar_wait(rbar + 8u * (pass & 1), (uint32_t)(pass >> 1) & 1u)) atomicExch(sp.status, (int)FBQ_ERR_TIMEOUT);
     };
 
-    uint4 tw = make_uint4(0u, 0u, 0u, 0u);
+    uint4 tw = make_uint4(0u, 0u, 0u, 0u);                                    // (no launch's number: a lane without an early look)
     int slot = 0, mt = 0;                                                     // mt: tiles this warp is through with
 #pragma unroll 1
     for (int pass = 0; pass < npass; ++pass) {

@@ -1,7 +1,9 @@
-"""The split kernel's count of launches, whose numbers the words of t carry: grids of more than 65536 CTAs."""
+"""The split kernel's count of launches, whose numbers the words of t carry: grids of more than 65536 CTAs, and
+counts at which a number of 32 bits, or of 31, comes round."""
 import pytest
 
-from gpu_utils import REL_F_TOL
+from gpu_utils import DeviceLinear, REL_F_TOL, check_parity
+from workloads import make_linear
 
 pytestmark = pytest.mark.gpu
 
@@ -42,3 +44,30 @@ def test_more_than_65536_ctas():
         assert float(((got - want).norm(dim=0) / want.norm(dim=0)).max()) < 0.02
         assert torch.equal(y_small, y[:, small])              # (one tile's sums do not depend on the grid: one K slice)
     assert fbq.poll_status() == 0
+
+
+@pytest.mark.parametrize("launches", [-2, -1, 2**31 - 2, 2**31 - 1, -2**31])
+@pytest.mark.parametrize("M,N,K,rank,ctas", [(16, 200, 1024, 64, 0), (8, 40, 512, 128, 0), (16, 1096, 1024, 64, 2)])
+def test_number_comes_round(launches, M, N, K, rank, ctas):
+    # fewer tiles than warps, so that some warps multiply no tile and have not looked at t when they take it in, and (the last
+    # one) tiles in several passes, where none has: each launch around the turn waits for its own t
+    import torch
+    import paper_2501_16385_b200 as fbq
+    inp = make_linear(M, N, K, 4, rank, seed=7700 + M + N, ab_std=0.141)
+    dev = DeviceLinear(inp, fbq)
+    assert fbq.split_plan(M, N, K, 128, 4, rank) is not None
+    fbq.set_option("gemv_ctas", ctas)
+    try:
+        check_parity(inp, fbq, threads=16)
+        want = dev.run(fbq)
+        other = -dev.x                                        # in between: another t in the same words
+        negative = dev.run(fbq, x=other)
+        torch.cuda.synchronize()
+        fbq.set_option("test_split_launches", launches)
+        for _ in range(4):
+            assert torch.equal(dev.run(fbq), want)
+            assert torch.equal(dev.run(fbq, x=other), negative)
+        torch.cuda.synchronize()
+    finally:
+        fbq.set_option("gemv_ctas", 0)
+    assert fbq.get_option("test_split_launches") == 0 and fbq.poll_status() == 0

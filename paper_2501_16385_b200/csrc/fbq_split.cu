@@ -31,6 +31,7 @@
 //
 // 3 to 16 tokens; one problem, or several problems that run as one launch.
 #include <algorithm>
+#include <cfloat>
 #include <cstring>
 #include <type_traits>
 #include <unordered_map>
@@ -53,6 +54,7 @@ constexpr int kStageA = 4096;                // of a stage of a t CTA: one group
 constexpr size_t kSmemAll = 227 * 1024;
 constexpr int kOffBar = 0;                   // one barrier per receive buffer
 constexpr int kOffDims = 64;
+constexpr int kOffOver = 256;                // a word per warp: tokens whose x it could not stage scaled up (stage_x)
 constexpr int kOffX = 512;
 
 struct alignas(16) SplitDims {
@@ -77,7 +79,7 @@ struct SplitParams {
     unsigned long long *epoch;               // 2^32 x the number of launches so far, plus the CTAs of this one that are through
     SplitDims p[kMostProblems];
 };
-static_assert(kOffDims + sizeof(SplitDims) <= kOffX, "");
+static_assert(kOffDims + sizeof(SplitDims) <= kOffOver && kOffOver + kW * 4 <= kOffX, "");
 
 template <typename T> __device__ __forceinline__ void mma16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -123,15 +125,12 @@ template <> __device__ __forceinline__ float2 pair_to_float<__nv_bfloat16>(uint3
 {
     return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
 }
-// The pair divided by 2^p (rounded once, exact but for underflow).
-template <typename T> __device__ __forceinline__ uint32_t pair_scaled(uint32_t v, int p)
+// The pair times f, rounded once.
+template <typename T> __device__ __forceinline__ uint32_t pair_scaled(uint32_t v, float f)
 {
-    if (p == 0) return v;
     using T2 = typename ActTraits<T>::T2;
-    const T f = ActTraits<T>::from_float(1.f / (float)(1 << p));
     T2 f2;
-    f2.x = f;
-    f2.y = f;
+    f2.x = f2.y = ActTraits<T>::from_float(f);
     const T2 r = __hmul2(*reinterpret_cast<const T2 *>(&v), f2);
     return *reinterpret_cast<const uint32_t *>(&r);
 }
@@ -171,10 +170,17 @@ template <typename T> __device__ __forceinline__ uint32_t pair_of(float v)
 // Two runs are on their way at a time, and never one too many: every CTA asks L2 for the same lines at the same moment, and a load
 // that only repeats another costs a launch 0.3 to 0.45 us (4096 -> 4096, 8 tokens, rank 128: with one 7.95 us, with two 8.4, with
 // none 7.6).
+// What is staged is up x / 2^p, 2^p the field weight of the code that meets x.  In fp16 x / 2^p would be rounded to multiples of 2^-24, so
+// `up` is 2^kUp, the largest field weight: nothing is rounded, and `finish` takes it out of the sums.  |x| of 65520 / up and more comes
+// out infinite then, which the sums tell: the return value names the tokens (bit t: token 2t of the eight, bit 4 + t: 2t + 1; the warps of
+// a part are a multiple of MT, so that all runs of a lane belong to one).  The part is staged again with up = 1 for these, where
+// a rounding of 2^-19 is nothing beside an x of 1000. 
+template <int BITS, typename T> constexpr int kUp = std::is_same_v<T, __half> ? (BITS == 4 ? 4 : 6) : 0;      // (bf16 has the exponents)
 template <int BITS, typename T, int MT>
-__device__ __forceinline__ void stage_x(const T *x, int K, int M, bool wide, uint8_t *xs, float4 *px, int groups, int part, int parts, int lane)
+__device__ __forceinline__ uint32_t stage_x(const T *x, int K, int M, bool wide, uint8_t *xs, float4 *px, int groups, int part, int parts, int lane, float up)
 {
     const int n = lane >> 2, t = lane & 3, total = groups * MT;
+    bool over0 = false, over1 = false;
     auto load = [&](int it, uint32_t (&e)[16]) {
         const int grp = it / MT, b = it - grp * MT;
         load_run(x + (size_t)min(8 * b + n, M - 1) * K + grp * kGroupFast + 32 * t, wide, e);
@@ -186,13 +192,18 @@ __device__ __forceinline__ void stage_x(const T *x, int K, int M, bool wide, uin
         for (int j = 0; j < 16; ++j) {
             constexpr auto div = [](int c) { return Unpack16<BITS, T>::div_log2(c); };
             const int c0 = pair_first<BITS>(j), c1 = pair_second<BITS>(j);
-            h[j] = pair_scaled<T>(__byte_perm(e[c0 >> 1], e[c1 >> 1], ((c0 & 1) ? 0x32u : 0x10u) | ((c1 & 1) ? 0x7600u : 0x5400u)), div(c0));
+            h[j] = __byte_perm(e[c0 >> 1], e[c1 >> 1], ((c0 & 1) ? 0x32u : 0x10u) | ((c1 & 1) ? 0x7600u : 0x5400u));
+            if (kUp<BITS, T> > 0 || div(c0) > 0) h[j] = pair_scaled<T>(h[j], up / (float)(1 << div(c0)));
             if (j & 1)
                 mma16<T>(d, pair_of<T>(1.f), pair_of<T>((float)(1 << div(pair_first<BITS>(j - 1)))), pair_of<T>(1.f), pair_of<T>((float)(1 << div(c0))), h[j - 1], h[j]);
         }
 #pragma unroll
         for (int q4 = 0; q4 < 4; ++q4)
             *reinterpret_cast<uint4 *>(xs + (((it * 4 + q4) * 32 + lane) << 4)) = make_uint4(h[4 * q4], h[4 * q4 + 1], h[4 * q4 + 2], h[4 * q4 + 3]);
+        if constexpr (kUp<BITS, T> > 0) {
+            over0 = over0 || !(fabsf(d[2]) <= FLT_MAX);
+            over1 = over1 || !(fabsf(d[3]) <= FLT_MAX);
+        }
         if (lane < 4) px[it * 4 + lane] = make_float4(-Unpack16<BITS, T>::kMagic * d[0], -Unpack16<BITS, T>::kMagic * d[1], d[2], d[3]);
     };
     int it = part;
@@ -209,6 +220,8 @@ __device__ __forceinline__ void stage_x(const T *x, int K, int M, bool wide, uin
         load(it, e);
         convert(it, e);
     }
+    if constexpr (kUp<BITS, T> > 0) return (__ballot_sync(0xFFFFFFFFu, over0) & 15u) | (__ballot_sync(0xFFFFFFFFu, over1) & 15u) << 4;
+    return 0u;
 }
 // The same for a t CTA: x as it is.
 template <typename T, int MT>
@@ -539,9 +552,29 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
     if (threadIdx.x == 0) mbar_expect_tx(rbar, (uint32_t)(owned(2 * min(PT, ntiles), cs_log2, crank) << (cs_log2 + wkl)) * MT * 512);
     pdl_wait();
     const uint32_t tag = launch_number(sp.epoch);
-    stage_x<BITS, T, MT>(x, K, M, wide, xs, px, mine, wr, wr_n, lane);
-    cp_async_wait_stage(stages);                                              // the first stage, and with it the scales and B
-    __syncthreads();
+    constexpr float kScaled = (float)(1 << kUp<BITS, T>);
+    uint32_t *overs = reinterpret_cast<uint32_t *>(smem + kOffOver);
+    auto over_of = [&](int b) {                                               // of the tokens 8b ..., in this warp's part of the slice
+        uint32_t v = 0u;
+#pragma unroll 1
+        for (int r = b; r < wr_n; r += MT) v |= overs[wk + (r << wkl)];
+        return v;
+    };
+    float up = kScaled;
+    bool again = false;
+#pragma unroll 1
+    for (;;) {
+        const uint32_t over = stage_x<BITS, T, MT>(x, K, M, wide, xs, px, mine, wr, wr_n, lane, up);
+        cp_async_wait_stage(stages);                                          // the first stage, and with it the scales and B
+        if constexpr (kUp<BITS, T> == 0) {
+            __syncthreads();
+            break;
+        }
+        if (lane == 0 && !again) overs[warp] = over;
+        if (!__syncthreads_or(!again && over != 0)) break;
+        again = true;
+        up = over_of(wr % MT) >> ((lane >> 3) + (lane & 4)) & 1u ? 1.f : kScaled;
+    }
     cluster_wait();                                                           // the other CTAs of the cluster have started
 
     // ---- granules of 16 rows that this CTA finishes: t.B^T, partial sums added in order, one rounding, store ----
@@ -595,7 +628,7 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
             T *ybuf = reinterpret_cast<T *>(rbase + ((((size_t)s << (cs_log2 + wkl)) * MT + b) << 9));
             __syncwarp();
 #pragma unroll
-            for (int c = 0; c < 4; ++c) ybuf[(2 * t + (c & 1)) * 16 + g + 8 * (c >> 1)] = ActTraits<T>::from_float(m4[c] + sum[c]);
+            for (int c = 0; c < 4; ++c) ybuf[(2 * t + (c & 1)) * 16 + g + 8 * (c >> 1)] = ActTraits<T>::from_float(fmaf(m4[c], 1.f / kScaled, sum[c]));
             __syncwarp();
             const int m = 8 * b + (lane >> 1), n = row0 + 8 * (lane & 1);
             if (lane < 16 && m < M && n < N) *reinterpret_cast<uint4 *>(y + (size_t)m * N + n) = *reinterpret_cast<const uint4 *>(ybuf + lane * 8);
@@ -636,6 +669,16 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
                 issue();
                 cp_async_commit();
                 if (++slot == stages) slot = 0;
+            }
+            if (again) {                                                      // tokens staged with up = 1: the factor that all sums carry
+#pragma unroll
+                for (int b = 0; b < MT; ++b) {
+                    const uint32_t over = over_of(b) >> t;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) acc[h][b][c] *= (over >> (4 * (c & 1))) & 1u ? kScaled : 1.f;
+                }
             }
             send_granule<MT>(recv, bar_r, 2 * ti, cs_log2, crank, wkl, wk, lane, acc[0]);
             send_granule<MT>(recv, bar_r, 2 * ti + 1, cs_log2, crank, wkl, wk, lane, acc[1]);

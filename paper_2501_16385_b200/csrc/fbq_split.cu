@@ -92,18 +92,6 @@ template <typename T> __device__ __forceinline__ void mma16(float (&d)[4], uint3
             : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
             : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// The same, started at (c0, c1) in both rows.
-template <typename T> __device__ __forceinline__ void mma16_from(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1, float c0, float c1)
-{
-    if constexpr (std::is_same_v<T, __half>)
-        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%10,%11};"
-            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c0), "f"(c1));
-    else
-        asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%10,%11};"
-            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c0), "f"(c1));
-}
 __device__ __forceinline__ void mma_tf32(float (&d)[4], const float (&a)[4], float b0, float b1)
 {
     asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -165,8 +153,13 @@ template <typename T> __device__ __forceinline__ uint32_t pair_of(float v)
 // x of the groups that this warp multiplies, as MMA column fragments [group][eight tokens][quarter of the run][lane] of 16 bytes.
 // Lane (token, t) of a fragment needs the run of 32 elements that codes run t of a weight row meet, so it loads that run itself:
 // nothing crosses lanes but what the two warps that share the groups stage for each other.  The unpacker's order and field
-// weights are applied to x here; (-P, X0) of a token and group, P = MAGIC sum of the staged x and X0 = sum of x, come out of
-// MMAs against rows of ones and of field weights, in the lanes that need them.  Tokens past M repeat the last one.
+// weights are applied to x here; (P, X0) of a token and group, the sums of (MAGIC + 2^p kMid) times the staged x and of x, come out of
+// MMAs against such rows and rows of field weights, in the lanes that need them.  Tokens past M repeat the last one.
+// The tensor core cuts its sums off towards zero, here 1024 times as large as what is left of them, and columns of x that are
+// large are so in every group: what a group's products lose, P has to lose as well.  So P is made by the same MMAs in the same order,
+// with codes of kMid, and subtracted at the end.  Relative error of y, INT3, fp16, 13824 inputs, one column of each group 1000 times
+// as large as the rest / all x of one sign: 2.3e-4 / 2.8e-4, of which the rounding of y is 2.1e-4.  (Products started from
+// -MAGIC sum x, an addition less: 1.2e-3 / 2.5e-4; kMid 0: 2.5e-4 / 1.1e-3, half way between the codes 2.4e-4 / 4.2e-4.)
 // Two runs are on their way at a time, and never one too many: every CTA asks L2 for the same lines at the same moment, and a load
 // that only repeats another costs a launch 0.3 to 0.45 us (4096 -> 4096, 8 tokens, rank 128: with one 7.95 us, with two 8.4, with
 // none 7.6).
@@ -174,7 +167,9 @@ template <typename T> __device__ __forceinline__ uint32_t pair_of(float v)
 // `up` is 2^kUp, the largest field weight: nothing is rounded, and `finish` takes it out of the sums.  |x| of 65520 / up and more comes
 // out infinite then, which the sums tell: the return value names the tokens (bit t: token 2t of the eight, bit 4 + t: 2t + 1; the warps of
 // a part are a multiple of MT, so that all runs of a lane belong to one).  The part is staged again with up = 1 for these, where
-// a rounding of 2^-19 is nothing beside an x of 1000. 
+// a rounding of 2^-19 is nothing beside an x of 1000.  (13B layer, 16 tokens, fp16:
+// 101.5 us, 99.8 with x / 2^p and no second pass; with small x found by the sum of |x| instead, and staged again scaled up, 103.0.)
+template <int BITS> constexpr float kMid = BITS == 4 ? 6.f : 2.f;
 template <int BITS, typename T> constexpr int kUp = std::is_same_v<T, __half> ? (BITS == 4 ? 4 : 6) : 0;      // (bf16 has the exponents)
 template <int BITS, typename T, int MT>
 __device__ __forceinline__ uint32_t stage_x(const T *x, int K, int M, bool wide, uint8_t *xs, float4 *px, int groups, int part, int parts, int lane, float up)
@@ -194,8 +189,11 @@ __device__ __forceinline__ uint32_t stage_x(const T *x, int K, int M, bool wide,
             const int c0 = pair_first<BITS>(j), c1 = pair_second<BITS>(j);
             h[j] = __byte_perm(e[c0 >> 1], e[c1 >> 1], ((c0 & 1) ? 0x32u : 0x10u) | ((c1 & 1) ? 0x7600u : 0x5400u));
             if (kUp<BITS, T> > 0 || div(c0) > 0) h[j] = pair_scaled<T>(h[j], up / (float)(1 << div(c0)));
-            if (j & 1)
-                mma16<T>(d, pair_of<T>(1.f), pair_of<T>((float)(1 << div(pair_first<BITS>(j - 1)))), pair_of<T>(1.f), pair_of<T>((float)(1 << div(c0))), h[j - 1], h[j]);
+            if (j & 1) {
+                constexpr float magic = Unpack16<BITS, T>::kMagic;
+                const float w0 = (float)(1 << div(pair_first<BITS>(j - 1))), w1 = (float)(1 << div(c0));
+                mma16<T>(d, pair_of<T>(magic + w0 * kMid<BITS>), pair_of<T>(w0), pair_of<T>(magic + w1 * kMid<BITS>), pair_of<T>(w1), h[j - 1], h[j]);
+            }
         }
 #pragma unroll
         for (int q4 = 0; q4 < 4; ++q4)
@@ -204,7 +202,7 @@ __device__ __forceinline__ uint32_t stage_x(const T *x, int K, int M, bool wide,
             over0 = over0 || !(fabsf(d[2]) <= FLT_MAX);
             over1 = over1 || !(fabsf(d[3]) <= FLT_MAX);
         }
-        if (lane < 4) px[it * 4 + lane] = make_float4(-Unpack16<BITS, T>::kMagic * d[0], -Unpack16<BITS, T>::kMagic * d[1], d[2], d[3]);
+        if (lane < 4) px[it * 4 + lane] = make_float4(d[0], d[1], d[2], d[3]);
     };
     int it = part;
 #pragma unroll 1
@@ -268,24 +266,23 @@ __device__ __forceinline__ void multiply_group(const uint8_t *codes, const uint8
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         fs[r] = __half2float(*reinterpret_cast<const __half *>(sc + r * srow8));
-        fz[r] = __half2float(*reinterpret_cast<const __half *>(sc + r * srow8 + zoff));
+        fz[r] = kMid<BITS> - __half2float(*reinterpret_cast<const __half *>(sc + r * srow8 + zoff));
     }
-    float d[2][MT][4], x0[MT][2];
+    float d[2][MT][4] = {}, p[MT][2], x0[MT][2];
 #pragma unroll
     for (int q4 = 0; q4 < 4; ++q4)
 #pragma unroll
         for (int b = 0; b < MT; ++b) {
             const uint4 xv = *reinterpret_cast<const uint4 *>(xg + (b * 4 + q4) * 512);
             if (q4 == 0) {
-                const float4 v = *reinterpret_cast<const float4 *>(pxg + b * 64);     // (-P, -P, X0, X0) of tokens 8b + 2t, 8b + 2t + 1
+                const float4 v = *reinterpret_cast<const float4 *>(pxg + b * 64);     // (P, P, X0, X0) of tokens 8b + 2t, 8b + 2t + 1
+                p[b][0] = v.x;
+                p[b][1] = v.y;
                 x0[b][0] = v.z;
                 x0[b][1] = v.w;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) mma16_from<T>(d[h][b], ha[h][0], hb[h][0], ha[h][1], hb[h][1], xv.x, xv.y, v.x, v.y);
-            } else {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) mma16<T>(d[h][b], ha[h][4 * q4], hb[h][4 * q4], ha[h][4 * q4 + 1], hb[h][4 * q4 + 1], xv.x, xv.y);
             }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) mma16<T>(d[h][b], ha[h][4 * q4], hb[h][4 * q4], ha[h][4 * q4 + 1], hb[h][4 * q4 + 1], xv.x, xv.y);
 #pragma unroll
             for (int h = 0; h < 2; ++h) mma16<T>(d[h][b], ha[h][4 * q4 + 2], hb[h][4 * q4 + 2], ha[h][4 * q4 + 3], hb[h][4 * q4 + 3], xv.z, xv.w);
         }
@@ -297,7 +294,7 @@ __device__ __forceinline__ void multiply_group(const uint8_t *codes, const uint8
             for (int b = 0; b < MT; ++b)
 #pragma unroll
                 for (int c = 0; c < 2; ++c)
-                    acc[h][b][2 * r + c] = fmaf(fs[2 * h + r], fmaf(-fz[2 * h + r], x0[b][c], d[h][b][2 * r + c]), acc[h][b][2 * r + c]);
+                    acc[h][b][2 * r + c] = fmaf(fs[2 * h + r], fmaf(fz[2 * h + r], x0[b][c], d[h][b][2 * r + c] - p[b][c]), acc[h][b][2 * r + c]);
         }
 }
 

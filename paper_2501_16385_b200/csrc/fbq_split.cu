@@ -415,8 +415,9 @@ __device__ __forceinline__ void t_program(const SplitParams &sp, const SplitDims
         }
 }
 
+// Returns whether one of this thread's sums is not finite.
 template <int BITS, typename T, int MT>
-__device__ __forceinline__ void main_program(const SplitParams &sp, const SplitDims &p, uint8_t *smem, int lc, int crank, int g0, int Gs)
+__device__ __forceinline__ bool main_program(const SplitParams &sp, const SplitDims &p, uint8_t *smem, int lc, int crank, int g0, int Gs)
 {
     constexpr int GB = BITS == 4 ? 64 : 48, kUnits = GB / 16;                 // bytes of a row and group, 16-byte units
     // (fields that are used past the wait are read here: shared memory would be read again after every barrier)
@@ -575,6 +576,7 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
     cluster_wait();                                                           // the other CTAs of the cluster have started
 
     // ---- granules of 16 rows that this CTA finishes: t.B^T, partial sums added in order, one rounding, store ----
+    uint32_t infinite = 0u;                                                   // 0 times the sums, as bits: NaN where one is not finite
     auto finish = [&](int pass) {
         const int pn = min(PT, ntiles - pass * PT), prow0 = nrow0 + pass * PT * kRows, pslot0 = (2 * pass * PT) >> cs_log2;
         uint8_t *rbase = recv0 + (pass & 1) * pass_bytes;
@@ -621,6 +623,7 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
 #pragma unroll
                 for (int k = 0; k < 4; ++k) { m4[0] += o[k].x; m4[1] += o[k].y; m4[2] += o[k].z; m4[3] += o[k].w; }
             }
+            infinite |= __float_as_uint(((m4[0] + m4[1]) + (m4[2] + m4[3])) * 0.f);
             // rows in order through shared memory (the place of this warp's own sums of the granule), whole 16 bytes per store
             T *ybuf = reinterpret_cast<T *>(rbase + ((((size_t)s << (cs_log2 + wkl)) * MT + b) << 9));
             __syncwarp();
@@ -710,6 +713,48 @@ __device__ __forceinline__ void main_program(const SplitParams &sp, const SplitD
             cluster_arrive();
         }
     }
+    return (infinite & 0x7F800000u) != 0;
+}
+
+// The outputs of this CTA that are not finite once more, product by product.  With an infinite x the sums of (MAGIC + 2^p q) x and P are
+// both infinite and their difference is NaN, where a weight times x is infinite; the largest x of bf16 overflow in P alone.
+// (What it costs launches that need none of it: 32 x 7 linears of a 7B model, 8 tokens, bf16, 2121 -> 2175 us, 13B layer, 16 tokens, fp16,
+// 101.4 -> 101.7; with this in `finish`, where a sum turns out so, 2198 and 103.8.)
+template <int BITS, typename T>
+__device__ __noinline__ void redo_rows(const SplitDims &p, const uint8_t *smem, int M, int lc, int crank, int cs_log2)
+{
+    constexpr int NW = BITS == 4 ? 4 : 3;
+    const int nrow0 = lc * p.R * kRows, ngran = 2 * min(p.R, p.tiles - lc * p.R);
+    T *y = static_cast<T *>(p.y);
+#pragma unroll 1
+    for (int e = threadIdx.x; e < 16 * M * owned(ngran, cs_log2, crank); e += kThr) {
+        const int slot = e / (16 * M), token = e / 16 % M, row = nrow0 + ((slot << cs_log2) + crank) * 16 + e % 16;
+        if (row >= p.N || fabsf(ActTraits<T>::to_float(y[(size_t)token * p.N + row])) <= FLT_MAX) continue;
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(p.qw) + (size_t)row * p.G * 4 * NW;
+        const unsigned short *x = static_cast<const unsigned short *>(p.x) + (size_t)token * p.K;
+        float sum = 0.f, sub = 0.f;
+#pragma unroll 1
+        for (int run = 0; run < 4 * p.G; ++run, w += NW, x += 32) {
+            const size_t at = (size_t)row * p.G + (run >> 2);
+            const float s = __half2float(p.scales[at]), z = __half2float(p.zeros[at]);
+            uint32_t h[16];
+            Unpack16<BITS, T>::run(w, h);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const int c0 = pair_first<BITS>(j), c1 = pair_second<BITS>(j);
+                const float2 q = pair_to_float<T>(h[j]);
+                const float down = 1.f / (float)(1 << Unpack16<BITS, T>::div_log2(c0));
+                const unsigned short x0 = __ldcg(x + c0), x1 = __ldcg(x + c1);
+                sum = fmaf(s * ((q.x - Unpack16<BITS, T>::kMagic) * down - z), ActTraits<T>::to_float(*reinterpret_cast<const T *>(&x0)), sum);
+                sum = fmaf(s * ((q.y - Unpack16<BITS, T>::kMagic) * down - z), ActTraits<T>::to_float(*reinterpret_cast<const T *>(&x1)), sum);
+            }
+        }
+        const T *b = reinterpret_cast<const T *>(smem + p.off_b + (slot * 16 + e % 16) * (p.rank * 2 + 16));
+        const float *t = reinterpret_cast<const float *>(smem + p.off_t) + token * (p.rank + 16);
+#pragma unroll 1
+        for (int j = 0; j < p.rank; ++j) sub = fmaf(t[j], ActTraits<T>::to_float(b[j]), sub);
+        y[(size_t)token * p.N + row] = ActTraits<T>::from_float(sum + sub);
+    }
 }
 
 template <int BITS, typename T, int MT>
@@ -740,12 +785,13 @@ __global__ void __launch_bounds__(kThr, 1) split_kernel(const __grid_constant__ 
             mbar_expect_tx(smem_u32(smem) + kOffBar, (uint32_t)(owned(ngran, sp.cs_log2, crank) << sp.cs_log2) * kTWK * MT * 512u);
         }
         t_program<T, MT>(sp, p, smem, lc, crank, g0, Gs);
+        __syncthreads();
     } else {
-        main_program<BITS, T, MT>(sp, p, smem, cluster - p.first_mc, crank, g0, Gs);
+        if (__syncthreads_or(main_program<BITS, T, MT>(sp, p, smem, cluster - p.first_mc, crank, g0, Gs)))
+            redo_rows<BITS, T>(p, smem, sp.M, cluster - p.first_mc, crank, sp.cs_log2);
     }
     // Every CTA read the launch's number before this; with the last one the count of launches goes up by one.  (The CTAs that are
     // through have 32 bits: grids of wide layers, 4096 -> 8 000 000, say, hold more than 65536 CTAs.)
-    __syncthreads();
     if (threadIdx.x == 0) atomicAdd(sp.epoch, blockIdx.x == 0 ? (1ull << 32) - (gridDim.x - 1) : 1ull);
 }
 

@@ -1,6 +1,6 @@
 """Calls of 3 to 16 tokens on inputs at the ends of the formats: x so small that its quotients by the field weights of the codes
 are subnormal in fp16, in all of a token, in some of its groups, beside larger ones, and in some tokens only; x so large that it
-cannot be scaled up against that; columns of x that are large in every group, and x of one sign."""
+cannot be scaled up against that; columns of x that are large in every group, and x of one sign; infinities and NaN."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -81,4 +81,38 @@ def test_large_columns(bits, M, K):
         x = x.half()
         want = x.double() @ w.T
         assert float(((run(x).double() - want).norm(dim=1) / want.norm(dim=1)).max()) <= 4e-4
+    assert fbq.poll_status() == 0
+
+
+@pytest.mark.parametrize("bits,dtype,M,K,rank", [(3, "f16", 16, 5120, 0), (4, "bf16", 16, 5120, 0), (4, "f16", 12, 5120, 32), (3, "bf16", 9, 13824, 0),
+                                                 (3, "f16", 4, 1152, 32), (4, "bf16", 8, 128, 0)])
+def test_infinite_and_huge_x(bits, dtype, M, K, rank):
+    # infinities of the sign of x times the weight, NaN where such meet or the weight is 0, in the tokens that hold them and no others
+    import torch
+    import paper_2501_16385_b200 as fbq
+    run, w, A, B, g = _problem(fbq, M, 72, K, bits, rank, dtype, 500 * bits + M)
+    act = torch.float16 if dtype == "f16" else torch.bfloat16
+    x = torch.randn((M, K), device="cuda", generator=g).to(act)
+    clean = run(x)
+    inf = float("inf")
+    x[0, 3], x[0, K - 1] = inf, inf
+    x[1, 77] = -inf
+    x[2, 5], x[2, K - 1 - 127] = inf, -inf
+    if M > 3:
+        x[M - 1, K // 2] = float("nan")
+    if M > 8 and dtype == "bf16":
+        x[8] = 2e35 * torch.rand((K,), device="cuda", generator=g).to(act)     # 128 times their sum is beyond fp32, y is not
+    want = (x.double()[:, None, :] * w[None]).sum(-1)
+    if rank:
+        t = (x.double()[:, None, :] * A.double()[None]).sum(-1)
+        want = want + (t[:, None, :] * B.double()[None]).sum(-1)
+    y = run(x)
+    assert torch.equal(y.isnan(), want.isnan()) and torch.equal(y.isinf(), want.isinf())
+    assert torch.equal(y[y.isinf()].sign().double(), want[want.isinf()].sign())
+    assert y[:2].isinf().any() or rank
+    same = [m for m in range(3, M - 1) if m != 8]
+    assert torch.equal(y[same], clean[same])
+    if M > 8 and dtype == "bf16":
+        assert float((y[8].double() - want[8]).norm() / want[8].norm()) < 2.0 ** -8
+    torch.cuda.synchronize()
     assert fbq.poll_status() == 0

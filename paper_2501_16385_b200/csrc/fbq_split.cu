@@ -62,7 +62,7 @@ struct alignas(16) SplitDims {
     const uint8_t *qw;
     const __half *scales, *zeros;
     void *y;
-    uint2 *t;                                // words of t, [token][rank]: value, number of the launch
+    unsigned long long *t;                   // words of t, [token][rank]: value, above it the number of the launch
     int N, K, G, rank;
     int tiles, R, PT;                        // tiles of the problem, of a cluster, of a pass
     int first_tc, first_mc;                  // first cluster
@@ -310,6 +310,19 @@ __device__ __forceinline__ void send_granule(uint32_t recv, uint32_t bar, int gi
 // Granules of `n` that CTA `crank` finishes.
 __device__ __forceinline__ int owned(int n, int cs_log2, int crank) { return (n + (1 << cs_log2) - 1 - crank) >> cs_log2; }
 
+// A word of t: value and number of the launch, an element of 64 bits to both accesses, so that whoever sees the number sees the value.
+// (Of the elements of a vector access nothing says that they are seen together.)
+__device__ __forceinline__ void store_t(unsigned long long *w, float v, uint32_t tag)
+{
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(w), "l"((unsigned long long)tag << 32 | __float_as_uint(v)));
+}
+__device__ __forceinline__ uint4 load_t2(const unsigned long long *w)        // two of them
+{
+    unsigned long long a, b;
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(w));
+    return make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
+}
+
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 // All but the latest n - 1 groups of copies of this thread have arrived.
 __device__ __forceinline__ void cp_async_wait_stage(int n)
@@ -361,7 +374,7 @@ __device__ __forceinline__ void t_program(const SplitParams &sp, const SplitDims
     uint8_t *xs = smem + kOffX + (size_t)gb * MT * 2048;
     const T *x = static_cast<const T *>(p.x) + (size_t)(g0 + gb) * kGroupFast;
     const bool wide = p.x_wide != 0;
-    uint2 *tw = p.t;
+    unsigned long long *tw = p.t;
     pdl_wait();
     const uint32_t tag = launch_number(sp.epoch);
     stage_x_plain<T, MT>(x, K, M, wide, xs, mine, wr, lane);
@@ -411,7 +424,7 @@ __device__ __forceinline__ void t_program(const SplitParams &sp, const SplitDims
                 for (int k = 0; k < kTWK; ++k) v += w[k];
             }
             const int l = (e >> 2) & 31, token = (e >> 7) * 8 + 2 * (l & 3) + (e & 1), row = row0 + gran * 16 + (l >> 2) + 8 * ((e >> 1) & 1);
-            if (token < M && row < rank && !sp.skip_t) __stcg(tw + (size_t)token * rank + row, make_uint2(__float_as_uint(v), tag));
+            if (token < M && row < rank && !sp.skip_t) store_t(tw + (size_t)token * rank + row, v, tag);
         }
 }
 
@@ -540,7 +553,7 @@ __device__ __forceinline__ bool main_program(const SplitParams &sp, const SplitD
     float4 *px = reinterpret_cast<float4 *>(smem + p.off_px) + gb * 4 * MT;
     const T *x = static_cast<const T *>(p.x) + (size_t)(g0 + gb) * kGroupFast;
     T *y = static_cast<T *>(p.y);
-    const uint4 *twords = reinterpret_cast<const uint4 *>(p.t);
+    const unsigned long long *twords = p.t;
     const bool wide = p.x_wide != 0;
     const uint8_t *codes0 = smem + p.off_ring + warp * stages * stage_bytes + g * GB + t * (GB / 4);
     const int rq = rank / 2, trow = rank + 16;                                // pairs of words of a token's t; floats of its row in shared memory
@@ -638,7 +651,7 @@ __device__ __forceinline__ bool main_program(const SplitParams &sp, const SplitD
         if (!waited && !mbar_wait(rbar + 8u * (pass & 1), (uint32_t)(pass >> 1) & 1u)) atomicExch(sp.status, (int)FBQ_ERR_TIMEOUT);
     };
 
-    uint4 tw = make_uint4(0u, 0u, 0u, 0u);                                    // (no launch's number: a lane without an early look)
+    uint4 tw = make_uint4(0u, 0u, 0u, 0u);                                     // (no launch's number: a lane without an early look)
     int slot = 0, mt = 0;                                                     // mt: tiles this warp is through with
 #pragma unroll 1
     for (int pass = 0; pass < npass; ++pass) {
@@ -652,7 +665,7 @@ __device__ __forceinline__ bool main_program(const SplitParams &sp, const SplitD
         if (pass > 0 && threadIdx.x == 0) mbar_expect_tx(bar_r, (uint32_t)(owned(2 * pn, cs_log2, crank) << (cs_log2 + wkl)) * MT * 512);
 #pragma unroll 1
         for (int ti = wr; ti < pn; ti += wr_n, ++mt) {
-            if (npass == 1 && mt == my_tiles - 1 && warp < M && lane < rq) tw = __ldcg(twords + warp * rq + lane);   // an early look at t
+            if (npass == 1 && mt == my_tiles - 1 && warp < M && lane < rq) tw = load_t2(twords + warp * rank + 2 * lane);     // an early look at t
             float acc[2][MT][4] = {};
             const uint8_t *scl = sc + ((pass * PT + ti) * 2 * kRows + g) * spitch + (sh + gb) * 2;
 #pragma unroll 1
@@ -693,7 +706,7 @@ __device__ __forceinline__ bool main_program(const SplitParams &sp, const SplitD
                         const unsigned long long t0 = global_ns();
 #pragma unroll 1
                         for (int looks = 1;; ++looks) {
-                            w = __ldcg(twords + m * rq + q);
+                            w = load_t2(twords + m * rank + 2 * q);
                             if (w.y == tag && w.w == tag) break;
                             if (sp.poll_limit > 0 ? looks >= sp.poll_limit : ((looks & 31) == 0 && global_ns() - t0 > kWaitNs)) {
                                 atomicExch(sp.status, (int)FBQ_ERR_TIMEOUT);
@@ -1061,7 +1074,7 @@ size_t split_scratch_bytes(const LinearArgs *a, int count)
 {
     size_t words = 16;                                               // the launch number's line
     for (int i = 0; i < count; ++i) words += t_words(a[i]);
-    return words * sizeof(uint2);
+    return words * sizeof(unsigned long long);
 }
 
 cudaError_t launch_split(const LinearArgs *a, int count, Workspace &ws, const GemvTuning &tune, cudaStream_t st, int *launches)
@@ -1078,7 +1091,7 @@ cudaError_t launch_split(const LinearArgs *a, int count, Workspace &ws, const Ge
         SplitDims &p = s.sp.p[i];
         p.x_wide = (reinterpret_cast<uintptr_t>(a[i].x) & 31) == 0;
         p.x = a[i].x; p.A = a[i].A; p.B = a[i].B; p.qw = reinterpret_cast<const uint8_t *>(a[i].qw); p.scales = a[i].scales; p.zeros = a[i].zeros; p.y = a[i].y;
-        p.t = reinterpret_cast<uint2 *>(ws.split) + words;
+        p.t = reinterpret_cast<unsigned long long *>(ws.split) + words;
         words += t_words(a[i]);
     }
     const bool pdl = tune.pdl != 0;

@@ -279,7 +279,9 @@ int fbq_split_plan(int M, int N, int K, int group, int bits, int rank, int act_i
  *   "gemv"          1 (default) = M <= 16 runs the streaming kernels where their domain allows (see fbq_linear),
  *                   0 = the other decode kernel at every M
  *   "gemv_ctas"     0 = automatic (one or two CTAs per SM), else an upper bound on the grid of the streaming kernels
- *                   (fbq_set_stream_option sets it for one stream)
+ *                   (fbq_set_stream_option sets it for one stream).  A call of 3 to 16 tokens takes several launches where its
+ *                   rows need more CTAs than that; the least grid is one cluster for the rows and one or two for t = x.A^T, of as
+ *                   many CTAs each (1, 2, 4, 8) as hold x of all tokens
  *   "t_poll_limit"  0 = default, else the number of looks the streaming kernels take at the t CTAs' words
  *                   before it gives up with FBQ_ERR_TIMEOUT
  *   "test_skip_t_arrive", "test_prefill_skip_flag", "prefill_flag_polls"

@@ -810,9 +810,10 @@ __global__ void __launch_bounds__(kThr, 1) split_kernel(const __grid_constant__ 
 
 // ---- host ----------------------------------------------------------------------------------------------------------
 struct Shape {
-    SplitParams sp;
+    SplitParams sp{};
     size_t smem = 0;
     int clusters = 0;
+    int launches = 1;                        // (several for one problem under a bound: each has `clusters` but the last)
     bool ok = false;
 };
 
@@ -884,13 +885,64 @@ bool fill_problem(const LinearArgs &a, SplitDims &p, int cs_log2, int wk_log2, s
     return true;
 }
 
+// Time of a main cluster with q.R tiles (microseconds), 2^w parts of a slice of Gs groups.
+double tiles_time(const SplitDims &q, int M, int Gs, int c, int w)
+{
+    const int MT = (M + 7) / 8, rounds = (q.R + (kW >> w) - 1) / (kW >> w), mine = (Gs + (1 << w) - 1) >> w;
+    const bool whole = q.stages * q.sg >= rounds * mine;
+    const double units = std::max(q.R * Gs * (0.05 + 0.035 * (MT - 1)), rounds * mine * (0.42 + 0.03 * (MT - 1)));
+    const double stream = q.R * Gs * 2.048 / (whole ? 44.0 : std::min(44.0, kW * q.stages * q.sg * 2.048 / 1.3));
+    return units + 0.3 * stream + 0.004 * Gs * M + 0.02 * (1 << (w + c)) + 0.01 * rounds * mine + (q.PT < q.R ? 0.5 : 0.0);
+}
+
+// One problem under a bound on the CTAs of a grid, those of t among them.  t may take as few clusters as hold it; tiles that a cluster's
+// tables do not hold are left to further launches.  The bound goes before the time; a cluster for t and one for the tiles there have
+// to be, of as many CTAs as hold x.
+Shape make_bounded_shape(const LinearArgs &a, int max_ctas)
+{
+    Shape best;
+    double best_cost = 1e30;
+    int best_excess = 1 << 30;
+    const int MT = (a.M + 7) / 8, G = a.K / kGroupFast, tiles = (a.N + kRows - 1) / kRows;
+    for (int c = 0; c <= (MT == 1 && !best.ok ? 4 : 3) && (1 << c) <= G; ++c)
+        for (int ngt = 1;; ngt *= 2) {
+            const int n_tc = (a.rank + 16 * ngt - 1) / (16 * ngt), room = std::max(1, (max_ctas >> c) - n_tc), Gs = (G + (1 << c) - 1) >> c;
+            const int excess = std::max(0, ((n_tc + room) << c) - max_ctas);
+            bool fits = false;
+            for (int R = (tiles + room - 1) / room; R >= 1 && !fits; R = R > 1 ? (R + 1) / 2 : 0)
+                for (int w = 3; w >= (c ? 1 : 2); --w) {
+                    SplitDims q{};
+                    q.N = a.N; q.K = a.K; q.G = G; q.rank = a.rank; q.tiles = tiles; q.R = R; q.ngt = ngt;
+                    size_t smem = 0;
+                    if (!fill_problem(a, q, c, w, &smem)) continue;
+                    fits = true;
+                    const int all = (tiles + R - 1) / R, launches = (all + room - 1) / room;
+                    const double t_time = a.rank > 0 ? 0.4 * ((ngt + kTWR - 1) / kTWR) * ((Gs + kTWK - 1) / kTWK) : 0.0;
+                    const double cost = launches * (std::max(tiles_time(q, a.M, Gs, c, w), t_time) + 0.3 * c + 4.0);
+                    if (excess > best_excess || (excess == best_excess && cost >= best_cost)) continue;
+                    best_excess = excess;
+                    best_cost = cost;
+                    best.sp = SplitParams{};
+                    best.sp.n = 1; best.sp.M = a.M; best.sp.cs_log2 = c; best.sp.n_tc = n_tc;
+                    q.first_mc = best.sp.first_mc[0] = n_tc;
+                    best.sp.p[0] = q;
+                    best.smem = smem;
+                    best.launches = launches;
+                    best.clusters = n_tc + (all + launches - 1) / launches;
+                    best.ok = true;
+                }
+            if (16 * ngt >= a.rank) break;
+        }
+    return best;
+}
+
 // The plan of a launch.  What is weighed (microseconds; measured on 4096, 5120, 11008 and 13824 wide layers, INT4, 4 to 16
 // tokens): staging x of the slice; the groups of the CTA (the SM's pipes) or of its fullest warp (latency); the stream of codes,
 // which a ring of few stages cannot keep up (about 1.3 us from request to arrival); sums to add; clusters, which cost more the
 // larger they are (and one of four or eight CTAs leaves SMs unused).  4096 -> 11008, 16 tokens, clusters of two, 8, 4, 2 parts
 // of the slice: 17.0, 15.2, 14.7 us; 11008 -> 4096, clusters of two, 8 parts, or of four, 2 parts: 4 tokens 12.4, 13.3, 8 tokens
 // 13.5, 14.3; 4096 -> 4096, 16 tokens, CTAs of a cluster 1, 2, 4, 8: 9.4, 8.2, 8.8, 9.8.
-Shape make_shape(const LinearArgs *a, int count, int max_ctas)
+Shape make_shape(const LinearArgs *a, int count)
 {
     Shape best;
     double best_cost = 1e30;
@@ -904,8 +956,6 @@ Shape make_shape(const LinearArgs *a, int count, int max_ctas)
         s.sp.M = M;
         s.sp.cs_log2 = c;
         int n_tc = 0, n_tcs[kMostProblems];
-        int room = resident_clusters(c);
-        if (max_ctas > 0) room = std::min(room, std::max(1, max_ctas >> c));
         for (int i = 0; i < count; ++i) {
             SplitDims &p = s.sp.p[i];
             p.N = a[i].N; p.K = a[i].K; p.G = a[i].K / kGroupFast; p.rank = a[i].rank;
@@ -915,7 +965,7 @@ Shape make_shape(const LinearArgs *a, int count, int max_ctas)
             n_tc += n_tcs[i];
         }
         // tiles per cluster: the least load of the fullest CTA that lets all main clusters be resident
-        const int main_room = std::max(count, max_ctas > 0 ? room : room - n_tc);
+        const int main_room = std::max(count, resident_clusters(c) - n_tc);
         auto slice = [&](int i) { return (s.sp.p[i].G + (1 << c) - 1) >> c; };
         auto tiles_for = [&](int i, int load) { return std::max(1, load / slice(i)); };
         auto total = [&](int load) {
@@ -947,11 +997,7 @@ Shape make_shape(const LinearArgs *a, int count, int max_ctas)
                     q.R = R;
                     size_t sm = 0;
                     if (!fill_problem(a[i], q, c, w, &sm)) continue;
-                    const int rounds = (R + (kW >> w) - 1) / (kW >> w), mine = (Gs + (1 << w) - 1) >> w, waves = (most + R - 1) / R;
-                    const bool whole = q.stages * q.sg >= rounds * mine;
-                    const double units = std::max(R * Gs * (0.05 + 0.035 * (MT - 1)), rounds * mine * (0.42 + 0.03 * (MT - 1)));
-                    const double stream = R * Gs * 2.048 / (whole ? 44.0 : std::min(44.0, kW * q.stages * q.sg * 2.048 / 1.3));
-                    const double ti = waves * (units + 0.3 * stream + 0.004 * Gs * M + 0.02 * (1 << (w + c)) + 0.01 * rounds * mine + (q.PT < q.R ? 0.5 : 0.0));
+                    const double ti = ((most + R - 1) / R) * tiles_time(q, M, Gs, c, w);
                     if (ti < t) {
                         t = ti;
                         pick = q;
@@ -994,7 +1040,7 @@ struct PlanHash {
         return (size_t)h;
     }
 };
-const Shape &shape_for(const LinearArgs *a, int count, int max_ctas)
+const Shape &shape_for(const LinearArgs *a, int count, int max_ctas)          // (one problem where there is a bound)
 {
     static thread_local std::unordered_map<PlanKey, Shape, PlanHash> plans;
     PlanKey k{};
@@ -1007,7 +1053,7 @@ const Shape &shape_for(const LinearArgs *a, int count, int max_ctas)
     const auto it = plans.find(k);
     if (it != plans.end()) return it->second;
     if (plans.size() >= 256) plans.clear();
-    return plans.emplace(k, make_shape(a, count, max_ctas)).first->second;
+    return plans.emplace(k, max_ctas > 0 ? make_bounded_shape(a[0], max_ctas) : make_shape(a, count)).first->second;
 }
 
 template <int BITS, typename T, int MT> cudaError_t launch_one(const Shape &s, bool pdl, cudaStream_t st)
@@ -1059,7 +1105,7 @@ bool split_supported(const LinearArgs &a)
 
 bool split_plan_exists(const LinearArgs *a, int count, const GemvTuning &tune)
 {
-    return count >= 1 && count <= kMostProblems && shape_for(a, count, tune.max_ctas).ok;
+    return count >= 1 && count <= kMostProblems && (count == 1 || tune.max_ctas == 0) && shape_for(a, count, tune.max_ctas).ok;
 }
 
 bool split_plan(const LinearArgs &a, const GemvTuning &tune, int *ctas, int *cluster)
@@ -1079,9 +1125,8 @@ size_t split_scratch_bytes(const LinearArgs *a, int count)
 
 cudaError_t launch_split(const LinearArgs *a, int count, Workspace &ws, const GemvTuning &tune, cudaStream_t st, int *launches)
 {
-    if (count < 1 || count > kMostProblems) return cudaErrorInvalidConfiguration;
+    if (!split_plan_exists(a, count, tune)) return cudaErrorInvalidConfiguration;
     Shape s = shape_for(a, count, tune.max_ctas);
-    if (!s.ok) return cudaErrorInvalidConfiguration;
     s.sp.poll_limit = tune.poll_limit;
     s.sp.skip_t = tune.test_skip_arrive;
     s.sp.status = ws.counters + kCtrStatus;
@@ -1095,10 +1140,18 @@ cudaError_t launch_split(const LinearArgs *a, int count, Workspace &ws, const Ge
         words += t_words(a[i]);
     }
     const bool pdl = tune.pdl != 0;
-    const cudaError_t e = a[0].bits == 4 ? (a[0].bf16 ? launch_mt<4, __nv_bfloat16>(s, pdl, st) : launch_mt<4, __half>(s, pdl, st))
-                                         : (a[0].bf16 ? launch_mt<3, __nv_bfloat16>(s, pdl, st) : launch_mt<3, __half>(s, pdl, st));
-    if (e == cudaSuccess) ++*launches;
-    return e;
+    const int main = s.clusters - s.sp.n_tc;                         // clusters of a launch
+    for (int l = 0; l < s.launches; ++l) {
+        if (l > 0) {                                                 // the tiles behind those of the launches before
+            s.sp.p[0].first_mc = s.sp.n_tc - l * main;
+            s.clusters = s.sp.n_tc + std::min(main, (s.sp.p[0].tiles + s.sp.p[0].R - 1) / s.sp.p[0].R - l * main);
+        }
+        const cudaError_t e = a[0].bits == 4 ? (a[0].bf16 ? launch_mt<4, __nv_bfloat16>(s, pdl, st) : launch_mt<4, __half>(s, pdl, st))
+                                             : (a[0].bf16 ? launch_mt<3, __nv_bfloat16>(s, pdl, st) : launch_mt<3, __half>(s, pdl, st));
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace fbq

@@ -1,5 +1,5 @@
 """The split kernel's count of launches, whose numbers the words of t carry: grids of more than 65536 CTAs, and
-counts at which a number of 32 bits, or of 31, comes round."""
+counts at which a number of 32 bits, or of 31, comes round; calls whose grid is bounded to less than holds their rows."""
 import pytest
 
 from gpu_utils import DeviceLinear, REL_F_TOL, check_parity
@@ -71,3 +71,26 @@ def test_number_comes_round(launches, M, N, K, rank, ctas):
     finally:
         fbq.set_option("gemv_ctas", 0)
     assert fbq.get_option("test_split_launches") == 0 and fbq.poll_status() == 0
+
+
+@pytest.mark.parametrize("bits,dtype,M,N,K,rank,ctas", [(4, "bf16", 8, 11008, 512, 128, 3), (3, "f16", 16, 4104, 1024, 64, 5), (4, "f16", 5, 90008, 128, 0, 1),
+                                                       (3, "bf16", 12, 2056, 5120, 32, 8)])
+def test_rows_in_several_launches(bits, dtype, M, N, K, rank, ctas):
+    import torch
+    import paper_2501_16385_b200 as fbq
+    inp = make_linear(M, N, K, bits, rank, dtype=dtype, seed=7900 + M + N)
+    assert fbq.split_plan(M, N, K, 128, bits, rank, dtype == "bf16", ctas)[0] <= ctas
+    dev = DeviceLinear(inp, fbq)
+    whole = dev.run(fbq)
+    fbq.set_option("gemv_ctas", ctas)
+    try:
+        before = fbq.launch_count()
+        ys = [dev.run(fbq) for _ in range(2)]
+        assert fbq.launch_count() - before > 2
+        torch.cuda.synchronize()
+    finally:
+        fbq.set_option("gemv_ctas", 0)
+    assert fbq.poll_status() == 0 and torch.equal(*ys)
+    # fp32 sums in another order, one rounding each
+    d = (ys[0].double() - whole.double()).norm(dim=0) / whole.double().norm(dim=0)
+    assert float(d.max()) < (2.0 ** -7 if dtype == "bf16" else 2.0 ** -10)

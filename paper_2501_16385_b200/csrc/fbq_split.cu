@@ -906,7 +906,7 @@ Shape make_bounded_shape(const LinearArgs &a, int max_ctas)
     const int MT = (a.M + 7) / 8, G = a.K / kGroupFast, tiles = (a.N + kRows - 1) / kRows;
     for (int c = 0; c <= (MT == 1 && !best.ok ? 4 : 3) && (1 << c) <= G; ++c)
         for (int ngt = 1;; ngt *= 2) {
-            const int n_tc = (a.rank + 16 * ngt - 1) / (16 * ngt), room = std::max(1, (max_ctas >> c) - n_tc), Gs = (G + (1 << c) - 1) >> c;
+            const int n_tc = (a.rank + 16 * ngt - 1) / (16 * ngt), room = std::max(1, std::min(max_ctas >> c, resident_clusters(c)) - n_tc), Gs = (G + (1 << c) - 1) >> c;
             const int excess = std::max(0, ((n_tc + room) << c) - max_ctas);
             bool fits = false;
             for (int R = (tiles + room - 1) / room; R >= 1 && !fits; R = R > 1 ? (R + 1) / 2 : 0)

@@ -152,8 +152,12 @@ int select_kernel(int M, int N, int K, int group, int bits, int rank, bool bf16)
     // head of its grid and wins at every rank up to 128; at M = 5 and 6 every CTA contributes to t and the tiles
     // wait for it, work that grows with M * rank, so M * rank above 128 goes to the tensor-core kernel.
     const bool streaming = g_opt.use_gemv != 0 && decode_ok && gemv_supported(a);
-    const bool decode_pays = streaming ? (M <= 8 || gemv_k_slices(M, K) == 1)
-                                       : (M <= kDecodePreferM && (M <= 4 ? rank <= 128 : M * rank <= 128));
+    bool decode_pays = streaming ? (M <= 8 || gemv_k_slices(M, K) == 1)
+                                 : (M <= kDecodePreferM && (M <= 4 ? rank <= 128 : M * rank <= 128));
+    // x of a K this deep (100480 with a sub-branch, 131200 without) is beyond the split kernel's clusters, and what is left of the decode
+    // kernels takes it in turns: 100480 -> 1024, INT4, us, other decode / tensor-core kernel: 3 tokens rank 16 69 / 79, rank 64 93 / 78;
+    // 4 tokens rank 16 85 / 79; 8 tokens rank 16 532 / 79, rank 128 982 / 79.
+    if (streaming && M > kGemvMaxM && K > kSplitAnyK && !split_plan_exists(&a, 1, GemvTuning{})) decode_pays = M == 3 && rank <= 16;
     if (decode_ok && (decode_pays || !prefill_ok)) return FBQ_KERNEL_DECODE;
     if (prefill_ok) return FBQ_KERNEL_PREFILL;
     return FBQ_KERNEL_GENERIC;

@@ -121,6 +121,7 @@ cudaError_t launch_gemv_batch(const LinearArgs *a, int count, Workspace &ws, con
 // The split kernel (fbq_split.cu): the same domain of widths and ranks, up to kSplitMaxM tokens, one problem or several in
 // one launch (cudaErrorInvalidConfiguration: no plan fits).  Scratch: Workspace::split, the status word of the counters.
 constexpr int kSplitMaxM = 16;
+constexpr int kSplitAnyK = 65536;     // up to eight tokens of this many inputs have a plan, with any N and rank
 bool split_supported(const LinearArgs &a);
 size_t split_scratch_bytes(const LinearArgs *a, int count);
 bool split_plan_exists(const LinearArgs *a, int count, const GemvTuning &tune);

@@ -116,3 +116,8 @@ def test_huge_and_non_finite_t(fbq):
     torch.cuda.synchronize()
     assert torch.all(y[0] == 0) and torch.all(y[2:] == 0) and not torch.any(torch.isfinite(y[1]))
     assert fbq.poll_status() == 0
+
+
+@pytest.mark.parametrize("M,K,rank", [(3, 100480, 16), (8, 100480, 64), (5, 131200, 0)])
+def test_just_past_the_deepest_layer(fbq, M, K, rank):
+    check_parity(make_linear(M, 40, K, 4, rank, seed=7700 + M), fbq, threads=16, floor=2e-5)

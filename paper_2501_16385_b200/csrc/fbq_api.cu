@@ -145,14 +145,15 @@ int select_kernel(int M, int N, int K, int group, int bits, int rank, bool bf16)
     if (g_opt.force_kernel == FBQ_KERNEL_DECODE && decode_ok) return FBQ_KERNEL_DECODE;
     if (g_opt.force_kernel == FBQ_KERNEL_PREFILL && prefill_ok) return FBQ_KERNEL_PREFILL;
     if (g_opt.force_kernel >= 0) return FBQ_KERNEL_GENERIC;
-    // In the streaming kernels' domain the decode class is one and two tokens (the streaming kernel) and as many as the split kernel
-    // is given by name: up to eight of any K, and up to sixteen while x of all K takes 136 KB.  A call of up to sixteen tokens that
-    // falls into the other class runs on the split kernel all the same (split_takes), so the line names a class, not a speed.
+    // In the streaming kernels' domain the decode class is up to eight tokens, and up to sixteen while x of all K (in whole stages of
+    // 1024, and 32 more) takes 136 KB.  A call of nine to sixteen tokens beyond that counts as a prompt, but the split kernel takes it
+    // all the same (split_takes).  The line is no crossover any more: callers of fbq_select_kernel know it, and in a batch it tells
+    // the problems of different x that run side by side from those that run one after another.
     // Outside that domain the other decode kernel keeps its own crossover: up to M = 4 it gets t from CTAs at the
     // head of its grid and wins at every rank up to 128; at M = 5 and 6 every CTA contributes to t and the tiles
     // wait for it, work that grows with M * rank, so M * rank above 128 goes to the tensor-core kernel.
     const bool streaming = g_opt.use_gemv != 0 && decode_ok && gemv_supported(a);
-    bool decode_pays = streaming ? (M <= 8 || gemv_k_slices(M, K) == 1)
+    bool decode_pays = streaming ? (M <= 8 || (size_t)M * ((K + 1023) / 1024 * 1024 + 32) * 2 <= 136 * 1024)
                                  : (M <= kDecodePreferM && (M <= 4 ? rank <= 128 : M * rank <= 128));
     // x of a K this deep (100480 with a sub-branch, 131200 without) is beyond the split kernel's clusters, and what is left of the decode
     // kernels takes it in turns: 100480 -> 1024, INT4, us, other decode / tensor-core kernel: 3 tokens rank 16 69 / 79, rank 64 93 / 78;
@@ -781,8 +782,8 @@ static int linear_batch_common(const fbq_problem *problems, int count, int M, in
     // Problems that read the same x (q, k and v; gate and up) share one launch of the streaming kernel, or of the split kernel, on
     // the caller's stream, and so do all problems of a call with host buffers, whose x arrive together.  (Seven linears of a 7B
     // layer, INT3, one token, pinned buffers, 51 us with the synchronisation: x over the bus 5 us, the launch of all seven 34, of which y over the bus is 3.5,
-    // and about 12 until the first kernel starts and after the last has ended.)  Above two tokens a problem of a single 16-row
-    // tile goes by itself.
+    // and about 12 until the first kernel starts and after the last has ended.)  Above two tokens a problem of 16 rows or less
+    // goes by itself, and the others with it, as it did when CTAs shared a tile in pairs: the split kernel could take it.
     if (g_opt.batch_single && count > 1 && count <= kGemvBatchMost) {
         bool together = true, one_x = true;
         for (int i = 0; i < count; ++i) {

@@ -41,6 +41,7 @@
 
 #include "fbq_common.cuh"
 #include "fbq_maps.h"
+#include "fbq_unpack16.cuh"
 
 #ifndef FBQ_NACC
 #define FBQ_NACC 2
@@ -192,13 +193,6 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-__device__ __forceinline__ uint32_t lop3_and_or(uint32_t a, uint32_t mask, uint32_t orv)
-{
-    uint32_t r;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(r) : "r"(a), "r"(mask), "r"(orv));   // (a & mask) | orv
-    return r;
-}
-
 template <typename T> struct Pk;   // packed-pair arithmetic on raw 32-bit registers
 template <> struct Pk<__half> {
     static __device__ __forceinline__ uint32_t sub(uint32_t a, uint32_t b)
@@ -261,113 +255,6 @@ template <> struct Pk<__nv_bfloat16> {
     }
 };
 
-// ------------------------------------------------------------------ unpackers
-// run(words, h) fills h[0..15] with one lane's 32 codes of one weight row as
-// packed 16-bit floats in "fragment order", using nothing but shifts and one
-// LOP3 per pair: a code field sitting at bit 3f (or 4e) of a 16-bit half is
-// OR-ed into the mantissa of MAGIC = 1024 (fp16) or 128 (bf16), which yields
-//        MAGIC + c*q      with c = 2^(field offset)  (kDiv below).
-//   INT4: h[4i+e]  = codes (8i+e , 8i+e+4)  of word i          (i = 0..3, e = 0..3)
-//   INT3: h[5i+f]  = codes (10i+f, 10i+5+f) of word i          (i = 0..2, f = 0..4)
-//         h[15]    = codes (30, 31)
-// No arithmetic is spent on removing MAGIC, c or the zero point per element:
-// x is stored in shared memory already divided by c (a power of two), so the
-// MMA yields  sum_k x_k*q_k + sum_k (MAGIC/c_k)*x_k ; the second sum and
-// sum_k x_k depend on the token and group only and are tabulated once per CTA
-// (P and X0), and the group's value is  s*(mma - P) - (s*z)*X0.
-template <int BITS, typename T> struct Unpack;
-
-template <> struct Unpack<4, __half> {
-    static constexpr int kWords = 4;
-    static constexpr float kMagic = 1024.f;
-    static __device__ __forceinline__ int div_log2(int c) { return ((c & 7) & 1) ? 4 : 0; }   // odd nibbles sit 4 bits up
-    static __device__ __forceinline__ void run(const uint32_t *w, uint32_t *h)
-    {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t a = w[i], b = w[i] >> 8;
-            h[4 * i + 0] = lop3_and_or(a, 0x000F000Fu, 0x64006400u);
-            h[4 * i + 1] = lop3_and_or(a, 0x00F000F0u, 0x64006400u);
-            h[4 * i + 2] = lop3_and_or(b, 0x000F000Fu, 0x64006400u);
-            h[4 * i + 3] = lop3_and_or(b, 0x00F000F0u, 0x64006400u);
-        }
-    }
-};
-template <> struct Unpack<4, __nv_bfloat16> {
-    static constexpr int kWords = 4;
-    static constexpr float kMagic = 128.f;                     // 0x4300 | q  is 128 + q in bf16 (7 mantissa bits)
-    static __device__ __forceinline__ int div_log2(int) { return 0; }
-    static __device__ __forceinline__ void run(const uint32_t *w, uint32_t *h)
-    {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) h[4 * i + e] = lop3_and_or(w[i] >> (4 * e), 0x000F000Fu, 0x43004300u);
-    }
-};
-template <> struct Unpack<3, __half> {
-    static constexpr int kWords = 3;
-    static constexpr float kMagic = 1024.f;
-    static __device__ __forceinline__ int div_log2(int c)
-    {
-        if (c >= 30) return 0;
-        const int f = (c % 10) % 5;                             // fields 0,3: bit 0; 1,4: bit 3; 2: bit 6 (3,4 after >> 9)
-        return (f == 2) ? 6 : ((f == 1 || f == 4) ? 3 : 0);
-    }
-    static __device__ __forceinline__ void run(const uint32_t *w, uint32_t *h)
-    {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const uint32_t a = w[i], b = w[i] >> 9;
-            h[5 * i + 0] = lop3_and_or(a, 0x00070007u, 0x64006400u);
-            h[5 * i + 1] = lop3_and_or(a, 0x00380038u, 0x64006400u);
-            h[5 * i + 2] = lop3_and_or(a, 0x01C001C0u, 0x64006400u);
-            h[5 * i + 3] = lop3_and_or(b, 0x00070007u, 0x64006400u);
-            h[5 * i + 4] = lop3_and_or(b, 0x00380038u, 0x64006400u);
-        }
-        uint32_t l = lop3_and_or(w[0] >> 15, 0x00010001u, 0x64006400u);
-        l = lop3_and_or(w[1] >> 14, 0x00020002u, l);
-        h[15] = lop3_and_or(w[2] >> 13, 0x00040004u, l);
-    }
-};
-template <> struct Unpack<3, __nv_bfloat16> {
-    static constexpr int kWords = 3;
-    static constexpr float kMagic = 128.f;
-    static __device__ __forceinline__ int div_log2(int c)
-    {
-        if (c >= 30) return 0;
-        const int f = (c % 10) % 5;                             // shifts 0, 6, 12: fields 0,2,4 at bit 0; 1,3 at bit 3
-        return (f == 1 || f == 3) ? 3 : 0;
-    }
-    static __device__ __forceinline__ void run(const uint32_t *w, uint32_t *h)
-    {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const uint32_t a = w[i], b = w[i] >> 6, c = w[i] >> 12;
-            h[5 * i + 0] = lop3_and_or(a, 0x00070007u, 0x43004300u);
-            h[5 * i + 1] = lop3_and_or(a, 0x00380038u, 0x43004300u);
-            h[5 * i + 2] = lop3_and_or(b, 0x00070007u, 0x43004300u);
-            h[5 * i + 3] = lop3_and_or(b, 0x00380038u, 0x43004300u);
-            h[5 * i + 4] = lop3_and_or(c, 0x00070007u, 0x43004300u);
-        }
-        uint32_t l = lop3_and_or(w[0] >> 15, 0x00010001u, 0x43004300u);
-        l = lop3_and_or(w[1] >> 14, 0x00020002u, l);
-        h[15] = lop3_and_or(w[2] >> 13, 0x00040004u, l);
-    }
-};
-
-// Position of code c (0..31) of a lane's 32-code run inside the fragment order
-// above: returns 2*h_index + (0 = low half, 1 = high half).
-template <int BITS> __device__ __forceinline__ int frag_pos(int c)
-{
-    if (BITS == 4) {
-        const int i = c >> 3, e8 = c & 7;
-        return 2 * (4 * i + (e8 & 3)) + (e8 >> 2);
-    }
-    if (c >= 30) return 2 * 15 + (c - 30);
-    const int i = c / 10, f = c - 10 * i;
-    return (f < 5) ? 2 * (5 * i + f) : 2 * (5 * i + f - 5) + 1;
-}
 // ------------------------------------------------- integer form (M <= 2)
 // A 3- or 4-bit code masked out of its word where it sits is already an unsigned
 // byte q * 2^j (j = the field's offset inside its byte): an operand of the 8-bit
@@ -680,7 +567,7 @@ __device__ __forceinline__ void decode_body(const DecodeParams &p, const CUtenso
     const int cta = cta_in_grid - p.n_t;
     extern __shared__ __align__(128) uint8_t smem[];
     constexpr int GB = (BITS == 4) ? 64 : 48;          // packed bytes of one group of one row
-    constexpr int NWORDS = Unpack<BITS, T>::kWords;    // words per lane per group
+    constexpr int NWORDS = BITS == 4 ? 4 : 3;    // words per lane per group
     // A stage in shared memory is [group][row][GB bytes], dense, as the tensor copy writes it: the
     // eight rows a warp reads at once are GB bytes apart, which spreads them over all banks (48 B:
     // 12 words, every lane of a 32-bit load in a bank of its own; 64 B: 128-bit loads, a quarter
@@ -1102,9 +989,9 @@ __device__ __forceinline__ void decode_body(const DecodeParams &p, const CUtenso
                     const float xf = ActTraits<T>::to_float(xe);
                     // exact division by the field weight (a power of two; up to fp16 underflow).
                     // P is summed from the stored value, so the MMA's bias term cancels exactly.
-                    const T xs = ActTraits<T>::from_float(ldexpf(xf, -Unpack<BITS, T>::div_log2(c)));
+                    const T xs = ActTraits<T>::from_float(ldexpf(xf, -Unpack16<BITS, T>::div_log2(c)));
                     h[pos >> 1] |= (uint32_t)(*reinterpret_cast<const uint16_t *>(&xs)) << (16 * (pos & 1));
-                    psum = fmaf(Unpack<BITS, T>::kMagic, ActTraits<T>::to_float(xs), psum);
+                    psum = fmaf(Unpack16<BITS, T>::kMagic, ActTraits<T>::to_float(xs), psum);
                     xsum += xf;
                 }
                 if (valid) {
@@ -1255,8 +1142,8 @@ __device__ __forceinline__ void decode_body(const DecodeParams &p, const CUtenso
                         }
                     }
                     uint32_t ha[16], hb[16];
-                    Unpack<BITS, T>::run(wa, ha);
-                    Unpack<BITS, T>::run(wb, hb);
+                    Unpack16<BITS, T>::run(wa, ha);
+                    Unpack16<BITS, T>::run(wb, hb);
 
 #pragma unroll
                     for (int b = 0; b < MT; ++b) {

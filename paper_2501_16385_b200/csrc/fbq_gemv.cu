@@ -1269,8 +1269,6 @@ Plan make_plan(const LinearArgs &a, const GemvTuning &tune)
     return make_plan_on(a, tune, 1);
 }
 
-// Slices of eight groups or more that x of all tokens has to be cut into to stay within 136 KB of shared memory.
-constexpr size_t kXLimit = 136 * 1024;
 // A plan is a function of the shape and the tuning alone and a call needs it twice (scratch, launch): the host thread
 // keeps the plans of the shapes it met last (a decoder has three or four).
 const Plan &plan_for(const LinearArgs &a, const GemvTuning &tune)
@@ -1321,16 +1319,6 @@ cudaError_t launch_variant(const Plan &pl, const CUtensorMap &wmap, const CUtens
 }
 
 }  // namespace
-
-int gemv_k_slices(int M, int K)
-{
-    if (M <= 2 || K < kGroupFast) return 1;
-    const int G = K / kGroupFast;
-    auto slice_of = [&](int k) { return ((G + k - 1) / k + kCW - 1) / kCW * kCW; };
-    int sk = 1;
-    while (sk < 16 && (size_t)M * ((size_t)slice_of(sk) * kGroupFast + 32) * 2 > kXLimit) sk *= 2;
-    return (G + slice_of(sk) - 1) / slice_of(sk);
-}
 
 bool gemv_supported(const LinearArgs &a)
 {

@@ -128,7 +128,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 __device__ __forceinline__ void prefetch_l2(const void *a) { asm volatile("prefetch.global.L2 [%0];" ::"l"(a)); }
 
 // Thread-block clusters: rank of this CTA, the shared::cluster address of a shared::cta address in another CTA of the
-// cluster, 16- and 8-byte stores there, and the cluster-wide barrier (every thread of every CTA arrives once per phase).
+// cluster, and the cluster-wide barrier (every thread of every CTA arrives once per phase).
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {
     uint32_t r;

@@ -1,4 +1,4 @@
-// Codes as packed 16-bit floats, shared by the kernels that multiply on warp-level 16-bit MMAs.
+// Codes as packed 16-bit floats, for the kernels that multiply on warp-level 16-bit MMAs (split kernel, 16-bit form of the decode kernel).
 #pragma once
 
 #include "fbq_common.cuh"
@@ -7,10 +7,10 @@ namespace fbq {
 
 // Codes become packed 16-bit floats with one LOP3 per pair ("bias-free" unpack): a field at bit p of a
 // 16-bit half, OR-ed into the mantissa of MAGIC = 1024 (fp16) or 128 (bf16), is MAGIC + 2^p q.  Nothing is
-// spent per element on removing MAGIC, 2^p or the zero point: x is staged divided by 2^p (exact) and
-// permuted into the order the unpacker produces, so the MMA yields sum x q + sum (MAGIC / 2^p) x; the second
-// sum (P) and sum x (X0) depend on token and group only and are tabulated when x is staged, and a group
-// contributes s (mma - P) - (s z) X0.
+// spent per element on removing MAGIC, 2^p or the zero point: x is staged divided by 2^p (in fp16 exact down to
+// 2^(p - 14); the split kernel scales it up against that) and permuted into the order the unpacker produces,
+// so the MMA yields sum x q + sum (MAGIC / 2^p) x; the second sum (P) and sum x (X0) depend on token and
+// group only and are tabulated when x is staged, and a group contributes s (mma - P) - (s z) X0.
 //   INT4: h[4i+e]  = codes (8i+e , 8i+e+4)  of word i          (i = 0..3, e = 0..3)
 //   INT3: h[5i+f]  = codes (10i+f, 10i+5+f) of word i          (i = 0..2, f = 0..4);  h[15] = codes (30, 31)
 __device__ __forceinline__ uint32_t lop3_and_or(uint32_t a, uint32_t mask, uint32_t orv)

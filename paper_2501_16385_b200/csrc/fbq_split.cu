@@ -92,6 +92,18 @@ template <typename T> __device__ __forceinline__ void mma16(float (&d)[4], uint3
             : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
             : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
+// The same, started at (c0, c1) in both rows.
+template <typename T> __device__ __forceinline__ void mma16_from(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1, float c0, float c1)
+{
+    if constexpr (std::is_same_v<T, __half>)
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%10,%11};"
+            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c0), "f"(c1));
+    else
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%10,%11};"
+            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c0), "f"(c1));
+}
 __device__ __forceinline__ void mma_tf32(float (&d)[4], const float (&a)[4], float b0, float b1)
 {
     asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -170,6 +182,9 @@ template <typename T> __device__ __forceinline__ uint32_t pair_of(float v)
 // a rounding of 2^-19 is nothing beside an x of 1000.  (13B layer, 16 tokens, fp16:
 // 101.5 us, 99.8 with x / 2^p and no second pass; with small x found by the sum of |x| instead, and staged again scaled up, 103.0.)
 template <int BITS> constexpr float kMid = BITS == 4 ? 6.f : 2.f;
+// Products start from -P all the same in bf16, whose 128 x cut off is lost in its rounding of y (1.7e-3), from nine tokens on: 16 tokens, rank 64,
+// 4096 -> 11008 15.26 -> 14.80 us, 11008 -> 4096 18.3 -> 17.8; with 8 tokens, rank 128, 13824 -> 5120 17.7 -> 18.3.
+template <typename T, int MT> constexpr bool kFromP = std::is_same_v<T, __nv_bfloat16> && MT == 2;
 template <int BITS, typename T> constexpr int kUp = std::is_same_v<T, __half> ? (BITS == 4 ? 4 : 6) : 0;      // (bf16 has the exponents)
 template <int BITS, typename T, int MT>
 __device__ __forceinline__ uint32_t stage_x(const T *x, int K, int M, bool wide, uint8_t *xs, float4 *px, int groups, int part, int parts, int lane, float up)
@@ -268,6 +283,7 @@ __device__ __forceinline__ void multiply_group(const uint8_t *codes, const uint8
         fs[r] = __half2float(*reinterpret_cast<const __half *>(sc + r * srow8));
         fz[r] = kMid<BITS> - __half2float(*reinterpret_cast<const __half *>(sc + r * srow8 + zoff));
     }
+    constexpr bool kFrom = kFromP<T, MT>;
     float d[2][MT][4] = {}, p[MT][2], x0[MT][2];
 #pragma unroll
     for (int q4 = 0; q4 < 4; ++q4)
@@ -282,7 +298,10 @@ __device__ __forceinline__ void multiply_group(const uint8_t *codes, const uint8
                 x0[b][1] = v.w;
             }
 #pragma unroll
-            for (int h = 0; h < 2; ++h) mma16<T>(d[h][b], ha[h][4 * q4], hb[h][4 * q4], ha[h][4 * q4 + 1], hb[h][4 * q4 + 1], xv.x, xv.y);
+            for (int h = 0; h < 2; ++h) {
+                if (kFrom && q4 == 0) mma16_from<T>(d[h][b], ha[h][4 * q4], hb[h][4 * q4], ha[h][4 * q4 + 1], hb[h][4 * q4 + 1], xv.x, xv.y, -p[b][0], -p[b][1]);
+                else mma16<T>(d[h][b], ha[h][4 * q4], hb[h][4 * q4], ha[h][4 * q4 + 1], hb[h][4 * q4 + 1], xv.x, xv.y);
+            }
 #pragma unroll
             for (int h = 0; h < 2; ++h) mma16<T>(d[h][b], ha[h][4 * q4 + 2], hb[h][4 * q4 + 2], ha[h][4 * q4 + 3], hb[h][4 * q4 + 3], xv.z, xv.w);
         }
@@ -294,7 +313,7 @@ __device__ __forceinline__ void multiply_group(const uint8_t *codes, const uint8
             for (int b = 0; b < MT; ++b)
 #pragma unroll
                 for (int c = 0; c < 2; ++c)
-                    acc[h][b][2 * r + c] = fmaf(fs[2 * h + r], fmaf(fz[2 * h + r], x0[b][c], d[h][b][2 * r + c] - p[b][c]), acc[h][b][2 * r + c]);
+                    acc[h][b][2 * r + c] = fmaf(fs[2 * h + r], fmaf(fz[2 * h + r], x0[b][c], kFrom ? d[h][b][2 * r + c] : d[h][b][2 * r + c] - p[b][c]), acc[h][b][2 * r + c]);
         }
 }
 

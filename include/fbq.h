@@ -57,8 +57,8 @@ typedef enum {
 typedef enum {
     FBQ_KERNEL_NONE = -1,
     FBQ_KERNEL_GENERIC = 0,   /* any supported shape, CUDA cores, two launches if rank>0 */
-    FBQ_KERNEL_DECODE = 1,    /* M <= 16 (chosen for M <= 8, and to 16 while M * K * 2 <= 136 KB): fused streaming kernels, one launch */
-    FBQ_KERNEL_PREFILL = 2    /* tcgen05 / TMEM tensor-core kernel, one launch (chosen from M = 9, or 7 outside the streaming kernel's domain) */
+    FBQ_KERNEL_DECODE = 1,    /* M <= 16 (named for M <= 8, and to 16 while M * K * 2 <= 136 KB): fused decode kernels, one launch */
+    FBQ_KERNEL_PREFILL = 2    /* tcgen05 / TMEM tensor-core kernel, one launch (named from M = 9, or 5 outside the streaming kernels' domain) */
 } fbq_kernel;
 
 /* Number of uint32 words of a packed N x K code matrix: N*K/8 (4 bits) or
@@ -85,12 +85,13 @@ int fbq_dequant(const uint32_t *qweight, const uint16_t *scales, const uint16_t 
 /* The fused layer, fp16 activations: x, A, B, y are fp16; scales, zeros fp16.
  *   rank == 0: A and B are ignored (may be NULL); y is the main path alone.
  *   M == 0: nothing is done.
- * Dispatch (fbq_select_kernel tells which kernel a shape gets): group == 128 and rank a multiple of 8
+ * Dispatch (fbq_select_kernel names the class, fbq_split_plan says where the split kernel runs): group == 128 and rank a multiple of 8
  * not above 256 are the fast kernels' domain.  The streaming kernels ("gemv" option, default on)
  * need N a multiple of 8, rank a multiple of 16 up to 128 and, at M <= 2, 16-byte aligned scales and zeros; there
- * the decode class is M <= 8 for every shape, and M <= 16 while M * K * 2 bytes stay within 136 KB.  One
+ * the decode class is M <= 8, and M <= 16 while M * K * 2 bytes stay within 136 KB.  One
  * kernel of it takes M <= 2, the split kernel (K cut over the CTAs of a cluster) 3 <= M <= 16, also where that
- * rule says prefill, unless a kernel is forced.  Elsewhere the other decode kernel
+ * rule says prefill, unless a kernel is forced, up to K = 24576 at M >= 9 (32768 at rank 0) and to 100352 (131072) at M <= 8;
+ * deeper layers of M <= 8 are prefill too, but for M = 3 with rank <= 16.  Elsewhere the other decode kernel
  * takes M <= 4 with rank <= 128 and M = 5, 6 with M * rank <= 128.  The prefill kernel (N a multiple of
  * 8) takes the rest of the domain; shapes outside its domain stay with a decode kernel up to M = 16;
  * everything else that is well formed -> generic kernel.
@@ -100,10 +101,14 @@ int fbq_dequant(const uint32_t *qweight, const uint16_t *scales, const uint16_t 
  * produces for groups that do not straddle zero); the decode and generic kernels any fp16 value.
  * Accumulation is fp32; t = x.A^T stays fp32 in the decode and
  * generic kernels (where a decode kernel multiplies it with B on tensor cores it enters as
- * two 16-bit terms, the rounded value and the remainder) and is rounded once to the activation
+ * two 16-bit terms, the rounded value and the remainder, two TF32 terms in the split kernel) and is rounded once to the activation
  * type in the prefill kernel (which also rounds the dequantised weights s*(q-z) once to that
  * type).  At M <= 2 the decode kernels read x in fixed point per group of 128, exact to 2^-17
- * of the group's largest element; a group that holds an Inf or a NaN makes its token's outputs NaN.
+ * of the group's largest element; a group that holds an Inf or a NaN makes its token's outputs NaN.  The
+ * split kernel reads x exactly (fp16 beside an |x| of 1024 and more, INT4 4096, of the same token: to 2^-19), and
+ * an Inf or a NaN goes into the outputs as in the sum of products.  The other decode kernel's 16-bit form
+ * (M >= 3) divides x by up to 16 (INT4) or 64 (INT3) in the activation type, which rounds fp16 below 2^-10 (2^-8), and
+ * makes an Inf NaN.
  * Summation order is fixed for a given shape and grid size (results are
  * reproducible run to run), except for t in the other decode kernel at M >= 3, which is
  * accumulated with floating-point atomics.
@@ -264,12 +269,13 @@ int fbq_linear_batch_hostio(const fbq_problem *problems, int count, int M, int g
 int fbq_sub_branch_unfused(const void *x, const void *A, const void *B, void *y, int M, int N, int K,
                            int rank, int act_is_bf16, void *stream);
 
-/* Which kernel fbq_linear / fbq_linear_bf16 would run for this shape, or
- * FBQ_KERNEL_NONE when the shape is rejected.  Pure host logic. */
+/* Which class of kernels this shape belongs to for fbq_linear / fbq_linear_bf16 (see Dispatch there), or
+ * FBQ_KERNEL_NONE when the shape is rejected.  Calls of 9 to 16 tokens named FBQ_KERNEL_PREFILL run on the split kernel
+ * where fbq_split_plan has a plan.  Pure host logic. */
 int fbq_select_kernel(int M, int N, int K, int group, int bits, int rank, int act_is_bf16);
 
-/* How the split kernel (3 to 16 tokens) would run this shape, as one problem: CTAs of its grid and of a cluster, under the bound
- * max_ctas (0: what "gemv_ctas" says).  FBQ_ERR_UNSUPPORTED where fbq_linear would not run that kernel.  Pure host logic, for
+/* How the split kernel (3 to 16 tokens) would run this shape, as one problem: CTAs of its (largest) grid and of a cluster, under the
+ * bound max_ctas (0: what "gemv_ctas" says).  FBQ_ERR_UNSUPPORTED where fbq_linear would not run that kernel.  Pure host logic, for
  * tests and tuning. */
 int fbq_split_plan(int M, int N, int K, int group, int bits, int rank, int act_is_bf16, int max_ctas, int *ctas, int *cluster);
 

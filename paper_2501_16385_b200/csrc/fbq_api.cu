@@ -236,7 +236,7 @@ int run_split(const LinearArgs *a, int count, const GemvTuning &gt, Workspace *w
 
 // Calls of 3 to 16 tokens in the streaming kernels' domain, also those that select_kernel counts among the prompts, unless a
 // kernel is forced.  Measured on B200, INT4, bf16, us per launch in a row, the kernels before it (a streaming one whose CTAs
-// staged x of all K, or the tensor-core one) / this one:
+// staged x of all K, or the tensor-core one) / this one, before small and infinite x were seen to (up to 2 % since, fp16 3 %):
 //                  4 tokens, rank 64  8 tokens, rank 128  16 tokens, rank 64
 //   4096 -> 4096        8.7 /  7.2        11.7 /  7.6       13.9 /  8.2
 //   4096 -> 11008      13.4 / 11.1        17.5 / 12.1       20.6 / 13.9

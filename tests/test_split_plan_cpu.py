@@ -26,5 +26,5 @@ def test_deep_layers_without_a_plan(M, rank):
     assert fbq.split_plan(M, 1024, deepest, 128, 4, rank) is not None
     assert fbq.select_kernel(M, 1024, deepest, 128, 4, rank) == fbq.KERNEL_DECODE
     assert fbq.split_plan(M, 1024, deepest + 128, 128, 4, rank) is None
-    # the other decode kernel only where it is ahead of the tensor cores there
+    # there the other decode kernel only where it is ahead of the tensor cores
     assert fbq.select_kernel(M, 1024, deepest + 128, 128, 4, rank) == (fbq.KERNEL_DECODE if M == 3 and rank <= 16 else fbq.KERNEL_PREFILL)
